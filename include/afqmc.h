@@ -47,7 +47,10 @@ typedef enum {
 enum { AFQMC_PHASELESS = 0, AFQMC_FREE = 1 };
 
 /* Arithmetic of the step.  Overlap ratios, phases and weights are float64 in every mode.
- *   AFQMC_FP64:   every contraction, the determinants and MGS in float64.
+ *   AFQMC_FP64:   every contraction, the determinants and MGS to float64 accuracy; the large
+ *                 contractions as error-free sums of BF16 digit products on the tensor cores
+ *                 (operands to 62 bits of their row's largest element, one rounding of the
+ *                 result), the rest on the FP64 pipe.
  *   AFQMC_BF16X3: every product over the Cholesky index or the orbital basis runs on the
  *                 tensor cores with split operands x = hi + lo (two bf16), three MMAs per
  *                 product (hi*hi + hi*lo + lo*hi) accumulated in FP32: the force bias

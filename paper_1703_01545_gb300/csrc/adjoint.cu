@@ -40,6 +40,16 @@ struct Arena {
     ptrs.push_back(p);
     return static_cast<T*>(p);
   }
+  // the same without failing the run: nullptr when there is no memory
+  uint8_t* try_get(size_t bytes) {
+    void* p = nullptr;
+    if (!ok || cudaMalloc(&p, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    ptrs.push_back(p);
+    return static_cast<uint8_t*>(p);
+  }
   ~Arena() {
     for (void* p : ptrs) cudaFree(p);
   }
@@ -160,6 +170,25 @@ afqmc_status adjoint_body(Ctx* h, Arena& ar, int n_steps, const double* fields, 
   double* h1bar = ar.get<double>(MM);
   if (!ar.ok) return fail(h, AFQMC_ERR_NOMEM, "cannot allocate the adjoint's checkpoints and scratch");
 
+  // scratch of the reverse pass's two large contractions in digit form (their K is M^2 and X);
+  // without the memory they run on the SIMT kernel
+  afq::F64Ws ws = c.ws64;
+  size_t need = 0;
+  if (afq::gemm_f64e_ok(X, 2 * Nw, MM)) need = afq::gemm_f64e_bytes(X, 2 * Nw, MM, (size_t)192 << 20);
+  if (afq::gemm_f64e_ok(NM, 2 * Nw, X))
+    need = std::max(need, afq::gemm_f64e_bytes(NM, 2 * Nw, X, (size_t)192 << 20));
+  if (need > ws.bytes) {
+    ADJ_CK(afq::prepare_gemm_f64e());
+    uint8_t* p = ar.try_get(need);
+    int* err = ws.err ? ws.err : reinterpret_cast<int*>(ar.try_get(sizeof(int)));
+    if (p && err) {
+      if (!ws.err) ADJ_CK(cudaMemsetAsync(err, 0, sizeof(int), s));
+      ws.buf = p;
+      ws.bytes = need;
+      ws.err = err;
+    }
+  }
+
   ADJ_CK(afq::prepare_adjoint_kernels(c));
   ADJ_CK(afq::launch_transpose(c.Ltil, LtilT, X, NM, s));   // [NM][X]
   ADJ_CK(cudaMemsetAsync(phibar, 0, sizeof(double) * nphi, s));
@@ -219,19 +248,21 @@ afqmc_status adjoint_body(Ctx* h, Arena& ar, int n_steps, const double* fields, 
       ADJ_CK(afq::adj_logdet(c, phibar, Y1, rbar, 1.0, s));
       ADJ_CK(afq::adj_outer(c, phibar, c.phi2, still, part, Ebar, s));
       ADJ_CK(afq::gemm_tn_f64(M, cols, M, 1.0, c.expK, M, 0, phibar, M, 0, 0.0, pbA, M, 0, 1, s,
-                              afq::GEMM_ONEBODY));
+                              afq::GEMM_ONEBODY, &ws));
       ADJ_CK(afq::gemm_tn_f64(M, cols, M, 1.0, c.expK, M, 0, tp.phi, M, 0, 0.0, phi1, M, 0, 1, s,
-                              afq::GEMM_ONEBODY));
+                              afq::GEMM_ONEBODY, &ws));
       ADJ_CK(afq::adj_taylor(c, phi1, pbA, terms, Abar, c.phi2, still, s));
       ADJ_CK(afq::adj_outer(c, pbA, tp.phi, still, part, Ebar, s));
       ADJ_CK(afq::gemm_tn_f64(M, cols, M, 1.0, c.expK, M, 0, pbA, M, 0, 0.0, phibar, M, 0, 1, s,
-                              afq::GEMM_ONEBODY));
+                              afq::GEMM_ONEBODY, &ws));
       // S[(p,w)][g] = sum_ij L_g,ij Abar[(p,w)][ij]
-      ADJ_CK(afq::gemm_tn_f64(X, 2 * Nw, MM, 1.0, c.L, MM, 0, Abar, MM, 0, 0.0, S, X, 0, 1, s));
+      ADJ_CK(afq::gemm_tn_f64(X, 2 * Nw, MM, 1.0, c.L, MM, 0, Abar, MM, 0, 0.0, S, X, 0, 1, s,
+                              afq::GEMM_GENERIC, &ws));
       ADJ_CK(afq::set_step(c, t0 + t, s));
       ADJ_CK(afq::adj_fields(c, field_t(t), S, rbar, lwbar, rbb, still, s));
       // Thetabar[(p,w)][(n,i)] = sum_g rhobarbar[(p,w)][g] Ltil[g][(n,i)]
-      ADJ_CK(afq::gemm_tn_f64(NM, 2 * Nw, X, 1.0, LtilT, X, 0, rbb, X, 0, 0.0, thb, NM, 0, 1, s));
+      ADJ_CK(afq::gemm_tn_f64(NM, 2 * Nw, X, 1.0, LtilT, X, 0, rbb, X, 0, 0.0, thb, NM, 0, 1, s,
+                              afq::GEMM_GENERIC, &ws));
       ADJ_CK(afq::adj_inv_overlap(c, tp.phi, Y2, logO_tmp, nullptr, still, s));
       ADJ_CK(afq::adj_overlap(c, tp.phi, Y2, thb, phibar, still, s));
       ADJ_CK(afq::adj_logdet(c, phibar, Y2, rbar, -1.0, s));
@@ -248,7 +279,10 @@ afqmc_status adjoint_body(Ctx* h, Arena& ar, int n_steps, const double* fields, 
   double E = 0;
   ADJ_CK(cudaMemcpyAsync(&E, e_acc, sizeof(double), cudaMemcpyDeviceToHost, s));
   if (dE_dh1) ADJ_CK(cudaMemcpyAsync(dE_dh1, h1bar, sizeof(double) * MM, cudaMemcpyDefault, s));
+  int expired = 0;
+  if (ws.err) ADJ_CK(cudaMemcpyAsync(&expired, ws.err, sizeof(int), cudaMemcpyDeviceToHost, s));
   ADJ_CK(cudaStreamSynchronize(s));
+  if (expired) return fail(h, AFQMC_ERR_TIMEOUT, "a tensor-core kernel's bounded wait expired");
   if (e_mixed) *e_mixed = E;
   if (!std::isfinite(E)) return fail(h, AFQMC_ERR_NUMERIC, "no live walker at a measurement");
   return AFQMC_OK;

@@ -83,6 +83,7 @@ void free_ctx(Ctx* h) {
                    h->rhobar32, h->rho_mf32})
     if (b) cudaFree(b);
   if (h->d_tc_err) cudaFree(h->d_tc_err);
+  if (h->ws64.buf) cudaFree(h->ws64.buf);
   for (double* b : {h->md_coef, h->md_psi, h->md_Ltil, h->md_htil, h->md_logO, h->md_theta,
                     h->md_share, h->md_rhobar, h->md_eloc})
     if (b) cudaFree(b);
@@ -293,28 +294,28 @@ afqmc_status step_launch_tangent(Ctx* h, const double* fields_t, cudaStream_t s)
   const int M = h->M, X = h->X, N = h->N, Nw = h->Nw;
   const int64_t NM = (int64_t)N * M;
   AFQ_CK(afq::gemm_tn_f64(X, 2 * Nw, (int)NM, 1.0, h->Ltil, NM, 0, h->theta, NM, 0, 0.0,
-                          h->rhobar, X, 0, 1, s, afq::GEMM_FORCE_BIAS));
+                          h->rhobar, X, 0, 1, s, afq::GEMM_FORCE_BIAS, &h->ws64));
   AFQ_CK(afq::gemm_tn_f64(X, 2 * Nw, (int)NM, 1.0, h->Ltil, NM, 0, h->dtheta, NM, 0, 0.0,
-                          h->drhobar, X, 0, 1, s, afq::GEMM_FORCE_BIAS));
+                          h->drhobar, X, 0, 1, s, afq::GEMM_FORCE_BIAS, &h->ws64));
   AFQ_CK(afq::launch_fields_tan(*h, fields_t, s));
   AFQ_CK(afq::gemm_tn_f64((int)h->P, 2 * Nw, X, 1.0, h->Lt, X, 0, h->U, X, 0, 0.0, h->Avhs,
-                          h->P, 0, 1, s, afq::GEMM_VHS));
+                          h->P, 0, 1, s, afq::GEMM_VHS, &h->ws64));
   AFQ_CK(afq::gemm_tn_f64((int)h->P, 2 * Nw, X, 1.0, h->Lt, X, 0, h->dU, X, 0, 0.0, h->dAvhs,
-                          h->P, 0, 1, s, afq::GEMM_VHS));
+                          h->P, 0, 1, s, afq::GEMM_VHS, &h->ws64));
   const int cols = 2 * Nw * N;
   AFQ_CK(afq::gemm_tn_f64(M, cols, M, 1.0, h->expK, M, 0, h->phi, M, 0, 0.0, h->phi2, M, 0, 1, s,
-                          afq::GEMM_ONEBODY));
+                          afq::GEMM_ONEBODY, &h->ws64));
   AFQ_CK(afq::gemm_tn_f64(M, cols, M, 1.0, h->dexpK, M, 0, h->phi, M, 0, 0.0, h->dphi2, M, 0, 1, s,
-                          afq::GEMM_ONEBODY));
+                          afq::GEMM_ONEBODY, &h->ws64));
   AFQ_CK(afq::gemm_tn_f64(M, cols, M, 1.0, h->expK, M, 0, h->dphi, M, 0, 1.0, h->dphi2, M, 0, 1, s,
-                          afq::GEMM_ONEBODY));
+                          afq::GEMM_ONEBODY, &h->ws64));
   AFQ_CK(afq::launch_taylor_tan(*h, s));
   AFQ_CK(afq::gemm_tn_f64(M, cols, M, 1.0, h->expK, M, 0, h->phi2, M, 0, 0.0, h->theta, M, 0, 1, s,
-                          afq::GEMM_ONEBODY));
+                          afq::GEMM_ONEBODY, &h->ws64));
   AFQ_CK(afq::gemm_tn_f64(M, cols, M, 1.0, h->dexpK, M, 0, h->phi2, M, 0, 0.0, h->dtheta, M, 0, 1, s,
-                          afq::GEMM_ONEBODY));
+                          afq::GEMM_ONEBODY, &h->ws64));
   AFQ_CK(afq::gemm_tn_f64(M, cols, M, 1.0, h->expK, M, 0, h->dphi2, M, 0, 1.0, h->dtheta, M, 0, 1, s,
-                          afq::GEMM_ONEBODY));
+                          afq::GEMM_ONEBODY, &h->ws64));
   AFQ_CK(afq::launch_overlap_tan(*h, afq::OV_UPDATE, s));
   AFQ_CK(afq::launch_step_advance(*h, s));
   return AFQMC_OK;
@@ -333,19 +334,19 @@ afqmc_status step_launch(Ctx* h, const double* fields_t, cudaStream_t s) {
       AFQ_CK(afq::md_force_bias(*h, s));
     } else {
       AFQ_CK(afq::gemm_tn_f64(X, 2 * Nw, (int)NM, 1.0, h->Ltil, NM, 0, h->theta, NM, 0, 0.0,
-                              h->rhobar, X, 0, 1, s, afq::GEMM_FORCE_BIAS));
+                              h->rhobar, X, 0, 1, s, afq::GEMM_FORCE_BIAS, &h->ws64));
     }
   }
   AFQ_CK(afq::launch_fields(*h, fields_t, s));
   // packed A[(p,w)][ij] = sum_g Lt[ij][g] U[(p,w)][g]                         (Eq. 11)
   AFQ_CK(afq::gemm_tn_f64((int)h->P, 2 * Nw, X, 1.0, h->Lt, X, 0, h->U, X, 0, 0.0, h->Avhs,
-                          h->P, 0, 1, s, afq::GEMM_VHS));
+                          h->P, 0, 1, s, afq::GEMM_VHS, &h->ws64));
   // e^{-dt K/2} on every column of every walker
   AFQ_CK(afq::gemm_tn_f64(M, 2 * Nw * N, M, 1.0, h->expK, M, 0, h->phi, M, 0, 0.0, h->phi2, M,
-                          0, 1, s, afq::GEMM_ONEBODY));
+                          0, 1, s, afq::GEMM_ONEBODY, &h->ws64));
   AFQ_CK(afq::launch_taylor(*h, h->phi2, s));
   AFQ_CK(afq::gemm_tn_f64(M, 2 * Nw * N, M, 1.0, h->expK, M, 0, h->phi2, M, 0, 0.0, h->theta,
-                          M, 0, 1, s, afq::GEMM_ONEBODY));
+                          M, 0, 1, s, afq::GEMM_ONEBODY, &h->ws64));
   // new overlaps, Theta, ratio, phase, weight; live walkers take the new determinant
   afqmc_status os = overlap_launch(h, h->theta, afq::OV_UPDATE, s);
   if (os != AFQMC_OK) return os;
@@ -533,6 +534,28 @@ afqmc_status afqmc_setup(afqmc_handle* out, const double* h1_in, const double* L
   } while (0)
 
   AFQ_SCK(afq::prepare_kernels(*h));
+  if (opt->precision == AFQMC_FP64) {
+    // digits of the step's contractions: as much as they can use, the walkers' operands in
+    // chunks of 192 MB (a chunk and its products then stay in L2); without the memory the
+    // contractions run on the SIMT kernel
+    size_t need = 0;
+    const int64_t gemms[3][3] = {{h->P, 2 * Nw, X}, {X, 2 * Nw, NM}, {M, 2 * Nw * N, M}};
+    for (const auto& g : gemms)
+      if (g[1] < (int64_t)1 << 31 && afq::gemm_f64e_ok((int)g[0], (int)g[1], (int)g[2]))
+        need = std::max(need, afq::gemm_f64e_bytes(g[0], g[1], (int)g[2], (size_t)192 << 20));
+    if (need > 0) {
+      AFQ_SCK(afq::prepare_gemm_f64e());
+      int* err = nullptr;
+      if (cudaMalloc(&err, sizeof(int)) == cudaSuccess) {
+        h->d_tc_err = err;
+        h->ws64.err = err;
+        AFQ_SCK(cudaMemsetAsync(err, 0, sizeof(int), s));
+        if (cudaMalloc(&h->ws64.buf, need) == cudaSuccess) h->ws64.bytes = need;
+        else h->ws64.buf = nullptr;
+      }
+      cudaGetLastError();
+    }
+  }
   AFQ_SCK(cudaMemcpyAsync(h->h1, h1_in, sizeof(double) * M * M, cudaMemcpyDefault, s));
   AFQ_SCK(cudaMemcpyAsync(h->L, L_in, sizeof(double) * X * M * M, cudaMemcpyDefault, s));
   AFQ_SCK(cudaMemcpyAsync(tmp, trial_in, sizeof(double) * NM, cudaMemcpyDefault, s));
@@ -884,14 +907,14 @@ afqmc_status afqmc_time_kernel(afqmc_handle h, int which, int reps, double* ms, 
       case AFQMC_K_VHS:   // split precision: in the form the propagation variant reads
         if (h->tc_L) return afq::vhs_launch(*h, afq::propagation_variant(*h), s);
         return afq::gemm_tn_f64((int)h->P, 2 * Nw, X, 1.0, h->Lt, X, 0, h->U, X, 0, 0.0, h->Avhs,
-                                h->P, 0, 1, s, afq::GEMM_VHS);
+                                h->P, 0, 1, s, afq::GEMM_VHS, &h->ws64);
       case AFQMC_K_FORCE_BIAS:
         if (h->n_det > 0) return afq::md_force_bias(*h, s);
         if (h->tc_Ltil)
           return afq::gemm_bf16x3(*h->tc_Ltil, *h->tc_Theta, X, 2 * Nw, 1.0f, h->rhobar32, X,
                                   h->d_tc_err, s);
         return afq::gemm_tn_f64(X, 2 * Nw, (int)NM, 1.0, h->Ltil, NM, 0, h->theta, NM, 0, 0.0,
-                                h->rhobar, X, 0, 1, s, afq::GEMM_FORCE_BIAS);
+                                h->rhobar, X, 0, 1, s, afq::GEMM_FORCE_BIAS, &h->ws64);
       case AFQMC_K_OVERLAP_UPDATE:   // Phi <- Phi (unchanged), Theta from the FP32 walkers
         return afq::launch_overlap_fast(*h, h->phi, afq::OV_UPDATE, s, h->phi32, false);
       case AFQMC_K_OVERLAP:
@@ -1149,10 +1172,11 @@ afqmc_status afqmc_test_gemm(int impl, int Md, int Nd, int K, const double* A, c
   float* fC = nullptr;
   __nv_bfloat16 *ah = nullptr, *al = nullptr, *bh = nullptr, *bl = nullptr;
   int* err = nullptr;
+  void* wbuf = nullptr;
   const int Kp = afq::pad64(K);
   auto cleanup = [&]() {
     for (void* p : {(void*)dA, (void*)dB, (void*)dC, (void*)fC, (void*)ah, (void*)al, (void*)bh,
-                    (void*)bl, (void*)err})
+                    (void*)bl, (void*)err, wbuf})
       if (p) cudaFree(p);
   };
   afqmc_status st = AFQMC_OK;
@@ -1166,7 +1190,19 @@ afqmc_status afqmc_test_gemm(int impl, int Md, int Nd, int K, const double* A, c
     if ((e = cudaMemcpyAsync(dA, A, sizeof(double) * Md * (size_t)K, cudaMemcpyDefault, s)) != cudaSuccess) break;
     if ((e = cudaMemcpyAsync(dB, B, sizeof(double) * Nd * (size_t)K, cudaMemcpyDefault, s)) != cudaSuccess) break;
     if (impl == 0) {
-      if ((e = afq::gemm_tn_f64(Md, Nd, K, alpha, dA, K, 0, dB, K, 0, 0.0, dC, Md, 0, 1, s)) != cudaSuccess) break;
+      afq::F64Ws ws;   // as on a handle: the digit form from gemm_f64e_ok on
+      if (afq::gemm_f64e_ok(Md, Nd, K)) {
+        ws.err = err;
+        ws.bytes = afq::gemm_f64e_bytes(Md, Nd, K, (size_t)192 << 20);
+        if ((e = afq::prepare_gemm_f64e()) != cudaSuccess) break;
+        if ((e = cudaMalloc(&wbuf, ws.bytes)) != cudaSuccess) break;
+        ws.buf = static_cast<uint8_t*>(wbuf);
+      }
+      if ((e = afq::gemm_tn_f64(Md, Nd, K, alpha, dA, K, 0, dB, K, 0, 0.0, dC, Md, 0, 1, s, afq::GEMM_GENERIC, &ws)) != cudaSuccess) break;
+      int herr = 0;
+      if ((e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess) break;
+      if ((e = cudaStreamSynchronize(s)) != cudaSuccess) break;
+      if (herr) { st = AFQMC_ERR_TIMEOUT; break; }
     } else {
       if ((e = afq::prepare_tc_kernels()) != cudaSuccess) break;
       const int Mp = afq::tc_pad_rows(Md), Np = afq::tc_pad_rows(Nd);

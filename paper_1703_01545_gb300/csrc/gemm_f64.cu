@@ -119,8 +119,14 @@ AFQ_GEMM_KERNEL(k_gemm_f64_onebody)
 cudaError_t gemm_tn_f64(int Md, int Nd, int Kd, double alpha, const double* A, int64_t lda,
                         int64_t sA, const double* B, int64_t ldb, int64_t sB, double beta,
                         double* C, int64_t ldc, int64_t sC, int batch, cudaStream_t s,
-                        GemmUse use) {
+                        GemmUse use, const F64Ws* ws) {
   if (Md <= 0 || Nd <= 0 || batch <= 0) return cudaSuccess;
+  if (ws && ws->buf && gemm_f64e_ok(Md, Nd, Kd)) {
+    cudaError_t e = cudaSuccess;
+    for (int z = 0; z < batch && e == cudaSuccess; ++z)
+      e = gemm_f64e(Md, Nd, Kd, alpha, A + z * sA, lda, B + z * sB, ldb, beta, C + z * sC, ldc, *ws, s);
+    if (e != cudaErrorMemoryAllocation) return e;   // else: the workspace is too small for this shape
+  }
   dim3 grid((Md + BM - 1) / BM, (Nd + BN - 1) / BN, batch);
   if (grid.y > 65535u || grid.z > 65535u) return cudaErrorInvalidConfiguration;
   auto k = use == GEMM_FORCE_BIAS ? k_gemm_f64_force_bias

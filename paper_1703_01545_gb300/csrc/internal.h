@@ -49,6 +49,14 @@ struct EnergyTc {
   int NP = 0, Kp = 0, RT = 0, NwP = 0;
 };
 
+// Scratch of the digit form of the FP64 contractions (gemm_f64e.cu); a null buf leaves them to
+// the SIMT kernel.  One handle's work runs on one stream at a time, so each handle has its own.
+struct F64Ws {
+  uint8_t* buf = nullptr;
+  size_t bytes = 0;
+  int* err = nullptr;         // set by an expired bounded wait
+};
+
 struct Ctx {
   int M = 0, X = 0, n_up = 0, n_dn = 0, N = 0, Nw = 0, R = 1;
   int64_t P = 0;              // packed size of a symmetric M x M matrix
@@ -109,6 +117,7 @@ struct Ctx {
   int tune_energy_wb = -1;    // local energy: 0 tensor cores, else walkers per CTA of the FP32 kernel (2, 4, 8)
   int tune_taylor_smem = -1;  // propagation: 2 fused kernel; Taylor kernel with A in shared memory (1) or L1 (0)
   int tune_mgs = -1;          // orthonormalisation: 1 Cholesky QR, 0 modified Gram-Schmidt kernels
+  F64Ws ws64;                 // digits of the FP64 contractions' operands (FP64 handles)
   // tangent mode (tangent.cu): derivative along h1 -> h1 + lambda P, FP64 path only
   bool tangent_on = false;
   double* Bneg = nullptr;     // [M][M]  -dt K / 2 (kept from setup)
@@ -145,7 +154,14 @@ enum GemmUse { GEMM_GENERIC = 0, GEMM_FORCE_BIAS = 1, GEMM_VHS = 2, GEMM_ONEBODY
 cudaError_t gemm_tn_f64(int Md, int Nd, int Kd, double alpha, const double* A, int64_t lda,
                         int64_t sA, const double* B, int64_t ldb, int64_t sB, double beta,
                         double* C, int64_t ldc, int64_t sC, int batch, cudaStream_t s,
-                        GemmUse use = GEMM_GENERIC);
+                        GemmUse use = GEMM_GENERIC, const F64Ws* ws = nullptr);
+// the same product from exact BF16 digit products on the tensor cores (gemm_f64e.cu), taken by
+// gemm_tn_f64 when it is given a workspace and gemm_f64e_ok
+bool gemm_f64e_ok(int Md, int Nd, int Kd);
+size_t gemm_f64e_bytes(int64_t Md, int64_t Nd, int Kd, size_t col_cap);   // workspace it can use
+cudaError_t prepare_gemm_f64e();
+cudaError_t gemm_f64e(int Md, int Nd, int Kd, double alpha, const double* A, int64_t lda, const double* B,
+                      int64_t ldb, double beta, double* C, int64_t ldc, const F64Ws& ws, cudaStream_t s);
 
 // ---- split-BF16 tensor-core GEMM (gemm_tc.cu) ----
 // A K-major operand split into bf16 hi/lo rows of Kp (multiple of 64) elements, with

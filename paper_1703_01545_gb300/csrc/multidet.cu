@@ -160,7 +160,7 @@ cudaError_t md_force_bias(const Ctx& c, cudaStream_t s) {
   const int64_t NM = (int64_t)c.N * c.M;
   cudaError_t e = gemm_tn_f64(c.X, 2 * c.Nw, (int)NM, 1.0, c.md_Ltil, NM, (int64_t)c.X * NM,
                               c.md_theta, NM, 2 * (int64_t)c.Nw * NM, 0.0, c.md_rhobar, c.X,
-                              2 * (int64_t)c.Nw * c.X, c.n_det, s, GEMM_FORCE_BIAS);
+                              2 * (int64_t)c.Nw * c.X, c.n_det, s, GEMM_FORCE_BIAS, &c.ws64);
   if (e != cudaSuccess) return e;
   k_md_mix<<<grid_for((int64_t)c.Nw * c.X), 256, 0, s>>>(c.md_share, c.md_rhobar, c.rhobar,
                                                           c.n_det, c.Nw, c.X);
