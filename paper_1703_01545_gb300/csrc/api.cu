@@ -84,6 +84,7 @@ void free_ctx(Ctx* h) {
     if (b) cudaFree(b);
   if (h->d_tc_err) cudaFree(h->d_tc_err);
   if (h->ws64.buf) cudaFree(h->ws64.buf);
+  if (h->e64) cudaFree(h->e64);
   for (double* b : {h->md_coef, h->md_psi, h->md_Ltil, h->md_htil, h->md_logO, h->md_theta,
                     h->md_share, h->md_rhobar, h->md_eloc})
     if (b) cudaFree(b);
@@ -543,6 +544,8 @@ afqmc_status afqmc_setup(afqmc_handle* out, const double* h1_in, const double* L
     for (const auto& g : gemms)
       if (g[1] < (int64_t)1 << 31 && afq::gemm_f64e_ok((int)g[0], (int)g[1], (int)g[2]))
         need = std::max(need, afq::gemm_f64e_bytes(g[0], g[1], (int)g[2], (size_t)192 << 20));
+    const bool en = afq::energy_f64e_ok(M, X, n_up, n_dn, (int)Nw);
+    if (en) need = std::max(need, afq::energy_f64e_ws(*h));
     if (need > 0) {
       AFQ_SCK(afq::prepare_gemm_f64e());
       int* err = nullptr;
@@ -552,6 +555,8 @@ afqmc_status afqmc_setup(afqmc_handle* out, const double* h1_in, const double* L
         AFQ_SCK(cudaMemsetAsync(err, 0, sizeof(int), s));
         if (cudaMalloc(&h->ws64.buf, need) == cudaSuccess) h->ws64.bytes = need;
         else h->ws64.buf = nullptr;
+        if (en && h->ws64.buf && cudaMalloc(&h->e64, afq::energy_f64e_scratch(*h)) != cudaSuccess)
+          h->e64 = nullptr;
       }
       cudaGetLastError();
     }

@@ -117,6 +117,7 @@ struct Ctx {
   int tune_energy_wb = -1;    // local energy: 0 tensor cores, else walkers per CTA of the FP32 kernel (2, 4, 8)
   int tune_taylor_smem = -1;  // propagation: 2 fused kernel; Taylor kernel with A in shared memory (1) or L1 (0)
   int tune_mgs = -1;          // orthonormalisation: 1 Cholesky QR, 0 modified Gram-Schmidt kernels
+  double* e64 = nullptr;      // scratch of the FP64 local energy in digit form
   F64Ws ws64;                 // digits of the FP64 contractions' operands (FP64 handles)
   // tangent mode (tangent.cu): derivative along h1 -> h1 + lambda P, FP64 path only
   bool tangent_on = false;
@@ -160,6 +161,40 @@ cudaError_t gemm_tn_f64(int Md, int Nd, int Kd, double alpha, const double* A, i
 bool gemm_f64e_ok(int Md, int Nd, int Kd);
 size_t gemm_f64e_bytes(int64_t Md, int64_t Nd, int Kd, size_t col_cap);   // workspace it can use
 cudaError_t prepare_gemm_f64e();
+// The parts of that form, for products whose operands stay in digits.  DigitOp: rows of K
+// elements as 8 BF16 digit planes [8][rp][Kp] with an exponent per row.
+struct DigitOp {
+  __nv_bfloat16* dig = nullptr;
+  int* ex = nullptr;
+  int64_t rp = 0;
+  int Kp = 0;
+};
+size_t digit_bytes(int64_t rows, int K);
+DigitOp digit_place(void* p, int64_t rows, int K);   // in digit_bytes of 256-byte-aligned memory
+// row r of the digits is row (r / grp) gstep + goff + r % grp of `in` (grp 0: row r)
+cudaError_t digits_of(const double* in, int64_t ld, int rows, int K, const DigitOp& d, cudaStream_t s,
+                      int grp = 0, int64_t gstep = 0, int goff = 0);
+// out[z * outz + c * ldc + r] (swap: [r * ldc + c]) = alpha sum_k rows[z rz + r][k] cols[z cz + c][k]
+// + beta out, r < R, c < Cn, z < nz.  ks > 1: ks partial sums over K ranges, `part` doubles apart,
+// without the rows' scales.  A row with NaN gives NaN; with infinities the float64 products of
+// rsrc and csrc (rows of ldr, ldcs; one batch element), or NaN without them.
+struct DigitGemm {
+  int R = 0, Cn = 0, nz = 1, rz = 0, cz = 0, ks = 1, swap = 0;
+  double alpha = 1.0, beta = 0.0;
+  double* out = nullptr;
+  int64_t ldc = 0, outz = 0, part = 0;
+  const double *rsrc = nullptr, *csrc = nullptr;
+  int64_t ldr = 0, ldcs = 0;
+  int K = 0;
+  int* err = nullptr;
+};
+// FP64 local energy with its contraction in digit form (energy_f64e.cu): taken by launch_energy
+// for all walkers of a handle that has its scratch (c.e64)
+bool energy_f64e_ok(int M, int X, int n_up, int n_dn, int Nw);
+size_t energy_f64e_scratch(const Ctx& c);
+size_t energy_f64e_ws(const Ctx& c);
+cudaError_t launch_energy_f64e(const Ctx& c, cudaStream_t s);
+cudaError_t digit_gemm(const DigitOp& rows, const DigitOp& cols, const DigitGemm& g, cudaStream_t s);
 cudaError_t gemm_f64e(int Md, int Nd, int Kd, double alpha, const double* A, int64_t lda, const double* B,
                       int64_t ldb, double beta, double* C, int64_t ldc, const F64Ws& ws, cudaStream_t s);
 

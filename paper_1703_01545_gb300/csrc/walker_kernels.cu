@@ -686,6 +686,7 @@ cudaError_t launch_mgs(const Ctx& c, cudaStream_t s) {
 }
 
 cudaError_t launch_energy(const Ctx& c, cudaStream_t s, int n_walkers) {
+  if (n_walkers <= 0 && c.e64) return launch_energy_f64e(c, s);
   const size_t smem = smem_energy(c);
   k_energy<<<n_walkers > 0 ? n_walkers : c.Nw, kThreads, smem, s>>>(c.theta, c.Ltil, c.htil, c.eloc, c.M, c.N, c.n_up, c.X, c.Nw);
   return cudaGetLastError();
