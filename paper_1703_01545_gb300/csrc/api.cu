@@ -546,6 +546,8 @@ afqmc_status afqmc_setup(afqmc_handle* out, const double* h1_in, const double* L
         need = std::max(need, afq::gemm_f64e_bytes(g[0], g[1], (int)g[2], (size_t)192 << 20));
     const bool en = afq::energy_f64e_ok(M, X, n_up, n_dn, (int)Nw);
     if (en) need = std::max(need, afq::energy_f64e_ws(*h));
+    const bool tay = afq::taylor_f64e_ok(M, N, (int)Nw, opt->taylor_order);
+    if (tay) need = std::max(need, afq::taylor_f64e_ws(M, N, (int)Nw));
     if (need > 0) {
       AFQ_SCK(afq::prepare_gemm_f64e());
       int* err = nullptr;
@@ -555,6 +557,7 @@ afqmc_status afqmc_setup(afqmc_handle* out, const double* h1_in, const double* L
         AFQ_SCK(cudaMemsetAsync(err, 0, sizeof(int), s));
         if (cudaMalloc(&h->ws64.buf, need) == cudaSuccess) h->ws64.bytes = need;
         else h->ws64.buf = nullptr;
+        h->taylor_dig = tay && h->ws64.buf;
         if (en && h->ws64.buf && cudaMalloc(&h->e64, afq::energy_f64e_scratch(*h)) != cudaSuccess)
           h->e64 = nullptr;
       }

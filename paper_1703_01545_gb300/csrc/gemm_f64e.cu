@@ -52,6 +52,7 @@
 #include <cstdint>
 #include <mutex>
 
+#include "gemm_f64e.cuh"
 #include "internal.h"
 #include "tc_device.cuh"
 
@@ -59,8 +60,8 @@ namespace afq {
 namespace {
 
 using namespace tc;
+using namespace dig;
 
-constexpr int kDig = 8;                        // digits per element
 constexpr int kBR = 128, kBK = 64;             // tile rows, K block
 constexpr int kChunk = 4;                      // K blocks per exact chunk (256 k)
 constexpr int kABytes = kBR * kBK * 2;
@@ -76,7 +77,6 @@ struct ELay {
   static_assert(kSmem <= 227 * 1024, "shared memory of a CTA");
 };
 constexpr uint64_t kWaitE = 2000000000ull;
-constexpr int kExpNaN = 4095, kExpInf = 4094;  // exponent marks of rows with NaN / infinities
 
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x,
                                             int y, int z) {
@@ -514,52 +514,26 @@ __global__ void __launch_bounds__(256) k_digits(const double* __restrict__ in, i
     double x[8];
     fetch(k, x);
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const uint32_t h = (uint32_t)__double2hiint(x[q]) & 0x7fffffffu;
-      mx = max(mx, h);
-      nan |= h > 0x7ff00000u || (h == 0x7ff00000u && __double2loint(x[q]) != 0);
-    }
+    for (int q = 0; q < 8; ++q) row_scan(x[q], mx, nan);
   }
-  mx = __reduce_max_sync(0xffffffffu, mx) >> 20;
-  nan = __any_sync(0xffffffffu, nan);
-  const bool special = mx == 0x7ffu;
-  int em = (int)mx;
-  if (mx == 0) {   // subnormal (or zero) row: its exponent continues below 1
+  int mark;
+  const int em = row_exponent(mx, nan, mark, [&]() {
     long long top = 0;
-    for (int k = lane; k < K; k += 32)
-      top = max(top, __double_as_longlong(__ldg(row + k)) & 0xfffffffffffffll);
-    for (int o = 16; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
-    em = top ? 12 - __clzll(top) : 1;
-  }
-  if (lane == 0) ex[r] = nan ? kExpNaN : special ? kExpInf : em;
+    for (int k = lane; k < K; k += 32) top = max(top, fraction_of(__ldg(row + k)));
+    return top;
+  });
+  if (lane == 0) ex[r] = mark;
   for (int k = 8 * lane; k < Kp; k += 256) {
     double x[8];
     fetch(k, x);
     uint32_t b[kDig][4];
 #pragma unroll
     for (int q = 0; q < 8; q += 2) {
-      uint32_t w[2][2];
+      uint32_t w0[2], w1[2];
+      digit_bytes_of(x[q], em, mark >= kExpInf, w0[0], w0[1]);
+      digit_bytes_of(x[q + 1], em, mark >= kExpInf, w1[0], w1[1]);
 #pragma unroll
-      for (int p = 0; p < 2; ++p) {
-        const uint64_t bits = (uint64_t)__double_as_longlong(x[q + p]);
-        const int e = (int)((bits >> 52) & 0x7ffu);
-        uint64_t m = bits & 0xfffffffffffffull;
-        if (e) m |= 0x10000000000000ull;
-        const int sh = 9 - (em - (e ? e : 1));
-        uint64_t y = sh >= 0 ? m << sh : (sh > -55 ? (m + (1ull << (-sh - 1))) >> -sh : 0ull);
-        if (special) y = 0;
-        if (bits >> 63) y = 0 - y;
-        y += 0x8080808080808080ull;   // digit + 128 in every byte
-        w[p][0] = (uint32_t)(y >> 32);
-        w[p][1] = (uint32_t)y;
-      }
-#pragma unroll
-      for (int j = 0; j < kDig; ++j) {
-        const uint32_t sel = 0x7440u | (uint32_t)(3 - (j & 3));   // 0x4b, 0, 0, byte
-        const float f0 = __uint_as_float(__byte_perm(w[0][j >> 2], 0x4b000000u, sel)) - 8388736.f;
-        const float f1 = __uint_as_float(__byte_perm(w[1][j >> 2], 0x4b000000u, sel)) - 8388736.f;
-        b[j][q >> 1] = __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632u);
-      }
+      for (int j = 0; j < kDig; ++j) b[j][q >> 1] = digit_pair(j, w0, w1);
     }
 #pragma unroll
     for (int j = 0; j < kDig; ++j)

@@ -117,6 +117,7 @@ struct Ctx {
   int tune_energy_wb = -1;    // local energy: 0 tensor cores, else walkers per CTA of the FP32 kernel (2, 4, 8)
   int tune_taylor_smem = -1;  // propagation: 2 fused kernel; Taylor kernel with A in shared memory (1) or L1 (0)
   int tune_mgs = -1;          // orthonormalisation: 1 Cholesky QR, 0 modified Gram-Schmidt kernels
+  int taylor_dig = 0;         // 1: the FP64 Taylor products in digit form (ws64 has the room)
   double* e64 = nullptr;      // scratch of the FP64 local energy in digit form
   F64Ws ws64;                 // digits of the FP64 contractions' operands (FP64 handles)
   // tangent mode (tangent.cu): derivative along h1 -> h1 + lambda P, FP64 path only
@@ -188,6 +189,11 @@ struct DigitGemm {
   int K = 0;
   int* err = nullptr;
 };
+// FP64 Taylor exponential in digit form (taylor_f64e.cu): taken by launch_taylor for handles whose
+// workspace was sized for it (c.taylor_dig)
+bool taylor_f64e_ok(int M, int N, int Nw, int order);
+size_t taylor_f64e_ws(int M, int N, int Nw);
+cudaError_t launch_taylor_f64e(const Ctx& c, double* phi, cudaStream_t s);
 // FP64 local energy with its contraction in digit form (energy_f64e.cu): taken by launch_energy
 // for all walkers of a handle that has its scratch (c.e64)
 bool energy_f64e_ok(int M, int X, int n_up, int n_dn, int Nw);

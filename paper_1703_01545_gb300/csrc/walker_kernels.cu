@@ -665,6 +665,7 @@ cudaError_t launch_fields(const Ctx& c, const double* fields, cudaStream_t s) {
 }
 
 cudaError_t launch_taylor(const Ctx& c, double* phi_io, cudaStream_t s) {
+  if (c.taylor_dig) return launch_taylor_f64e(c, phi_io, s);
   const int NM = c.N * c.M;
   const size_t smem = smem_taylor(c);
   const int opt = opt_for(NM);
