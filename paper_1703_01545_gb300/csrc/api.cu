@@ -535,6 +535,10 @@ afqmc_status afqmc_setup(afqmc_handle* out, const double* h1_in, const double* L
   } while (0)
 
   AFQ_SCK(afq::prepare_kernels(*h));
+  if (opt->precision == AFQMC_FP64 && afq::overlap64_ok(*h)) {
+    AFQ_SCK(afq::prepare_overlap64(*h));
+    if (dalloc(h, &h->ovdet, 8 * (size_t)Nw) != AFQMC_OK) return bail(AFQMC_ERR_NOMEM);
+  }
   if (opt->precision == AFQMC_FP64) {
     // digits of the step's contractions: as much as they can use, the walkers' operands in
     // chunks of 192 MB (a chunk and its products then stay in L2); without the memory the
@@ -683,6 +687,15 @@ afqmc_status afqmc_setup_multidet(afqmc_handle* out, const double* h1, const dou
       dalloc(h, &h->md_eloc, (size_t)n_det * 2 * Nw) != AFQMC_OK ||
       dalloc(h, &tmp, (size_t)(n_det + 1) * NM) != AFQMC_OK)
     return fail_with(AFQMC_ERR_NOMEM);
+  if (h->ovdet) {   // one record per determinant
+    cudaStreamSynchronize(s);
+    cudaFree(h->ovdet);
+    h->ovdet = nullptr;
+    if (dalloc(h, &h->ovdet, 8 * (size_t)n_det * Nw) != AFQMC_OK) {
+      cudaFree(tmp);
+      return fail_with(AFQMC_ERR_NOMEM);
+    }
+  }
   cudaError_t e = cudaMemcpyAsync(h->md_coef, c.data(), sizeof(double) * n_det,
                                   cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)

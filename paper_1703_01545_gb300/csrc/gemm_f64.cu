@@ -12,6 +12,8 @@
 // only job is to keep that pipe busy: 64x64 CTA tile, 16-deep k slices staged
 // through shared memory (transposed, so the inner loop reads contiguous rows),
 // 4x4 outputs per thread, fused alpha/beta epilogue with coalesced stores.
+#include <cmath>
+
 #include "internal.h"
 
 namespace afq {
@@ -100,6 +102,55 @@ __device__ __forceinline__ void gemm_tn_body(int Md, int Nd, int Kd, double alph
     }
   }
 }
+// Small products: 16 x 16 tiles, one output per thread, the same order of the sums.  A 64 x 64 tile
+// occupies one SM's FP64 pipe (2 multiply-adds per clock) for 2048 cycles per k, so a product of a
+// few such tiles leaves most SMs idle: V_HS of the smallest pair (36 x 256, k = 24) took 35 us on 4
+// SMs; 16 x 16 tiles use 48 of them and take 3.1 us.  The 2M x 2M products of the exponential's
+// derivative at M = 96: 200 -> 15 us.
+constexpr int ST = 16, SK = 32;
+__global__ void __launch_bounds__(ST * ST)
+    k_gemm_f64_small(int Md, int Nd, int Kd, double alpha, const double* __restrict__ A, int64_t lda, int64_t sA,
+                     const double* __restrict__ B, int64_t ldb, int64_t sB, double beta,
+                     double* __restrict__ C, int64_t ldc, int64_t sC) {
+  __shared__ double As[2][SK][ST + 1], Bs[2][SK][ST + 1];
+  const int tid = threadIdx.x, tx = tid % ST, ty = tid / ST;
+  const int64_t z = blockIdx.z;
+  const int m0 = blockIdx.x * ST, n0 = blockIdx.y * ST;
+  // a thread stages 2 elements of each operand: row ty, k = tx and tx + 16
+  const bool ar = m0 + ty < Md, br = n0 + ty < Nd;
+  const double* Ap = A + z * sA + (int64_t)(m0 + ty) * lda;
+  const double* Bp = B + z * sB + (int64_t)(n0 + ty) * ldb;
+  double ra[2], rb[2];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int k = k0 + tx + ST * q;
+      ra[q] = ar && k < Kd ? __ldg(Ap + k) : 0.0;
+      rb[q] = br && k < Kd ? __ldg(Bp + k) : 0.0;
+    }
+  };
+  fetch(0);
+  double acc = 0.0;
+  int buf = 0;
+  for (int k0 = 0; k0 < Kd; k0 += SK, buf ^= 1) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      As[buf][tx + ST * q][ty] = ra[q];
+      Bs[buf][tx + ST * q][ty] = rb[q];
+    }
+    __syncthreads();
+    if (k0 + SK < Kd) fetch(k0 + SK);
+    const int kn = min(SK, Kd - k0);
+#pragma unroll 8
+    for (int kk = 0; kk < kn; ++kk) acc = fma(As[buf][kk][tx], Bs[buf][kk][ty], acc);
+  }
+  const int m = m0 + tx, n = n0 + ty;
+  if (m < Md && n < Nd) {
+    double* Cp = C + z * sC + (int64_t)n * ldc + m;
+    *Cp = (beta != 0.0) ? fma(alpha, acc, beta * *Cp) : alpha * acc;
+  }
+}
+
 // One kernel symbol per use, so profiles and launch lists name the contraction.
 #define AFQ_GEMM_KERNEL(name)                                                                    \
   __global__ void __launch_bounds__(NT) name(int Md, int Nd, int Kd, double alpha,              \
@@ -128,6 +179,14 @@ cudaError_t gemm_tn_f64(int Md, int Nd, int Kd, double alpha, const double* A, i
     if (e != cudaErrorMemoryAllocation) return e;   // else: the workspace is too small for this shape
   }
   dim3 grid((Md + BM - 1) / BM, (Nd + BN - 1) / BN, batch);
+  const dim3 gs((Md + ST - 1) / ST, (Nd + ST - 1) / ST, batch);
+  // multiply-adds of the busiest SM in both tilings (tiles of a batch run side by side)
+  const double t64 = (double)grid.x * grid.y * batch, t16 = (double)gs.x * gs.y * batch;
+  if (gs.y <= 65535u && gs.z <= 65535u &&
+      1.1 * std::ceil(t16 / 152) * ST * ST < std::ceil(t64 / 152) * BM * BN) {
+    k_gemm_f64_small<<<gs, ST * ST, 0, s>>>(Md, Nd, Kd, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC);
+    return cudaGetLastError();
+  }
   if (grid.y > 65535u || grid.z > 65535u) return cudaErrorInvalidConfiguration;
   auto k = use == GEMM_FORCE_BIAS ? k_gemm_f64_force_bias
            : use == GEMM_VHS      ? k_gemm_f64_vhs

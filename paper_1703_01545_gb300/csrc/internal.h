@@ -312,6 +312,10 @@ cudaError_t prepare_fast_walker_kernels(const Ctx& c);
 // with_weights = false launches the overlap kernel without the per-walker weight kernel
 cudaError_t launch_overlap_fast(const Ctx& c, const double* src, int mode, cudaStream_t s,
                                 const float* src32 = nullptr, bool with_weights = true);
+// FP64 overlaps with spin blocks of at most 16 (walker_fast.cu); c.ovdet: [Nd or 1][Nw][8]
+bool overlap64_ok(const Ctx& c);
+cudaError_t prepare_overlap64(const Ctx& c);
+cudaError_t launch_overlap64(const Ctx& c, const double* src, int mode, cudaStream_t s);
 // update_logO: subtract log det R (the column norms) from log O instead of recomputing it
 cudaError_t launch_mgs_warp(const Ctx& c, cudaStream_t s, bool update_logO = false);
 bool mgs_chol_ok(const Ctx& c);

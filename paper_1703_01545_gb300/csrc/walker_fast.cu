@@ -49,6 +49,9 @@ struct FastOvArgs {
   double* det;        // [Nw][8]: per spin the determinant mantissa (re, im), the summed
                       // power-of-two exponent, the singular flag (k_overlap_fast -> k_overlap_weights)
   int M, N, n_up, Nw, mode, free_proj;
+  double* theta64;    // FP64 form (k_overlap64): Theta
+  // mode OV_DET (grid row d = determinant d): psi, Theta, log O and det of d start d * det_* on
+  int64_t det_psi, det_theta, det_logO, det_det;
   int fp64_copy;      // 1: Phi also staged in FP64 shared memory (every mode but the FP32 update)
   double log_shift;
 };
@@ -152,7 +155,10 @@ __device__ __forceinline__ void lu_block(T* __restrict__ ar, T* __restrict__ ai,
         dexp += eh - S::bias();
       }
     }
-    const T rinv = S::rcp(S::fm(vr, vr, vi * vi));
+    const T vv = S::fm(vr, vr, vi * vi);
+    // FP64: a pivot whose square leaves the range counts as singular (or not finite) too
+    if (sizeof(T) == 8 && go && !(vv > T(0) && S::key(vv) < S::kInf)) bad = true;
+    const T rinv = S::rcp(vv);
     const T ir = vr * rinv, ii = -vi * rinv;          // 1 / pivot
     __syncwarp();
     if (go && l >= k && l < ns) {
@@ -487,13 +493,169 @@ __global__ void __launch_bounds__(256) k_overlap_fast(FastOvArgs a) {
   }
 }
 
-// Per walker, after k_overlap_fast: log det O, the overlap ratio and the weight update.
+// The FP64 path's overlap, determinant and Theta for spin blocks of at most 16, everything in
+// float64: the sums of O_s = Psi_s^T Phi_s (4 lanes an entry), the warp LU above, and Theta_s =
+// Phi_s O_s^{-1} by triangular solves, one orbital row of a spin per thread (half the operations of
+// forming the inverse and multiplying).  Bound by the FP64 pipe (2 multiply-adds per clock and SM):
+// at M = 64, 8/8 about 52 k of them per walker, 0.18 ms for 2048 walkers; measured 0.23 ms, against
+// 0.52 ms of the block-wide Gauss-Jordan kernel (k_overlap, now for larger blocks only), which waits at
+// its barriers for as long again.  128 walkers at M = 8, 2/2: 22 -> 9.4 us.
+// Modes as k_overlap: OV_UPDATE takes src as the walker if it lives, else recomputes from Phi
+// (Theta's buffer held the propagated walkers); OV_DET: grid row = determinant, no walker changes.
+template <int ROWS, int NSM>
+__global__ void __launch_bounds__(256) k_overlap64(FastOvArgs a) {
+  extern __shared__ double smo[];
+  const int wk = blockIdx.x, tid = threadIdx.x, M = a.M, N = a.N, NM = N * M;
+  const int MP = M + 1, NMP = N * MP;   // columns M + 1 apart: the solves' and sums' reads spread
+  constexpr int LDA = NSM == 8 ? 8 : kLd, PLN = NSM * LDA, SPB = 2 * PLN;
+  const int lane = tid & 31, warp = tid >> 5;
+  double* pr = smo;            // [N][MP]
+  double* pi = pr + NMP;
+  double* aug = pi + NMP;      // LU factors: spin s at aug + s * SPB, re, im [NSM][LDA]
+  __shared__ double s_det[2][2];
+  __shared__ int s_dexp[2], s_bad[2];
+  __shared__ int s_piv[2][kNsMax];
+  __shared__ unsigned long long s_perm[2];
+  const bool upd = a.mode == OV_UPDATE && a.alive[wk] != 0;
+  const double* psi = a.psi + blockIdx.y * a.det_psi;
+  double* theta = a.theta64 + blockIdx.y * a.det_theta;
+  const double* src = (upd || (a.mode == OV_DET && a.src)) ? a.src : a.phi;
+  const int64_t plane = (int64_t)a.Nw * NM, wbase = (int64_t)wk * NM;
+  for (int e = tid; e < NM; e += blockDim.x) {
+    const int es = e + e / M;
+    const double xr = src[wbase + e], xi = src[plane + wbase + e];
+    if (upd) {
+      a.phi[wbase + e] = xr;
+      a.phi[plane + wbase + e] = xi;
+    }
+    pr[es] = xr;
+    pi[es] = xi;
+  }
+  if (tid < 2) { s_det[tid][0] = 1.0; s_det[tid][1] = 0.0; s_dexp[tid] = 0; s_bad[tid] = 0; }
+  __syncthreads();
+  const int nu = a.n_up, nd = N - nu, nn = nu * nu + nd * nd;
+  for (int base = 0; base < nn * 4; base += blockDim.x) {
+    const int q = base + tid, ent = q >> 2, part = q & 3;
+    double re = 0.0, im = 0.0;
+    int sp = 0, r = 0, c = 0;
+    if (ent < nn) {
+      if (ent < nu * nu) { r = ent / nu; c = ent % nu; }
+      else { sp = 1; const int e2 = ent - nu * nu; r = e2 / nd; c = e2 % nd; }
+      const int n0 = sp ? nu : 0;
+      const double* ps = psi + (int64_t)(n0 + r) * M;
+      const double* fr = pr + (n0 + c) * MP;
+      const double* fi = pi + (n0 + c) * MP;
+      for (int i = part; i < M; i += 4) {
+        const double p = __ldg(ps + i);
+        re = fma(p, fr[i], re);
+        im = fma(p, fi[i], im);
+      }
+    }
+    re += __shfl_xor_sync(0xffffffffu, re, 1);
+    im += __shfl_xor_sync(0xffffffffu, im, 1);
+    re += __shfl_xor_sync(0xffffffffu, re, 2);
+    im += __shfl_xor_sync(0xffffffffu, im, 2);
+    if (ent < nn && part == 0) {
+      aug[sp * SPB + r * LDA + c] = re;
+      aug[sp * SPB + PLN + r * LDA + c] = im;
+    }
+  }
+  __syncthreads();
+  // NSM = 8: both blocks in warp 0, 16 lanes each; else a warp per block
+  if (warp < (NSM == 8 ? 1 : 2)) {
+    const int sp = NSM == 8 ? lane >> 4 : warp, l = NSM == 8 ? lane & 15 : lane, ns = sp ? nd : nu;
+    double* ar = aug + sp * SPB;
+    double dr, di;
+    int dexp;
+    bool bad;
+    if (NSM == 8) lu_block<16, 4, LDA>(ar, ar + PLN, l, ns, nu > nd ? nu : nd, s_piv[sp], dr, di, dexp, bad);
+    else lu_block<32, ROWS, LDA>(ar, ar + PLN, l, ns, ns, s_piv[sp], dr, di, dexp, bad);
+    if (l == 0) {
+      s_det[sp][0] = dr;
+      s_det[sp][1] = di;
+      s_dexp[sp] = dexp;
+      s_bad[sp] = bad ? 1 : 0;
+    }
+  }
+  __syncthreads();
+  const bool bad = s_bad[0] || s_bad[1];
+  if (tid < 2) {   // P from the interchanges, in order, as 4-bit row indices
+    const int ns = tid ? nd : nu;
+    unsigned long long pw = 0xfedcba9876543210ull;
+    if (!bad)
+      for (int k = 0; k < ns; ++k) {
+        const int p = s_piv[tid][k];
+        const unsigned long long x = (pw >> (4 * k)) & 15ull, y = (pw >> (4 * p)) & 15ull;
+        pw ^= ((x ^ y) << (4 * k)) | ((x ^ y) << (4 * p));
+      }
+    s_perm[tid] = pw;
+  }
+  __syncthreads();
+  if (bad) {
+    for (int e = tid; e < NM; e += blockDim.x) theta[wbase + e] = theta[plane + wbase + e] = 0.0;
+  } else {
+    // y U = phi_i (U unit upper), z L = y (L lower, 1 / pivot on the diagonal), theta_i[perm[j]] = z_j
+    for (int t = tid; t < 2 * M; t += blockDim.x) {
+      const int sp = t / M, i = t - sp * M, ns = sp ? nd : nu, n0 = sp ? nu : 0;
+      const double* Lr = aug + sp * SPB;
+      const double* Li = Lr + PLN;
+      double yr[NSM], yi[NSM];
+#pragma unroll
+      for (int j = 0; j < NSM; ++j) {
+        yr[j] = j < ns ? pr[(n0 + j) * MP + i] : 0.0;
+        yi[j] = j < ns ? pi[(n0 + j) * MP + i] : 0.0;
+      }
+#pragma unroll
+      for (int j = 1; j < NSM; ++j)
+        if (j < ns) {
+#pragma unroll
+          for (int k = 0; k < j; ++k) {
+            const double ur = Lr[k * LDA + j], ui = Li[k * LDA + j];
+            yr[j] = fma(-yr[k], ur, fma(yi[k], ui, yr[j]));
+            yi[j] = fma(-yr[k], ui, fma(-yi[k], ur, yi[j]));
+          }
+        }
+#pragma unroll
+      for (int j = NSM - 1; j >= 0; --j)
+        if (j < ns) {
+          double tr = yr[j], ti = yi[j];
+#pragma unroll
+          for (int k = j + 1; k < NSM; ++k)
+            if (k < ns) {
+              const double lr = Lr[k * LDA + j], li = Li[k * LDA + j];
+              tr = fma(-yr[k], lr, fma(yi[k], li, tr));
+              ti = fma(-yr[k], li, fma(-yi[k], lr, ti));
+            }
+          const double qr = Lr[j * LDA + j], qi = Li[j * LDA + j];
+          yr[j] = fma(tr, qr, -ti * qi);
+          yi[j] = fma(tr, qi, ti * qr);
+        }
+      const unsigned long long pw = s_perm[sp];
+#pragma unroll
+      for (int j = 0; j < NSM; ++j)
+        if (j < ns) {
+          const int64_t gi = wbase + (n0 + (int)((pw >> (4 * j)) & 15ull)) * M + i;
+          theta[gi] = yr[j];
+          theta[plane + gi] = yi[j];
+        }
+    }
+  }
+  if (tid < 6) {
+    double v = bad ? 1.0 : 0.0;
+    if (tid < 4) v = s_det[tid >> 1][tid & 1];
+    else if (tid == 4) v = (double)(s_dexp[0] + s_dexp[1]);
+    a.det[blockIdx.y * a.det_det + 8 * (int64_t)wk + tid] = v;
+  }
+}
+
+// Per walker, after k_overlap_fast or k_overlap64: log det O, the overlap ratio and the weight update.
 __global__ void __launch_bounds__(32) k_overlap_weights(FastOvArgs a) {
   const int wk = blockIdx.x * blockDim.x + threadIdx.x;
   if (wk >= a.Nw) return;
   const bool upd = (a.mode == OV_UPDATE) && a.alive[wk] != 0;
   if (a.mode == OV_UPDATE && !upd) return;
-  const double* dt = a.det + 8 * (int64_t)wk;
+  const double* dt = a.det + blockIdx.y * a.det_det + 8 * (int64_t)wk;
+  double* logO = a.logO + blockIdx.y * a.det_logO;
   const bool bad = dt[5] != 0.0;
   // log det O = log(d_up d_dn) + (e_up + e_dn) ln 2
   const double d0r = dt[0], d0i = dt[1], d1r = dt[2], d1i = dt[3];
@@ -501,6 +663,11 @@ __global__ void __launch_bounds__(32) k_overlap_weights(FastOvArgs a) {
   const double ld_re = 0.5 * log(fma(pr_, pr_, pi_ * pi_)) + dt[4] * M_LN2;
   const double ld_im = atan2(pi_, pr_);
   if (bad || !isfinite(ld_re) || !isfinite(ld_im)) {
+    if (a.mode == OV_DET) {   // this determinant contributes nothing to the trial
+      logO[wk] = -INFINITY;
+      logO[a.Nw + wk] = 0.0;
+      return;
+    }
     atomicAdd(a.flags, 1);
     if (upd || a.mode == OV_REFRESH) {
       a.w[wk] = 0.0;
@@ -510,8 +677,8 @@ __global__ void __launch_bounds__(32) k_overlap_weights(FastOvArgs a) {
     return;
   }
   if (!upd) {
-    a.logO[wk] = ld_re;
-    a.logO[a.Nw + wk] = ld_im;
+    logO[wk] = ld_re;
+    logO[a.Nw + wk] = ld_im;
     return;
   }
   const double* x = a.aux + 4 * (int64_t)wk;
@@ -915,7 +1082,7 @@ cudaError_t prepare_fast_walker_kernels(const Ctx& c) {
 
 cudaError_t launch_overlap_fast(const Ctx& c, const double* src, int mode, cudaStream_t s,
                                 const float* src32, bool with_weights) {
-  FastOvArgs a;
+  FastOvArgs a{};
   a.src = src;
   a.src32 = c.psi32h ? src32 : nullptr;
   a.psih = c.psi32h;
@@ -939,6 +1106,63 @@ cudaError_t launch_overlap_fast(const Ctx& c, const double* src, int mode, cudaS
   else k_overlap_fast<8, 16><<<c.Nw, nt, sm, s>>>(a);
   // one warp per CTA: the FP64 chain of each warp gets an SM's FP64 pipe to itself
   if (with_weights) k_overlap_weights<<<(c.Nw + 31) / 32, 32, 0, s>>>(a);
+  return cudaGetLastError();
+}
+
+namespace {
+size_t smem_overlap64(const Ctx& c) {
+  const int nmax = std::max(c.n_up, c.N - c.n_up);
+  return sizeof(double) * (2 * (size_t)c.N * (c.M + 1) + 4 * (nmax <= 8 ? 8 * 8 : kNsMax * kLd));
+}
+SmemLimits g_ov64_limits;
+}  // namespace
+
+bool overlap64_ok(const Ctx& c) {
+  return c.n_up <= kNsMax && c.N - c.n_up <= kNsMax && smem_overlap64(c) <= 200 * 1024;
+}
+
+cudaError_t prepare_overlap64(const Ctx& c) {
+  const size_t sm = smem_overlap64(c);
+  auto raise = [&](int slot, auto k) {
+    return g_ov64_limits.raise(slot, sm, [&] {
+      return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    });
+  };
+  cudaError_t e = raise(0, k_overlap64<4, 8>);
+  if (e == cudaSuccess) e = raise(1, k_overlap64<4, 16>);
+  if (e == cudaSuccess) e = raise(2, k_overlap64<8, 16>);
+  return e;
+}
+
+// FP64 overlaps of the walkers (OV_REFRESH, OV_UPDATE) or of every determinant (OV_DET, n_det rows)
+cudaError_t launch_overlap64(const Ctx& c, const double* src, int mode, cudaStream_t s) {
+  FastOvArgs a{};
+  const bool dets = mode == OV_DET;
+  a.src = src;
+  a.phi = c.phi;
+  a.psi = dets ? c.md_psi : c.psi;
+  a.theta64 = dets ? c.md_theta : c.theta;
+  a.logO = dets ? c.md_logO : c.logO;
+  a.w = c.w; a.alive = c.alive; a.aux = c.aux; a.flags = c.d_flags; a.det = c.ovdet;
+  a.M = c.M; a.N = c.N; a.n_up = c.n_up; a.Nw = c.Nw; a.mode = mode;
+  a.free_proj = c.opt.mode == AFQMC_FREE;
+  a.log_shift = -c.opt.dt * (c.c_mf - c.e_trial);
+  if (dets) {
+    a.det_psi = (int64_t)c.N * c.M;
+    a.det_theta = 2 * (int64_t)c.Nw * c.N * c.M;
+    a.det_logO = 2 * (int64_t)c.Nw;
+    a.det_det = 8 * (int64_t)c.Nw;
+  }
+  const int nd = dets ? c.n_det : 1, nmax = std::max(c.n_up, c.N - c.n_up);
+  const size_t sm = smem_overlap64(c);
+  const dim3 grid(c.Nw, nd);
+  const int rows = nmax > 0 ? (nmax + (32 / nmax) - 1) / (32 / nmax) : 1;   // LU rows of a lane
+  // as many threads as the entries' lanes or the solves' rows can use
+  const int nt = std::max(64, std::min(256, std::max(2 * c.M, 4 * nmax * nmax) / 32 * 32));
+  if (nmax <= 8) k_overlap64<4, 8><<<grid, nt, sm, s>>>(a);
+  else if (rows <= 4) k_overlap64<4, 16><<<grid, nt, sm, s>>>(a);
+  else k_overlap64<8, 16><<<grid, nt, sm, s>>>(a);
+  k_overlap_weights<<<dim3((c.Nw + 31) / 32, nd), 32, 0, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -2,6 +2,7 @@
 // determinant, so every small dense operation (overlap, Gauss-Jordan inverse,
 // Taylor products, Gram-Schmidt, exchange trace) runs out of shared memory with
 // coalesced loads from the planar walker layout [2][Nw][N][M].
+#include <algorithm>
 #include <cmath>
 #include <cuda_bf16.h>
 #include "device_util.cuh"
@@ -406,6 +407,90 @@ __global__ void __launch_bounds__(kThreads) k_taylor(double* __restrict__ phi, c
   }
 }
 
+// The same for M <= 32: the walker's A expanded to a full matrix in shared memory (16 KB at most),
+// as many threads as outputs, and two partial sums over j, so that a round is a chain of M
+// multiply-adds.  k_taylor reads A element by element from the packed triangle: at M = 8, 4 columns,
+// a chain of 192 global loads (25 us for 128 walkers; 13.4 us here).
+template <int OPT>
+__global__ void __launch_bounds__(kThreads) k_taylor_small(double* __restrict__ phi, const double* __restrict__ Ap,
+                                                           int M, int N, int Nw, int64_t P, int order) {
+  extern __shared__ double sm[];
+  const int wk = blockIdx.x, tid = threadIdx.x, nt = blockDim.x, NM = N * M, MM = M * M;
+  double* xr = sm;             // A [M][M]
+  double* xi = xr + MM;
+  double* tr = xi + MM;        // [M][N] current term
+  double* ti = tr + NM;
+  double* nr = ti + NM;        // next term
+  double* ni = nr + NM;
+  const int64_t plane = (int64_t)Nw * NM, base = (int64_t)wk * NM;
+  const double* ar = Ap + (int64_t)wk * P;
+  const double* ai = ar + (int64_t)Nw * P;
+  double acc_r[OPT], acc_i[OPT];
+#pragma unroll
+  for (int q = 0; q < OPT; ++q) {
+    const int o = tid + q * nt;
+    acc_r[q] = acc_i[q] = 0.0;
+    if (o < NM) {
+      const int i = o / N, b = o - i * N;
+      acc_r[q] = phi[base + (int64_t)b * M + i];
+      acc_i[q] = phi[plane + base + (int64_t)b * M + i];
+      tr[o] = acc_r[q];
+      ti[o] = acc_i[q];
+    }
+  }
+  for (int e = tid; e < MM; e += nt) {
+    const int i = e / M, j = e - i * M, lo = min(i, j), hi = max(i, j);
+    const int p = lo * (M - 1) - lo * (lo - 1) / 2 + hi;
+    xr[e] = ar[p];
+    xi[e] = ai[p];
+  }
+  __syncthreads();
+  for (int m = 1; m <= order; ++m) {
+    const double inv = 1.0 / (double)m;
+#pragma unroll
+    for (int q = 0; q < OPT; ++q) {
+      const int o = tid + q * nt;
+      if (o < NM) {
+        const int i = o / N, b = o - i * N;
+        const double* pr = xr + i * M;
+        const double* pi = xi + i * M;
+        double s0 = 0, s1 = 0, u0 = 0, u1 = 0;
+        int j = 0;
+#pragma unroll 4
+        for (; j + 1 < M; j += 2) {
+          const double y0 = tr[j * N + b], z0 = ti[j * N + b], y1 = tr[(j + 1) * N + b], z1 = ti[(j + 1) * N + b];
+          s0 = fma(pr[j], y0, fma(-pi[j], z0, s0));
+          u0 = fma(pr[j], z0, fma(pi[j], y0, u0));
+          s1 = fma(pr[j + 1], y1, fma(-pi[j + 1], z1, s1));
+          u1 = fma(pr[j + 1], z1, fma(pi[j + 1], y1, u1));
+        }
+        if (j < M) {
+          const double y0 = tr[j * N + b], z0 = ti[j * N + b];
+          s0 = fma(pr[j], y0, fma(-pi[j], z0, s0));
+          u0 = fma(pr[j], z0, fma(pi[j], y0, u0));
+        }
+        const double sr = (s0 + s1) * inv, si = (u0 + u1) * inv;
+        nr[o] = sr;
+        ni[o] = si;
+        acc_r[q] += sr;
+        acc_i[q] += si;
+      }
+    }
+    __syncthreads();
+    double* t0 = tr; tr = nr; nr = t0;
+    double* t1 = ti; ti = ni; ni = t1;
+  }
+#pragma unroll
+  for (int q = 0; q < OPT; ++q) {
+    const int o = tid + q * nt;
+    if (o < NM) {
+      const int i = o / N, b = o - i * N;
+      phi[base + (int64_t)b * M + i] = acc_r[q];
+      phi[plane + base + (int64_t)b * M + i] = acc_i[q];
+    }
+  }
+}
+
 // ---------------------------------------------------------------------------
 // Modified Gram-Schmidt per spin block (Sec. II.D): for each column j in order,
 // subtract its projections on the already orthonormal columns one at a time,
@@ -611,6 +696,19 @@ cudaError_t prepare_kernels(const Ctx& c) {
   if ((e = ensure_smem(k_overlap<true>, 7, smem_overlap(c))) != cudaSuccess) return e;
   if ((e = ensure_smem(k_mgs, 1, smem_mgs(c))) != cudaSuccess) return e;
   if ((e = ensure_smem(k_energy, 2, smem_energy(c))) != cudaSuccess) return e;
+  if (c.M <= 32) {   // N <= 64 columns: 80 KB at most
+    static SmemLimits small;
+    const size_t sm = smem_taylor(c) + sizeof(double) * 2 * (size_t)c.M * c.M;
+    auto raise = [&](int slot, auto k) {
+      return small.raise(slot, sm, [&] {
+        return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      });
+    };
+    if ((e = raise(0, k_taylor_small<1>)) != cudaSuccess) return e;
+    if ((e = raise(1, k_taylor_small<2>)) != cudaSuccess) return e;
+    if ((e = raise(2, k_taylor_small<4>)) != cudaSuccess) return e;
+    if ((e = raise(3, k_taylor_small<8>)) != cudaSuccess) return e;
+  }
   const size_t st = smem_taylor(c);
   if ((e = ensure_smem(k_taylor<2>, 3, st)) != cudaSuccess) return e;
   if ((e = ensure_smem(k_taylor<4>, 4, st)) != cudaSuccess) return e;
@@ -621,6 +719,7 @@ cudaError_t prepare_kernels(const Ctx& c) {
 
 cudaError_t launch_overlap(const Ctx& c, const double* src, int mode, cudaStream_t s,
                            int n_walkers) {
+  if (c.ovdet && !c.theta32 && n_walkers <= 0 && overlap64_ok(c)) return launch_overlap64(c, src, mode, s);
   OverlapArgs a;
   a.theta32 = c.theta32;
   a.op_hi = c.tc_Theta ? c.tc_Theta->hi : nullptr;
@@ -641,6 +740,7 @@ cudaError_t launch_overlap(const Ctx& c, const double* src, int mode, cudaStream
 
 cudaError_t launch_overlap_dets(const Ctx& c, const double* src, cudaStream_t s) {
   if (c.n_det < 1 || c.n_det > 65535) return cudaErrorInvalidValue;
+  if (c.ovdet && overlap64_ok(c)) return launch_overlap64(c, src, OV_DET, s);
   OverlapArgs a = {};
   a.src = src; a.phi = c.phi; a.alive = c.alive; a.aux = c.aux; a.flags = c.d_flags;
   a.psi = c.md_psi; a.theta = c.md_theta; a.logO = c.md_logO; a.w = c.w;
@@ -667,6 +767,18 @@ cudaError_t launch_fields(const Ctx& c, const double* fields, cudaStream_t s) {
 cudaError_t launch_taylor(const Ctx& c, double* phi_io, cudaStream_t s) {
   if (c.taylor_dig) return launch_taylor_f64e(c, phi_io, s);
   const int NM = c.N * c.M;
+  if (c.M <= 32) {
+    const size_t sm = smem_taylor(c) + sizeof(double) * 2 * (size_t)c.M * c.M;
+    const int nt = std::min(kThreads, (NM + 31) / 32 * 32), per = (NM + nt - 1) / nt;
+#define AFQ_TAYLOR(K)                                                                                    \
+  k_taylor_small<K><<<c.Nw, nt, sm, s>>>(phi_io, c.Avhs, c.M, c.N, c.Nw, c.P, c.opt.taylor_order);
+    if (per <= 1) { AFQ_TAYLOR(1) }
+    else if (per <= 2) { AFQ_TAYLOR(2) }
+    else if (per <= 4) { AFQ_TAYLOR(4) }
+    else { AFQ_TAYLOR(8) }
+#undef AFQ_TAYLOR
+    return cudaGetLastError();
+  }
   const size_t smem = smem_taylor(c);
   const int opt = opt_for(NM);
 #define AFQ_TAYLOR(K)                                                                          \
