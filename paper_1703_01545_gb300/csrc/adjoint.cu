@@ -177,6 +177,11 @@ afqmc_status adjoint_body(Ctx* h, Arena& ar, int n_steps, const double* fields, 
   if (afq::gemm_f64e_ok(X, 2 * Nw, MM)) need = afq::gemm_f64e_bytes(X, 2 * Nw, MM, (size_t)192 << 20);
   if (afq::gemm_f64e_ok(NM, 2 * Nw, X))
     need = std::max(need, afq::gemm_f64e_bytes(NM, 2 * Nw, X, (size_t)192 << 20));
+  // the Taylor series' reverse and the measurement's in digit form, where the forward ones are
+  const bool rev_t = afq::taylor_f64e_ok(M, N, Nw, c.opt.taylor_order);
+  const bool rev_e = afq::energy_f64e_ok(M, X, c.n_up, nd, Nw);
+  if (rev_t) need = std::max(need, afq::taylor_rev_f64e_ws(M, N, Nw, c.opt.taylor_order));
+  if (rev_e) need = std::max(need, afq::energy_rev_f64e_ws(c));
   if (need > ws.bytes) {
     ADJ_CK(afq::prepare_gemm_f64e());
     uint8_t* p = ar.try_get(need);
@@ -188,6 +193,10 @@ afqmc_status adjoint_body(Ctx* h, Arena& ar, int n_steps, const double* fields, 
       ws.err = err;
     }
   }
+  const bool room = ws.buf && ws.bytes >= need;
+  double* vterms = rev_t && room ? reinterpret_cast<double*>(ar.try_get(sizeof(double) * nphi * c.opt.taylor_order))
+                                 : nullptr;
+  double* erev = rev_e && room ? reinterpret_cast<double*>(ar.try_get(afq::energy_rev_f64e_scratch(c))) : nullptr;
 
   ADJ_CK(afq::prepare_adjoint_kernels(c));
   ADJ_CK(afq::launch_transpose(c.Ltil, LtilT, X, NM, s));   // [NM][X]
@@ -234,7 +243,8 @@ afqmc_status adjoint_body(Ctx* h, Arena& ar, int n_steps, const double* fields, 
       // measurement after step t: E_m = sum w Re E_L / sum w on the (orthonormalised) walkers
       if (meas_at(t)) {
         ADJ_CK(afq::adj_meas_weights(c, ebar, 1.0 / n_meas, s));
-        ADJ_CK(afq::adj_energy(c, c.theta, ebar, thb, eloc_r, c.alive, s));
+        if (erev) ADJ_CK(afq::launch_energy_rev_f64e(c, ws, erev, c.theta, ebar, thb, eloc_r, c.alive, s));
+        else ADJ_CK(afq::adj_energy(c, c.theta, ebar, thb, eloc_r, c.alive, s));
         ADJ_CK(afq::adj_meas_finish(c, eloc_r, ebar, lwbar, e_acc, (double)n_meas, s));
         ADJ_CK(afq::adj_theta_avg(c, c.theta, ebar, avg, s));
         ADJ_CK(afq::adj_inv_overlap(c, c.phi, Y1, logO_tmp, nullptr, c.alive, s));
@@ -251,7 +261,8 @@ afqmc_status adjoint_body(Ctx* h, Arena& ar, int n_steps, const double* fields, 
                               afq::GEMM_ONEBODY, &ws));
       ADJ_CK(afq::gemm_tn_f64(M, cols, M, 1.0, c.expK, M, 0, tp.phi, M, 0, 0.0, phi1, M, 0, 1, s,
                               afq::GEMM_ONEBODY, &ws));
-      ADJ_CK(afq::adj_taylor(c, phi1, pbA, terms, Abar, c.phi2, still, s));
+      if (vterms) ADJ_CK(afq::launch_taylor_rev_f64e(c, ws, phi1, pbA, terms, vterms, Abar, still, s));
+      else ADJ_CK(afq::adj_taylor(c, phi1, pbA, terms, Abar, c.phi2, still, s));
       ADJ_CK(afq::adj_outer(c, pbA, tp.phi, still, part, Ebar, s));
       ADJ_CK(afq::gemm_tn_f64(M, cols, M, 1.0, c.expK, M, 0, pbA, M, 0, 0.0, phibar, M, 0, 1, s,
                               afq::GEMM_ONEBODY, &ws));

@@ -17,6 +17,7 @@
 #include <cstdint>
 
 #include "device_util.cuh"
+#include "gemm_f64e.cuh"
 #include "internal.h"
 
 namespace afq {
@@ -128,6 +129,107 @@ __global__ void __launch_bounds__(128) k_energy_sum(const double* __restrict__ t
   }
 }
 
+// Ltil rows (g, b) of a spin as columns: element (orbital i, k = g ns + b)
+struct LtilColumns {
+  const double* ltil;
+  int ns, n0, N, M;
+  __device__ double at(int, int i, int k) const {
+    const int g = k / ns;
+    return ltil[((int64_t)g * N + n0 + k - g * ns) * M + i];
+  }
+};
+
+// W[(p, wl, a)][(g, b)] = conj(rhobar_g) delta_ab - conj(T_g[a][b]) as digits, from the chunk's T
+// ([(p, wl, b)][(g, a)]) and the traces tr[spin][p][w][g] of both spins.  A CTA per (wl, p): the rows'
+// exponents in a first pass, then gb Cholesky vectors at a time staged as [a][(g, b)], so that T is
+// read along its rows and the digits are written along theirs.  gb ns is even.
+__global__ void __launch_bounds__(256) k_energy_w(const double* __restrict__ T, int64_t ldt, int ns, int X, int w0, int Nw,
+                                                  const double* __restrict__ tr, int nspin, int gb, int Kp, int64_t rp,
+                                                  uint16_t* __restrict__ out, int* __restrict__ ex) {
+  using namespace dig;
+  extern __shared__ double sm[];   // [ns][gb ns + 1]
+  __shared__ uint32_t smx[32], snan[32];
+  __shared__ unsigned long long sfr[32];
+  __shared__ int sem[32], smark[32];
+  const int wl = blockIdx.x, nwc = gridDim.x, p = blockIdx.y, tid = threadIdx.x, K = X * ns;
+  const int lane = tid & 31, warp = tid >> 5, ld = gb * ns + 1;
+  const int64_t tsp = 2 * (int64_t)Nw * X, to = ((int64_t)p * Nw + w0 + wl) * X;
+  const double* Tw = T + ((int64_t)(p * nwc + wl) * ns) * ldt;
+  auto value = [&](int a, int b, int g, double t) -> double {
+    double v = p ? t : -t;
+    if (a == b) {
+      double rho = 0.0;
+      for (int s = 0; s < nspin; ++s) rho += tr[s * tsp + to + g];
+      v += p ? -rho : rho;
+    }
+    return v;
+  };
+  if (tid < 32) {
+    smx[tid] = snan[tid] = 0u;
+    sfr[tid] = 0ull;
+  }
+  __syncthreads();
+  for (int b = 0; b < ns; ++b)
+    for (int r = tid; r < K; r += 256) {
+      const int g = r / ns, a = r - g * ns;
+      const double x = value(a, b, g, Tw[(int64_t)b * ldt + r]);
+      uint32_t mx = 0, nan = 0;
+      row_scan(x, mx, nan);
+      if (mx > smx[a]) atomicMax(&smx[a], mx);
+      if (nan) snan[a] = 1u;
+      if ((mx >> 20) == 0) atomicMax(&sfr[a], (unsigned long long)fraction_of(x));
+    }
+  __syncthreads();
+  if (tid < ns) {
+    const uint32_t mx = smx[tid] >> 20;
+    const int em = mx ? (int)mx : sfr[tid] ? 12 - __clzll((long long)sfr[tid]) : 1;
+    sem[tid] = em;
+    smark[tid] = snan[tid] ? kExpNaN : mx == 0x7ffu ? kExpInf : em;
+    ex[(int64_t)(p * nwc + wl) * ns + tid] = smark[tid];
+  }
+  for (int k0 = 0; k0 < Kp; k0 += gb * ns) {
+    const int g0 = k0 / ns, len = min(gb * ns, Kp - k0);   // (the last step pads K with zeros)
+    __syncthreads();
+    for (int b = warp; b < ns; b += 8)
+      for (int r = lane; r < gb * ns; r += 32) {
+        const int g = r / ns, a = r - g * ns;
+        sm[a * ld + g * ns + b] = g0 + g < X ? value(a, b, g0 + g, Tw[(int64_t)b * ldt + (int64_t)g0 * ns + r]) : 0.0;
+      }
+    __syncthreads();
+    for (int a = warp; a < ns; a += 8)
+      for (int k = 2 * lane; k < len; k += 64) {
+        uint32_t x[2], y[2];
+        digit_bytes_of(sm[a * ld + k], sem[a], smark[a] >= kExpInf, x[0], x[1]);
+        digit_bytes_of(sm[a * ld + k + 1], sem[a], smark[a] >= kExpInf, y[0], y[1]);
+        const int64_t row = (int64_t)(p * nwc + wl) * ns + a;
+#pragma unroll
+        for (int j = 0; j < kDig; ++j)
+          *reinterpret_cast<uint32_t*>(out + ((int64_t)j * rp + row) * Kp + k0 + k) = digit_pair(j, x, y);
+      }
+  }
+}
+
+// thb[(p, w, n0 + a)][i] = ebar_w (htil[n0 + a][i] (real plane) + G[(p, wl, a)][i]), 0 for walkers out
+// of the sweep
+__global__ void __launch_bounds__(256) k_energy_thb(const double* __restrict__ G, const double* __restrict__ htil,
+                                                    const double* __restrict__ ebar, const int* __restrict__ mask,
+                                                    int ns, int n0, int N, int M, int w0, int nwc, int Nw,
+                                                    double* __restrict__ thb) {
+  const int64_t total = 2 * (int64_t)nwc * ns * M;
+  for (int64_t e = blockIdx.x * 256 + threadIdx.x; e < total; e += (int64_t)gridDim.x * 256) {
+    const int i = (int)(e % M), a = (int)(e / M % ns), wl = (int)(e / ((int64_t)M * ns) % nwc);
+    const int p = (int)(e / ((int64_t)M * ns * nwc)), w = w0 + wl;
+    const double v = mask[w] ? ebar[w] * (p ? G[e] : G[e] + htil[(n0 + a) * M + i]) : 0.0;
+    thb[(((int64_t)p * Nw + w) * N + n0 + a) * M + i] = v;
+  }
+}
+
+__global__ void k_energy_masked(const double* __restrict__ el, const int* __restrict__ mask, int Nw,
+                                double* __restrict__ eloc) {
+  const int w = blockIdx.x * blockDim.x + threadIdx.x;
+  if (w < Nw) eloc[w] = mask[w] ? el[w] : 0.0;
+}
+
 // Walkers per chunk: T of both planes within kTBytes for the larger spin (one at least).
 int chunk_walkers(const Ctx& c) {
   const int ns = std::max(c.n_up, c.N - c.n_up);
@@ -162,6 +264,39 @@ size_t energy_f64e_ws(const Ctx& c) {
   return digit_bytes((int64_t)c.X * ns, c.M) + digit_bytes(2 * (int64_t)chunk_walkers(c) * ns, c.M);
 }
 
+namespace {
+
+// T of one spin for walkers w0 .. w0 + nw - 1, and from it the exchange sums and traces (spin index
+// sp); `cols` memory for the columns' digits
+cudaError_t chunk_of(const Ctx& c, const F64Ws& ws, const double* theta, const DigitOp& da, void* cols, int sp, int n0,
+                     int ns, int w0, int nw, int nsplit, double* T, double* tr, double* ex, cudaStream_t s) {
+  const int NM = c.N * c.M, nc = 2 * nw * ns, rows = c.X * ns;
+  const DigitOp db = digit_place(cols, nc, c.M);
+  for (int p = 0; p < 2; ++p) {
+    DigitOp dp = db;
+    dp.dig += (int64_t)p * nw * ns * db.Kp;
+    dp.ex += p * nw * ns;
+    const cudaError_t e = digits_of(theta + ((int64_t)p * c.Nw + w0) * NM, c.M, nw * ns, c.M, dp, s, ns, c.N, n0);
+    if (e != cudaSuccess) return e;
+  }
+  DigitGemm g;
+  g.R = rows;
+  g.Cn = nc;
+  g.out = T;
+  g.ldc = rows;
+  g.K = c.M;
+  g.err = ws.err;
+  const cudaError_t e = digit_gemm(da, db, g, s);
+  if (e != cudaSuccess) return e;
+  int gb = 32;
+  while (gb > 1 && (size_t)2 * ns * ns * (gb + 1) * sizeof(double) > kStage) gb /= 2;
+  k_exchange<<<dim3(nw, nsplit), kEx, (size_t)2 * ns * ns * (gb + 1) * sizeof(double), s>>>(
+      T, rows, ns, c.X, w0, c.Nw, gb, ex + (size_t)sp * nsplit * 2 * c.Nw, tr + (size_t)sp * 2 * c.Nw * c.X);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
 cudaError_t launch_energy_f64e(const Ctx& c, cudaStream_t s) {
   const int NM = c.N * c.M, nwc = chunk_walkers(c), nsmax = std::max(c.n_up, c.N - c.n_up);
   const int nsplit = splits(c, nwc);
@@ -173,38 +308,110 @@ cudaError_t launch_energy_f64e(const Ctx& c, cudaStream_t s) {
   for (int s0 = 0; s0 < 2 && e == cudaSuccess; ++s0) {
     const int n0 = s0 ? c.n_up : 0, ns = s0 ? c.N - c.n_up : c.n_up;
     if (ns == 0) continue;
-    const int rows = c.X * ns;
-    const DigitOp da = digit_place(c.ws64.buf, rows, c.M);
-    e = digits_of(c.Ltil, c.M, rows, c.M, da, s, ns, c.N, n0);
-    for (int w0 = 0; w0 < c.Nw && e == cudaSuccess; w0 += nwc) {
-      const int nw = std::min(nwc, c.Nw - w0), cols = 2 * nw * ns;
-      const DigitOp db = digit_place(c.ws64.buf + digit_bytes(rows, c.M), cols, c.M);
-      for (int p = 0; p < 2 && e == cudaSuccess; ++p) {
-        DigitOp dp = db;
-        dp.dig += (int64_t)p * nw * ns * db.Kp;
-        dp.ex += p * nw * ns;
-        e = digits_of(c.theta + ((int64_t)p * c.Nw + w0) * NM, c.M, nw * ns, c.M, dp, s, ns, c.N, n0);
-      }
-      if (e != cudaSuccess) break;
-      DigitGemm g;
-      g.R = rows;
-      g.Cn = cols;
-      g.out = T;
-      g.ldc = rows;
-      g.K = c.M;
-      g.err = c.ws64.err;
-      if ((e = digit_gemm(da, db, g, s)) != cudaSuccess) break;
-      int gb = 32;
-      while (gb > 1 && (size_t)2 * ns * ns * (gb + 1) * sizeof(double) > kStage) gb /= 2;
-      k_exchange<<<dim3(nw, nsplit), kEx, (size_t)2 * ns * ns * (gb + 1) * sizeof(double), s>>>(
-          T, rows, ns, c.X, w0, c.Nw, gb, ex + (size_t)sp * nsplit * 2 * c.Nw,
-          tr + (size_t)sp * 2 * c.Nw * c.X);
-      e = cudaGetLastError();
-    }
+    const DigitOp da = digit_place(c.ws64.buf, c.X * ns, c.M);
+    e = digits_of(c.Ltil, c.M, c.X * ns, c.M, da, s, ns, c.N, n0);
+    for (int w0 = 0; w0 < c.Nw && e == cudaSuccess; w0 += nwc)
+      e = chunk_of(c, c.ws64, c.theta, da, c.ws64.buf + digit_bytes(c.X * ns, c.M), sp, n0, ns, w0,
+                   std::min(nwc, c.Nw - w0), nsplit, T, tr, ex, s);
     ++sp;
   }
   if (e != cudaSuccess) return e;
   k_energy_sum<<<c.Nw, 128, 0, s>>>(c.theta, c.htil, tr, ex, sp, nsplit, NM, c.X, c.Nw, c.eloc);
+  return cudaGetLastError();
+}
+
+// Reverse: T of both spins of a chunk, W and Ltil's columns as digits, G and its partial sums.
+namespace {
+constexpr size_t kRevPart = (size_t)64 << 20;
+// walkers whose T (both spins) takes 320 MB at most: the reverse reads it twice only, and needs as
+// many (walker, plane) CTAs as there are SMs
+int rev_chunk(const Ctx& c) {
+  const int ns = std::max(c.n_up, c.N - c.n_up);
+  const size_t per = 4 * (size_t)c.X * ns * ns * sizeof(double);
+  return (int)std::max<size_t>(1, std::min<size_t>((size_t)c.Nw, ((size_t)320 << 20) / per));
+}
+}  // namespace
+
+size_t energy_rev_f64e_scratch(const Ctx& c) {
+  const int ns = std::max(c.n_up, c.N - c.n_up), nwc = rev_chunk(c);
+  return sizeof(double) * (4 * (size_t)c.X * ns * ns * nwc + 2 * (size_t)nwc * ns * c.M + 4 * (size_t)c.Nw * c.X +
+                           4 * (size_t)kMaxSplit * c.Nw + 2 * (size_t)c.Nw) + kRevPart;
+}
+
+size_t energy_rev_f64e_ws(const Ctx& c) {
+  const int ns = std::max(c.n_up, c.N - c.n_up), nwc = rev_chunk(c);
+  return 2 * digit_bytes((int64_t)c.X * ns, c.M) + 2 * digit_bytes(c.M, c.X * ns) +
+         std::max(digit_bytes(2 * (int64_t)nwc * ns, c.M), digit_bytes(2 * (int64_t)nwc * ns, c.X * ns));
+}
+
+// 15.7 ms in the walker kernel (k_energy_rev) at M = 96, X = 480, 12/12, 128 walkers, 3.6 ms here.
+// E_L of every walker and thb = ebar (htil + sum_g conj(rhobar_g) Ltil_g - sum_g conj(T_g) Ltil_g), the
+// second product as one contraction over (g, b).
+cudaError_t launch_energy_rev_f64e(const Ctx& c, const F64Ws& ws, double* scratch, const double* theta,
+                                   const double* ebar, double* thb, double* eloc, const int* mask, cudaStream_t s) {
+  const int NM = c.N * c.M, nwc = rev_chunk(c), nsmax = std::max(c.n_up, c.N - c.n_up);
+  const int nsplit = splits(c, nwc);
+  const size_t tlen = 2 * (size_t)c.X * nsmax * nsmax * nwc;
+  double* part = scratch;
+  double* T[2] = {part + kRevPart / sizeof(double), part + kRevPart / sizeof(double) + tlen};
+  double* G = T[1] + tlen;
+  double* tr = G + 2 * (size_t)nwc * nsmax * c.M;
+  double* ex = tr + 4 * (size_t)c.Nw * c.X;
+  double* el = ex + 4 * (size_t)kMaxSplit * c.Nw;
+  uint8_t* at = ws.buf;
+  DigitOp da[2], dl[2];
+  int n0s[2], nss[2], nspin = 0;
+  cudaError_t e = cudaSuccess;
+  for (int s0 = 0; s0 < 2 && e == cudaSuccess; ++s0) {
+    const int n0 = s0 ? c.n_up : 0, ns = s0 ? c.N - c.n_up : c.n_up;
+    if (ns == 0) continue;
+    const int rows = c.X * ns;
+    n0s[nspin] = n0;
+    nss[nspin] = ns;
+    da[nspin] = digit_place(at, rows, c.M);
+    at += digit_bytes(rows, c.M);
+    dl[nspin] = digit_place(at, c.M, rows);
+    at += digit_bytes(c.M, rows);
+    e = digits_of(c.Ltil, c.M, rows, c.M, da[nspin], s, ns, c.N, n0);
+    if (e != cudaSuccess) break;
+    const LtilColumns f{c.Ltil, ns, n0, c.N, c.M};
+    dig::k_strided_digits<<<dim3(1, (c.M + 31) / 32), 1024, 0, s>>>(
+        f, c.M, rows, dl[nspin].Kp, dl[nspin].rp, c.M, 0, reinterpret_cast<uint16_t*>(dl[nspin].dig), dl[nspin].ex);
+    e = cudaGetLastError();
+    ++nspin;
+  }
+  for (int w0 = 0; w0 < c.Nw && e == cudaSuccess; w0 += nwc) {
+    const int nw = std::min(nwc, c.Nw - w0);
+    for (int sp = 0; sp < nspin && e == cudaSuccess; ++sp)
+      e = chunk_of(c, ws, theta, da[sp], at, sp, n0s[sp], nss[sp], w0, nw, nsplit, T[sp], tr, ex, s);
+    for (int sp = 0; sp < nspin && e == cudaSuccess; ++sp) {
+      const int ns = nss[sp], rows = c.X * ns;
+      const DigitOp dw = digit_place(at, 2 * nw * ns, rows);
+      // staged vectors: an even number (gb ns has to be even) within kStage
+      const int gb = std::max(2, (int)(kStage / (sizeof(double) * ns * ns)) / 2 * 2);
+      const int gs = std::min(gb, 32);
+      k_energy_w<<<dim3(nw, 2), 256, sizeof(double) * ns * ((size_t)gs * ns + 1), s>>>(T[sp], rows, ns, c.X, w0, c.Nw, tr, nspin, gs, dw.Kp, dw.rp,
+                                             reinterpret_cast<uint16_t*>(dw.dig), dw.ex);
+      if ((e = cudaGetLastError()) != cudaSuccess) break;
+      DigitGemm g;
+      g.R = 2 * nw * ns;
+      g.Cn = c.M;
+      g.swap = 1;
+      g.out = G;
+      g.ldc = c.M;
+      g.K = rows;
+      g.err = ws.err;
+      if ((e = digit_gemm_sum(dw, dl[sp], g, part, kRevPart, s)) != cudaSuccess) break;
+      const int64_t total = 2 * (int64_t)nw * ns * c.M;
+      k_energy_thb<<<(int)std::min<int64_t>((total + 255) / 256, 152 * 8), 256, 0, s>>>(
+          G, c.htil, ebar, mask, ns, n0s[sp], c.N, c.M, w0, nw, c.Nw, thb);
+      e = cudaGetLastError();
+    }
+  }
+  if (e != cudaSuccess) return e;
+  k_energy_sum<<<c.Nw, 128, 0, s>>>(theta, c.htil, tr, ex, nspin, nsplit, NM, c.X, c.Nw, el);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  k_energy_masked<<<(c.Nw + 255) / 256, 256, 0, s>>>(el, mask, c.Nw, eloc);
   return cudaGetLastError();
 }
 

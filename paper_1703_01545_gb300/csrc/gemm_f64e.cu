@@ -562,11 +562,11 @@ constexpr size_t kPartBytes = 64u << 20;   // room for the partial sums of a spl
 // K ranges for `tiles` tiles of nkb K blocks: the split that minimises the waves' length, in
 // cycles of one K block (4.8 k) and of an item's fixed part (6 k: pipeline fill, the last
 // chunk's drain), with the partial sums' round trip (16 bytes per output and range).
-int k_ranges(int64_t tiles, int nkb) {
+int k_ranges(int64_t tiles, int nkb, size_t part_bytes) {
   int best = 1;
   double bt = 1e300;
   for (int ks = 1; ks <= std::max(1, nkb / 2) && ks <= 64; ++ks) {
-    if ((size_t)(tiles * kBR * 64) * 8 * ks > kPartBytes && ks > 1) break;
+    if ((size_t)(tiles * kBR * 64) * 8 * ks > part_bytes && ks > 1) break;
     const int kbs = (nkb + ks - 1) / ks;
     if ((nkb + kbs - 1) / kbs != ks) continue;
     const double waves = std::ceil((double)(tiles * ks) / kSms);
@@ -583,7 +583,7 @@ int k_ranges(int64_t tiles, int nkb) {
 cudaError_t digit_map(CUtensorMap* map, const DigitOp& d, int box_rows, int box_dig) {
   auto fn = encode_tiled_fn();
   if (!fn) return cudaErrorNotSupported;
-  cuuint64_t dims[3] = {(cuuint64_t)d.Kp, (cuuint64_t)d.rp, (cuuint64_t)kDig};
+  cuuint64_t dims[3] = {(cuuint64_t)d.Kp, (cuuint64_t)(d.rp - d.off), (cuuint64_t)kDig};
   cuuint64_t strides[2] = {(cuuint64_t)d.Kp * 2, (cuuint64_t)d.rp * d.Kp * 2};
   cuuint32_t box[3] = {(cuuint32_t)kBK, (cuuint32_t)box_rows, (cuuint32_t)box_dig};
   cuuint32_t estr[3] = {1, 1, 1};
@@ -674,6 +674,29 @@ cudaError_t digit_gemm(const DigitOp& rows, const DigitOp& cols, const DigitGemm
   }
 }
 
+// digit_gemm of one batch element over as many K ranges as pay, their partial sums in `part`.
+cudaError_t digit_gemm_sum(const DigitOp& rows, const DigitOp& cols, DigitGemm g, double* part, size_t part_bytes,
+                           cudaStream_t s) {
+  const int64_t tiles = ((int64_t)(g.R + kBR - 1) / kBR) * ((g.Cn + 63) / 64);
+  g.ks = k_ranges(tiles, rows.Kp / kBK, part_bytes);
+  if (g.ks <= 1) return digit_gemm(rows, cols, g, s);
+  // the partial sums are dense, the operand whose index is contiguous in `out` innermost
+  const int in = g.swap ? g.Cn : g.R, outer = g.swap ? g.R : g.Cn;
+  DigitGemm q = g;
+  q.alpha = 1.0;
+  q.beta = 0.0;
+  q.out = part;
+  q.ldc = in;
+  q.part = (int64_t)in * outer;
+  cudaError_t e = digit_gemm(rows, cols, q, s);
+  if (e != cudaSuccess) return e;
+  const int64_t total = (int64_t)in * outer;
+  k_sum_ranges<<<(int)std::min<int64_t>((total + 255) / 256, kSms * 16), 256, 0, s>>>(
+      part, q.part, g.ks, in, total, g.swap ? cols.ex : rows.ex, g.swap ? rows.ex : cols.ex, g.alpha, g.beta, g.out,
+      g.ldc);
+  return cudaGetLastError();
+}
+
 // The digit form pays where its launches (about 12 us in all) and its 36 products of the padded
 // operands (1.2 PFLOP/s) take less than the FP64 pipe's 1.1 TFLOP/s.  At M = 8 and 128 walkers the
 // pipe's 17 us win; from 3e7 products on it needs 55 us and more.
@@ -726,31 +749,17 @@ cudaError_t gemm_f64e(int Md, int Nd, int Kd, double alpha, const double* A, int
     g.swap = t1 < t0;
     g.R = g.swap ? nr : Md;
     g.Cn = g.swap ? Md : nr;
-    g.ks = k_ranges(std::min(t0, t1), da.Kp / kBK);
     g.alpha = alpha;
     g.beta = beta;
     g.out = Cn;
     g.ldc = ldc;
-    if (g.ks > 1) {
-      g.alpha = 1.0;
-      g.beta = 0.0;
-      g.out = part;
-      g.ldc = Md;
-      g.part = (int64_t)Md * nr;
-    }
     g.rsrc = g.swap ? B + n0 * ldb : A;
     g.ldr = g.swap ? ldb : lda;
     g.csrc = g.swap ? A : B + n0 * ldb;
     g.ldcs = g.swap ? lda : ldb;
     g.K = Kd;
     g.err = ws.err;
-    if ((e = digit_gemm(g.swap ? db : da, g.swap ? da : db, g, s)) != cudaSuccess) break;
-    if (g.ks > 1) {
-      const int64_t total = (int64_t)Md * nr;
-      k_sum_ranges<<<(int)std::min<int64_t>((total + 255) / 256, kSms * 16), 256, 0, s>>>(
-          part, g.part, g.ks, Md, total, da.ex, db.ex, alpha, beta, Cn, ldc);
-      e = cudaGetLastError();
-    }
+    e = digit_gemm_sum(g.swap ? db : da, g.swap ? da : db, g, part, kPartBytes, s);
   }
   return e;
 }

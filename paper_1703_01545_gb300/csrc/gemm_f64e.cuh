@@ -61,5 +61,71 @@ __device__ __forceinline__ long long fraction_of(double x) {
   return __double_as_longlong(x) & 0xfffffffffffffll;
 }
 
+// Rows r0 .. of a batch element as digits, K strided in memory: a CTA per batch element and 32 rows,
+// element (row, k) from f.at(z, row, k), which is contiguous in the row.  The first pass takes the
+// rows' exponents, the second cuts 64 k x 32 rows at a time through shared memory (32 warps, as a
+// single batch element has few rows and a long K).  `quarter`: pairs
+// (k even: re, odd: im) give a second set of rows, rows2 further on, with (-im, re).
+template <class F>
+__global__ void __launch_bounds__(1024) k_strided_digits(const F f, int rows, int K, int Kp, int64_t rp, int rz,
+                                                        int rows2, uint16_t* __restrict__ out,
+                                                        int* __restrict__ ex) {
+  __shared__ double tile[32][65];
+  __shared__ uint32_t smx[32][32], snan[32][32];
+  __shared__ long long sfr[32][32];
+  __shared__ int sem[32], smark[32];
+  const int z = blockIdx.x, r0 = blockIdx.y * 32, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int row = r0 + lane;
+  uint32_t mx = 0, nan = 0;
+  long long fr = 0;
+  for (int k = warp; k < K; k += 32) {
+    const double x = row < rows ? f.at(z, row, k) : 0.0;
+    row_scan(x, mx, nan);
+    fr = max(fr, fraction_of(x));
+  }
+  smx[warp][lane] = mx;
+  snan[warp][lane] = nan;
+  sfr[warp][lane] = fr;
+  __syncthreads();
+  if (warp == 0) {
+    for (int w = 1; w < 32; ++w) {
+      mx = max(mx, smx[w][lane]);
+      nan |= snan[w][lane];
+      fr = max(fr, sfr[w][lane]);
+    }
+    mx >>= 20;
+    // (the largest fraction is the row's largest element only in a subnormal row)
+    const int em = mx ? (int)mx : fr ? 12 - __clzll(fr) : 1;
+    const int mark = nan ? kExpNaN : mx == 0x7ffu ? kExpInf : em;
+    sem[lane] = em;
+    smark[lane] = mark;
+    if (row < rows) {
+      ex[(int64_t)z * rz + row] = mark;
+      if (rows2) ex[(int64_t)z * rz + rows2 + row] = mark;
+    }
+  }
+  for (int k0 = 0; k0 < Kp; k0 += 64) {
+    __syncthreads();
+    for (int k = warp; k < 64; k += 32)
+      tile[lane][k] = row < rows && k0 + k < K ? f.at(z, row, k0 + k) : 0.0;
+    __syncthreads();
+    const int q = warp;
+    if (r0 + q < rows) {
+      uint32_t a[2], b[2];
+      digit_bytes_of(tile[q][2 * lane], sem[q], smark[q] >= kExpInf, a[0], a[1]);
+      digit_bytes_of(tile[q][2 * lane + 1], sem[q], smark[q] >= kExpInf, b[0], b[1]);
+      const int64_t o = ((int64_t)z * rz + r0 + q) * Kp + k0 + 2 * lane;
+#pragma unroll
+      for (int j = 0; j < kDig; ++j) {
+        const uint32_t d = digit_pair(j, a, b);
+        *reinterpret_cast<uint32_t*>(out + (int64_t)j * rp * Kp + o) = d;
+        if (rows2)
+          *reinterpret_cast<uint32_t*>(out + (int64_t)j * rp * Kp + o + (int64_t)rows2 * Kp) =
+              __byte_perm(d, d, 0x1032u) ^ 0x00008000u;
+      }
+    }
+  }
+}
+
 }  // namespace dig
 }  // namespace afq

@@ -168,6 +168,7 @@ struct DigitOp {
   __nv_bfloat16* dig = nullptr;
   int* ex = nullptr;
   int64_t rp = 0;
+  int64_t off = 0;   // rows of the planes before dig (a view that starts further down)
   int Kp = 0;
 };
 size_t digit_bytes(int64_t rows, int K);
@@ -201,6 +202,16 @@ size_t energy_f64e_scratch(const Ctx& c);
 size_t energy_f64e_ws(const Ctx& c);
 cudaError_t launch_energy_f64e(const Ctx& c, cudaStream_t s);
 cudaError_t digit_gemm(const DigitOp& rows, const DigitOp& cols, const DigitGemm& g, cudaStream_t s);
+cudaError_t digit_gemm_sum(const DigitOp& rows, const DigitOp& cols, DigitGemm g, double* part, size_t part_bytes,
+                           cudaStream_t s);
+size_t taylor_rev_f64e_ws(int M, int N, int Nw, int order);
+cudaError_t launch_taylor_rev_f64e(const Ctx& c, const F64Ws& ws, const double* phi1, double* pbar, double* u,
+                                   double* v, double* Abar, const int* mask, cudaStream_t s);
+// E_L and the adjoint of ebar Re E_L (adj_energy), eloc [Nw]; scratch: energy_rev_f64e_scratch doubles
+size_t energy_rev_f64e_ws(const Ctx& c);
+size_t energy_rev_f64e_scratch(const Ctx& c);
+cudaError_t launch_energy_rev_f64e(const Ctx& c, const F64Ws& ws, double* scratch, const double* theta,
+                                   const double* ebar, double* thb, double* eloc, const int* mask, cudaStream_t s);
 cudaError_t gemm_f64e(int Md, int Nd, int Kd, double alpha, const double* A, int64_t lda, const double* B,
                       int64_t ldb, double beta, double* C, int64_t ldc, const F64Ws& ws, cudaStream_t s);
 

@@ -100,20 +100,41 @@ __global__ void __launch_bounds__(512) k_vhs_digits(const double* __restrict__ A
   }
 }
 
+// What a term kernel does with the round's product U (of A, or of conj(A) in the reverse sweep).
+enum TermKind {
+  kFirst = 0,   // x = in
+  kSum = 1,     // x = U, acc += coef x
+  kKeep = 2,    // x = U, out = coef x
+  kRev = 3      // x = in + coef U, out = x (where the walker's mask allows)
+};
+
+struct TermArgs {
+  const double* prod;    // products of walkers w0 .., [z][2 N][R]
+  const double* in;      // [2][Nw][N][M]
+  double* out;           // [2][Nw][N][M], or null
+  const int* mask;       // kRev: walkers whose out is written, or null
+  double coef;
+  int M, N, Nw, w0, nw, stack, M2;
+  int conj;              // the digits' products are with conj(A) (and so were kRev's)
+  int more;              // digits of x as the next round's columns
+  int Kp;
+  int64_t rp;
+  __nv_bfloat16* dig;
+  int* ex;
+};
+
 // One term of walkers w0 .. : a warp per (walker, column n), lanes over pairs of orbitals.
-// FIRST: U = Phi; else U = the round's products and Phi += coef U.  `more`: the digits of U as the
-// next round's columns.
-template <int NP, bool FIRST>
-__global__ void __launch_bounds__(256) k_term(const double* __restrict__ prod, double* __restrict__ phi, int M, int N,
-                                              int Nw, int w0, int nw, int stack, int M2, double coef, int more,
-                                              int Kp, int64_t rp, __nv_bfloat16* __restrict__ out,
-                                              int* __restrict__ ex) {
-  const int task = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (task >= nw * N) return;
-  const int z = task / N, n = task - z * N, R = stack ? 2 * M : M;
-  const int64_t base = ((int64_t)(w0 + z) * N + n) * M, plane = (int64_t)Nw * N * M;
-  const double* pr = prod + ((int64_t)z * 2 * N + n) * R;       // column n of the real half
+// Columns n and N + n of the next product, joined K: [x_r | -x_i], [x_i | x_r] for A, [x_r | x_i],
+// [x_i | -x_r] for conj(A); stacked rows: x_r, x_i for both.
+template <int NP, int KIND>
+__global__ void __launch_bounds__(256) k_term(const TermArgs a) {
+  const int task = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31, M = a.M, N = a.N;
+  if (task >= a.nw * N) return;
+  const int z = task / N, n = task - z * N, R = a.stack ? 2 * M : M;
+  const int64_t base = ((int64_t)(a.w0 + z) * N + n) * M, plane = (int64_t)a.Nw * N * M;
+  const double* pr = a.prod + ((int64_t)z * 2 * N + n) * R;     // column n of the real half
   const double* pi = pr + (int64_t)N * R;
+  const bool write = KIND != kRev || (a.out && (!a.mask || a.mask[a.w0 + z]));
   double x[NP][2][2];   // [pair][element][re, im]
   uint32_t mx = 0, nan = 0;
 #pragma unroll
@@ -123,19 +144,36 @@ __global__ void __launch_bounds__(256) k_term(const double* __restrict__ prod, d
       const int i = 64 * t + 2 * lane + q;
       double re = 0.0, im = 0.0;
       if (i < M) {
-        if (FIRST) {
-          re = phi[base + i];
-          im = phi[plane + base + i];
+        if (KIND == kFirst) {
+          re = a.in[base + i];
+          im = a.in[plane + base + i];
         } else {
-          if (stack) {
-            re = pr[i] - pi[M + i];
-            im = pi[i] + pr[M + i];
-          } else {
+          if (!a.stack) {
             re = pr[i];
             im = pi[i];
+          } else if (KIND == kRev) {
+            re = pr[i] + pi[M + i];
+            im = pi[i] - pr[M + i];
+          } else {
+            re = pr[i] - pi[M + i];
+            im = pi[i] + pr[M + i];
           }
-          phi[base + i] = fma(coef, re, phi[base + i]);
-          phi[plane + base + i] = fma(coef, im, phi[plane + base + i]);
+          if (KIND == kSum) {
+            a.out[base + i] = fma(a.coef, re, a.out[base + i]);
+            a.out[plane + base + i] = fma(a.coef, im, a.out[plane + base + i]);
+          }
+          if (KIND == kRev) {
+            re = fma(a.coef, re, a.in[base + i]);
+            im = fma(a.coef, im, a.in[plane + base + i]);
+          }
+          if (KIND == kKeep) {
+            a.out[base + i] = a.coef * re;
+            a.out[plane + base + i] = a.coef * im;
+          }
+          if (KIND == kRev && write) {
+            a.out[base + i] = re;
+            a.out[plane + base + i] = im;
+          }
         }
       }
       x[t][q][0] = re;
@@ -143,7 +181,7 @@ __global__ void __launch_bounds__(256) k_term(const double* __restrict__ prod, d
       row_scan(re, mx, nan);
       row_scan(im, mx, nan);
     }
-  if (!more) return;
+  if (!a.more) return;
   int mark;
   const int em = row_exponent(mx, nan, mark, [&]() {
     long long f = 0;
@@ -154,49 +192,103 @@ __global__ void __launch_bounds__(256) k_term(const double* __restrict__ prod, d
     return f;
   });
   const int64_t r0 = (int64_t)z * 2 * N + n, r1 = r0 + N;
-  if (lane == 0) ex[r0] = ex[r1] = mark;
+  if (lane == 0) a.ex[r0] = a.ex[r1] = mark;
+  const uint32_t neg_re = a.conj ? 0u : 0x80008000u, neg_im = a.conj ? 0x80008000u : 0u;
 #pragma unroll
   for (int t = 0; t < NP; ++t) {
     const int k = 64 * t + 2 * lane;
     if (k >= M) break;
-    uint32_t a[2], b[2], c[2], d[2];
-    digit_bytes_of(x[t][0][0], em, mark >= kExpInf, a[0], a[1]);
-    digit_bytes_of(x[t][1][0], em, mark >= kExpInf, b[0], b[1]);
-    digit_bytes_of(x[t][0][1], em, mark >= kExpInf, c[0], c[1]);
-    digit_bytes_of(x[t][1][1], em, mark >= kExpInf, d[0], d[1]);
+    uint32_t b[2], c[2], d[2], e[2];
+    digit_bytes_of(x[t][0][0], em, mark >= kExpInf, b[0], b[1]);
+    digit_bytes_of(x[t][1][0], em, mark >= kExpInf, c[0], c[1]);
+    digit_bytes_of(x[t][0][1], em, mark >= kExpInf, d[0], d[1]);
+    digit_bytes_of(x[t][1][1], em, mark >= kExpInf, e[0], e[1]);
 #pragma unroll
     for (int j = 0; j < kDig; ++j) {
-      const uint32_t re = digit_pair(j, a, b), im = digit_pair(j, c, d);
-      uint32_t* p0 = reinterpret_cast<uint32_t*>(out + ((int64_t)j * rp + r0) * Kp + k);
-      uint32_t* p1 = reinterpret_cast<uint32_t*>(out + ((int64_t)j * rp + r1) * Kp + k);
+      const uint32_t re = digit_pair(j, b, c), im = digit_pair(j, d, e);
+      uint32_t* p0 = reinterpret_cast<uint32_t*>(a.dig + ((int64_t)j * a.rp + r0) * a.Kp + k);
+      uint32_t* p1 = reinterpret_cast<uint32_t*>(a.dig + ((int64_t)j * a.rp + r1) * a.Kp + k);
       *p0 = re;
       *p1 = im;
-      if (!stack) {
-        p0[M2 / 2] = im ^ 0x80008000u;
-        p1[M2 / 2] = re;
+      if (!a.stack) {
+        p0[a.M2 / 2] = im ^ neg_re;
+        p1[a.M2 / 2] = re ^ neg_im;
       }
     }
   }
 }
 
-template <bool FIRST>
-cudaError_t launch_term(const Ctx& c, const Plan& p, const double* prod, double* phi, int w0, int nw, double coef,
-                        int more, const DigitOp& b, cudaStream_t s) {
-  const int grid = (nw * c.N + 7) / 8, st = stacked(c.M), M2 = even(c.M);
-  switch ((c.M + 63) / 64) {
-#define AFQ_TERM(NP)                                                                                        \
-  case NP:                                                                                                  \
-    k_term<NP, FIRST><<<grid, 256, 0, s>>>(prod, phi, c.M, c.N, c.Nw, w0, nw, st, M2, coef, more, b.Kp, b.rp, \
-                                           b.dig, b.ex);                                                    \
-    break;
-    AFQ_TERM(1)
-    AFQ_TERM(2)
-    AFQ_TERM(3)
-    AFQ_TERM(4)
-#undef AFQ_TERM
+template <int KIND>
+cudaError_t launch_term(const TermArgs& a, cudaStream_t s) {
+  const int grid = (a.nw * a.N + 7) / 8;
+  switch ((a.M + 63) / 64) {
+    case 1: k_term<1, KIND><<<grid, 256, 0, s>>>(a); break;
+    case 2: k_term<2, KIND><<<grid, 256, 0, s>>>(a); break;
+    case 3: k_term<3, KIND><<<grid, 256, 0, s>>>(a); break;
+    case 4: k_term<4, KIND><<<grid, 256, 0, s>>>(a); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
+}
+
+// A chunk of walkers in the workspace: digits of A and of the terms, products.
+struct Chunk {
+  DigitOp a, b;
+  double* prod;
+  uint8_t* end;
+  DigitGemm g;
+  TermArgs t;
+};
+
+cudaError_t start_chunk(const Ctx& c, const F64Ws& ws, const Plan& p, int w0, int nw, Chunk& k, cudaStream_t s) {
+  k.a = digit_place(ws.buf, (int64_t)nw * p.R, p.K);
+  uint8_t* pb = ws.buf + digit_bytes((int64_t)nw * p.R, p.K);
+  k.b = digit_place(pb, (int64_t)nw * p.Cn, p.K);
+  k.prod = reinterpret_cast<double*>(pb + digit_bytes((int64_t)nw * p.Cn, p.K));
+  k.end = reinterpret_cast<uint8_t*>(k.prod) + (sizeof(double) * (size_t)nw * p.R * p.Cn + 255) / 256 * 256;
+  DigitGemm& g = k.g;
+  g.R = p.R;
+  g.Cn = p.Cn;
+  g.nz = nw;
+  g.rz = p.R;
+  g.cz = p.Cn;
+  g.out = k.prod;
+  g.ldc = p.R;
+  g.outz = (int64_t)p.R * p.Cn;
+  g.K = p.K;
+  g.err = ws.err;
+  k.t = TermArgs{k.prod, nullptr, nullptr, nullptr, 0.0, c.M, c.N, c.Nw, w0, nw, stacked(c.M), even(c.M),
+                 0, 1, k.b.Kp, k.b.rp, k.b.dig, k.b.ex};
+  k_vhs_digits<<<nw, 512, 0, s>>>(c.Avhs, c.P, c.M, c.Nw, w0, stacked(c.M), even(c.M), k.a.Kp, k.a.rp, k.a.dig,
+                                  k.a.ex);
+  cudaError_t e = cudaGetLastError();
+  // the columns' padding in K meets zero digits of A, but must be finite
+  if (e == cudaSuccess) e = cudaMemsetAsync(k.b.dig, 0, (size_t)k.b.rp * k.b.Kp * 2 * kDig, s);
+  return e;
+}
+
+// Terms of the Taylor series at orbital i, k = (n N + b) 2 + re / im: x[n][plane][w][b][i].
+struct TermRows {
+  const double* x;
+  int64_t nstride, plane;   // one term, one plane
+  int N, M, w0;
+  __device__ double at(int z, int i, int k) const {
+    const int p = k & 1, nb = k >> 1, n = nb / N, b = nb - n * N;
+    return x[n * nstride + p * plane + ((int64_t)(w0 + z) * N + b) * M + i];
+  }
+};
+
+// Abar of the walkers that are out of the reverse sweep
+__global__ void __launch_bounds__(256) k_zero_masked(double* __restrict__ Abar, const int* __restrict__ mask, int MM,
+                                                     int Nw) {
+  const int w = blockIdx.x;
+  if (mask[w]) return;
+  for (int p = 0; p < 2; ++p)
+    for (int e = threadIdx.x; e < MM; e += 256) Abar[((int64_t)p * Nw + w) * MM + e] = 0.0;
+}
+
+size_t outer_bytes(int M, int K2, int nw) {
+  return digit_bytes((int64_t)nw * M, K2) + digit_bytes(2 * (int64_t)nw * M, K2);
 }
 
 }  // namespace
@@ -226,35 +318,105 @@ cudaError_t launch_taylor_f64e(const Ctx& c, double* phi, cudaStream_t s) {
   const int order = c.opt.taylor_order;
   cudaError_t e = cudaSuccess;
   for (int w0 = 0; w0 < c.Nw && e == cudaSuccess; w0 += p.nw) {
-    const int nw = std::min(p.nw, c.Nw - w0);
-    const DigitOp a = digit_place(c.ws64.buf, (int64_t)nw * p.R, p.K);
-    uint8_t* pb = c.ws64.buf + digit_bytes((int64_t)nw * p.R, p.K);
-    const DigitOp b = digit_place(pb, (int64_t)nw * p.Cn, p.K);
-    double* prod = reinterpret_cast<double*>(pb + digit_bytes((int64_t)nw * p.Cn, p.K));
-    k_vhs_digits<<<nw, 512, 0, s>>>(c.Avhs, c.P, c.M, c.Nw, w0, stacked(c.M), even(c.M), a.Kp, a.rp, a.dig, a.ex);
-    if ((e = cudaGetLastError()) != cudaSuccess) break;
-    // the columns' padding in K meets zero digits of A, but must be finite
-    if ((e = cudaMemsetAsync(b.dig, 0, (size_t)b.rp * b.Kp * 2 * kDig, s)) != cudaSuccess) break;
-    if ((e = launch_term<true>(c, p, prod, phi, w0, nw, 0.0, 1, b, s)) != cudaSuccess) break;
-    double coef = 1.0;
+    Chunk k;
+    if ((e = start_chunk(c, c.ws64, p, w0, std::min(p.nw, c.Nw - w0), k, s)) != cudaSuccess) break;
+    k.t.in = phi;
+    if ((e = launch_term<kFirst>(k.t, s)) != cudaSuccess) break;
+    k.t.out = phi;
+    k.t.coef = 1.0;
     for (int m = 1; m <= order && e == cudaSuccess; ++m) {
-      DigitGemm g;
-      g.R = p.R;
-      g.Cn = p.Cn;
-      g.nz = nw;
-      g.rz = p.R;
-      g.cz = p.Cn;
-      g.out = prod;
-      g.ldc = p.R;
-      g.outz = (int64_t)p.R * p.Cn;
-      g.K = p.K;
-      g.err = c.ws64.err;
-      if ((e = digit_gemm(a, b, g, s)) != cudaSuccess) break;
-      coef /= m;
-      e = launch_term<false>(c, p, prod, phi, w0, nw, coef, m < order, b, s);
+      if ((e = digit_gemm(k.a, k.b, k.g, s)) != cudaSuccess) break;
+      k.t.coef /= m;
+      k.t.more = m < order;
+      e = launch_term<kSum>(k.t, s);
     }
   }
   return e;
+}
+
+size_t taylor_rev_f64e_ws(int M, int N, int Nw, int order) {
+  const Plan p = plan_of(M, N, Nw);
+  return taylor_f64e_ws(M, N, Nw) + outer_bytes(M, 2 * order * N, p.nw);
+}
+
+// Reverse of the Taylor series at the walkers' A (adj_taylor): with U_n = A^n Phi1 and
+//   V_order = Pbar2,  V_(n-1) = Pbar2 + conj(A) V_n / n,
+// pbar <- V_0 and Abar = sum_n V_n (U_(n-1) / n!)^H (u keeps U_(n-1) / n!), the last as one contraction over (n, b, re / im)
+// per walker.  u, v: [order][2][Nw][N][M] each.  Abar comes out transposed, [2][Nw][j][i], which its
+// only use, the trace with the symmetric L_g, does not see.  At M = 96, 12/12, 128 walkers, order 6:
+// 4.93 ms in the walker kernel (k_taylor_rev), 0.55 ms here.
+cudaError_t launch_taylor_rev_f64e(const Ctx& c, const F64Ws& ws, const double* phi1, double* pbar, double* u,
+                                   double* v, double* Abar, const int* mask, cudaStream_t s) {
+  const Plan p = plan_of(c.M, c.N, c.Nw);
+  const int order = c.opt.taylor_order, M = c.M, MM = M * M, K2 = 2 * order * c.N;
+  const int64_t nphi = 2 * (int64_t)c.Nw * c.N * M;
+  cudaError_t e = cudaSuccess;
+  for (int w0 = 0; w0 < c.Nw && e == cudaSuccess; w0 += p.nw) {
+    const int nw = std::min(p.nw, c.Nw - w0);
+    // U_0 and V_order of the chunk as they are
+    for (int q = 0; q < 2 && e == cudaSuccess; ++q) {
+      const int64_t o = ((int64_t)q * c.Nw + w0) * c.N * M;
+      const size_t by = sizeof(double) * (size_t)nw * c.N * M;
+      e = cudaMemcpyAsync(u + o, phi1 + o, by, cudaMemcpyDeviceToDevice, s);
+      if (e == cudaSuccess)
+        e = cudaMemcpyAsync(v + (order - 1) * nphi + o, pbar + o, by, cudaMemcpyDeviceToDevice, s);
+    }
+    Chunk k;
+    if (e != cudaSuccess || (e = start_chunk(c, ws, p, w0, nw, k, s)) != cudaSuccess) break;
+    k.t.in = phi1;
+    k.t.more = order > 1;
+    if ((e = launch_term<kFirst>(k.t, s)) != cudaSuccess) break;
+    k.t.coef = 1.0;
+    for (int m = 1; m < order && e == cudaSuccess; ++m) {
+      if ((e = digit_gemm(k.a, k.b, k.g, s)) != cudaSuccess) break;
+      k.t.coef /= m + 1;
+      k.t.out = u + m * nphi;
+      k.t.more = m + 1 < order;
+      e = launch_term<kKeep>(k.t, s);
+    }
+    k.t.conj = 1;
+    k.t.more = 1;
+    k.t.in = v + (order - 1) * nphi;
+    if (e == cudaSuccess) e = launch_term<kFirst>(k.t, s);
+    for (int n = order; n >= 1 && e == cudaSuccess; --n) {
+      if ((e = digit_gemm(k.a, k.b, k.g, s)) != cudaSuccess) break;
+      k.t.coef = 1.0 / n;
+      k.t.out = n > 1 ? v + (n - 2) * nphi : pbar;
+      k.t.mask = n > 1 ? nullptr : mask;
+      k.t.more = n > 1;
+      e = launch_term<kRev>(k.t, s);
+    }
+    if (e != cudaSuccess) break;
+    // V[(n-1)] holds V_n, u[(n-1)] U_(n-1): both at index n - 1
+    const DigitOp dv = digit_place(k.end, (int64_t)nw * M, K2);
+    const DigitOp du = digit_place(k.end + digit_bytes((int64_t)nw * M, K2), 2 * (int64_t)nw * M, K2);
+    const dim3 grid(nw, (M + 31) / 32);
+    const TermRows fv{v, nphi, nphi / 2, c.N, M, w0}, fu{u, nphi, nphi / 2, c.N, M, w0};
+    k_strided_digits<<<grid, 1024, 0, s>>>(fv, M, K2, dv.Kp, dv.rp, M, 0, reinterpret_cast<uint16_t*>(dv.dig), dv.ex);
+    if ((e = cudaGetLastError()) != cudaSuccess) break;
+    k_strided_digits<<<grid, 1024, 0, s>>>(fu, M, K2, du.Kp, du.rp, 2 * M, M, reinterpret_cast<uint16_t*>(du.dig), du.ex);
+    if ((e = cudaGetLastError()) != cudaSuccess) break;
+    for (int q = 0; q < 2 && e == cudaSuccess; ++q) {   // re: [U_r | U_i], im: [-U_i | U_r]
+      DigitOp dq = du;
+      dq.dig += (int64_t)q * M * du.Kp;
+      dq.ex += q * M;
+      dq.off = q * M;
+      DigitGemm g;
+      g.R = g.Cn = M;
+      g.nz = nw;
+      g.rz = M;
+      g.cz = 2 * M;
+      g.out = Abar + ((int64_t)q * c.Nw + w0) * MM;
+      g.ldc = M;
+      g.outz = MM;
+      g.K = K2;
+      g.err = ws.err;
+      e = digit_gemm(dv, dq, g, s);
+    }
+  }
+  if (e != cudaSuccess) return e;
+  k_zero_masked<<<c.Nw, 256, 0, s>>>(Abar, mask, MM, c.Nw);
+  return cudaGetLastError();
 }
 
 }  // namespace afq
