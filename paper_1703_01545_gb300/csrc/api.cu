@@ -85,6 +85,7 @@ void free_ctx(Ctx* h) {
   if (h->d_tc_err) cudaFree(h->d_tc_err);
   if (h->ws64.buf) cudaFree(h->ws64.buf);
   if (h->e64) cudaFree(h->e64);
+  if (h->e64_tan) cudaFree(h->e64_tan);
   for (double* b : {h->md_coef, h->md_psi, h->md_Ltil, h->md_htil, h->md_logO, h->md_theta,
                     h->md_share, h->md_rhobar, h->md_eloc})
     if (b) cudaFree(b);
@@ -1085,6 +1086,10 @@ afqmc_status afqmc_set_tangent(afqmc_handle h, const double* P, cudaStream_t s) 
     if ((st = dalloc(h, &h->daux, 4 * (size_t)Nw)) != AFQMC_OK) return st;
     if ((st = dalloc(h, &h->deloc, 2 * (size_t)Nw)) != AFQMC_OK) return st;
     if ((st = dalloc(h, &h->desum, 4 * (size_t)h->R)) != AFQMC_OK) return st;
+    if (h->e64 && cudaMalloc(&h->e64_tan, afq::energy_tan_f64e_scratch(*h)) != cudaSuccess) {
+      cudaGetLastError();
+      h->e64_tan = nullptr;   // the walker kernel then
+    }
   }
   AFQ_CK(afq::prepare_tangent_kernels(*h));
   double *dP = nullptr, *dE = nullptr;

@@ -129,6 +129,94 @@ __global__ void __launch_bounds__(128) k_energy_sum(const double* __restrict__ t
   }
 }
 
+// Tangent mode: beside ex and tr of T, the derivatives dex = sum_g sum_ab T_ab dT_ba (of half the
+// exchange sum) and dtr = sum_a dT_aa, from dT = Ltil dTheta in the same layout.
+__global__ void __launch_bounds__(kEx) k_exchange_tan(const double* __restrict__ T, const double* __restrict__ dT,
+                                                      int64_t ldt, int ns, int X, int w0, int Nw, int gb,
+                                                      double* __restrict__ ex, double* __restrict__ tr) {
+  extern __shared__ double sm[];
+  __shared__ double red[4 * (kEx / 32)];
+  const int wl = blockIdx.x, nwc = gridDim.x, q = blockIdx.y, tid = threadIdx.x, w = w0 + wl;
+  const int g0 = (int)((int64_t)X * q / gridDim.y), g1 = (int)((int64_t)X * (q + 1) / gridDim.y);
+  const int nsq = ns * ns, gs = gb + 1, pl = nsq * gs;   // planes: T re, T im, dT re, dT im
+  const int lg = tid & (gb - 1), slot = tid / gb, nslot = kEx / gb;
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int gc = g0; gc < g1; gc += gb) {
+    const int ng = min(gb, g1 - gc), len = ng * ns;
+    __syncthreads();
+    for (int col = tid >> 5; col < 4 * ns; col += kEx / 32) {
+      const int pp = col / ns, b = col - pp * ns;
+      const double* src = (pp >= 2 ? dT : T) + ((int64_t)((pp & 1) * nwc + wl) * ns + b) * ldt + (int64_t)gc * ns;
+      for (int k = tid & 31; k < len; k += 32) {
+        const int g = k / ns;
+        sm[(col * ns + k - g * ns) * gs + g] = src[k];
+      }
+    }
+    __syncthreads();
+    if (lg < ng)
+      for (int r = slot; r < nsq; r += nslot) {
+        const int b = r / ns, a = r - b * ns;
+        const double* xy = sm + r * gs + lg;               // (a, b)
+        const double* yx = sm + (a * ns + b) * gs + lg;    // (b, a)
+        const double xr = xy[0], xi = xy[pl], dr = yx[2 * pl], di = yx[3 * pl];
+        acc[2] = fma(xr, dr, fma(-xi, di, acc[2]));
+        acc[3] = fma(xr, di, fma(xi, dr, acc[3]));
+        if (a <= b) {
+          const double f = a == b ? 1.0 : 2.0, yr = f * yx[0], yi = f * yx[pl];
+          acc[0] = fma(xr, yr, fma(-xi, yi, acc[0]));
+          acc[1] = fma(xr, yi, fma(xi, yr, acc[1]));
+        }
+      }
+    for (int e = tid; e < 4 * ng; e += kEx) {
+      const int p = e / ng, g = e - p * ng;
+      double t = 0.0;
+      for (int a = 0; a < ns; ++a) t += sm[p * pl + (a * ns + a) * gs + g];
+      tr[((int64_t)p * Nw + w) * X + gc + g] = t;
+    }
+  }
+  block_sum<4>(acc, red);
+  if (tid == 0)
+    for (int p = 0; p < 4; ++p) ex[((int64_t)q * 4 + p) * Nw + w] = acc[p];
+}
+
+// E_L and dE_L of a walker; tr[spin][4][w][g], ex[spin][range][4][w] as above
+__global__ void __launch_bounds__(128) k_energy_sum_tan(const double* __restrict__ theta, const double* __restrict__ dtheta,
+                                                        const double* __restrict__ htil, const double* __restrict__ htilP,
+                                                        const double* __restrict__ tr, const double* __restrict__ ex,
+                                                        int nspin, int nsplit, int NM, int X, int Nw,
+                                                        double* __restrict__ eloc, double* __restrict__ deloc) {
+  __shared__ double red[4 * 4];
+  const int w = blockIdx.x;
+  const int64_t plane = (int64_t)Nw * NM, base = (int64_t)w * NM, tp = (int64_t)Nw * X;
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int e = threadIdx.x; e < NM; e += 128) {
+    const double h = __ldg(htil + e), hp = __ldg(htilP + e), vr = theta[base + e], vi = theta[plane + base + e];
+    acc[0] = fma(h, vr, acc[0]);
+    acc[1] = fma(h, vi, acc[1]);
+    acc[2] = fma(hp, vr, fma(h, dtheta[base + e], acc[2]));
+    acc[3] = fma(hp, vi, fma(h, dtheta[plane + base + e], acc[3]));
+  }
+  for (int g = threadIdx.x; g < X; g += 128) {
+    double c[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int s = 0; s < nspin; ++s)
+      for (int p = 0; p < 4; ++p) c[p] += tr[(4 * s + p) * tp + (int64_t)w * X + g];
+    acc[0] = fma(0.5 * c[0], c[0], fma(-0.5 * c[1], c[1], acc[0]));
+    acc[1] = fma(c[0], c[1], acc[1]);
+    acc[2] = fma(c[0], c[2], fma(-c[1], c[3], acc[2]));
+    acc[3] = fma(c[0], c[3], fma(c[1], c[2], acc[3]));
+  }
+  block_sum<4>(acc, red);
+  if (threadIdx.x == 0) {
+    double x[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int q = 0; q < nspin * nsplit; ++q)
+      for (int p = 0; p < 4; ++p) x[p] += ex[((int64_t)q * 4 + p) * Nw + w];
+    eloc[w] = acc[0] - 0.5 * x[0];
+    eloc[Nw + w] = acc[1] - 0.5 * x[1];
+    deloc[w] = acc[2] - x[2];
+    deloc[Nw + w] = acc[3] - x[3];
+  }
+}
+
 // Ltil rows (g, b) of a spin as columns: element (orbital i, k = g ns + b)
 struct LtilColumns {
   const double* ltil;
@@ -259,6 +347,10 @@ size_t energy_f64e_scratch(const Ctx& c) {
   const size_t t = 2 * (size_t)c.X * ns * ns * chunk_walkers(c);
   return sizeof(double) * (t + 4 * (size_t)c.Nw * c.X + 4 * (size_t)kMaxSplit * c.Nw);
 }
+// tangent mode: traces of T and dT of both spins and their exchange sums (T and dT share the T chunk)
+size_t energy_tan_f64e_scratch(const Ctx& c) {
+  return sizeof(double) * (8 * (size_t)c.Nw * c.X + 8 * (size_t)kMaxSplit * c.Nw);
+}
 size_t energy_f64e_ws(const Ctx& c) {
   const int ns = std::max(c.n_up, c.N - c.n_up);
   return digit_bytes((int64_t)c.X * ns, c.M) + digit_bytes(2 * (int64_t)chunk_walkers(c) * ns, c.M);
@@ -266,10 +358,9 @@ size_t energy_f64e_ws(const Ctx& c) {
 
 namespace {
 
-// T of one spin for walkers w0 .. w0 + nw - 1, and from it the exchange sums and traces (spin index
-// sp); `cols` memory for the columns' digits
-cudaError_t chunk_of(const Ctx& c, const F64Ws& ws, const double* theta, const DigitOp& da, void* cols, int sp, int n0,
-                     int ns, int w0, int nw, int nsplit, double* T, double* tr, double* ex, cudaStream_t s) {
+// T of one spin for walkers w0 .. w0 + nw - 1; `cols` memory for the columns' digits
+cudaError_t products_of(const Ctx& c, const F64Ws& ws, const double* theta, const DigitOp& da, void* cols, int n0,
+                        int ns, int w0, int nw, double* T, cudaStream_t s) {
   const int NM = c.N * c.M, nc = 2 * nw * ns, rows = c.X * ns;
   const DigitOp db = digit_place(cols, nc, c.M);
   for (int p = 0; p < 2; ++p) {
@@ -286,16 +377,62 @@ cudaError_t chunk_of(const Ctx& c, const F64Ws& ws, const double* theta, const D
   g.ldc = rows;
   g.K = c.M;
   g.err = ws.err;
-  const cudaError_t e = digit_gemm(da, db, g, s);
-  if (e != cudaSuccess) return e;
+  return digit_gemm(da, db, g, s);
+}
+
+// Cholesky vectors staged at a time by the exchange kernels: a power of two within kStage
+int staged(int ns, int planes) {
   int gb = 32;
-  while (gb > 1 && (size_t)2 * ns * ns * (gb + 1) * sizeof(double) > kStage) gb /= 2;
+  while (gb > 1 && (size_t)planes * ns * ns * (gb + 1) * sizeof(double) > kStage) gb /= 2;
+  return gb;
+}
+
+// T of a spin and from it the exchange sums and traces (spin index sp)
+cudaError_t chunk_of(const Ctx& c, const F64Ws& ws, const double* theta, const DigitOp& da, void* cols, int sp, int n0,
+                     int ns, int w0, int nw, int nsplit, double* T, double* tr, double* ex, cudaStream_t s) {
+  const cudaError_t e = products_of(c, ws, theta, da, cols, n0, ns, w0, nw, T, s);
+  if (e != cudaSuccess) return e;
+  const int gb = staged(ns, 2);
   k_exchange<<<dim3(nw, nsplit), kEx, (size_t)2 * ns * ns * (gb + 1) * sizeof(double), s>>>(
-      T, rows, ns, c.X, w0, c.Nw, gb, ex + (size_t)sp * nsplit * 2 * c.Nw, tr + (size_t)sp * 2 * c.Nw * c.X);
+      T, c.X * ns, ns, c.X, w0, c.Nw, gb, ex + (size_t)sp * nsplit * 2 * c.Nw, tr + (size_t)sp * 2 * c.Nw * c.X);
   return cudaGetLastError();
 }
 
 }  // namespace
+
+// E_L and dE_L of every walker from Theta and dTheta (tangent mode)
+cudaError_t launch_energy_tan_f64e(const Ctx& c, cudaStream_t s) {
+  const int NM = c.N * c.M, nwc = std::max(1, chunk_walkers(c) / 2), nsmax = std::max(c.n_up, c.N - c.n_up);
+  const int nsplit = splits(c, nwc);
+  double* T = c.e64;
+  double* dT = T + 2 * (size_t)c.X * nsmax * nsmax * nwc;
+  double* tr = c.e64_tan;
+  double* ex = tr + 8 * (size_t)c.Nw * c.X;
+  cudaError_t e = cudaSuccess;
+  int sp = 0;
+  for (int s0 = 0; s0 < 2 && e == cudaSuccess; ++s0) {
+    const int n0 = s0 ? c.n_up : 0, ns = s0 ? c.N - c.n_up : c.n_up;
+    if (ns == 0) continue;
+    const DigitOp da = digit_place(c.ws64.buf, c.X * ns, c.M);
+    uint8_t* cols = c.ws64.buf + digit_bytes(c.X * ns, c.M);
+    e = digits_of(c.Ltil, c.M, c.X * ns, c.M, da, s, ns, c.N, n0);
+    for (int w0 = 0; w0 < c.Nw && e == cudaSuccess; w0 += nwc) {
+      const int nw = std::min(nwc, c.Nw - w0), gb = staged(ns, 4);
+      e = products_of(c, c.ws64, c.theta, da, cols, n0, ns, w0, nw, T, s);
+      if (e == cudaSuccess) e = products_of(c, c.ws64, c.dtheta, da, cols, n0, ns, w0, nw, dT, s);
+      if (e != cudaSuccess) break;
+      k_exchange_tan<<<dim3(nw, nsplit), kEx, (size_t)4 * ns * ns * (gb + 1) * sizeof(double), s>>>(
+          T, dT, c.X * ns, ns, c.X, w0, c.Nw, gb, ex + (size_t)sp * nsplit * 4 * c.Nw,
+          tr + (size_t)sp * 4 * c.Nw * c.X);
+      e = cudaGetLastError();
+    }
+    ++sp;
+  }
+  if (e != cudaSuccess) return e;
+  k_energy_sum_tan<<<c.Nw, 128, 0, s>>>(c.theta, c.dtheta, c.htil, c.htilP, tr, ex, sp, nsplit, NM, c.X, c.Nw, c.eloc,
+                                        c.deloc);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_energy_f64e(const Ctx& c, cudaStream_t s) {
   const int NM = c.N * c.M, nwc = chunk_walkers(c), nsmax = std::max(c.n_up, c.N - c.n_up);

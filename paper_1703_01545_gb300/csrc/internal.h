@@ -118,6 +118,7 @@ struct Ctx {
   int tune_taylor_smem = -1;  // propagation: 2 fused kernel; Taylor kernel with A in shared memory (1) or L1 (0)
   int tune_mgs = -1;          // orthonormalisation: 1 Cholesky QR, 0 modified Gram-Schmidt kernels
   int taylor_dig = 0;         // 1: the FP64 Taylor products in digit form (ws64 has the room)
+  double* e64_tan = nullptr;  // traces and exchange sums of the tangent local energy in digit form
   double* e64 = nullptr;      // scratch of the FP64 local energy in digit form
   F64Ws ws64;                 // digits of the FP64 contractions' operands (FP64 handles)
   // tangent mode (tangent.cu): derivative along h1 -> h1 + lambda P, FP64 path only
@@ -200,10 +201,14 @@ cudaError_t launch_taylor_f64e(const Ctx& c, double* phi, cudaStream_t s);
 bool energy_f64e_ok(int M, int X, int n_up, int n_dn, int Nw);
 size_t energy_f64e_scratch(const Ctx& c);
 size_t energy_f64e_ws(const Ctx& c);
+size_t energy_tan_f64e_scratch(const Ctx& c);   // beside c.e64, for tangent mode (c.e64_tan)
+cudaError_t launch_energy_tan_f64e(const Ctx& c, cudaStream_t s);
 cudaError_t launch_energy_f64e(const Ctx& c, cudaStream_t s);
 cudaError_t digit_gemm(const DigitOp& rows, const DigitOp& cols, const DigitGemm& g, cudaStream_t s);
 cudaError_t digit_gemm_sum(const DigitOp& rows, const DigitOp& cols, DigitGemm g, double* part, size_t part_bytes,
                            cudaStream_t s);
+bool taylor_tan_f64e_ok(const Ctx& c);
+cudaError_t launch_taylor_tan_f64e(const Ctx& c, double* phi, double* dphi, cudaStream_t s);
 size_t taylor_rev_f64e_ws(int M, int N, int Nw, int order);
 cudaError_t launch_taylor_rev_f64e(const Ctx& c, const F64Ws& ws, const double* phi1, double* pbar, double* u,
                                    double* v, double* Abar, const int* mask, cudaStream_t s);

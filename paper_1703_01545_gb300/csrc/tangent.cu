@@ -649,6 +649,7 @@ cudaError_t launch_fields_tan(const Ctx& c, const double* fields, cudaStream_t s
 }
 
 cudaError_t launch_taylor_tan(const Ctx& c, cudaStream_t s) {
+  if (taylor_tan_f64e_ok(c)) return launch_taylor_tan_f64e(c, c.phi2, c.dphi2, s);
   k_taylor_tan<<<c.Nw, kT, smem_taylor_tan(c), s>>>(c.phi2, c.dphi2, c.Avhs, c.dAvhs, c.M, c.N,
                                                     c.Nw, c.P, c.opt.taylor_order);
   return cudaGetLastError();
@@ -673,6 +674,7 @@ cudaError_t launch_mgs_tan(const Ctx& c, cudaStream_t s) {
 }
 
 cudaError_t launch_energy_tan(const Ctx& c, cudaStream_t s) {
+  if (c.e64 && c.e64_tan) return launch_energy_tan_f64e(c, s);
   k_energy_tan<<<c.Nw, kT, smem_energy_tan(c), s>>>(c.theta, c.dtheta, c.Ltil, c.htil, c.htilP,
                                                     c.eloc, c.deloc, c.M, c.N, c.n_up, c.X, c.Nw);
   return cudaGetLastError();

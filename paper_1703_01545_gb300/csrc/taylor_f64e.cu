@@ -231,6 +231,88 @@ cudaError_t launch_term(const TermArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// Tangent mode: U = A U' and dU = dA U' + A dU' of a round; products of [U' | dU'] with A ([z][4 N][R])
+// and of U' with dA ([z][2 N][R]).  FIRST: U = Phi, dU = dPhi; else Phi += coef U, dPhi += coef dU.
+// Columns of a walker: U's real, U's imaginary, dU's real, dU's imaginary ones.
+template <int NP, bool FIRST>
+__global__ void __launch_bounds__(256) k_term_tan(const double* __restrict__ prod, const double* __restrict__ dprod,
+                                                  double* __restrict__ phi, double* __restrict__ dphi, int M, int N,
+                                                  int Nw, int w0, int nw, int stack, int M2, double coef, int more,
+                                                  int Kp, int64_t rp, __nv_bfloat16* __restrict__ out,
+                                                  int* __restrict__ ex) {
+  const int task = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (task >= 2 * nw * N) return;
+  const int d = task & 1, zn = task >> 1, z = zn / N, n = zn - z * N, R = stack ? 2 * M : M;   // d = 1: dU
+  const int64_t base = ((int64_t)(w0 + z) * N + n) * M, plane = (int64_t)Nw * N * M;
+  double* x0 = d ? dphi : phi;
+  const double* pr = prod + ((int64_t)z * 4 * N + d * 2 * N + n) * R;
+  const double* pi = pr + (int64_t)N * R;
+  const double* qr = dprod + ((int64_t)z * 2 * N + n) * R;
+  const double* qi = qr + (int64_t)N * R;
+  double x[NP][2][2];
+  uint32_t mx = 0, nan = 0;
+#pragma unroll
+  for (int t = 0; t < NP; ++t)
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int i = 64 * t + 2 * lane + q;
+      double re = 0.0, im = 0.0;
+      if (i < M) {
+        if (FIRST) {
+          re = x0[base + i];
+          im = x0[plane + base + i];
+        } else {
+          re = stack ? pr[i] - pi[M + i] : pr[i];
+          im = stack ? pi[i] + pr[M + i] : pi[i];
+          if (d) {
+            re += stack ? qr[i] - qi[M + i] : qr[i];
+            im += stack ? qi[i] + qr[M + i] : qi[i];
+          }
+          x0[base + i] = fma(coef, re, x0[base + i]);
+          x0[plane + base + i] = fma(coef, im, x0[plane + base + i]);
+        }
+      }
+      x[t][q][0] = re;
+      x[t][q][1] = im;
+      row_scan(re, mx, nan);
+      row_scan(im, mx, nan);
+    }
+  if (!more) return;
+  int mark;
+  const int em = row_exponent(mx, nan, mark, [&]() {
+    long long f = 0;
+#pragma unroll
+    for (int t = 0; t < NP; ++t)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) f = max(f, fraction_of(x[t][q >> 1][q & 1]));
+    return f;
+  });
+  const int64_t r0 = (int64_t)z * 4 * N + d * 2 * N + n, r1 = r0 + N;
+  if (lane == 0) ex[r0] = ex[r1] = mark;
+#pragma unroll
+  for (int t = 0; t < NP; ++t) {
+    const int k = 64 * t + 2 * lane;
+    if (k >= M) break;
+    uint32_t a[2], b[2], c[2], e[2];
+    digit_bytes_of(x[t][0][0], em, mark >= kExpInf, a[0], a[1]);
+    digit_bytes_of(x[t][1][0], em, mark >= kExpInf, b[0], b[1]);
+    digit_bytes_of(x[t][0][1], em, mark >= kExpInf, c[0], c[1]);
+    digit_bytes_of(x[t][1][1], em, mark >= kExpInf, e[0], e[1]);
+#pragma unroll
+    for (int j = 0; j < kDig; ++j) {
+      const uint32_t re = digit_pair(j, a, b), im = digit_pair(j, c, e);
+      uint32_t* p0 = reinterpret_cast<uint32_t*>(out + ((int64_t)j * rp + r0) * Kp + k);
+      uint32_t* p1 = reinterpret_cast<uint32_t*>(out + ((int64_t)j * rp + r1) * Kp + k);
+      *p0 = re;
+      *p1 = im;
+      if (!stack) {
+        p0[M2 / 2] = im ^ 0x80008000u;
+        p1[M2 / 2] = re;
+      }
+    }
+  }
+}
+
 // A chunk of walkers in the workspace: digits of A and of the terms, products.
 struct Chunk {
   DigitOp a, b;
@@ -329,6 +411,93 @@ cudaError_t launch_taylor_f64e(const Ctx& c, double* phi, cudaStream_t s) {
       k.t.coef /= m;
       k.t.more = m < order;
       e = launch_term<kSum>(k.t, s);
+    }
+  }
+  return e;
+}
+
+namespace {
+// bytes of the workspace a walker takes in tangent mode: digits of A, dA and four sets of columns
+// (each with its padding to 128 rows over the chunk, below), products
+size_t tan_per(const Plan& p) {
+  return (size_t)(2 * p.R + 2 * p.Cn) * ((size_t)pad64(p.K) * 2 * kDig + 4) + sizeof(double) * 3 * (size_t)p.R * p.Cn;
+}
+int tan_chunk(const Ctx& c, const Plan& p) {
+  const size_t pad = 3 * digit_bytes(128, p.K) + 4096;
+  if (!c.ws64.buf || c.ws64.bytes <= pad) return 0;
+  return (int)std::min<size_t>((size_t)c.Nw, (c.ws64.bytes - pad) / tan_per(p));
+}
+}  // namespace
+
+// Where the plain series runs in digit form and the handle's workspace holds a chunk of some size.
+bool taylor_tan_f64e_ok(const Ctx& c) {
+  if (!c.taylor_dig || !taylor_f64e_ok(c.M, c.N, c.Nw, c.opt.taylor_order)) return false;
+  return tan_chunk(c, plan_of(c.M, c.N, c.Nw)) >= std::min(c.Nw, 38);
+}
+
+// Phi <- T_n(A) Phi and dPhi <- its derivative along dA and dPhi, in place.
+cudaError_t launch_taylor_tan_f64e(const Ctx& c, double* phi, double* dphi, cudaStream_t s) {
+  const Plan p = plan_of(c.M, c.N, c.Nw);
+  const int nwc = tan_chunk(c, p), order = c.opt.taylor_order, M2 = even(c.M), st = stacked(c.M);
+  cudaError_t e = cudaSuccess;
+  for (int w0 = 0; w0 < c.Nw && e == cudaSuccess; w0 += nwc) {
+    const int nw = std::min(nwc, c.Nw - w0), cn = 2 * p.Cn;
+    uint8_t* at = c.ws64.buf;
+    DigitOp a[2];
+    for (int q = 0; q < 2 && e == cudaSuccess; ++q) {
+      a[q] = digit_place(at, (int64_t)nw * p.R, p.K);
+      at += digit_bytes((int64_t)nw * p.R, p.K);
+      k_vhs_digits<<<nw, 512, 0, s>>>(q ? c.dAvhs : c.Avhs, c.P, c.M, c.Nw, w0, st, M2, a[q].Kp, a[q].rp, a[q].dig,
+                                      a[q].ex);
+      e = cudaGetLastError();
+    }
+    const DigitOp b = digit_place(at, (int64_t)nw * cn, p.K);
+    at += digit_bytes((int64_t)nw * cn, p.K);
+    double* prod = reinterpret_cast<double*>(at);
+    double* dprod = prod + (size_t)nw * p.R * cn;
+    if (e == cudaSuccess) e = cudaMemsetAsync(b.dig, 0, (size_t)b.rp * b.Kp * 2 * kDig, s);
+    auto term = [&](bool first, double coef, int more) -> cudaError_t {
+      const int grid = (2 * nw * c.N + 7) / 8;
+#define AFQ_TERM(NP)                                                                                             \
+  case NP:                                                                                                       \
+    if (first)                                                                                                   \
+      k_term_tan<NP, true><<<grid, 256, 0, s>>>(prod, dprod, phi, dphi, c.M, c.N, c.Nw, w0, nw, st, M2, coef, more, \
+                                                b.Kp, b.rp, b.dig, b.ex);                                        \
+    else                                                                                                         \
+      k_term_tan<NP, false><<<grid, 256, 0, s>>>(prod, dprod, phi, dphi, c.M, c.N, c.Nw, w0, nw, st, M2, coef,   \
+                                                 more, b.Kp, b.rp, b.dig, b.ex);                                 \
+    break;
+      switch ((c.M + 63) / 64) {
+        AFQ_TERM(1)
+        AFQ_TERM(2)
+        AFQ_TERM(3)
+        AFQ_TERM(4)
+        default: return cudaErrorInvalidValue;
+      }
+#undef AFQ_TERM
+      return cudaGetLastError();
+    };
+    if (e != cudaSuccess || (e = term(true, 0.0, 1)) != cudaSuccess) break;
+    double coef = 1.0;
+    for (int m = 1; m <= order && e == cudaSuccess; ++m) {
+      DigitGemm g;
+      g.R = p.R;
+      g.Cn = cn;
+      g.nz = nw;
+      g.rz = p.R;
+      g.cz = cn;
+      g.out = prod;
+      g.ldc = p.R;
+      g.outz = (int64_t)p.R * cn;
+      g.K = p.K;
+      g.err = c.ws64.err;
+      if ((e = digit_gemm(a[0], b, g, s)) != cudaSuccess) break;
+      g.Cn = p.Cn;
+      g.out = dprod;
+      g.outz = (int64_t)p.R * p.Cn;
+      if ((e = digit_gemm(a[1], b, g, s)) != cudaSuccess) break;
+      coef /= m;
+      e = term(false, coef, m < order);
     }
   }
   return e;
