@@ -54,6 +54,17 @@ bool is_device_ptr(const void* p) {
   return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// Memory of the current device itself: kernels may read and write it in place of a staged copy.
+bool is_local_device_ptr(const void* p) {
+  cudaPointerAttributes a;
+  int dev = -1;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == dev;
+}
+
 void free_ctx(Ctx* h) {
   afq::destroy_pair_cache(h);
   double* bufs[] = {h->h1, h->L, h->Lt, h->Ltil, h->htil, h->psi, h->expK, h->rho_mf, h->phi,
@@ -85,6 +96,7 @@ void free_ctx(Ctx* h) {
   if (h->d_tc_err) cudaFree(h->d_tc_err);
   if (h->ws64.buf) cudaFree(h->ws64.buf);
   if (h->e64) cudaFree(h->e64);
+  if (h->ov_O) cudaFree(h->ov_O);
   if (h->e64_tan) cudaFree(h->e64_tan);
   for (double* b : {h->md_coef, h->md_psi, h->md_Ltil, h->md_htil, h->md_logO, h->md_theta,
                     h->md_share, h->md_rhobar, h->md_eloc})
@@ -152,6 +164,19 @@ afqmc_status setup_mixed(Ctx* h, cudaStream_t s) {
   if ((st = dalloc(h, &h->rhobar32, 2 * (size_t)Nw * X)) != AFQMC_OK) return st;
   if ((st = dalloc(h, &h->rho_mf32, (size_t)X)) != AFQMC_OK) return st;
   AFQ_CK(cudaMemsetAsync(h->d_tc_err, 0, sizeof(int), s));
+  if (afq::fast_walker_kernels_ok(*h) && afq::refresh_f64e_ok(*h)) {
+    // without the memory the refresh sums run in its kernel
+    const size_t nu = h->n_up, nd = N - h->n_up, need = afq::refresh_f64e_ws(*h);
+    AFQ_CK(afq::prepare_gemm_f64e());
+    if (cudaMalloc(&h->ws64.buf, need) != cudaSuccess) {
+      h->ws64.buf = nullptr;
+    } else {
+      h->ws64.bytes = need;
+      h->ws64.err = h->d_tc_err;
+      if (cudaMalloc(&h->ov_O, sizeof(double) * 2 * Nw * (nu * nu + nd * nd)) != cudaSuccess) h->ov_O = nullptr;
+    }
+    cudaGetLastError();
+  }
   // L as rows ij with g contiguous: transpose [X][M*M] -> [M*M][X] through phi2 (large enough
   // only when 2*Nw*N*M >= X*M*M; otherwise a temporary)
   double* tmp = nullptr;
@@ -747,9 +772,13 @@ afqmc_status afqmc_set_walkers(afqmc_handle h, const double* phi, const double* 
   if (!h) return AFQMC_ERR_ARG;
   if (!phi) return set_err(h, AFQMC_ERR_ARG, "phi is NULL");
   const int64_t n = 2 * (int64_t)h->Nw * h->N * h->M;
-  // stage the external layout in theta, convert into phi
-  AFQ_CK(cudaMemcpyAsync(h->theta, phi, sizeof(double) * n, cudaMemcpyDefault, s));
-  AFQ_CK(afq::launch_phi_layout(h->theta, h->phi, h->Nw, h->M, h->N, 1, s));
+  // the external layout (of other memory: staged in theta) into phi
+  const double* in = phi;
+  if (!is_local_device_ptr(phi)) {
+    AFQ_CK(cudaMemcpyAsync(h->theta, phi, sizeof(double) * n, cudaMemcpyDefault, s));
+    in = h->theta;
+  }
+  AFQ_CK(afq::launch_phi_layout(in, h->phi, h->Nw, h->M, h->N, 1, s));
   const double* wd = nullptr;
   if (w) {
     AFQ_CK(cudaMemcpyAsync(h->eloc, w, sizeof(double) * 2 * h->Nw, cudaMemcpyDefault, s));
@@ -819,8 +848,9 @@ afqmc_status afqmc_get_state(afqmc_handle h, double* phi, double* logO, double* 
   if (!h) return AFQMC_ERR_ARG;
   if (phi) {
     const int64_t n = 2 * (int64_t)h->Nw * h->N * h->M;
-    AFQ_CK(afq::launch_phi_layout(h->phi, h->phi2, h->Nw, h->M, h->N, 0, s));
-    AFQ_CK(cudaMemcpyAsync(phi, h->phi2, sizeof(double) * n, cudaMemcpyDefault, s));
+    const bool local = is_local_device_ptr(phi);
+    AFQ_CK(afq::launch_phi_layout(h->phi, local ? phi : h->phi2, h->Nw, h->M, h->N, 0, s));
+    if (!local) AFQ_CK(cudaMemcpyAsync(phi, h->phi2, sizeof(double) * n, cudaMemcpyDefault, s));
   }
   if (logO) AFQ_CK(cudaMemcpyAsync(logO, h->logO, sizeof(double) * 2 * h->Nw, cudaMemcpyDefault, s));
   if (w) AFQ_CK(cudaMemcpyAsync(w, h->w, sizeof(double) * 2 * h->Nw, cudaMemcpyDefault, s));

@@ -118,6 +118,7 @@ struct Ctx {
   int tune_taylor_smem = -1;  // propagation: 2 fused kernel; Taylor kernel with A in shared memory (1) or L1 (0)
   int tune_mgs = -1;          // orthonormalisation: 1 Cholesky QR, 0 modified Gram-Schmidt kernels
   int taylor_dig = 0;         // 1: the FP64 Taylor products in digit form (ws64 has the room)
+  double* ov_O = nullptr;     // split precision: FP64 overlap sums of a refresh [spin][a][(p, w, b)]
   double* e64_tan = nullptr;  // traces and exchange sums of the tangent local energy in digit form
   double* e64 = nullptr;      // scratch of the FP64 local energy in digit form
   F64Ws ws64;                 // digits of the FP64 contractions' operands (FP64 handles)
@@ -329,6 +330,9 @@ cudaError_t prepare_fast_walker_kernels(const Ctx& c);
 cudaError_t launch_overlap_fast(const Ctx& c, const double* src, int mode, cudaStream_t s,
                                 const float* src32 = nullptr, bool with_weights = true);
 // FP64 overlaps with spin blocks of at most 16 (walker_fast.cu); c.ovdet: [Nd or 1][Nw][8]
+// overlap sums of a split-precision refresh in digit form (c.ov_O, c.ws64)
+bool refresh_f64e_ok(const Ctx& c);
+size_t refresh_f64e_ws(const Ctx& c);
 bool overlap64_ok(const Ctx& c);
 cudaError_t prepare_overlap64(const Ctx& c);
 cudaError_t launch_overlap64(const Ctx& c, const double* src, int mode, cudaStream_t s);

@@ -52,6 +52,7 @@ struct FastOvArgs {
   double* theta64;    // FP64 form (k_overlap64): Theta
   // mode OV_DET (grid row d = determinant d): psi, Theta, log O and det of d start d * det_* on
   int64_t det_psi, det_theta, det_logO, det_det;
+  const double* O;    // FP64 overlap sums [spin][a][(p, w, b)] (refresh), or null: summed here
   int fp64_copy;      // 1: Phi also staged in FP64 shared memory (every mode but the FP32 update)
   double log_shift;
 };
@@ -206,11 +207,11 @@ __global__ void __launch_bounds__(256) k_overlap_fast(FastOvArgs a) {
   const int lane = tid & 31, warp = tid >> 5;
   double* pr = smo;            // [N][MP] (only when a.fp64_copy: the FP64 overlap sums)
   double* pi = pr + NMP;       // [N][MP]
-  double* aug = a.fp64_copy ? pi + NMP : smo;   // LU factors: spin s at aug + s * SPB, re, im [NSM][LDA]
+  double* aug = a.fp64_copy ? pi + NMP : smo;   // LU factors (at smo too when O is given): spin s at aug + s * SPB, re, im [NSM][LDA]
   // FP32 copies for Theta: converting once here keeps double->float conversions (which run
   // on the FP64 pipe) off the Theta loop
-  float* pfr = a.fp64_copy ? reinterpret_cast<float*>(aug + 2 * SPB)   // [N][MP]
-                           : reinterpret_cast<float*>(smo);
+  float* pfr = a.fp64_copy || a.O ? reinterpret_cast<float*>(aug + 2 * SPB)   // [N][MP]
+                                  : reinterpret_cast<float*>(smo);
   float* pfi = pfr + NMP;
   float* invf = pfi + NMP;     // spin s at invf + s * 2 * 16 * 16: re [16][16], im [16][16]
   __shared__ double s_det[2][2];   // per spin: determinant mantissa (re, im) ...
@@ -263,17 +264,28 @@ __global__ void __launch_bounds__(256) k_overlap_fast(FastOvArgs a) {
         a.phi[wbase + e] = xr;
         a.phi[plane + wbase + e] = xi;
       }
-      pr[es] = xr;               // the FP64 copy feeds the FP64 overlap sums
-      pi[es] = xi;
-      pfr[es] = (float)xr;
-      pfi[es] = (float)xi;
+      if (a.fp64_copy) {
+        pr[es] = xr;             // the FP64 copy feeds the FP64 overlap sums
+        pi[es] = xi;
+      }
+      pfr[es] = f64_to_f32_rn(xr);   // on the integer pipe
+      pfi[es] = f64_to_f32_rn(xi);
     }
   }
   if (tid < 2) { s_det[tid][0] = 1.0; s_det[tid][1] = 0.0; s_dexp[tid] = 0; s_bad[tid] = 0; }
   __syncthreads();
   // O_s[a][b] = sum_i psi[n0+a][i] phi[n0+b][i]; 4 threads per entry, shuffle-combined
   const int nu = a.n_up, nd = N - nu, nn = nu * nu + nd * nd;
-  for (int base = 0; base < nn * 4; base += blockDim.x) {
+  if (a.O)
+    for (int e = tid; e < nn; e += blockDim.x) {
+      const bool dn = e >= nu * nu;
+      const int ns = dn ? nd : nu, r = (dn ? e - nu * nu : e) / ns, c = (dn ? e - nu * nu : e) % ns;
+      const double* o = a.O + (dn ? 2 * (int64_t)a.Nw * nu * nu : 0) + (int64_t)r * 2 * a.Nw * ns + c;
+      double* ar = aug + (dn ? SPB : 0);
+      ar[r * LDA + c] = o[(int64_t)wk * ns];
+      ar[PLN + r * LDA + c] = o[((int64_t)a.Nw + wk) * ns];
+    }
+  for (int base = 0; base < (a.O ? 0 : nn * 4); base += blockDim.x) {
     const int q = base + tid, ent = q >> 2, part = q & 3;
     double re = 0.0, im = 0.0;
     float sr = 0.f, cr = 0.f, si = 0.f, ci = 0.f;   // FP32-pair partial sums (update mode)
@@ -886,8 +898,8 @@ __global__ void __launch_bounds__(128) k_mgs_chol(double* __restrict__ phi, cons
   const int wk = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
   if (!alive[wk]) return;
   const int64_t NM = (int64_t)N * M, plane = (int64_t)Nw * NM, base = (int64_t)wk * NM;
-  const int RS = N + 1;                                              // row stride (float2)
-  float2* X2 = reinterpret_cast<float2*>(smc);                       // [M][N + 1]
+  const int RS = N | 1;   // row stride (float2): odd, so that the rows' accesses spread over the banks
+  float2* X2 = reinterpret_cast<float2*>(smc);                       // [M][RS]
   float* Sre = reinterpret_cast<float*>(X2 + (size_t)M * RS);        // [N][N] (block diagonal)
   float* Sim = Sre + (size_t)N * N;
   float2* R2 = reinterpret_cast<float2*>(Sim + (size_t)N * N);       // [N][N]  R in FP32
@@ -1015,16 +1027,25 @@ __global__ void __launch_bounds__(128) k_mgs_chol(double* __restrict__ phi, cons
     const bool dn = it >= M;
     const int i = dn ? it - M : it, ns = dn ? nd : nu, o = dn ? nu : 0;
     float2* row = X2 + (size_t)i * RS + o;
-    for (int j = 0; j < ns; ++j) {
-      float2 x = row[j];
-      for (int k = 0; k < j; ++k) {
-        const float2 q = row[k], rv = R2[(size_t)(o + k) * N + o + j];
-        x.x = fmaf(-q.x, rv.x, fmaf(q.y, rv.y, x.x));
-        x.y = fmaf(-q.x, rv.y, fmaf(-q.y, rv.x, x.y));
+    float2 q[kNsMax];   // the row in registers: the R entries are all that is read per product
+#pragma unroll
+    for (int j = 0; j < kNsMax; ++j) q[j] = j < ns ? row[j] : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int j = 0; j < kNsMax; ++j)
+      if (j < ns) {
+        float2 x = q[j];
+#pragma unroll
+        for (int k = 0; k < j; ++k) {
+          const float2 rv = R2[(size_t)(o + k) * N + o + j];
+          x.x = fmaf(-q[k].x, rv.x, fmaf(q[k].y, rv.y, x.x));
+          x.y = fmaf(-q[k].x, rv.y, fmaf(-q[k].y, rv.x, x.y));
+        }
+        const float inv = Rd[o + j];
+        q[j] = make_float2(x.x * inv, x.y * inv);
       }
-      const float inv = Rd[o + j];
-      row[j] = make_float2(x.x * inv, x.y * inv);
-    }
+#pragma unroll
+    for (int j = 0; j < kNsMax; ++j)
+      if (j < ns) row[j] = q[j];
   }
   __syncthreads();
   for (int64_t e = tid; e < NM; e += blockDim.x) {
@@ -1041,12 +1062,12 @@ size_t smem_mgs_chol(const Ctx& c) {
          sizeof(float2) * (size_t)c.N * c.N + sizeof(float) * (size_t)c.N;
 }
 
-size_t smem_fast_overlap(const Ctx& c, bool fp64_copy = true) {
+size_t smem_fast_overlap(const Ctx& c, bool fp64_copy = true, bool given = false) {
   const size_t nmp = (size_t)c.N * (c.M + kPad);
   const bool small = std::max(c.n_up, c.N - c.n_up) <= 8;   // the NSM = 8 factor layout
   const size_t aug = small ? 2 * 2 * 8 * 8 : 2 * 2 * kNsMax * kLd;
   // the FP32 update factorises in the FP32 factor arrays: no FP64 copy of Phi, no FP64 factors
-  return sizeof(double) * (fp64_copy ? 2 * nmp + aug : 0) +
+  return sizeof(double) * (fp64_copy ? 2 * nmp + aug : given ? aug : 0) +
          sizeof(float) * (2 * nmp + 2 * 2 * kNsMax * kNsMax);
 }
 size_t smem_mgs_warp(const Ctx& c) { return sizeof(double) * 4 * (size_t)c.N * c.M; }   // two walkers
@@ -1080,6 +1101,58 @@ cudaError_t prepare_fast_walker_kernels(const Ctx& c) {
   });
 }
 
+// The overlap sums of a refresh (2 M sum_s N_s^2 complex by real multiply-adds per walker, 0.85 ms of the
+// FP64 pipe at M = 128, 16/16, 4096 walkers) as digit contractions: rows (p, w, b) of a spin's columns,
+// columns the trial's orbitals a.  Walkers in chunks whose digits stay in L2.
+namespace {
+constexpr size_t kRefreshChunk = (size_t)64 << 20;
+int refresh_chunk(const Ctx& c) {
+  const int nmax = std::max(c.n_up, c.N - c.n_up);
+  return (int)std::max<size_t>(1, std::min<size_t>((size_t)c.Nw, kRefreshChunk / ((size_t)nmax * pad64(c.M) * 16)));
+}
+
+cudaError_t refresh_sums(const Ctx& c, cudaStream_t s) {
+  const int nwc = refresh_chunk(c), NM = c.N * c.M;
+  double* out = c.ov_O;
+  cudaError_t e = cudaSuccess;
+  for (int sp = 0; sp < 2 && e == cudaSuccess; ++sp) {
+    const int n0 = sp ? c.n_up : 0, ns = sp ? c.N - c.n_up : c.n_up;
+    if (ns == 0) continue;
+    const DigitOp dp = digit_place(c.ws64.buf, ns, c.M);
+    e = digits_of(c.psi + (int64_t)n0 * c.M, c.M, ns, c.M, dp, s);
+    for (int p = 0; p < 2; ++p)
+      for (int w0 = 0; w0 < c.Nw && e == cudaSuccess; w0 += nwc) {
+        const int nw = std::min(nwc, c.Nw - w0);
+        const DigitOp db = digit_place(c.ws64.buf + digit_bytes(ns, c.M), (int64_t)nw * ns, c.M);
+        e = digits_of(c.phi + ((int64_t)p * c.Nw + w0) * NM, c.M, nw * ns, c.M, db, s, ns, c.N, n0);
+        if (e != cudaSuccess) break;
+        DigitGemm g;
+        g.R = nw * ns;
+        g.Cn = ns;
+        g.out = out + ((int64_t)p * c.Nw + w0) * ns;
+        g.ldc = 2 * (int64_t)c.Nw * ns;
+        g.K = c.M;
+        g.err = c.ws64.err;
+        e = digit_gemm(db, dp, g, s);
+      }
+    out += 2 * (int64_t)c.Nw * ns * ns;
+  }
+  return e;
+}
+}  // namespace
+
+// Where the sums' time on the FP64 pipe (1.1 TFLOP/s) exceeds that of the digits (24 bytes per element
+// of Phi at 5 TB/s) and their launches by half.
+bool refresh_f64e_ok(const Ctx& c) {
+  const int nu = c.n_up, nd = c.N - nu;
+  const double pipe = 4.0 * c.M * (nu * nu + nd * nd) * (double)c.Nw / 1.1e6;
+  return pipe > 1.5 * (25.0 + 48.0 * c.N * c.M * (double)c.Nw / 5.0e6);
+}
+size_t refresh_f64e_ws(const Ctx& c) {
+  const int nmax = std::max(c.n_up, c.N - c.n_up);
+  return digit_bytes(nmax, c.M) + digit_bytes((int64_t)refresh_chunk(c) * nmax, c.M);
+}
+
 cudaError_t launch_overlap_fast(const Ctx& c, const double* src, int mode, cudaStream_t s,
                                 const float* src32, bool with_weights) {
   FastOvArgs a{};
@@ -1094,10 +1167,16 @@ cudaError_t launch_overlap_fast(const Ctx& c, const double* src, int mode, cudaS
   a.free_proj = c.opt.mode == AFQMC_FREE;
   a.log_shift = -c.opt.dt * (c.c_mf - c.e_trial);
   a.fp64_copy = !(mode == OV_UPDATE && a.src32 != nullptr);
+  if (mode == OV_REFRESH && !src && c.ov_O) {
+    const cudaError_t e = refresh_sums(c, s);
+    if (e != cudaSuccess) return e;
+    a.O = c.ov_O;
+    a.fp64_copy = 0;
+  }
   auto rows = [](int ns) { return ns > 0 ? (ns + 32 / ns - 1) / (32 / ns) : 0; };
   const int nmax = std::max(c.n_up, c.N - c.n_up);
   const int need = std::max(rows(c.n_up), rows(c.N - c.n_up));
-  const size_t sm = smem_fast_overlap(c, a.fp64_copy != 0);
+  const size_t sm = smem_fast_overlap(c, a.fp64_copy != 0, a.O != nullptr);
   // the FP32 update (FP32-pair sums, smaller shared footprint) runs more CTAs of 128 threads
   // per SM, so more LU warps overlap; the FP64 sums of the other modes use 256
   const int nt = a.fp64_copy ? 256 : 128;
