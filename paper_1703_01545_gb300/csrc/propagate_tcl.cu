@@ -10,19 +10,27 @@
 // Both B operands are windows of one buffer of 3 Np rows [-T_im; T_re; T_im] (K = orbital j):
 // rows Np..3Np serve A_re and E - I, rows 0..2Np serve A_im.
 //
-// A is not held in shared memory: its split-BF16 tiles (128 rows x 64 K, hi and lo, written in
-// that form by the V_HS contraction) stream through a TMA ring for every round, so the ring
-// and the term operand fit two CTAs per SM at M = 128.  A hi tile is consumed by two MMAs per
-// 16-wide K step (hi * T_hi, hi * T_lo), a lo tile by one (lo * T_hi): the three split
-// products, accumulated in FP32 in tensor memory.  The running sum S of the series lives in
-// tensor memory beside the accumulator, so the epilogue threads hold no more than 16 columns
-// at a time.
+// A is not held in shared memory.  M <= 128: a walker's A (and E - I where it fits) is copied to tensor
+// memory once and every round reads it there.  M > 128: its split-BF16 tiles (128 rows x 64 K, hi and lo,
+// written in that form by the V_HS contraction) stream through a TMA ring for every round, 32 KB (a hi
+// tile and its lo tile) a stage.  A hi tile is consumed by two MMAs per 16-wide K step (hi * T_hi,
+// hi * T_lo), a lo tile by one (lo * T_hi): the three split products, accumulated in FP32 in tensor
+// memory.  The running sum S of the series lives in tensor memory beside the accumulator, so the
+// epilogue threads hold no more than 16 columns at a time.
 //
-// Roles (persistent CTA over walkers, 192 threads):
+// The streamed form at M = 200, N = 18 fills 512 KB of stages a Taylor round (26 bytes a cycle per SM at
+// the measured time, near what L2 delivers to all SMs at once) for 156 MMAs of some 45 cycles.  Scalar
+// work of the issuing lane between two MMAs costs more than the MMA, so a stage's MMAs are unrolled and
+// stages are counted, not divided; the first row tile's epilogue runs under the second tile's MMAs, which
+// needs a second copy of the term operand.  2048 walkers: 1.16 ms per launch with one CTA per SM and two
+// copies, 1.26 ms with one copy and a ring of four stages, 2.06 ms with 16 KB stages and one barrier for
+// both row tiles.
+//
+// Roles (persistent CTA over walkers, 4 or 8 epilogue warps):
 //   warp 0 / lane 0  TMA producer: the tiles of every round of every walker, in order
 //   warp 1 / lane 0  MMA issuer: per round, waits for the term operand, consumes the tiles,
-//                    commits "D full"
-//   warps 2..5       epilogue: thread r owns orbital row i = 128 t + r of every tile t (TMEM
+//                    commits "D full" per row tile
+//   warps 2..        epilogue: thread r owns orbital row i = 128 t + r of every tile t (TMEM
 //                    lane r); reads D and S, forms the next term, writes it into the operand
 //                    (split BF16, 128-byte swizzle), arrives on "B ready"
 // Every wait is bounded by %globaltimer; on expiry the kernel sets *err and a shared abort
@@ -46,7 +54,8 @@ using namespace tc;
 
 constexpr uint64_t kWaitNs = 2000000000ull;
 constexpr int kTile = 128 * 64 * 2;       // one 128-row x 64-K bf16 tile, 128-byte swizzle
-constexpr int kMaxStages = 12;
+constexpr int kStage = 2 * kTile;         // a ring stage: a hi tile and its lo tile
+constexpr int kMaxStages = 6;
 constexpr int kXu = 4;                    // staged-X elements per epilogue thread and round
 
 __device__ __forceinline__ uint32_t idesc_n(int n) {
@@ -155,6 +164,27 @@ __device__ __forceinline__ void mma_round_tmem(uint32_t d, uint32_t abase, uint6
     }
 }
 
+// The MMAs of one streamed tile: NKS 16-wide K steps of A at `a` against B hi (and, for a hi tile, B
+// lo).  Fully unrolled, the first one accumulating or not by `acc`: scalar work between two MMAs (a loop
+// counter, a branch) costs the issuing lane more than the MMA itself at these N.
+template <int NKS, bool HI>
+__device__ __forceinline__ void mma_tile(uint32_t d, uint64_t a, uint64_t bh, uint64_t bl, uint32_t idesc,
+                                         uint32_t acc) {
+#pragma unroll
+  for (int ks = 0; ks < NKS; ++ks) {
+    mma_bf16(d, a + (uint64_t)(2 * ks), bh + (uint64_t)(2 * ks), idesc, ks ? 1u : acc);   // 16 bf16 = 32 bytes
+    if (HI) mma_bf16(d, a + (uint64_t)(2 * ks), bl + (uint64_t)(2 * ks), idesc, 1u);
+  }
+}
+template <bool HI>
+__device__ __forceinline__ void mma_tile_n(int nks, uint32_t d, uint64_t a, uint64_t bh, uint64_t bl, uint32_t idesc,
+                                           uint32_t acc) {
+  if (nks == 4) mma_tile<4, HI>(d, a, bh, bl, idesc, acc);
+  else if (nks == 3) mma_tile<3, HI>(d, a, bh, bl, idesc, acc);
+  else if (nks == 2) mma_tile<2, HI>(d, a, bh, bl, idesc, acc);
+  else mma_tile<1, HI>(d, a, bh, bl, idesc, acc);
+}
+
 // Static shape of one launch (host-computed).
 struct TclShape {
   const __nv_bfloat16 *ahi, *alo;   // V_HS split planes [2][Nw][M][Mp] (L2 prefetch of the next walker)
@@ -168,6 +198,9 @@ struct TclShape {
   int acol;              // resident form: TMEM column of A (plane P, K block kb at acol + 32 (P KB + kb))
   int eres, ecol;        // 1: e^{-dt K/2} - I also in tensor memory (hi, lo planes from ecol), loaded
                          // once per CTA; the one-body rounds then need no ring
+  int bbuf;              // bytes from one copy of the term operand to the other, 0: one copy.  With two
+                         // (two row tiles, one CTA per SM) the epilogue of the first row tile writes the
+                         // next term while the second tile's MMAs still read this one
   int bkb;               // bytes of one K block of the term operand (3 Np rows x 128 bytes)
   int dcol;              // TMEM column stride between tiles (D and S regions)
   uint32_t tcols;        // TMEM columns allocated
@@ -179,8 +212,8 @@ struct TclShape {
 };
 
 // Round q of a walker: 0 and order + 1 are the one-body products, 1..order the Taylor terms.
-// Tiles of a round, in order: for each row tile t and K block kb: E hi, E lo (one-body) or
-// A_re hi, A_re lo, A_im hi, A_im lo (Taylor).
+// Stages of a round, in order: for each row tile t and K block kb: E (one-body) or A_re, A_im (Taylor),
+// hi and lo tile each.
 
 template <int EPI>
 __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
@@ -198,7 +231,8 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
   const uint32_t done = smem_u32(bars + 2 * kMaxStages + 2);
   const uint32_t afull = smem_u32(bars + 2 * kMaxStages + 3), acopied = smem_u32(bars + 2 * kMaxStages + 4);
   const uint32_t xfull = smem_u32(bars + 2 * kMaxStages + 5), xread = smem_u32(bars + 2 * kMaxStages + 6);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kMaxStages + 7);
+  const uint32_t dfull1 = smem_u32(bars + 2 * kMaxStages + 7);   // the second row tile's accumulator
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kMaxStages + 8);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rounds = sh.order + 2;
@@ -210,6 +244,7 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
       mbar_init(empty0 + 8 * q, 1);
     }
     mbar_init(dfull, 1);
+    mbar_init(dfull1, 1);
     mbar_init(bready, 32 * EPI);
     mbar_init(done, 1);
     mbar_init(afull, 1);
@@ -220,7 +255,7 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   // the term operand starts at zero: padded rows and K beyond M stay zero throughout
-  for (int e = threadIdx.x; e < 2 * sh.KB * sh.bkb / 16; e += blockDim.x)
+  for (int e = threadIdx.x; e < (sh.bbuf ? 4 : 2) * sh.KB * sh.bkb / 16; e += blockDim.x)
     reinterpret_cast<uint4*>(smem + sh.bhi_off)[e] = make_uint4(0u, 0u, 0u, 0u);
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // visible to the tensor core
   if (warp == 1) {
@@ -239,7 +274,8 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
   if (warp == 0) {
     if (lane == 0) {
       // ---- TMA producer: the same walker and tile order the MMA issuer consumes ----
-      int g = 0, aw = 0;
+      int g = 0, aw = 0, st = 0;
+      uint32_t ph = 0;   // parity of the stage's current use
       bool ok = true;
       const uint64_t abytes = (uint64_t)sh.M * sh.Mp * 2;   // one plane of A, hi or lo
       const uint64_t pbytes = (uint64_t)NM * 8;             // one plane of Phi
@@ -284,24 +320,25 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
           if (sh.resident && (taylor || sh.eres)) continue;
           for (int t = 0; t < sh.MT && ok; ++t)
             for (int kb = 0; kb < sh.KB && ok; ++kb)
-              for (int u = 0; u < (taylor ? 4 : 2); ++u, ++g) {
-                const int st = g % sh.nst, use = g / sh.nst;
+              for (int u = 0; u < (taylor ? 2 : 1); ++u, ++g) {
                 if (*abort_flag) { ok = false; break; }
-                if (g >= sh.nst && !mbar_wait(empty0 + 8 * st, (use - 1) & 1, err, wait_ns)) {
+                if (g >= sh.nst && !mbar_wait(empty0 + 8 * st, ph ^ 1u, err, wait_ns)) {
                   fail();
                   ok = false;
                   break;
                 }
-                const uint32_t dst = smem_u32(smem + sh.ring_off + st * kTile);
+                const uint32_t dst = smem_u32(smem + sh.ring_off + st * kStage);
                 const uint32_t fb = full0 + 8 * st;
-                mbar_expect_tx(fb, kTile);
-                if (taylor) {
-                  // u: 0 A_re hi, 1 A_re lo, 2 A_im hi, 3 A_im lo; z = (plane, walker)
-                  const int z = (u >> 1) * sh.Nw + w;
-                  tma_load_3d(dst, (u & 1) ? &tmAlo : &tmAhi, fb, kb * 64, t * 128, z);
+                mbar_expect_tx(fb, kStage);
+                if (taylor) {   // u: 0 A_re, 1 A_im; z = (plane, walker)
+                  const int z = u * sh.Nw + w;
+                  tma_load_3d(dst, &tmAhi, fb, kb * 64, t * 128, z);
+                  tma_load_3d(dst + kTile, &tmAlo, fb, kb * 64, t * 128, z);
                 } else {
-                  tma_load_2d(dst, (u & 1) ? &tmElo : &tmEhi, fb, kb * 64, t * 128);
+                  tma_load_2d(dst, &tmEhi, fb, kb * 64, t * 128);
+                  tma_load_2d(dst + kTile, &tmElo, fb, kb * 64, t * 128);
                 }
+                if (++st == sh.nst) { st = 0; ph ^= 1u; }
               }
         }
       }
@@ -315,10 +352,13 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
     // and one elected lane issues; lane 0 polls the barriers and broadcasts the outcome ----
     const uint32_t idesc = idesc_n(sh.n2);
     const uint32_t bhi = smem_u32(smem + sh.bhi_off), blo = smem_u32(smem + sh.blo_off);
-    const uint64_t dbh = sw128_desc(bhi), dbl = sw128_desc(blo);
+    const uint64_t dbh0 = sw128_desc(bhi), dbl0 = sw128_desc(blo);
     const uint32_t bkb16 = (uint32_t)(sh.bkb >> 4), np16 = (uint32_t)(sh.Np * 8);
     const int nks_last = min(4, (sh.M - 64 * (sh.KB - 1) + 15) / 16);
-    int g = 0, rq = 0;
+    int rq = 0, st = 0;
+    uint32_t ph = 0;   // parity of the ring stage's current use
+    const int nst = sh.nst, KB = sh.KB, MT = sh.MT;
+    const uint64_t dring = sw128_desc(smem_u32(smem + sh.ring_off));
     bool ok = true;
     auto wait_all = [&](uint32_t bar, int parity) {
       int okw = 1;
@@ -331,6 +371,7 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
       if (alive && !alive[w]) continue;
       for (int q = 0; q < rounds && ok; ++q, ++rq) {
         const bool taylor = q >= 1 && q <= sh.order;
+        const uint64_t boff = (uint64_t)((rq & 1) * (sh.bbuf >> 4)), dbh = dbh0 + boff, dbl = dbl0 + boff;
         if (!wait_all(bready, rq & 1)) { ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (sh.resident && (taylor || sh.eres)) {
@@ -352,33 +393,33 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
           __syncwarp();
           continue;
         }
-        for (int t = 0; t < sh.MT && ok; ++t) {
+        // (counters instead of divisions, a stage of two tiles: the chain of scalar work between two
+        // stages kept the tensor core waiting for 500 of every 1000 cycles)
+        const int npair = taylor ? 2 : 1;
+        for (int t = 0; t < MT && ok; ++t) {
           const uint32_t d = tmem + (uint32_t)(t * sh.dcol);
-          for (int kb = 0; kb < sh.KB && ok; ++kb) {
-            const int nks = kb == sh.KB - 1 ? nks_last : 4;   // K steps holding orbitals
-            for (int u = 0; u < (taylor ? 4 : 2); ++u, ++g) {
-              const int st = g % sh.nst, use = g / sh.nst;
-              if (!wait_all(full0 + 8 * st, use & 1)) { ok = false; break; }
+          for (int kb = 0; kb < KB && ok; ++kb) {
+            const int nks = kb == KB - 1 ? nks_last : 4;   // K steps holding orbitals
+            for (int u = 0; u < npair; ++u) {
+              if (!__all_sync(0xffffffffu, mbar_try(full0 + 8 * st, ph)) && !wait_all(full0 + 8 * st, (int)ph)) {
+                ok = false;
+                break;
+              }
               asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
               if (elect_one()) {
-                const uint64_t a = sw128_desc(smem_u32(smem + sh.ring_off + st * kTile));
-                // A_im (u >= 2) takes rows 0..2Np of the term operand, A_re and E - I rows Np..3Np
-                const uint64_t roff = (uint64_t)(kb * bkb16 + ((taylor && u >= 2) ? 0u : np16));
-                const bool hi = (u & 1) == 0;
-                for (int ks = 0; ks < nks; ++ks) {
-                  const uint64_t dk = roff + (uint64_t)(2 * ks);   // 16 bf16 = 32 bytes along K
-                  mma_bf16(d, a + (uint64_t)(2 * ks), dbh + dk, idesc, (kb | u | ks) != 0 ? 1u : 0u);
-                  if (hi) mma_bf16(d, a + (uint64_t)(2 * ks), dbl + dk, idesc, 1u);
-                }
+                const uint64_t a = dring + (uint64_t)(st * (kStage >> 4));
+                // A_im (u = 1) takes rows 0..2Np of the term operand, A_re and E - I rows Np..3Np
+                const uint64_t roff = (uint64_t)(kb * bkb16 + (u ? 0u : np16));
+                mma_tile_n<true>(nks, d, a, dbh + roff, dbl + roff, idesc, (kb | u) != 0 ? 1u : 0u);
+                mma_tile_n<false>(nks, d, a + (uint64_t)(kTile >> 4), dbh + roff, dbl + roff, idesc, 1u);
                 mma_commit(empty0 + 8 * st);
+                // a row tile's accumulator is complete: its epilogue runs beside the next tile's MMAs
+                if (kb == KB - 1 && u == npair - 1) mma_commit(t ? dfull1 : dfull);
               }
               __syncwarp();
+              if (++st == nst) { st = 0; ph ^= 1u; }
             }
           }
-        }
-        if (ok) {
-          if (elect_one()) mma_commit(dfull);
-          __syncwarp();
         }
       }
     }
@@ -392,7 +433,7 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
     const int qd = warp & 3, r = 32 * qd + lane;
     const int half = EPI == 8 ? (warp - 2) >> 2 : 0, cstep = EPI == 8 ? 32 : 16;
     const uint32_t lanes = (uint32_t)(32 * qd) << 16;
-    const uint32_t bhi_s = smem_u32(smem + sh.bhi_off), blo_s = smem_u32(smem + sh.blo_off);
+    const uint32_t bhi_s0 = smem_u32(smem + sh.bhi_off), blo_s0 = smem_u32(smem + sh.blo_off);
     const uint32_t sreg = (uint32_t)(sh.MT * sh.dcol);   // S region after the D columns
     const int jj = lane >> 3, kk = lane & 7, fr = lane >> 2, fc = 2 * (lane & 3);
     // fragment element j: lane offset fr (+ 8), column offset fc (+ 1) (+ 8)
@@ -404,7 +445,9 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
     };
     // the block's values (orbitals i0b .., columns c0 ..) into operand rows Np + c, and with neg,
     // -value into rows c - Np for the imaginary columns c >= Np
-    auto put_block = [&](const float (&v)[8], int i0b, int c0, bool neg) {
+    int rq = 0, jw = 0;
+    auto put_block = [&](const float (&v)[8], int i0b, int c0, bool neg, int round) {
+      const uint32_t bo = (uint32_t)((round & 1) * sh.bbuf), bhi_s = bhi_s0 + bo, blo_s = blo_s0 + bo;
       uint32_t h[4], l[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) split_pair(v[2 * j], v[2 * j + 1], h[j], l[j]);
@@ -428,7 +471,6 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
         stsm_x2_t(chunk(blo_s, cn, i0), l[2], l[3]);
       }
     };
-    int rq = 0, jw = 0;
     bool ok = true;
     // resident A: the staging tiles into tensor memory; lane r takes row r of every tile (16-byte
     // chunks in the 128-byte swizzle), the two warps of a lane quadrant take planes
@@ -519,7 +561,7 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
             v[j] = __float_as_uint(x[j]);
           }
           tmem_st_frag(tl + sreg + (uint32_t)(t * sh.dcol + c0), v);
-          if (i0b < 64 * sh.KB) put_block(x, i0b, c0, false);
+          if (i0b < 64 * sh.KB) put_block(x, i0b, c0, false, rq);
         }
         mbar_arrive(xread);   // the staged X may take the next walker's once all have read it
       } else
@@ -556,7 +598,7 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
             v[j] = __float_as_uint(x[j]);
           }
           tmem_st_frag(tl + sreg + (uint32_t)(t * sh.dcol + c0), v);
-          if (i0b < 64 * sh.KB) put_block(x, i0b, c0, false);
+          if (i0b < 64 * sh.KB) put_block(x, i0b, c0, false, rq);
         }
       }
       if (!ok) break;
@@ -588,12 +630,19 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
               if (xi >= sh.M) { xi -= sh.M; ++xc; }
             }
           }
+        // the first row tile's products; all of them when its epilogue overwrites their operand
         bool okw = !*abort_flag && mbar_wait(dfull, rq & 1, err, wait_ns);
+        if (sh.MT > 1 && !sh.bbuf) okw = okw && !*abort_flag && mbar_wait(dfull1, rq & 1, err, wait_ns);
         if (pre && q == 0) okw = okw && !*abort_flag && mbar_wait(xread, kw & 1, err, wait_ns);
         if (!__all_sync(0xffffffffu, okw)) { fail(); ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const float inv = (q >= 1 && q <= sh.order) ? 1.f / (float)q : 1.f;
-        for (int t = 0; t < sh.MT; ++t)
+        for (int t = 0; t < sh.MT && ok; ++t) {
+          if (t && sh.bbuf) {
+            okw = !*abort_flag && mbar_wait(dfull1, rq & 1, err, wait_ns);
+            if (!__all_sync(0xffffffffu, okw)) { fail(); ok = false; break; }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          }
           for (int sl = 0; sl < 2; ++sl) {
             const int i0b = 128 * t + 32 * qd + 16 * sl;
             const bool in_b = i0b < 64 * sh.KB;
@@ -612,7 +661,7 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
                   sv[j] = __float_as_uint(x[j]);
                 }
                 tmem_st_frag(tl + sreg + (uint32_t)(t * sh.dcol + c0), sv);
-                if (in_b) put_block(x, i0b, c0, true);
+                if (in_b) put_block(x, i0b, c0, true, rq + 1);
               } else if (!last) {
                 // T_q = A T_{q-1} / q; S += T_q; operand = T_q, or S after the last term
                 float y[8];
@@ -623,7 +672,7 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
                   sv[j] = __float_as_uint(y[j]);
                 }
                 tmem_st_frag(tl + sreg + (uint32_t)(t * sh.dcol + c0), sv);
-                if (in_b) put_block(q < sh.order ? x : y, i0b, c0, q < sh.order);
+                if (in_b) put_block(q < sh.order ? x : y, i0b, c0, q < sh.order, rq + 1);
               } else {
                 // Phi' = S + (E - I) S
 #pragma unroll
@@ -639,6 +688,8 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
               }
             }
           }
+        }
+        if (!ok) break;
         if (!last) {
           asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -708,7 +759,7 @@ cudaError_t make_map(CUtensorMap* map, void* base, int M, int Mp, int64_t nz) {
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-TclShape shape_of(const Ctx& c, int nst, int resident) {
+TclShape shape_of(const Ctx& c, int nst, int resident, int two = 0) {
   TclShape s{};
   s.ahi = c.tcl_ahi;
   s.alo = c.tcl_alo;
@@ -736,32 +787,33 @@ TclShape shape_of(const Ctx& c, int nst, int resident) {
   // (the staging covers kXu elements per epilogue thread and round)
   s.xs = resident && s.eres && s.n2 * s.M <= kXu * 32 * 8 * (s.order + 2);
   s.xs_ld = s.M + 4;   // rows 4 floats apart: the fragment reads below fall in distinct banks
-  s.ares_off = s.xs ? (s.n2 * s.xs_ld * 4 + 1023) / 1024 * 1024 : nst * kTile;
+  s.ares_off = s.xs ? (s.n2 * s.xs_ld * 4 + 1023) / 1024 * 1024 : nst * kStage;
   s.bhi_off = s.ares_off + (resident ? 4 * s.KB * kTile : 0);
   s.blo_off = s.bhi_off + s.KB * s.bkb;
-  s.bar_off = s.blo_off + s.KB * s.bkb;
-  s.smem_bytes = s.bar_off + 8 * (2 * kMaxStages + 7) + 16 + 1024;
+  s.bbuf = two ? 2 * s.KB * s.bkb : 0;   // [hi][lo] of round parity 0, then of parity 1
+  s.bar_off = s.blo_off + s.KB * s.bkb + s.bbuf;
+  s.smem_bytes = s.bar_off + 8 * (2 * kMaxStages + 8) + 16 + 1024;
   return s;
 }
 
-// Launch form: A resident with a 2-stage ring for e^{-dt K/2} - I and 8 epilogue warps, one CTA
-// per SM (M <= 128); else A streamed, two CTAs per SM of 4 epilogue warps when a ring of at
-// least 4 stages fits 113 KB, otherwise one CTA per SM of 8 epilogue warps with the deepest
-// ring that fits.
+// Launch form: A resident with 8 epilogue warps, one CTA per SM (M <= 128); else A streamed, two CTAs
+// per SM of 4 epilogue warps when a ring of at least 2 stages (of 32 KB) fits 113 KB, otherwise one
+// CTA per SM of 8 epilogue warps with two copies of the term operand and the deepest ring that fits (two
+// stages at N M = 4096, the largest system).
 TclShape plan(const Ctx& c) {
   if (c.M <= 128) {
-    const TclShape s = shape_of(c, 2, 1);
+    const TclShape s = shape_of(c, 1, 1);
     if (s.smem_bytes <= 227 * 1024) return s;
   }
-  for (int nst = 8; nst >= 4; --nst) {
+  for (int nst = 4; nst >= 2; --nst) {
     const TclShape s = shape_of(c, nst, 0);
     if (s.smem_bytes <= 113 * 1024) return s;
   }
   for (int nst = kMaxStages; nst >= 2; --nst) {
-    const TclShape s = shape_of(c, nst, 0);
+    const TclShape s = shape_of(c, nst, 0, 1);
     if (s.smem_bytes <= 227 * 1024) return s;
   }
-  return shape_of(c, 2, 0);
+  return shape_of(c, 2, 0, 1);
 }
 
 bool two_per_sm(const TclShape& s) { return !s.resident && s.smem_bytes <= 113 * 1024; }
@@ -774,7 +826,9 @@ bool propagate_tcl_ok(const Ctx& c) {
   return s.smem_bytes <= 227 * 1024 && s.tcols <= (two_per_sm(s) ? 256u : 512u);
 }
 
-int propagate_tcl_mp(int M) { return (M + 7) / 8 * 8; }
+// Elements per orbital row of the split planes: whole 128-byte lines, so that no row of a TMA box
+// straddles two (at M = 200 a pitch of 400 bytes made every 128-byte row of a box two requests).
+int propagate_tcl_mp(int M) { return (M + 63) / 64 * 64; }
 
 cudaError_t prepare_propagate_tcl() {
   cudaError_t e = cudaFuncSetAttribute(k_propagate_tcl<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -27,22 +27,30 @@ __device__ __forceinline__ uint64_t global_ns() {
   return t;
 }
 
+// One wait for the phase with the given parity, of up to about a millisecond: the thread is suspended
+// until the phase completes instead of polling.  Without the time hint the wait returns at once, and the
+// polls of eight epilogue warps kept the issuing warp's own barrier and shuffle instructions waiting
+// hundreds of cycles each.
+__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity), "r"(1000000u)
+      : "memory");
+  return ok != 0;
+}
+
 // Bounded wait for the phase with the given parity; false (and *err set) on expiry.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* err,
                                           uint64_t limit_ns) {
+  if (mbar_try(bar, parity)) return true;
   const uint64_t t0 = global_ns();
-  for (uint32_t it = 0;; ++it) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (ok) return true;
-    if ((it & 255u) == 255u && global_ns() - t0 > limit_ns) break;
-  }
+  do {
+    if (mbar_try(bar, parity)) return true;
+  } while (global_ns() - t0 <= limit_ns);
   atomicOr(err, 1);
   return false;
 }

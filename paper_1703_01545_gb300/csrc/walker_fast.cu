@@ -1108,7 +1108,7 @@ namespace {
 constexpr size_t kRefreshChunk = (size_t)64 << 20;
 int refresh_chunk(const Ctx& c) {
   const int nmax = std::max(c.n_up, c.N - c.n_up);
-  return (int)std::max<size_t>(1, std::min<size_t>((size_t)c.Nw, kRefreshChunk / ((size_t)nmax * pad64(c.M) * 16)));
+  return (int)std::max<size_t>(1, std::min<size_t>(2 * (size_t)c.Nw, kRefreshChunk / ((size_t)nmax * pad64(c.M) * 16)));
 }
 
 cudaError_t refresh_sums(const Ctx& c, cudaStream_t s) {
@@ -1120,9 +1120,11 @@ cudaError_t refresh_sums(const Ctx& c, cudaStream_t s) {
     if (ns == 0) continue;
     const DigitOp dp = digit_place(c.ws64.buf, ns, c.M);
     e = digits_of(c.psi + (int64_t)n0 * c.M, c.M, ns, c.M, dp, s);
-    for (int p = 0; p < 2; ++p)
-      for (int w0 = 0; w0 < c.Nw && e == cudaSuccess; w0 += nwc) {
-        const int nw = std::min(nwc, c.Nw - w0);
+    // a small population: both planes' rows (p, w, b) at once
+    const int planes = 2 * c.Nw <= nwc ? 1 : 2;
+    for (int p = 0; p < planes; ++p)
+      for (int w0 = 0; w0 < c.Nw && e == cudaSuccess; w0 += planes == 1 ? c.Nw : nwc) {
+        const int nw = planes == 1 ? 2 * c.Nw : std::min(nwc, c.Nw - w0);
         const DigitOp db = digit_place(c.ws64.buf + digit_bytes(ns, c.M), (int64_t)nw * ns, c.M);
         e = digits_of(c.phi + ((int64_t)p * c.Nw + w0) * NM, c.M, nw * ns, c.M, db, s, ns, c.N, n0);
         if (e != cudaSuccess) break;
@@ -1146,7 +1148,7 @@ cudaError_t refresh_sums(const Ctx& c, cudaStream_t s) {
 bool refresh_f64e_ok(const Ctx& c) {
   const int nu = c.n_up, nd = c.N - nu;
   const double pipe = 4.0 * c.M * (nu * nu + nd * nd) * (double)c.Nw / 1.1e6;
-  return pipe > 1.5 * (25.0 + 48.0 * c.N * c.M * (double)c.Nw / 5.0e6);
+  return pipe > 1.5 * (45.0 + 48.0 * c.N * c.M * (double)c.Nw / 5.0e6);
 }
 size_t refresh_f64e_ws(const Ctx& c) {
   const int nmax = std::max(c.n_up, c.N - c.n_up);
