@@ -14,7 +14,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(ROOT, "_build")
 LIB = os.path.join(HERE, "libafqmc_gb300.so")
-SOURCES = ["gemm_f64.cu", "gemm_f64e.cu", "energy_f64e.cu", "taylor_f64e.cu", "walker_kernels.cu", "setup_kernels.cu", "api.cu", "pair.cu", "stats.cpp",
+SOURCES = ["gemm_f64.cu", "gemm_f64e.cu", "energy_f64e.cu", "taylor_f64e.cu", "step_small.cu", "walker_kernels.cu", "setup_kernels.cu", "api.cu", "pair.cu", "stats.cpp",
            "noalloc.cu", "gemm_tc.cu", "mixed_kernels.cu", "walker_fast.cu", "autotune.cu",
            "tangent.cu", "adjoint_kernels.cu", "adjoint.cu",
            "energy_tc.cu", "propagate_f32.cu",

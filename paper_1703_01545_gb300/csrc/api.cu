@@ -381,6 +381,18 @@ afqmc_status step_launch(Ctx* h, const double* fields_t, cudaStream_t s) {
   return AFQMC_OK;
 }
 
+// n_steps steps; fields [n_steps][Nw][X] or null.
+afqmc_status steps_launch(Ctx* h, int n_steps, const double* fields, cudaStream_t s) {
+  if (!h->tangent_on && afq::step_small_ok(*h)) {
+    AFQ_CK(afq::launch_steps_small(*h, n_steps, fields, s));
+    return AFQMC_OK;
+  }
+  const int64_t per = (int64_t)h->Nw * h->X;
+  afqmc_status st = AFQMC_OK;
+  for (int t = 0; t < n_steps && st == AFQMC_OK; ++t) st = step_launch(h, fields ? fields + per * t : nullptr, s);
+  return st;
+}
+
 // Overlap / Theta / weight kernel: the warp-synchronous variant in split-precision mode.
 afqmc_status overlap_launch(Ctx* h, const double* src, int mode, cudaStream_t s,
                             const float* src32) {
@@ -439,7 +451,7 @@ afqmc_status check_opts(const afqmc_options* o, std::string& why) {
 }  // namespace
 
 namespace afq {
-afqmc_status pair_step(Ctx* h, cudaStream_t s) { return step_launch(h, nullptr, s); }
+afqmc_status pair_steps(Ctx* h, int n, cudaStream_t s) { return steps_launch(h, n, nullptr, s); }
 afqmc_status run_step(Ctx* h, const double* fields_t, cudaStream_t s) { return step_launch(h, fields_t, s); }
 afqmc_status pair_ortho(Ctx* h, cudaStream_t s) { return ortho_launch(h, s); }
 afqmc_status pair_energy(Ctx* h, cudaStream_t s) { return energy_launch(h, s); }
@@ -563,6 +575,7 @@ afqmc_status afqmc_setup(afqmc_handle* out, const double* h1_in, const double* L
   AFQ_SCK(afq::prepare_kernels(*h));
   if (opt->precision == AFQMC_FP64 && afq::overlap64_ok(*h)) {
     AFQ_SCK(afq::prepare_overlap64(*h));
+    if (afq::step_small_ok(*h)) AFQ_SCK(afq::prepare_step_small(*h));
     if (dalloc(h, &h->ovdet, 8 * (size_t)Nw) != AFQMC_OK) return bail(AFQMC_ERR_NOMEM);
   }
   if (opt->precision == AFQMC_FP64) {
@@ -895,8 +908,7 @@ afqmc_status afqmc_propagate(afqmc_handle h, int n_steps, const double* fields, 
       fd = staged;
     }
   }
-  afqmc_status st = AFQMC_OK;
-  for (int t = 0; t < n_steps && st == AFQMC_OK; ++t) st = step_launch(h, fd ? fd + per * t : nullptr, s);
+  const afqmc_status st = steps_launch(h, n_steps, fd, s);
   if (staged) {
     cudaStreamSynchronize(s);
     cudaFree(staged);

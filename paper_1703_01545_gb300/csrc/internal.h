@@ -416,7 +416,11 @@ cudaError_t launch_mgs(const Ctx& c, cudaStream_t s);
 cudaError_t launch_energy(const Ctx& c, cudaStream_t s, int n_walkers = -1);
 cudaError_t launch_mixed_sum(const Ctx& c, double* out, const int* slot, int slot_stride,
                              cudaStream_t s);
-cudaError_t launch_step_advance(const Ctx& c, cudaStream_t s);
+cudaError_t launch_step_advance(const Ctx& c, cudaStream_t s, int n_steps = 1);
+// Whole FP64 steps of small systems in one kernel (step_small.cu)
+bool step_small_ok(const Ctx& c);
+cudaError_t prepare_step_small(const Ctx& c);
+cudaError_t launch_steps_small(const Ctx& c, int n_steps, const double* fields, cudaStream_t s);
 
 // setup helpers
 cudaError_t launch_transpose(const double* in, double* out, int rows, int cols, cudaStream_t s);

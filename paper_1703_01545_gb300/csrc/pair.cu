@@ -15,7 +15,7 @@
 struct afqmc_ctx : afq::Ctx {};
 
 namespace afq {
-afqmc_status pair_step(Ctx* h, cudaStream_t s);
+afqmc_status pair_steps(Ctx* h, int n, cudaStream_t s);
 afqmc_status pair_ortho(Ctx* h, cudaStream_t s);
 afqmc_status pair_energy(Ctx* h, cudaStream_t s);
 afqmc_status pair_check(Ctx* h);
@@ -80,13 +80,15 @@ afqmc_status record_block(afqmc_ctx* A, afqmc_ctx* B, Res* r, F last) {
   afqmc_status st = AFQMC_OK;
   cudaError_t ce = cudaEventRecord(r->fork, r->cs);
   if (ce == cudaSuccess) ce = cudaStreamWaitEvent(r->cs2, r->fork, 0);
-  for (int j = 0; j < r->ee && st == AFQMC_OK && ce == cudaSuccess; ++j) {
-    st = afq::pair_step(A, r->cs);
-    if (st == AFQMC_OK) st = afq::pair_step(B, r->cs2);
-    if (st == AFQMC_OK && (j + 1) % r->me == 0) {
-      st = afq::pair_ortho(A, r->cs);
-      if (st == AFQMC_OK) st = afq::pair_ortho(B, r->cs2);
+  // steps of A and B recorded in turn, or all up to the orthonormalisation where a kernel takes several
+  const int run = afq::step_small_ok(*A) && afq::step_small_ok(*B) ? r->me : 1;
+  for (int j = 0; j < r->ee && st == AFQMC_OK && ce == cudaSuccess; j += r->me) {   // ee is a multiple of me
+    for (int k = 0; k < r->me && st == AFQMC_OK; k += run) {
+      st = afq::pair_steps(A, run, r->cs);
+      if (st == AFQMC_OK) st = afq::pair_steps(B, run, r->cs2);
     }
+    if (st == AFQMC_OK) st = afq::pair_ortho(A, r->cs);
+    if (st == AFQMC_OK) st = afq::pair_ortho(B, r->cs2);
   }
   if (st == AFQMC_OK && ce == cudaSuccess) st = afq::pair_energy(A, r->cs);
   if (st == AFQMC_OK && ce == cudaSuccess) st = afq::pair_energy(B, r->cs2);

@@ -657,9 +657,9 @@ __global__ void __launch_bounds__(256) k_mixed_sum(const double* __restrict__ w,
   }
 }
 
-__global__ void k_step_advance(unsigned long long* step, int* meas, int bump_meas) {
+__global__ void k_step_advance(unsigned long long* step, int n, int* meas, int bump_meas) {
   if (threadIdx.x == 0 && blockIdx.x == 0) {
-    if (step) *step += 1ull;
+    if (step) *step += (unsigned long long)n;
     if (meas && bump_meas) *meas += 1;
   }
 }
@@ -813,12 +813,12 @@ cudaError_t launch_mixed_sum(const Ctx& c, double* out, const int* slot, int slo
 }
 
 cudaError_t launch_meas_advance(int* meas, cudaStream_t s) {
-  k_step_advance<<<1, 32, 0, s>>>(nullptr, meas, 1);
+  k_step_advance<<<1, 32, 0, s>>>(nullptr, 0, meas, 1);
   return cudaGetLastError();
 }
 
-cudaError_t launch_step_advance(const Ctx& c, cudaStream_t s) {
-  k_step_advance<<<1, 32, 0, s>>>(c.d_step, nullptr, 0);
+cudaError_t launch_step_advance(const Ctx& c, cudaStream_t s, int n_steps) {
+  k_step_advance<<<1, 32, 0, s>>>(c.d_step, n_steps, nullptr, 0);
   return cudaGetLastError();
 }
 
