@@ -26,6 +26,15 @@
 // copies, 1.26 ms with one copy and a ring of four stages, 2.06 ms with 16 KB stages and one barrier for
 // both row tiles.
 //
+// M <= 128 and more than 8 columns: the columns form two groups with an accumulator, a term operand and 8
+// epilogue warps each.  The groups take turns at the tensor core, so the MMAs of one run beside the epilogue
+// of the other; at these N an MMA's time falls with N (16 cycles at N = 32, 32 at N = 64, A in tensor
+// memory), so halving N costs no tensor time.  The sizes are template constants: with run-time strides the
+// issuing lane took 50 cycles an MMA, now 20.  M = 128, N = 32, 4096 walkers, beside the
+// other system's kernels: 0.79 -> 0.66 ms per launch (M = 101, N = 21, 777 walkers, alone: 162 -> 137 us).  A
+// round of both groups takes 5.1 k cycles: 2 x 2 k of MMAs,
+// slowed by the other group's tensor-memory traffic, beside 1.5 k of epilogue.
+//
 // Roles (persistent CTA over walkers, 4 or 8 epilogue warps):
 //   warp 0 / lane 0  TMA producer: the tiles of every round of every walker, in order
 //   warp 1 / lane 0  MMA issuer: per round, waits for the term operand, consumes the tiles,
@@ -56,6 +65,8 @@ constexpr uint64_t kWaitNs = 2000000000ull;
 constexpr int kTile = 128 * 64 * 2;       // one 128-row x 64-K bf16 tile, 128-byte swizzle
 constexpr int kStage = 2 * kTile;         // a ring stage: a hi tile and its lo tile
 constexpr int kMaxStages = 6;
+constexpr int kDcol2 = 32;                // accumulator columns of a group (two-group form)
+constexpr int kBars = 2 * kMaxStages + 16;
 constexpr int kXu = 4;                    // staged-X elements per epilogue thread and round
 
 __device__ __forceinline__ uint32_t idesc_n(int n) {
@@ -164,6 +175,22 @@ __device__ __forceinline__ void mma_round_tmem(uint32_t d, uint32_t abase, uint6
     }
 }
 
+// The same with constant sizes: KS K steps, operand rows NP.
+template <int KS, int NPL, int NP>
+__device__ __forceinline__ void mma_round_const(uint32_t d, uint32_t abase, uint64_t dbh, uint64_t dbl) {
+  constexpr int KB = (KS + 3) / 4;
+  constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(2 * NP >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+#pragma unroll
+  for (int k = 0; k < KS; ++k)
+#pragma unroll
+    for (int u = 0; u < NPL; ++u) {
+      const uint32_t ta = abase + (uint32_t)(32 * (u * KB + k / 4) + 8 * (k % 4));
+      const uint64_t dk = (uint64_t)(k / 4 * (3 * NP * 8) + (u >= 2 ? 0 : NP * 8) + 2 * (k % 4));
+      mma_bf16_ta(d, ta, dbh + dk, idesc, (k | u) != 0 ? 1u : 0u);
+      if ((u & 1) == 0) mma_bf16_ta(d, ta, dbl + dk, idesc, 1u);
+    }
+}
+
 // The MMAs of one streamed tile: NKS 16-wide K steps of A at `a` against B hi (and, for a hi tile, B
 // lo).  Fully unrolled, the first one accumulating or not by `acc`: scalar work between two MMAs (a loop
 // counter, a branch) costs the issuing lane more than the MMA itself at these N.
@@ -189,7 +216,10 @@ __device__ __forceinline__ void mma_tile_n(int nks, uint32_t d, uint64_t a, uint
 struct TclShape {
   const __nv_bfloat16 *ahi, *alo;   // V_HS split planes [2][Nw][M][Mp] (L2 prefetch of the next walker)
   int Mp;                // elements per orbital row of the split planes
-  int M, N, Np, n2;      // orbitals, occupied columns, N rounded up to 8, MMA N = 2 Np
+  int M, N, Np, n2;      // orbitals, occupied columns, a group's columns rounded up to 8, MMA N = 2 Np
+  int G;                 // column groups (resident form): 1, or 2 of Np columns each that take turns, the
+                         // MMAs of one beside the epilogue of the other
+  int gop, gxs;          // bytes from one group's term operand, staged X to the other's
   int MT, KB;            // 128-row tiles of orbitals, 64-wide K blocks
   int nst;               // ring stages
   int resident;          // 1: A of a walker held in tensor memory for all its Taylor rounds,
@@ -215,8 +245,10 @@ struct TclShape {
 // Stages of a round, in order: for each row tile t and K block kb: E (one-body) or A_re, A_im (Taylor),
 // hi and lo tile each.
 
-template <int EPI>
-__global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
+// KS, NP (G == 2): 16-wide K steps of a product, Np.  As constants they leave no arithmetic between two
+// MMAs: with run-time strides the issuing lane needed some 60 cycles an MMA, 16 of them at this N.
+template <int EPI, int G, int KS, int NP>
+__global__ void __launch_bounds__(64 + 32 * EPI * G, EPI == 4 ? 2 : 1)
     k_propagate_tcl(const __grid_constant__ CUtensorMap tmAhi, const __grid_constant__ CUtensorMap tmAlo,
                     const __grid_constant__ CUtensorMap tmEhi, const __grid_constant__ CUtensorMap tmElo,
                     const TclShape sh, const double* phi_in, double* phi_out,
@@ -227,35 +259,44 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
                                              ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + sh.bar_off);
   const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + kMaxStages);
+  // (G == 2: group 1's dfull, bready, xfull and xread are kG barriers further on)
+  constexpr uint32_t kG = 8 * 9;
   const uint32_t dfull = smem_u32(bars + 2 * kMaxStages), bready = smem_u32(bars + 2 * kMaxStages + 1);
   const uint32_t done = smem_u32(bars + 2 * kMaxStages + 2);
   const uint32_t afull = smem_u32(bars + 2 * kMaxStages + 3), acopied = smem_u32(bars + 2 * kMaxStages + 4);
   const uint32_t xfull = smem_u32(bars + 2 * kMaxStages + 5), xread = smem_u32(bars + 2 * kMaxStages + 6);
   const uint32_t dfull1 = smem_u32(bars + 2 * kMaxStages + 7);   // the second row tile's accumulator
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kMaxStages + 8);
+  const uint32_t afree = smem_u32(bars + 2 * kMaxStages + 8);    // G == 2: both groups are done with A
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kBars);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rounds = sh.order + 2;
   const int64_t NM = (int64_t)sh.N * sh.M, plane = (int64_t)sh.Nw * NM;
+  const int Np = G == 2 ? NP : sh.Np, n2 = 2 * Np, KB = G == 2 ? (KS + 3) / 4 : sh.KB, bkb = 3 * Np * 128;
+  const int dcol = G == 2 ? kDcol2 : sh.dcol, gop = 2 * KB * bkb;
+  const int acol = G == 2 ? 4 * kDcol2 : sh.acol, ecol = G == 2 ? 4 * kDcol2 + 128 * KB : sh.ecol;
 
   if (threadIdx.x == 0) {
     for (int q = 0; q < sh.nst; ++q) {
       mbar_init(full0 + 8 * q, 1);
       mbar_init(empty0 + 8 * q, 1);
     }
-    mbar_init(dfull, 1);
     mbar_init(dfull1, 1);
-    mbar_init(bready, 32 * EPI);
     mbar_init(done, 1);
     mbar_init(afull, 1);
-    mbar_init(acopied, 32 * EPI);
-    mbar_init(xfull, 32 * EPI);
-    mbar_init(xread, 32 * EPI);
+    mbar_init(acopied, 32 * EPI * G);
+    mbar_init(afree, 1);
+    for (int g = 0; g < G; ++g) {
+      mbar_init(dfull + g * kG, 1);
+      mbar_init(bready + g * kG, 32 * EPI);
+      mbar_init(xfull + g * kG, 32 * EPI);
+      mbar_init(xread + g * kG, 32 * EPI);
+    }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   // the term operand starts at zero: padded rows and K beyond M stay zero throughout
-  for (int e = threadIdx.x; e < (sh.bbuf ? 4 : 2) * sh.KB * sh.bkb / 16; e += blockDim.x)
+  for (int e = threadIdx.x; e < (sh.bbuf || G == 2 ? 4 : 2) * KB * bkb / 16; e += blockDim.x)
     reinterpret_cast<uint4*>(smem + sh.bhi_off)[e] = make_uint4(0u, 0u, 0u, 0u);
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // visible to the tensor core
   if (warp == 1) {
@@ -281,8 +322,8 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
       const uint64_t pbytes = (uint64_t)NM * 8;             // one plane of Phi
       if (sh.eres) {
         // e^{-dt K/2} - I through the staging region into tensor memory, once per CTA
-        mbar_expect_tx(afull, 2 * sh.KB * kTile);
-        for (int kb = 0; kb < sh.KB; ++kb)
+        mbar_expect_tx(afull, 2 * KB * kTile);
+        for (int kb = 0; kb < KB; ++kb)
           for (int u = 0; u < 2; ++u)
             tma_load_2d(smem_u32(smem + sh.ares_off + (kb * 4 + u) * kTile), u ? &tmElo : &tmEhi, afull,
                         kb * 64, 0);
@@ -310,8 +351,8 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
               ok = false;
               break;
             }
-            mbar_expect_tx(afull, 4 * sh.KB * kTile);
-            for (int kb = 0; kb < sh.KB; ++kb)
+            mbar_expect_tx(afull, 4 * KB * kTile);
+            for (int kb = 0; kb < KB; ++kb)
               for (int u = 0; u < 4; ++u)
                 tma_load_3d(smem_u32(smem + sh.ares_off + (kb * 4 + u) * kTile),
                             (u & 1) ? &tmAlo : &tmAhi, afull, kb * 64, 0, (u >> 1) * sh.Nw + w);
@@ -319,7 +360,7 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
           }
           if (sh.resident && (taylor || sh.eres)) continue;
           for (int t = 0; t < sh.MT && ok; ++t)
-            for (int kb = 0; kb < sh.KB && ok; ++kb)
+            for (int kb = 0; kb < KB && ok; ++kb)
               for (int u = 0; u < (taylor ? 2 : 1); ++u, ++g) {
                 if (*abort_flag) { ok = false; break; }
                 if (g >= sh.nst && !mbar_wait(empty0 + 8 * st, ph ^ 1u, err, wait_ns)) {
@@ -350,14 +391,14 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
   } else if (warp == 1) {
     // ---- MMA issuer: the whole warp follows the loop, so every operand address is warp-uniform,
     // and one elected lane issues; lane 0 polls the barriers and broadcasts the outcome ----
-    const uint32_t idesc = idesc_n(sh.n2);
+    const uint32_t idesc = idesc_n(n2);
     const uint32_t bhi = smem_u32(smem + sh.bhi_off), blo = smem_u32(smem + sh.blo_off);
     const uint64_t dbh0 = sw128_desc(bhi), dbl0 = sw128_desc(blo);
-    const uint32_t bkb16 = (uint32_t)(sh.bkb >> 4), np16 = (uint32_t)(sh.Np * 8);
-    const int nks_last = min(4, (sh.M - 64 * (sh.KB - 1) + 15) / 16);
-    int rq = 0, st = 0;
+    const uint32_t bkb16 = (uint32_t)(bkb >> 4), np16 = (uint32_t)(Np * 8);
+    const int nks_last = min(4, (sh.M - 64 * (KB - 1) + 15) / 16);
+    int rq = 0, st = 0, jw = 0;
     uint32_t ph = 0;   // parity of the ring stage's current use
-    const int nst = sh.nst, KB = sh.KB, MT = sh.MT;
+    const int nst = sh.nst, MT = sh.MT;
     const uint64_t dring = sw128_desc(smem_u32(smem + sh.ring_off));
     bool ok = true;
     auto wait_all = [&](uint32_t bar, int parity) {
@@ -371,22 +412,43 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
       if (alive && !alive[w]) continue;
       for (int q = 0; q < rounds && ok; ++q, ++rq) {
         const bool taylor = q >= 1 && q <= sh.order;
+        if constexpr (G == 2) {
+          // E (before the first walker) and this walker's A (before its first term) in tensor memory
+          if ((jw == 0 || q == 1) && !wait_all(acopied, jw++ & 1)) { ok = false; break; }
+#pragma unroll
+          for (int g = 0; g < G; ++g) {
+            if (!wait_all(bready + g * kG, rq & 1)) { ok = false; break; }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            if (elect_one()) {
+              const uint64_t go = (uint64_t)(g * (gop >> 4));
+              const uint32_t d = tmem + (uint32_t)(g * dcol);
+              if (taylor)
+                mma_round_const<KS, 4, NP>(d, tmem + (uint32_t)acol, dbh0 + go, dbl0 + go);
+              else
+                mma_round_const<KS, 2, NP>(d, tmem + (uint32_t)ecol, dbh0 + go, dbl0 + go);
+              mma_commit(dfull + g * kG);
+              if (g == 1 && q == sh.order) mma_commit(afree);
+            }
+            __syncwarp();
+          }
+          continue;
+        }
         const uint64_t boff = (uint64_t)((rq & 1) * (sh.bbuf >> 4)), dbh = dbh0 + boff, dbl = dbl0 + boff;
         if (!wait_all(bready, rq & 1)) { ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (sh.resident && (taylor || sh.eres)) {
           // every A plane in tensor memory (one tile row, MT = 1)
           if (elect_one()) {
-            if (sh.KB == 2) {
+            if (KB == 2) {
               if (taylor)
-                mma_round_tmem<2, 4>(tmem, tmem + (uint32_t)sh.acol, dbh, dbl, bkb16, np16, idesc, nks_last);
+                mma_round_tmem<2, 4>(tmem, tmem + (uint32_t)acol, dbh, dbl, bkb16, np16, idesc, nks_last);
               else
-                mma_round_tmem<2, 2>(tmem, tmem + (uint32_t)sh.ecol, dbh, dbl, bkb16, np16, idesc, nks_last);
+                mma_round_tmem<2, 2>(tmem, tmem + (uint32_t)ecol, dbh, dbl, bkb16, np16, idesc, nks_last);
             } else {
               if (taylor)
-                mma_round_tmem<1, 4>(tmem, tmem + (uint32_t)sh.acol, dbh, dbl, bkb16, np16, idesc, nks_last);
+                mma_round_tmem<1, 4>(tmem, tmem + (uint32_t)acol, dbh, dbl, bkb16, np16, idesc, nks_last);
               else
-                mma_round_tmem<1, 2>(tmem, tmem + (uint32_t)sh.ecol, dbh, dbl, bkb16, np16, idesc, nks_last);
+                mma_round_tmem<1, 2>(tmem, tmem + (uint32_t)ecol, dbh, dbl, bkb16, np16, idesc, nks_last);
             }
             mma_commit(dfull);
           }
@@ -397,7 +459,7 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
         // stages kept the tensor core waiting for 500 of every 1000 cycles)
         const int npair = taylor ? 2 : 1;
         for (int t = 0; t < MT && ok; ++t) {
-          const uint32_t d = tmem + (uint32_t)(t * sh.dcol);
+          const uint32_t d = tmem + (uint32_t)(t * dcol);
           for (int kb = 0; kb < KB && ok; ++kb) {
             const int nks = kb == KB - 1 ? nks_last : 4;   // K steps holding orbitals
             for (int u = 0; u < npair; ++u) {
@@ -431,17 +493,23 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
     // take alternate 16-column groups.  The term operand is written by transposed 8x8 stores:
     // one 16-byte row chunk holds 8 consecutive orbitals of one operand row ----
     const int qd = warp & 3, r = 32 * qd + lane;
-    const int half = EPI == 8 ? (warp - 2) >> 2 : 0, cstep = EPI == 8 ? 32 : 16;
+    const int grp = G == 2 ? (warp - 2) / EPI : 0, ew = warp - 2 - grp * EPI;
+    const int half = EPI == 8 ? ew >> 2 : 0, cstep = EPI == 8 ? 32 : 16;
+    // this group's columns, barriers and accumulator
+    const int col0 = grp * Np, ncol = G == 2 ? min(Np, sh.N - col0) : sh.N;
+    const uint32_t tmg = tmem + (uint32_t)(grp * dcol), gb = grp * kG;
+    const uint32_t dfullg = dfull + gb, breadyg = bready + gb, xfullg = xfull + gb, xreadg = xread + gb;
     const uint32_t lanes = (uint32_t)(32 * qd) << 16;
-    const uint32_t bhi_s0 = smem_u32(smem + sh.bhi_off), blo_s0 = smem_u32(smem + sh.blo_off);
-    const uint32_t sreg = (uint32_t)(sh.MT * sh.dcol);   // S region after the D columns
+    const uint32_t bhi_s0 = smem_u32(smem + sh.bhi_off) + (uint32_t)(grp * gop);
+    const uint32_t blo_s0 = smem_u32(smem + sh.blo_off) + (uint32_t)(grp * gop);
+    const uint32_t sreg = (uint32_t)(G * sh.MT * dcol);   // S region after the D columns
     const int jj = lane >> 3, kk = lane & 7, fr = lane >> 2, fc = 2 * (lane & 3);
     // fragment element j: lane offset fr (+ 8), column offset fc (+ 1) (+ 8)
     auto lane_of = [&](int j) { return fr + ((j & 2) ? 8 : 0); };
     auto col_of = [&](int j) { return fc + (j & 1) + ((j & 4) ? 8 : 0); };
     // shared address of the row chunk (operand row R, orbitals i0 .. i0 + 7) of one 8x8 store
     auto chunk = [&](uint32_t buf, int R, int i0) {
-      return buf + (uint32_t)((i0 >> 6) * sh.bkb + R * 128 + ((((i0 & 63) >> 3) ^ (R & 7)) << 4));
+      return buf + (uint32_t)((i0 >> 6) * bkb + R * 128 + ((((i0 & 63) >> 3) ^ (R & 7)) << 4));
     };
     // the block's values (orbitals i0b .., columns c0 ..) into operand rows Np + c, and with neg,
     // -value into rows c - Np for the imaginary columns c >= Np
@@ -453,33 +521,34 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
       for (int j = 0; j < 4; ++j) split_pair(v[2 * j], v[2 * j + 1], h[j], l[j]);
       // matrix jj: orbitals i0b + 8 (jj & 1) .., columns c0 + 8 (jj >> 1) ..; this lane: row kk
       const int i0 = i0b + 8 * (jj & 1), c = c0 + 8 * (jj >> 1) + kk;
-      stsm_x4_t(chunk(bhi_s, sh.Np + c, i0), h);
-      stsm_x4_t(chunk(blo_s, sh.Np + c, i0), l);
-      if (!neg || c0 + 8 < sh.Np) return;   // no imaginary column in the group
+      stsm_x4_t(chunk(bhi_s, Np + c, i0), h);
+      stsm_x4_t(chunk(blo_s, Np + c, i0), l);
+      if (!neg || c0 + 8 < Np) return;   // no imaginary column in the group
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         h[j] ^= 0x80008000u;
         l[j] ^= 0x80008000u;
       }
-      if (c0 >= sh.Np) {
-        stsm_x4_t(chunk(bhi_s, c - sh.Np, i0), h);
-        stsm_x4_t(chunk(blo_s, c - sh.Np, i0), l);
+      if (c0 >= Np) {
+        stsm_x4_t(chunk(bhi_s, c - Np, i0), h);
+        stsm_x4_t(chunk(blo_s, c - Np, i0), l);
       } else {
         // only the second 8-column block is imaginary: matrices 2, 3 (lanes 0..15 give rows)
-        const int cn = c0 + 8 + kk - sh.Np;
+        const int cn = c0 + 8 + kk - Np;
         stsm_x2_t(chunk(bhi_s, cn, i0), h[2], h[3]);
         stsm_x2_t(chunk(blo_s, cn, i0), l[2], l[3]);
       }
     };
     bool ok = true;
     // resident A: the staging tiles into tensor memory; lane r takes row r of every tile (16-byte
-    // chunks in the 128-byte swizzle), the two warps of a lane quadrant take planes
-    // {2 half, 2 half + 1} of the first np planes, from TMEM column col0
-    auto copy_planes = [&](int np, int col0) {
+    // chunks in the 128-byte swizzle), the 2 G warps of a lane quadrant take 2 / G of the first np
+    // planes each, from TMEM column tcol on
+    auto copy_planes = [&](int np, int tcol) {
       const bool okw = !*abort_flag && mbar_wait(afull, jw & 1, err, wait_ns);
       if (!__all_sync(0xffffffffu, okw)) { fail(); return false; }
-      for (int u = 2 * half; u < 2 * half + 2 && u < np; ++u)
-        for (int kb = 0; kb < sh.KB; ++kb) {
+      const int u0 = G == 2 ? 2 * grp + half : 2 * half;
+      for (int u = u0; u < u0 + 2 / G && u < np; ++u)
+        for (int kb = 0; kb < KB; ++kb) {
           const uint4* row = reinterpret_cast<const uint4*>(smem + sh.ares_off + (kb * 4 + u) * kTile + r * 128);
           uint32_t v[32];
 #pragma unroll
@@ -487,30 +556,31 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
             const uint4 c = row[j ^ (r & 7)];
             v[4 * j] = c.x; v[4 * j + 1] = c.y; v[4 * j + 2] = c.z; v[4 * j + 3] = c.w;
           }
-          const uint32_t ta = tmem + lanes + (uint32_t)(col0 + 32 * (u * sh.KB + kb));
+          const uint32_t ta = tmem + lanes + (uint32_t)(tcol + 32 * (u * KB + kb));
           tmem_st16(ta, *reinterpret_cast<const uint32_t(*)[16]>(v));
           tmem_st16(ta + 16, *reinterpret_cast<const uint32_t(*)[16]>(v + 16));
         }
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      if (G == 2) asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");   // the MMA warp waits for it
       mbar_arrive(acopied);   // the staging region may take the next tiles
       ++jw;
       return true;
     };
     // this warp's (tile, slab, 16-column group) items: item it -> tile it / (2 ngh), slab
     // (it % 2 ngh) / ngh, columns 16 half + (it % ngh) cstep
-    const int ngh = (sh.n2 - 16 * half + cstep - 1) / cstep;
+    const int ngh = (n2 - 16 * half + cstep - 1) / cstep;
     const int nitems = sh.MT * 2 * ngh;
-    if (sh.eres && !copy_planes(2, sh.ecol)) ok = false;
+    if (sh.eres && !copy_planes(2, ecol)) ok = false;
     // staged X: element e of a walker is column c = e / M, orbital i = e % M (FP32); thread t of
     // the epilogue takes e = t + 32 EPI (q + rounds u) in round q, so a walker's X is loaded
     // during the previous walker's rounds, each load issued before the round's wait
-    float* xst = reinterpret_cast<float*>(smem + sh.ring_off);
-    const int et = threadIdx.x - 64, nte = 32 * EPI, nx = sh.n2 * sh.M;
+    float* xst = reinterpret_cast<float*>(smem + sh.ring_off + grp * sh.gxs);
+    const int et = 32 * ew + lane, nte = 32 * EPI, nx = n2 * sh.M;
     const int xu = (nx + nte * rounds - 1) / (nte * rounds);     // elements per thread and round
     const int xdc = nte / sh.M, xdi = nte - (nte / sh.M) * sh.M;
     auto x_elem = [&](int wn, int e) -> double {
-      const int c = e / sh.M, i = e - c * sh.M, b = c < sh.Np ? c : c - sh.Np;
-      return b < sh.N ? phi_in[(c < sh.Np ? 0 : plane) + ((int64_t)wn * sh.N + b) * sh.M + i] : 0.0;
+      const int c = e / sh.M, i = e - c * sh.M, b = c < Np ? c : c - Np;
+      return b < ncol ? phi_in[(c < Np ? 0 : plane) + ((int64_t)wn * sh.N + col0 + b) * sh.M + i] : 0.0;
     };
     auto x_put = [&](int e, double v) {
       const int c = e / sh.M, i = e - c * sh.M;
@@ -533,7 +603,7 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
           for (int u = 0; u < 4; ++u)
             if (e0 + u * nte < nx) x_put(e0 + u * nte, v[u]);
         }
-      mbar_arrive(xfull);
+      mbar_arrive(xfullg);
     }
     int kx = 0;   // live walkers of this CTA so far
     for (int w = blockIdx.x; w < sh.Nw && ok; w += gridDim.x) {
@@ -545,13 +615,14 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
       int xe = et, xc = et / sh.M, xi = et - (et / sh.M) * sh.M;
       if (sh.xs) {
         // this walker's X, staged by every epilogue thread, is complete
-        const bool okx = !*abort_flag && mbar_wait(xfull, kw & 1, err, wait_ns);
+        const bool okx = !*abort_flag && mbar_wait(xfullg, kw & 1, err, wait_ns) &&
+                         (G == 1 || kw == 0 || mbar_wait(afree, (kw - 1) & 1, err, wait_ns));
         if (!__all_sync(0xffffffffu, okx)) { fail(); ok = false; break; }
-        if (!copy_planes(4, sh.acol)) { ok = false; break; }
+        if (!copy_planes(4, acol)) { ok = false; break; }
         for (int it = 0; it < nitems; ++it) {
           const int t = it / (2 * ngh), sl = (it % (2 * ngh)) / ngh;
           const int c0 = 16 * half + (it % ngh) * cstep, i0b = 128 * t + 32 * qd + 16 * sl;
-          const uint32_t tl = tmem + ((uint32_t)(32 * qd + 16 * sl) << 16);
+          const uint32_t tl = tmg + ((uint32_t)(32 * qd + 16 * sl) << 16);
           float x[8];
           uint32_t v[8];
 #pragma unroll
@@ -560,11 +631,11 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
             x[j] = i < sh.M ? xst[c * sh.xs_ld + i] : 0.f;
             v[j] = __float_as_uint(x[j]);
           }
-          tmem_st_frag(tl + sreg + (uint32_t)(t * sh.dcol + c0), v);
-          if (i0b < 64 * sh.KB) put_block(x, i0b, c0, false, rq);
+          tmem_st_frag(tl + sreg + (uint32_t)(t * dcol + c0), v);
+          if (i0b < 64 * KB) put_block(x, i0b, c0, false, rq);
         }
-        mbar_arrive(xread);   // the staged X may take the next walker's once all have read it
-      } else
+        mbar_arrive(xreadg);   // the staged X may take the next walker's once all have read it
+      } else if constexpr (G == 1)
       // S = X (this walker's columns) and the operand [X_re; X_im] for the first one-body round.
       // The (tile, slab, column group) items of this warp go in batches of 4: every load of a
       // batch is issued first, so the walker pays one memory latency per batch, and the first
@@ -577,19 +648,19 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
           const int c0 = 16 * half + (it % ngh) * cstep, i0b = 128 * t + 32 * qd + 16 * sl;
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            const int i = i0b + lane_of(j), c = c0 + col_of(j), b = c < sh.Np ? c : c - sh.Np;
+            const int i = i0b + lane_of(j), c = c0 + col_of(j), b = c < Np ? c : c - Np;
             xv[u][j] = (it < nitems && i < sh.M && b < sh.N)
-                           ? phi_in[(c < sh.Np ? 0 : plane) + ((int64_t)w * sh.N + b) * sh.M + i]
+                           ? phi_in[(c < Np ? 0 : plane) + ((int64_t)w * sh.N + b) * sh.M + i]
                            : 0.0;
           }
         }
-        if (b0 == 0 && sh.resident && !copy_planes(4, sh.acol)) { ok = false; break; }
+        if (b0 == 0 && sh.resident && !copy_planes(4, acol)) { ok = false; break; }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           const int it = b0 + u, t = it / (2 * ngh), sl = (it % (2 * ngh)) / ngh;
           const int c0 = 16 * half + (it % ngh) * cstep, i0b = 128 * t + 32 * qd + 16 * sl;
           if (it >= nitems) break;
-          const uint32_t tl = tmem + ((uint32_t)(32 * qd + 16 * sl) << 16);
+          const uint32_t tl = tmg + ((uint32_t)(32 * qd + 16 * sl) << 16);
           float x[8];
           uint32_t v[8];
 #pragma unroll
@@ -597,15 +668,15 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
             x[j] = f64_to_f32_rn(xv[u][j]);
             v[j] = __float_as_uint(x[j]);
           }
-          tmem_st_frag(tl + sreg + (uint32_t)(t * sh.dcol + c0), v);
-          if (i0b < 64 * sh.KB) put_block(x, i0b, c0, false, rq);
+          tmem_st_frag(tl + sreg + (uint32_t)(t * dcol + c0), v);
+          if (i0b < 64 * KB) put_block(x, i0b, c0, false, rq);
         }
       }
       if (!ok) break;
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      mbar_arrive(bready);
+      mbar_arrive(breadyg);
       for (int q = 0; q < rounds && ok; ++q, ++rq) {
         const bool last = q == rounds - 1;
         // this round's share of the next walker's X: loaded now, staged after the round's
@@ -618,9 +689,9 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
 #pragma unroll
           for (int u = 0; u < kXu; ++u) {
             const bool v = u < xu && xe < nx;
-            const int b = xc < sh.Np ? xc : xc - sh.Np;
-            xp[u] = v && b < sh.N
-                        ? phi_in[(xc < sh.Np ? 0 : plane) + ((int64_t)wn * sh.N + b) * sh.M + xi]
+            const int b = xc < Np ? xc : xc - Np;
+            xp[u] = v && b < ncol
+                        ? phi_in[(xc < Np ? 0 : plane) + ((int64_t)wn * sh.N + col0 + b) * sh.M + xi]
                         : 0.0;
             xo[u] = v ? xc * sh.xs_ld + xi : -1;
             if (v) {   // the thread's next element: e + nte
@@ -631,9 +702,9 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
             }
           }
         // the first row tile's products; all of them when its epilogue overwrites their operand
-        bool okw = !*abort_flag && mbar_wait(dfull, rq & 1, err, wait_ns);
+        bool okw = !*abort_flag && mbar_wait(dfullg, rq & 1, err, wait_ns);
         if (sh.MT > 1 && !sh.bbuf) okw = okw && !*abort_flag && mbar_wait(dfull1, rq & 1, err, wait_ns);
-        if (pre && q == 0) okw = okw && !*abort_flag && mbar_wait(xread, kw & 1, err, wait_ns);
+        if (pre && q == 0) okw = okw && !*abort_flag && mbar_wait(xreadg, kw & 1, err, wait_ns);
         if (!__all_sync(0xffffffffu, okw)) { fail(); ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const float inv = (q >= 1 && q <= sh.order) ? 1.f / (float)q : 1.f;
@@ -645,12 +716,12 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
           }
           for (int sl = 0; sl < 2; ++sl) {
             const int i0b = 128 * t + 32 * qd + 16 * sl;
-            const bool in_b = i0b < 64 * sh.KB;
-            const uint32_t tl = tmem + ((uint32_t)(32 * qd + 16 * sl) << 16);
-            for (int c0 = 16 * half; c0 < sh.n2; c0 += cstep) {
+            const bool in_b = i0b < 64 * KB;
+            const uint32_t tl = tmg + ((uint32_t)(32 * qd + 16 * sl) << 16);
+            for (int c0 = 16 * half; c0 < n2; c0 += cstep) {
               uint32_t dv[8], sv[8];
-              tmem_ld_frag(tl + (uint32_t)(t * sh.dcol + c0), dv);
-              tmem_ld_frag(tl + sreg + (uint32_t)(t * sh.dcol + c0), sv);
+              tmem_ld_frag(tl + (uint32_t)(t * dcol + c0), dv);
+              tmem_ld_frag(tl + sreg + (uint32_t)(t * dcol + c0), sv);
               tmem_wait_ld();
               float x[8];
               if (q == 0) {
@@ -660,7 +731,7 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
                   x[j] = __uint_as_float(sv[j]) + __uint_as_float(dv[j]);
                   sv[j] = __float_as_uint(x[j]);
                 }
-                tmem_st_frag(tl + sreg + (uint32_t)(t * sh.dcol + c0), sv);
+                tmem_st_frag(tl + sreg + (uint32_t)(t * dcol + c0), sv);
                 if (in_b) put_block(x, i0b, c0, true, rq + 1);
               } else if (!last) {
                 // T_q = A T_{q-1} / q; S += T_q; operand = T_q, or S after the last term
@@ -671,16 +742,16 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
                   y[j] = __uint_as_float(sv[j]) + x[j];
                   sv[j] = __float_as_uint(y[j]);
                 }
-                tmem_st_frag(tl + sreg + (uint32_t)(t * sh.dcol + c0), sv);
+                tmem_st_frag(tl + sreg + (uint32_t)(t * dcol + c0), sv);
                 if (in_b) put_block(q < sh.order ? x : y, i0b, c0, q < sh.order, rq + 1);
               } else {
                 // Phi' = S + (E - I) S
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                  const int i = i0b + lane_of(j), c = c0 + col_of(j), b = c < sh.Np ? c : c - sh.Np;
-                  if (i < sh.M && b < sh.N) {
+                  const int i = i0b + lane_of(j), c = c0 + col_of(j), b = c < Np ? c : c - Np;
+                  if (i < sh.M && b < ncol) {
                     const float y = __uint_as_float(sv[j]) + __uint_as_float(dv[j]);
-                    const int64_t gi = (c < sh.Np ? 0 : plane) + ((int64_t)w * sh.N + b) * sh.M + i;
+                    const int64_t gi = (c < Np ? 0 : plane) + ((int64_t)w * sh.N + col0 + b) * sh.M + i;
                     phi_out[gi] = f32_to_f64(y);
                     if (phi_out32) phi_out32[gi] = y;
                   }
@@ -694,13 +765,13 @@ __global__ void __launch_bounds__(64 + 32 * EPI, EPI == 4 ? 2 : 1)
           asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-          mbar_arrive(bready);
+          mbar_arrive(breadyg);
         }
         if (pre) {
 #pragma unroll
           for (int u = 0; u < kXu; ++u)
             if (xo[u] >= 0) xst[xo[u]] = f64_to_f32_rn(xp[u]);
-          if (last) mbar_arrive(xfull);   // the next walker's X is staged
+          if (last) mbar_arrive(xfullg);   // the next walker's X is staged
         }
       }
     }
@@ -759,21 +830,22 @@ cudaError_t make_map(CUtensorMap* map, void* base, int M, int Mp, int64_t nz) {
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-TclShape shape_of(const Ctx& c, int nst, int resident, int two = 0) {
+TclShape shape_of(const Ctx& c, int nst, int resident, int two = 0, int G = 1) {
   TclShape s{};
   s.ahi = c.tcl_ahi;
   s.alo = c.tcl_alo;
   s.Mp = propagate_tcl_mp(c.M);
   s.M = c.M;
   s.N = c.N;
-  s.Np = (c.N + 7) / 8 * 8;
+  s.G = G;
+  s.Np = ((c.N + G - 1) / G + 7) / 8 * 8;
   s.n2 = 2 * s.Np;
   s.MT = (c.M + 127) / 128;
   s.KB = (c.M + 63) / 64;
   s.nst = nst;
   s.bkb = 3 * s.Np * 128;
-  s.dcol = (s.n2 + 63) / 64 * 64;
-  s.acol = 2 * s.MT * s.dcol;
+  s.dcol = G == 2 ? kDcol2 : (s.n2 + 63) / 64 * 64;
+  s.acol = 2 * G * s.MT * s.dcol;
   uint32_t need = (uint32_t)(s.acol + (resident ? 4 * 32 * s.KB : 0)), cols = 32;
   s.ecol = (int)need;
   s.eres = resident && need + 2 * 32 * s.KB <= 512u;
@@ -787,21 +859,29 @@ TclShape shape_of(const Ctx& c, int nst, int resident, int two = 0) {
   // (the staging covers kXu elements per epilogue thread and round)
   s.xs = resident && s.eres && s.n2 * s.M <= kXu * 32 * 8 * (s.order + 2);
   s.xs_ld = s.M + 4;   // rows 4 floats apart: the fragment reads below fall in distinct banks
-  s.ares_off = s.xs ? (s.n2 * s.xs_ld * 4 + 1023) / 1024 * 1024 : nst * kStage;
+  s.gxs = (s.n2 * s.xs_ld * 4 + 1023) / 1024 * 1024;
+  s.ares_off = s.xs ? G * s.gxs : nst * kStage;
   s.bhi_off = s.ares_off + (resident ? 4 * s.KB * kTile : 0);
   s.blo_off = s.bhi_off + s.KB * s.bkb;
   s.bbuf = two ? 2 * s.KB * s.bkb : 0;   // [hi][lo] of round parity 0, then of parity 1
-  s.bar_off = s.blo_off + s.KB * s.bkb + s.bbuf;
-  s.smem_bytes = s.bar_off + 8 * (2 * kMaxStages + 8) + 16 + 1024;
+  s.gop = 2 * s.KB * s.bkb;
+  s.bar_off = s.bhi_off + G * s.gop + s.bbuf;
+  s.smem_bytes = s.bar_off + 8 * kBars + 16 + 1024;
   return s;
 }
 
-// Launch form: A resident with 8 epilogue warps, one CTA per SM (M <= 128); else A streamed, two CTAs
+// Launch form: M <= 128: A resident, one CTA per SM, two column groups of 8 epilogue warps if there are more
+// than 8 columns (below, one group fills an MMA of N = 16 and a second would be padding) and the rounds cover
+// the next walker's loads, else one group; else A streamed, two CTAs
 // per SM of 4 epilogue warps when a ring of at least 2 stages (of 32 KB) fits 113 KB, otherwise one
 // CTA per SM of 8 epilogue warps with two copies of the term operand and the deepest ring that fits (two
 // stages at N M = 4096, the largest system).
 TclShape plan(const Ctx& c) {
   if (c.M <= 128) {
+    if (c.N > 8) {
+      const TclShape s = shape_of(c, 1, 1, 0, 2);
+      if (s.xs && s.tcols <= 512 && s.smem_bytes <= 227 * 1024) return s;
+    }
     const TclShape s = shape_of(c, 1, 1);
     if (s.smem_bytes <= 227 * 1024) return s;
   }
@@ -814,6 +894,15 @@ TclShape plan(const Ctx& c) {
     if (s.smem_bytes <= 227 * 1024) return s;
   }
   return shape_of(c, 2, 0, 1);
+}
+
+// The two-group kernel for ks K steps (even: one step of zero padding at most) and groups of np columns.
+using GroupsKernel = decltype(&k_propagate_tcl<8, 2, 8, 16>);
+GroupsKernel groups_kernel(int ks, int np) {
+#define AFQ_G(NP) \
+  (ks <= 2 ? k_propagate_tcl<8, 2, 2, NP> : ks <= 4 ? k_propagate_tcl<8, 2, 4, NP> : ks <= 6 ? k_propagate_tcl<8, 2, 6, NP> : k_propagate_tcl<8, 2, 8, NP>)
+  return np == 8 ? AFQ_G(8) : AFQ_G(16);
+#undef AFQ_G
 }
 
 bool two_per_sm(const TclShape& s) { return !s.resident && s.smem_bytes <= 113 * 1024; }
@@ -831,10 +920,14 @@ bool propagate_tcl_ok(const Ctx& c) {
 int propagate_tcl_mp(int M) { return (M + 63) / 64 * 64; }
 
 cudaError_t prepare_propagate_tcl() {
-  cudaError_t e = cudaFuncSetAttribute(k_propagate_tcl<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(k_propagate_tcl<4, 1, 0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        227 * 1024);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_propagate_tcl<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    e = cudaFuncSetAttribute(k_propagate_tcl<8, 1, 0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  for (int np = 8; np <= 16; np += 8)
+    for (int ks = 2; ks <= 8; ks += 2)
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(groups_kernel(ks, np), cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   return e;
 }
 
@@ -865,12 +958,16 @@ cudaError_t launch_propagate_tcl(const Ctx& c, double* out, float* out32, cudaSt
   if (!propagate_tcl_ok(c) || !c.tcl_maps) return cudaErrorInvalidValue;
   const TclShape sh = plan(c);
   const int* al = out == c.phi ? c.alive : nullptr;
-  if (two_per_sm(sh)) {
-    k_propagate_tcl<4><<<std::min(c.Nw, 2 * 152), 64 + 32 * 4, sh.smem_bytes, s>>>(
+  if (sh.G == 2) {
+    groups_kernel((c.M + 15) / 16, sh.Np)<<<std::min(c.Nw, 152), 64 + 32 * 16, sh.smem_bytes, s>>>(
+        c.tcl_maps[0], c.tcl_maps[1], c.tcl_maps[2], c.tcl_maps[3], sh, c.phi, out, out32, al,
+        c.d_tc_err, kWaitNs);
+  } else if (two_per_sm(sh)) {
+    k_propagate_tcl<4, 1, 0, 0><<<std::min(c.Nw, 2 * 152), 64 + 32 * 4, sh.smem_bytes, s>>>(
         c.tcl_maps[0], c.tcl_maps[1], c.tcl_maps[2], c.tcl_maps[3], sh, c.phi, out, out32, al,
         c.d_tc_err, kWaitNs);
   } else {
-    k_propagate_tcl<8><<<std::min(c.Nw, 152), 64 + 32 * 8, sh.smem_bytes, s>>>(
+    k_propagate_tcl<8, 1, 0, 0><<<std::min(c.Nw, 152), 64 + 32 * 8, sh.smem_bytes, s>>>(
         c.tcl_maps[0], c.tcl_maps[1], c.tcl_maps[2], c.tcl_maps[3], sh, c.phi, out, out32, al,
         c.d_tc_err, kWaitNs);
   }
