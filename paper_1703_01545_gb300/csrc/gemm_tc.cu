@@ -76,73 +76,80 @@ __device__ __forceinline__ void tri_tile(int tm, int& a, int& b, int& h) {
   b = q - a * (a + 1) / 2;
 }
 
-// Split output of 32 accumulator columns of the index pair (i, j) (skipped outside the
-// M x M matrix); with `stg`, the pair's hi and lo values also go to column q of the staging
-// arrays [32][128] at row r, for the transposed write of the mirror block.
-__device__ __forceinline__ void store_split_ij(const SplitOut& so, int i, int j, int n0, int Nd,
-                                               float alpha, const uint32_t (&v)[32],
-                                               __nv_bfloat16* stg, int r) {
-  const bool in = i < so.M && j < so.M;
-  const int64_t off = (int64_t)i * so.Mp + j;
+// Split output of 16 accumulator columns of a half block of the lower triangle, by the 128 threads of an
+// epilogue group (thread r holds the index pair (i, j) = (i0 + r / 16, j0 + r % 16)).  A pair of lanes
+// (j even, j + 1) exchanges columns, so that each writes both of its j for half of them, 4 bytes at a time
+// (rows of V are whole 16-byte units: what an odd M's last pair writes beyond j < M is the padding's zero).
+// With `stg` ([16 columns][16 j][8 i] packed hi | lo words, the 16-byte halves of a j's 32 bytes swapped by
+// bit 2 of j, so that neither side meets a bank conflict beyond two lanes) the values are also staged for
+// the mirror block.
+__device__ __forceinline__ void store_tri16(const SplitOut& so, int i, int j, int n0, int Nd, float alpha,
+                                            const uint32_t (&v)[16], uint32_t* stg, int r) {
+  const bool in = i < so.M && (j & ~1) < so.M;
+  const int odd = j & 1, jj = r & 15, ii = r >> 4;
+  const int64_t off = (int64_t)i * so.Mp + (j & ~1);
+  uint32_t* sw = stg ? stg + jj * 8 + ((((ii >> 2) ^ (jj >> 2)) & 1) << 2) + (ii & 3) : nullptr;
 #pragma unroll
-  for (int q = 0; q < 32; ++q) {
-    const int n = n0 + q;
-    const float x = alpha * __uint_as_float(v[q]);
-    const __nv_bfloat16 h = __float2bfloat16_rn(x);
-    const __nv_bfloat16 l = __float2bfloat16_rn(x - __bfloat162float(h));
+  for (int q = 0; q < 16; q += 2) {
+    uint32_t w[2];   // columns q, q + 1: hi in the low half
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const float x = alpha * __uint_as_float(v[q + u]);
+      const __nv_bfloat16 h = __float2bfloat16_rn(x);
+      const __nv_bfloat16 l = __float2bfloat16_rn(x - __bfloat162float(h));
+      w[u] = (uint32_t)__bfloat16_as_ushort(h) | ((uint32_t)__bfloat16_as_ushort(l) << 16);
+      if (sw) sw[(q + u) * 128] = w[u];
+    }
+    // even lanes write column q, odd ones q + 1
+    const uint32_t got = __shfl_xor_sync(0xffffffffu, odd ? w[0] : w[1], 1);
+    const uint32_t lo_j = odd ? got : w[0], hi_j = odd ? w[1] : got;
+    const int n = n0 + q + odd;
     if (in && n < Nd) {
-      so.hi[(int64_t)n * so.ld + off] = h;
-      so.lo[(int64_t)n * so.ld + off] = l;
-    }
-    if (stg) {
-      stg[q * BM + r] = h;
-      stg[32 * BM + q * BM + r] = l;
+      *reinterpret_cast<uint32_t*>(so.hi + (int64_t)n * so.ld + off) = __byte_perm(lo_j, hi_j, 0x5410);
+      *reinterpret_cast<uint32_t*>(so.lo + (int64_t)n * so.ld + off) = __byte_perm(lo_j, hi_j, 0x7632);
     }
   }
 }
 
-// The staged 8 x 16 (i, j) half block of 32 columns written transposed: V[j][i0 .. i0 + 7]
-// for the 16 j of the block, 16 bytes per (column, j, hi / lo); task t of the 128 epilogue
-// threads' 1024.
-__device__ __forceinline__ void store_mirror(const SplitOut& so, const __nv_bfloat16* stg, int i0,
-                                             int j0, int n0, int Nd, int tid) {
-  for (int task = tid; task < 32 * 16 * 2; task += 128) {
-    const int q = task >> 5, jj = (task >> 1) & 15, hl = task & 1;
-    const int n = n0 + q, j = j0 + jj;
-    if (n >= Nd || j >= so.M) continue;
-    const __nv_bfloat16* src = stg + hl * 32 * BM + q * BM + jj;   // row r = 16 ii + jj
-    __nv_bfloat16* dst = (hl ? so.lo : so.hi) + (int64_t)n * so.ld + (int64_t)j * so.Mp + i0;
-    if (i0 + 8 <= so.M) {
-      __align__(16) __nv_bfloat16 pk[8];
+// The staged half block written transposed: V[j][i0 .. i0 + 7] for the 16 j, 16 bytes per (column, j, hi /
+// lo); two (column, j) tasks for each of the group's 128 threads.
+__device__ __forceinline__ void store_mirror16(const SplitOut& so, const uint32_t* stg, int i0, int j0, int n0,
+                                               int Nd, int tid) {
 #pragma unroll
-      for (int ii = 0; ii < 8; ++ii) pk[ii] = src[16 * ii];
-      *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(pk);
-    } else {
-      for (int ii = 0; ii < 8 && i0 + ii < so.M; ++ii) dst[ii] = src[16 * ii];
+  for (int task = tid; task < 16 * 16; task += 128) {
+    const int q = task >> 4, jj = task & 15, n = n0 + q, j = j0 + jj;
+    const uint32_t* src = stg + q * 128 + jj * 8;
+    const int f = (jj >> 2) & 1;
+    const uint4 a = *reinterpret_cast<const uint4*>(src + 4 * f), b = *reinterpret_cast<const uint4*>(src + 4 * (f ^ 1));
+    if (n >= Nd || j >= so.M) continue;
+    const uint4 hi = make_uint4(__byte_perm(a.x, a.y, 0x5410), __byte_perm(a.z, a.w, 0x5410),
+                                __byte_perm(b.x, b.y, 0x5410), __byte_perm(b.z, b.w, 0x5410));
+    const uint4 lo = make_uint4(__byte_perm(a.x, a.y, 0x7632), __byte_perm(a.z, a.w, 0x7632),
+                                __byte_perm(b.x, b.y, 0x7632), __byte_perm(b.z, b.w, 0x7632));
+    const int64_t off = (int64_t)n * so.ld + (int64_t)j * so.Mp + i0;
+    if (i0 < so.M) {   // a row's 8 elements lie within its pitch; beyond i < M they are zero
+      *reinterpret_cast<uint4*>(so.hi + off) = hi;
+      *reinterpret_cast<uint4*>(so.lo + off) = lo;
     }
   }
 }
 
-// AND of `ok` over the 256 epilogue threads (named barrier 3): they leave the tile loop
-// together, so none is left waiting at a staging barrier.
+// AND of `ok` over the epilogue threads (named barrier 5): they leave the tile loop together, so none is
+// left waiting at a staging barrier.
+template <int THREADS>
 __device__ __forceinline__ bool epilogue_all(bool ok) {
   uint32_t r;
   asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.and.pred q, 3, 256, p;\n\t"
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.and.pred q, 5, %2, p;\n\t"
       "selp.u32 %0, 1, 0, q;\n\t}"
       : "=r"(r)
-      : "r"((uint32_t)ok)
+      : "r"((uint32_t)ok), "n"(THREADS)
       : "memory");
   return r != 0;
 }
 
 // The four warps of epilogue group g (named barrier 1 + g, 128 threads).
-__device__ __forceinline__ void group_sync(int g) {
-  if (g == 0)
-    asm volatile("bar.sync 1, 128;" ::: "memory");
-  else
-    asm volatile("bar.sync 2, 128;" ::: "memory");
-}
+__device__ __forceinline__ void group_sync(int g) { asm volatile("bar.sync %0, 128;" ::"r"(1 + g) : "memory"); }
 
 template <int BN, int STAGES, class TC>
 __global__ void __launch_bounds__(NTHREADS, 1)
@@ -267,11 +274,29 @@ struct PLayoutG {
   static constexpr int A_BYTES = BM * BK * 2;
   static constexpr int B_BYTES = PBN * BK * 2;
   static constexpr int STAGE_BYTES = 2 * A_BYTES + 2 * B_BYTES;
-  static constexpr int STG_OFFSET = PSTAGES * STAGE_BYTES;   // mirror staging per epilogue
-  static constexpr int STG_GROUP = 2 * 32 * BM;               // group: hi, lo [32][128] bf16
-  static constexpr int BAR_OFFSET = STG_OFFSET + 2 * STG_GROUP * 2;
+  static constexpr int BAR_OFFSET = PSTAGES * STAGE_BYTES;
   static constexpr int SMEM_BYTES = BAR_OFFSET + 256 + 1024;
 };
+
+// Accumulator columns cbeg .. cbeg + cnt - 1 of the lanes at TMEM address `acc`: output row m of the thread.
+__device__ __forceinline__ void store_columns(const SplitOut& so, float* __restrict__ C, int64_t ldc, uint32_t acc,
+                                              int m, int n0, int cbeg, int cnt, int Md, int Nd, float alpha) {
+  for (int c0 = cbeg; c0 < cbeg + cnt; c0 += 32) {
+    uint32_t v[32];
+    tmem_ld32(acc + (uint32_t)c0, v);
+    if (m < Md) {
+      if (so.hi) {
+        store_split(so, m, n0 + c0, Nd, alpha, v);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+          const int n = n0 + c0 + j;
+          if (n < Nd) C[(int64_t)n * ldc + m] = alpha * __uint_as_float(v[j]);
+        }
+      }
+    }
+  }
+}
 
 __global__ void __launch_bounds__(PTHREADS, 1)
     k_gemm_bf16x3_tc_persist(const __grid_constant__ CUtensorMap tmAh, const __grid_constant__ CUtensorMap tmAl,
@@ -376,53 +401,14 @@ __global__ void __launch_bounds__(PTHREADS, 1)
     // ---- epilogue: warp w drains TMEM lanes 32 (w % 4) .. + 31 (output rows m) of its
     // group's columns 128 g .. 128 g + 127 ----
     int i = 0;
-    const int grp = warp >> 2, wq = warp & 3, cbeg = grp * (PBN / 2), cend = cbeg + PBN / 2;
-    __nv_bfloat16* stg =
-        reinterpret_cast<__nv_bfloat16*>(smem + Lay::STG_OFFSET) + grp * Lay::STG_GROUP;
+    const int grp = warp >> 2, wq = warp & 3;
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++i) {
       const int b = i & 1, m0 = (t % mt) * BM, n0 = (t / mt) * PBN;
       const bool ok = mbar_wait(tfull0 + 8 * b, (i >> 1) & 1, err, wait_ns);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      if (so.tri) {
-        if (!epilogue_all(ok)) break;
-        // lower-triangle block rows: V[i][j] directly and, off the diagonal, V[j][i] through
-        // the staging arrays
-        int ta, tb, th;
-        tri_tile(t % mt, ta, tb, th);
-        const int r = wq * 32 + lane;
-        const int ri = 16 * ta + 8 * th + (r >> 4), rj = 16 * tb + (r & 15);
-        const bool mirror = ta != tb;
-        for (int c0 = cbeg; c0 < cend; c0 += 32) {
-          uint32_t v[32];
-          tmem_ld32(tmem + ((uint32_t)(wq * 32) << 16) + (uint32_t)(b * PBN + c0), v);
-          store_split_ij(so, ri, rj, n0 + c0, Nd, alpha, v, mirror ? stg : nullptr, r);
-          if (mirror) {
-            group_sync(grp);   // the half block's 32 columns are staged
-            store_mirror(so, stg, 16 * ta + 8 * th, 16 * tb, n0 + c0, Nd, r);
-            group_sync(grp);   // and written: the group's staging arrays are free again
-          }
-        }
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        mbar_arrive(tempty0 + 8 * b);
-        continue;
-      }
       if (!__all_sync(0xffffffffu, ok)) break;
-      const int m = m0 + wq * 32 + lane;
-      for (int c0 = cbeg; c0 < cend; c0 += 32) {
-        uint32_t v[32];
-        tmem_ld32(tmem + ((uint32_t)(wq * 32) << 16) + (uint32_t)(b * PBN + c0), v);
-        if (m < Md) {
-          if (so.hi) {
-            store_split(so, m, n0 + c0, Nd, alpha, v);
-          } else {
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              const int n = n0 + c0 + j;
-              if (n < Nd) C[(int64_t)n * ldc + m] = alpha * __uint_as_float(v[j]);
-            }
-          }
-        }
-      }
+      store_columns(so, C, ldc, tmem + (uint32_t)(b * PBN) + ((uint32_t)(wq * 32) << 16), m0 + wq * 32 + lane, n0,
+                    grp * (PBN / 2), PBN / 2, Md, Nd, alpha);
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       mbar_arrive(tempty0 + 8 * b);
     }
@@ -434,6 +420,268 @@ __global__ void __launch_bounds__(PTHREADS, 1)
   if (warp == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u)
                  : "memory");
+}
+
+// The persistent kernel by pairs of SMs (cta_group::2): a cluster of two CTAs computes a 256 x 256 tile,
+// each with 128 of its rows (A and the accumulator) and half of its columns' B operand in its own shared
+// memory; the first CTA issues the MMAs for both.  A 64-wide k slice of hi and lo operands is 64 KB a CTA
+// instead of the 96 KB of a 128 x 256 tile: with 12 MMAs of some 131 cycles a slice, one CTA per tile
+// asked L2 for 61 bytes a cycle and SM, 7.7 TB/s over the chip, which bounded it.  Ring of 3 stages.
+//   warp 16 / lane 0  TMA producer of its CTA's operands; every byte of both CTAs counts on the first
+//                     CTA's "full" barrier
+//   warp 17 / lane 0  (first CTA) MMA issuer; its commits arrive on the barriers of both CTAs
+//   warps 0..15       epilogue of the CTA's own 128 rows, four groups of four warps with 64 columns each;
+//                     "tile empty" counts the warps of both
+// The V_HS epilogue (split, transposed for the mirror block) was the longer side of a tile with 8 warps
+// and 2-byte accesses (36 k cycles beside 19 k of MMAs at K = 768), hence 16 warps, 4-byte stores of lane
+// pairs and 16-byte staging reads.  V_HS at M = 128, X = 768, 4096 walkers, beside the other system's
+// kernels: 344 us with one CTA per tile, 313 us by pairs with the old epilogue, 273 us so (tensor pipe 54 %
+// active, L2 45 %, the last of the tiles' waves half empty at smaller sizes); M = 64, 2048 walkers:
+// 32.4 -> 28.8 us; M = 200: 495 -> 436 us.
+constexpr int QSTAGES = 3, QEPI = 512, QTHREADS = QEPI + 64;
+struct QLayout {
+  static constexpr int T_BYTES = 128 * BK * 2;
+  static constexpr int STAGE_BYTES = 4 * T_BYTES;   // A hi, lo, B hi, lo
+  static constexpr int STG_OFFSET = QSTAGES * STAGE_BYTES;
+  static constexpr int STG_BYTES = 16 * 16 * 8 * 4;   // mirror staging of an epilogue group
+  static constexpr int BAR_OFFSET = STG_OFFSET + 4 * STG_BYTES;
+  static constexpr int SMEM_BYTES = BAR_OFFSET + 256 + 1024;
+};
+
+// Address of the same shared-memory location in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+// TMA load into this CTA whose bytes count on a barrier of either CTA of the pair.
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, "
+      "%3}], [%4];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
+      : "memory");
+}
+__device__ __forceinline__ void mma_bf16_pair(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc,
+                                              uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+      "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// Arrives on the barrier at this offset in both CTAs once the MMAs issued so far have completed.
+__device__ __forceinline__ void mma_commit_pair(uint32_t bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+      "h"((uint16_t)3)
+      : "memory");
+}
+__device__ __forceinline__ void arrive_remote(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ bool try_wait_cluster(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity), "r"(1000000u)
+      : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ bool wait_cluster(uint32_t bar, uint32_t parity, int* err, uint64_t limit_ns) {
+  const uint64_t t0 = global_ns();
+  do {
+    if (try_wait_cluster(bar, parity)) return true;
+  } while (global_ns() - t0 <= limit_ns);
+  atomicOr(err, 1);
+  return false;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(QTHREADS, 1)
+    k_gemm_bf16x3_tc_pair(const __grid_constant__ CUtensorMap tmAh, const __grid_constant__ CUtensorMap tmAl,
+                          const __grid_constant__ CUtensorMap tmBh, const __grid_constant__ CUtensorMap tmBl,
+                          int Md, int Nd, int nkb, float alpha, float* __restrict__ C, int64_t ldc,
+                          SplitOut so, int* err, uint64_t wait_ns) {
+  using Lay = QLayout;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                             ~uintptr_t(1023));
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Lay::BAR_OFFSET);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * QSTAGES + 5);
+  const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + QSTAGES);
+  const uint32_t tfull0 = smem_u32(bars + 2 * QSTAGES), tempty0 = smem_u32(bars + 2 * QSTAGES + 2);
+  const uint32_t done = smem_u32(bars + 2 * QSTAGES + 4);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = (int)(blockIdx.x & 1), pair = (int)(blockIdx.x >> 1), npairs = (int)(gridDim.x >> 1);
+  const int mt = (Md + 2 * BM - 1) / (2 * BM), ntiles = mt * ((Nd + PBN - 1) / PBN);
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < QSTAGES; ++s) {
+      mbar_init(full0 + 8 * s, 1);
+      mbar_init(empty0 + 8 * s, 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(tfull0 + 8 * b, 1);
+      mbar_init(tempty0 + 8 * b, 2 * (QEPI / 32));
+    }
+    mbar_init(done, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(tmem_slot)),
+                 "r"(512u)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  }
+  __syncthreads();
+  cluster_sync();   // both CTAs' barriers are initialised
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == 16) {
+    if (lane == 0) {
+      // ---- TMA producer ----
+      int s = 0, g = 0;
+      uint32_t ph = 0;   // parity of the stage's current use
+      bool ok = true;
+      for (int t = pair; t < ntiles && ok; t += npairs) {
+        const int m0 = (2 * (t % mt) + rank) * BM, n0 = (t / mt) * PBN + rank * (PBN / 2);
+        for (int kb = 0; kb < nkb; ++kb, ++g) {
+          if (g >= QSTAGES && !mbar_wait(empty0 + 8 * s, ph ^ 1u, err, wait_ns)) { ok = false; break; }
+          const uint32_t st = smem_u32(smem + s * Lay::STAGE_BYTES);
+          const uint32_t fb = map_rank(full0 + 8 * s, 0);
+          if (rank == 0) mbar_expect_tx(full0 + 8 * s, 2 * Lay::STAGE_BYTES);
+          tma_load_2d_pair(st, &tmAh, fb, kb * BK, m0);
+          tma_load_2d_pair(st + Lay::T_BYTES, &tmAl, fb, kb * BK, m0);
+          tma_load_2d_pair(st + 2 * Lay::T_BYTES, &tmBh, fb, kb * BK, n0);
+          tma_load_2d_pair(st + 3 * Lay::T_BYTES, &tmBl, fb, kb * BK, n0);
+          if (++s == QSTAGES) { s = 0; ph ^= 1u; }
+        }
+      }
+      // every issued stage of both CTAs must have landed before either may exit (the other one's bytes
+      // and this one's count here)
+      if (rank == 0) {
+        const int left = g < QSTAGES ? g : QSTAGES;
+        for (int q = g - left; q < g; ++q)
+          mbar_wait(full0 + 8 * (q % QSTAGES), (q / QSTAGES) & 1, err, wait_ns);
+      }
+    }
+  } else if (warp == 17) {
+    if (lane == 0 && rank == 0) {
+      // ---- MMA issuer ----
+      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(PBN >> 3) << 17) |
+                             ((uint32_t)(2 * BM >> 4) << 24);
+      int s = 0, i = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int t = pair; t < ntiles && ok; t += npairs, ++i) {
+        const int b = i & 1;
+        if (i >= 2 && !wait_cluster(tempty0 + 8 * b, ((i >> 1) - 1) & 1, err, wait_ns)) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t d = tmem + (uint32_t)(b * PBN);
+        for (int kb = 0; kb < nkb; ++kb) {
+          if (!mbar_wait(full0 + 8 * s, ph, err, wait_ns)) { ok = false; break; }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint32_t st = smem_u32(smem + s * Lay::STAGE_BYTES);
+          const uint64_t ah = sw128_desc(st), al = sw128_desc(st + Lay::T_BYTES);
+          const uint64_t bh = sw128_desc(st + 2 * Lay::T_BYTES), bl = sw128_desc(st + 3 * Lay::T_BYTES);
+#pragma unroll
+          for (int kk = 0; kk < BK / 16; ++kk) {
+            const uint64_t dk = (uint64_t)((kk * 32) >> 4);
+            mma_bf16_pair(d, ah + dk, bh + dk, idesc, (kb | kk) != 0);
+            mma_bf16_pair(d, ah + dk, bl + dk, idesc, 1u);
+            mma_bf16_pair(d, al + dk, bh + dk, idesc, 1u);
+          }
+          mma_commit_pair(empty0 + 8 * s);
+          if (++s == QSTAGES) { s = 0; ph ^= 1u; }
+        }
+        if (ok) mma_commit_pair(tfull0 + 8 * b);
+      }
+      mma_commit_pair(done);   // arrives once every issued MMA has completed
+    }
+  } else {
+    // ---- epilogue ----
+    int i = 0;
+    const int grp = warp >> 2, wq = warp & 3, r = wq * 32 + lane;
+    uint32_t* stg = reinterpret_cast<uint32_t*>(smem + Lay::STG_OFFSET + grp * Lay::STG_BYTES);
+    for (int t = pair; t < ntiles; t += npairs, ++i) {
+      const int b = i & 1, tm = 2 * (t % mt) + rank, n0 = (t / mt) * PBN;
+      const bool ok = mbar_wait(tfull0 + 8 * b, (i >> 1) & 1, err, wait_ns);
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      if (!epilogue_all<QEPI>(ok)) break;
+      const uint32_t acc = tmem + (uint32_t)(b * PBN) + ((uint32_t)(wq * 32) << 16);
+      if (so.tri) {
+        // lower-triangle block rows: V[i][j] directly and, off the diagonal, V[j][i] through the staging
+        int ba, bb, bh;
+        tri_tile(tm, ba, bb, bh);
+        const int i0 = 16 * ba + 8 * bh, j0 = 16 * bb;
+        const bool mirror = ba != bb;
+        for (int c0 = 64 * grp; c0 < 64 * grp + 64; c0 += 16) {
+          uint32_t v[16];
+          tmem_ld16(acc + (uint32_t)c0, v);
+          store_tri16(so, i0 + (r >> 4), j0 + (r & 15), n0 + c0, Nd, alpha, v, mirror ? stg : nullptr, r);
+          if (mirror) {
+            group_sync(grp);   // the half block's 16 columns are staged
+            store_mirror16(so, stg, i0, j0, n0 + c0, Nd, r);
+            group_sync(grp);   // and written: the group's staging array is free again
+          }
+        }
+      } else {
+        store_columns(so, C, ldc, acc, tm * BM + r, n0, 64 * grp, 64, Md, Nd, alpha);
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) arrive_remote(map_rank(tempty0 + 8 * b, 0));
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) mbar_wait(done, 0, err, wait_ns);   // no MMA may still write TMEM
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  __syncthreads();
+  // neither CTA's shared or tensor memory, nor its barriers, are used by the other any more
+  cluster_sync();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u)
+                 : "memory");
+}
+
+// Clusters of the pair kernel that the device holds at once (its grid: a cluster that waited for an SM
+// would run its tiles after the others').
+int find_pair_clusters() {
+  static int have[64] = {};
+  static std::mutex mu;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  std::lock_guard<std::mutex> lock(mu);
+  if (!have[dev]) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(152);
+    cfg.blockDim = dim3(QTHREADS);
+    cfg.dynamicSmemBytes = QLayout::SMEM_BYTES;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, k_gemm_bf16x3_tc_pair, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      n = 0;
+    }
+    have[dev] = n > 0 ? n : -1;
+  }
+  return std::max(have[dev], 0);
 }
 
 // ---- operand preparation ----
@@ -550,11 +798,16 @@ cudaError_t split_bf16_tri(const double* in, int64_t ld_in, int M, int K, int Kp
   return cudaGetLastError();
 }
 
-// The persistent kernel (the only one with the lower-triangle output) takes a product of at
-// least two 128 x 256 tiles per SM whose B rows are whole 256-row tiles.
+// The persistent kernels take a product of at least two 128 x 256 tiles per SM whose B rows are whole
+// 256-row tiles.
 bool tc_persistent_ok(int Md, int Nd, int b_rows) {
   const int64_t tiles = (int64_t)((Md + BM - 1) / BM) * ((Nd + PBN - 1) / PBN);
   return tiles >= 2 * 152 && b_rows % PBN == 0;
+}
+
+// The lower-triangle output is the pair kernel's.
+bool vhs_tri_ok(int M, int Nd, int b_rows) {
+  return tc_persistent_ok(vhs_tri_rows(M), Nd, b_rows) && find_pair_clusters() > 0;
 }
 
 // A operand boxes are BM = 128 rows; B operand boxes are tc_bn() rows.  Operand buffers
@@ -571,7 +824,16 @@ cudaError_t gemm_f32_or_split(const TcOperand& A, const TcOperand& B, int Md, in
   // next tile's MMAs; B tiles of 256 rows stay inside the operand's padded rows (a multiple of
   // 256 here), or read the TMA fill value beyond them
   const int64_t tiles = (int64_t)((Md + BM - 1) / BM) * ((Nd + PBN - 1) / PBN);
-  if (so.tri && !tc_persistent_ok(Md, Nd, B.rows)) return cudaErrorInvalidValue;
+  if (so.tri && !vhs_tri_ok(so.M, Nd, B.rows)) return cudaErrorInvalidValue;
+  // by pairs of SMs unless an odd last row tile would leave a CTA idle for more than a tenth of the work
+  const int mt = (Md + BM - 1) / BM, np = find_pair_clusters();
+  if (tc_persistent_ok(Md, Nd, B.rows) && (mt % 2 == 0 || mt > 9) && np > 0) {
+    const int64_t pt = (int64_t)((mt + 1) / 2) * ((Nd + PBN - 1) / PBN);
+    k_gemm_bf16x3_tc_pair<<<2 * (int)std::min<int64_t>(pt, np), QTHREADS, QLayout::SMEM_BYTES, s>>>(
+        A.map_hi, A.map_lo, B.map_hi, B.map_lo, Md, Nd, A.Kp / BK, alpha, C, ldc, so, err,
+        kWaitLimitNs);
+    return cudaGetLastError();
+  }
   if (tc_persistent_ok(Md, Nd, B.rows)) {
     const int grid = (int)std::min<int64_t>(tiles, 152);
     k_gemm_bf16x3_tc_persist<<<grid, PTHREADS, PLayoutG::SMEM_BYTES, s>>>(
@@ -627,6 +889,10 @@ cudaError_t prepare_tc_kernels() {
     if (st == cudaSuccess)
       st = cudaFuncSetAttribute(k_gemm_bf16x3_tc_persist, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 PLayoutG::SMEM_BYTES);
+    if (st == cudaSuccess)
+      st = cudaFuncSetAttribute(k_gemm_bf16x3_tc_pair, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                QLayout::SMEM_BYTES);
+    find_pair_clusters();   // asked for here, not under a capture
   });
   return st;
 }

@@ -258,6 +258,7 @@ struct SplitOut {
 // the rest.
 int vhs_tri_rows(int M);
 bool tc_persistent_ok(int Md, int Nd, int b_rows);
+bool vhs_tri_ok(int M, int Nd, int b_rows);
 cudaError_t split_bf16_tri(const double* in, int64_t ld_in, int M, int K, int Kp, __nv_bfloat16* hi,
                            __nv_bfloat16* lo, cudaStream_t s);
 cudaError_t gemm_bf16x3_split_out(const TcOperand& A, const TcOperand& B, int Md, int Nd,
