@@ -67,9 +67,74 @@ __device__ __forceinline__ void df_add(float& s, float& c, float s2, float c2) {
   c = __fadd_rn(c, __fadd_rn(err, c2));
 }
 
+// The overlap matrices of an FP32 update by the 4 warps of a CTA: warp = (spin, tile row bit 1), lane =
+// (part of the sum, tile row bit 0, tile column); a thread holds the RT x RT tile of rows rt + 4 k, columns
+// ct + 4 l and adds every fourth i, so 3 RT loads serve 2 RT^2 multiply-adds (one entry a thread: 3 loads
+// for 2).  The four parts are combined by a reduce-scatter of FP32 pairs with error-free leading sums.
+template <int RT>
+__device__ __forceinline__ void overlap_sums(const float* __restrict__ psih, const float* pfr, const float* pfi,
+                                             float* invf, int M, int MP, int nu, int nd, int warp, int lane) {
+  const int sp = warp >> 1, ns = sp ? nd : nu, n0 = sp ? nu : 0;
+  const int ct = lane & 3, rt = ((lane >> 2) & 1) + 2 * (warp & 1), part = lane >> 3;
+  const float *ps[RT], *xr[RT], *xi[RT];
+#pragma unroll
+  for (int k = 0; k < RT; ++k) {
+    const int r = min(rt + 4 * k, ns - 1), c = min(ct + 4 * k, ns - 1);
+    ps[k] = psih + (int64_t)(n0 + r) * M;
+    xr[k] = pfr + (n0 + c) * MP;
+    xi[k] = pfi + (n0 + c) * MP;
+  }
+  float s[2][RT][RT];
+#pragma unroll
+  for (int e = 0; e < 2 * RT * RT; ++e) (&s[0][0][0])[e] = 0.f;
+#pragma unroll 2
+  for (int i = part; i < M; i += 4) {
+    float h[RT], a[RT], b[RT];
+#pragma unroll
+    for (int k = 0; k < RT; ++k) {
+      h[k] = __ldg(ps[k] + i);
+      a[k] = xr[k][i];
+      b[k] = xi[k][i];
+    }
+#pragma unroll
+    for (int k = 0; k < RT; ++k)
+#pragma unroll
+      for (int l = 0; l < RT; ++l) {
+        s[0][k][l] = fmaf(h[k], a[l], s[0][k][l]);
+        s[1][k][l] = fmaf(h[k], b[l], s[1][k][l]);
+      }
+  }
+  // parts 0, 2 keep the real sums, 1, 3 the imaginary ones; then parts 0, 1 the first half of the rows
+  const bool im = part & 1, up = part & 2;
+  float c[RT][RT], t[RT][RT];
+#pragma unroll
+  for (int k = 0; k < RT; ++k)
+#pragma unroll
+    for (int l = 0; l < RT; ++l) {
+      t[k][l] = im ? s[1][k][l] : s[0][k][l];
+      c[k][l] = 0.f;
+      df_add(t[k][l], c[k][l], __shfl_xor_sync(0xffffffffu, im ? s[0][k][l] : s[1][k][l], 8), 0.f);
+    }
+#pragma unroll
+  for (int k = 0; k < RT / 2; ++k)
+#pragma unroll
+    for (int l = 0; l < RT; ++l) {
+      float t0 = up ? t[k + RT / 2][l] : t[k][l], c0 = up ? c[k + RT / 2][l] : c[k][l];
+      const float t2 = __shfl_xor_sync(0xffffffffu, up ? t[k][l] : t[k + RT / 2][l], 16);
+      const float c2 = __shfl_xor_sync(0xffffffffu, up ? c[k][l] : c[k + RT / 2][l], 16);
+      df_add(t0, c0, t2, c2);
+      const int r = rt + 4 * (k + (up ? RT / 2 : 0)), col = ct + 4 * l;
+      if (r < ns && col < ns)
+        invf[sp * 2 * kNsMax * kNsMax + (im ? kNsMax * kNsMax : 0) + r * kNsMax + col] = t0 + c0;
+    }
+}
+
 // One CTA (128 or 256 threads) per walker.  Shared: phi [2][N][M + kPad] in FP64 (not in the
 // FP32 update), per spin the overlap matrix factorised in place (re and im [NSM][LDA], FP64),
 // FP32 copies of phi and of the factors.
+// The FP32 update is bound by instruction issue and latency (41 % of the issue slots at 4 to 5 CTAs an SM):
+// at M = 128, 16/16 a walker takes 41 k warp instructions, 56 k with one overlap entry a thread and factors
+// read one float at a time.  1024 walkers: 115 -> 88 us; 4096 beside the other system's kernels 373 -> 304 us.
 // NSM: the larger spin block is at most 8 (both blocks factorised by warp 0, 16 lanes each) or
 // 16 (one warp per block, ROWS = ceil(ns / (32 / ns)) rows per lane, 4 or 8).
 template <int ROWS, int NSM>
@@ -91,7 +156,8 @@ __global__ void __launch_bounds__(256) k_overlap_fast(FastOvArgs a) {
   float* pfr = a.fp64_copy || a.O ? reinterpret_cast<float*>(aug + 2 * SPB)   // [N][MP]
                                   : reinterpret_cast<float*>(smo);
   float* pfi = pfr + NMP;
-  float* invf = pfi + NMP;     // spin s at invf + s * 2 * 16 * 16: re [16][16], im [16][16]
+  float* invf = pfr + ((2 * NMP + 3) & ~3);   // (16-byte aligned) spin s at invf + s * 2 * 16 * 16: re [16][16], im [16][16]
+  float2* facf = reinterpret_cast<float2*>(invf + 4 * kNsMax * kNsMax);   // spin s at facf + s * 16 * 16
   __shared__ double s_det[2][2];   // per spin: determinant mantissa (re, im) ...
   __shared__ int s_dexp[2];        // ... and its power-of-two exponent
   __shared__ int s_bad[2];
@@ -163,67 +229,39 @@ __global__ void __launch_bounds__(256) k_overlap_fast(FastOvArgs a) {
       ar[r * LDA + c] = o[(int64_t)wk * ns];
       ar[PLN + r * LDA + c] = o[((int64_t)a.Nw + wk) * ns];
     }
+  if (f32) {
+    // phi is FP32 here (the propagator's FP32 output): FP32 products of psi (rounded to FP32) and phi,
+    // summed in FP32 (~2^-24 relative to sum |terms| per part; the log determinant then carries ~1e-6 of
+    // rounding, far below the step's other FP32 and split-BF16 errors)
+    if ((warp >> 1 ? nd : nu) > 0) overlap_sums<NSM / 4>(a.psih, pfr, pfi, invf, M, MP, nu, nd, warp, lane);
+  } else
   for (int base = 0; base < (a.O ? 0 : nn * 4); base += blockDim.x) {
     const int q = base + tid, ent = q >> 2, part = q & 3;
     double re = 0.0, im = 0.0;
-    float sr = 0.f, cr = 0.f, si = 0.f, ci = 0.f;   // FP32-pair partial sums (update mode)
     int sp = 0, r = 0, c = 0;
     if (ent < nn) {
       if (ent < nu * nu) { r = ent / nu; c = ent % nu; }
       else { sp = 1; const int e2 = ent - nu * nu; r = e2 / nd; c = e2 % nd; }
       const int n0 = sp ? nu : 0;
-      if (f32) {
-        // phi is FP32 here (the propagator's FP32 output): FP32 products of psi (rounded to
-        // FP32) and phi, summed in FP32 (~2^-24 relative to sum |terms| per part; the log
-        // determinant then carries ~1e-6 of rounding, far below the step's other FP32 and
-        // split-BF16 errors); the FP64 pipe sees only the final conversions
-        const float* hs = a.psih + (int64_t)(n0 + r) * M;
-        const float* xr = pfr + (n0 + c) * MP;
-        const float* xi = pfi + (n0 + c) * MP;
-        for (int i = part; i < M; i += 4) {
-          const float h = __ldg(hs + i);
-          sr = fmaf(h, xr[i], sr);
-          si = fmaf(h, xi[i], si);
-        }
-      } else {
-        const double* ps = a.psi + (int64_t)(n0 + r) * M;
-        const double* fr = pr + (n0 + c) * MP;
-        const double* fi = pi + (n0 + c) * MP;
-        for (int i = part; i < M; i += 4) {
-          const double p = __ldg(ps + i);
-          re = fma(p, fr[i], re);
-          im = fma(p, fi[i], im);
-        }
+      const double* ps = a.psi + (int64_t)(n0 + r) * M;
+      const double* fr = pr + (n0 + c) * MP;
+      const double* fi = pi + (n0 + c) * MP;
+      for (int i = part; i < M; i += 4) {
+        const double p = __ldg(ps + i);
+        re = fma(p, fr[i], re);
+        im = fma(p, fi[i], im);
       }
     }
     // combine the 4 partial sums of each entry (every lane takes part in the shuffles)
-    if (f32) {
-      // FP32 pairs with error-free additions: the FP64 pipe sees one conversion per component
-#pragma unroll
-      for (int o = 1; o <= 2; o <<= 1) {
-        const float s2r = __shfl_xor_sync(0xffffffffu, sr, o), c2r = __shfl_xor_sync(0xffffffffu, cr, o);
-        const float s2i = __shfl_xor_sync(0xffffffffu, si, o), c2i = __shfl_xor_sync(0xffffffffu, ci, o);
-        df_add(sr, cr, s2r, c2r);
-        df_add(si, ci, s2i, c2i);
-      }
-      // every lane of the entry holds the combined pair; part 0 converts the real sum and
-      // part 1 the imaginary one, so each lane issues 2 conversions and 1 add
-      // (FP32 update: the factorisation below runs in FP32 on these)
-      const bool odd = part & 1;
-      if (ent < nn && part < 2)
-        invf[sp * 2 * kNsMax * kNsMax + (odd ? kNsMax * kNsMax : 0) + r * kNsMax + c] =
-            (odd ? si : sr) + (odd ? ci : cr);
-    } else {
-      re += __shfl_xor_sync(0xffffffffu, re, 1);
-      im += __shfl_xor_sync(0xffffffffu, im, 1);
-      re += __shfl_xor_sync(0xffffffffu, re, 2);
-      im += __shfl_xor_sync(0xffffffffu, im, 2);
-      if (ent < nn && part == 0) {
-        double* ar = aug + sp * SPB;
-        double* ai = ar + PLN;
-        ar[r * LDA + c] = re;
-        ai[r * LDA + c] = im;
-      }
+    re += __shfl_xor_sync(0xffffffffu, re, 1);
+    im += __shfl_xor_sync(0xffffffffu, im, 1);
+    re += __shfl_xor_sync(0xffffffffu, re, 2);
+    im += __shfl_xor_sync(0xffffffffu, im, 2);
+    if (ent < nn && part == 0) {
+      double* ar = aug + sp * SPB;
+      double* ai = ar + PLN;
+      ar[r * LDA + c] = re;
+      ai[r * LDA + c] = im;
     }
   }
   __syncthreads();
@@ -304,15 +342,21 @@ __global__ void __launch_bounds__(256) k_overlap_fast(FastOvArgs a) {
       }
     s_perm[tid] = pw;
   }
-  if (!f32)
-  for (int e = tid; e < nn; e += blockDim.x) {   // the factors (and 1/pivot) to FP32, once
+  // the factors (and 1 / pivot) as FP32 (re, im) pairs, column by column: the solves read a column's
+  // entries four floats at a time
+  for (int e = tid; e < nn; e += blockDim.x) {
     int sp = 0, r, c;
     if (e < nu * nu) { r = e / nu; c = e % nu; }
     else { sp = 1; r = (e - nu * nu) / nd; c = (e - nu * nu) % nd; }
-    const double* ar = aug + sp * SPB;
-    float* fr = invf + sp * 2 * kNsMax * kNsMax;
-    fr[r * kNsMax + c] = (float)ar[r * LDA + c];
-    fr[kNsMax * kNsMax + r * kNsMax + c] = (float)ar[PLN + r * LDA + c];
+    float2 v;
+    if (f32) {
+      const float* fr = invf + sp * 2 * kNsMax * kNsMax;
+      v = make_float2(fr[r * kNsMax + c], fr[kNsMax * kNsMax + r * kNsMax + c]);
+    } else {
+      const double* ar = aug + sp * SPB;
+      v = make_float2((float)ar[r * LDA + c], (float)ar[PLN + r * LDA + c]);
+    }
+    facf[sp * kNsMax * kNsMax + c * kNsMax + r] = v;
   }
   __syncthreads();
   // Theta_s = Phi_s O_s^{-1} = ((Phi_s U^{-1}) L^{-1}) P, one orbital row i of one spin per
@@ -334,8 +378,7 @@ __global__ void __launch_bounds__(256) k_overlap_fast(FastOvArgs a) {
   } else {
     for (int t = tid; t < 2 * M; t += blockDim.x) {
       const int sp = t / M, i = t - sp * M, ns = sp ? nd : nu, n0 = sp ? nu : 0;
-      const float* Lr = invf + sp * 2 * kNsMax * kNsMax;
-      const float* Li = Lr + kNsMax * kNsMax;
+      const float2* fc = facf + sp * kNsMax * kNsMax;   // column j at fc + j * 16
       float yr[NSM], yi[NSM];
 #pragma unroll
       for (int j = 0; j < NSM; ++j) {
@@ -346,26 +389,38 @@ __global__ void __launch_bounds__(256) k_overlap_fast(FastOvArgs a) {
       for (int j = 1; j < NSM; ++j)
         if (j < ns) {
 #pragma unroll
-          for (int k = 0; k < j; ++k) {
-            const float ur = Lr[k * kNsMax + j], ui = Li[k * kNsMax + j];
-            yr[j] = fmaf(-yr[k], ur, fmaf(yi[k], ui, yr[j]));
-            yi[j] = fmaf(-yr[k], ui, fmaf(-yi[k], ur, yi[j]));
+          for (int k = 0; k < j; k += 2) {
+            const float4 u = *reinterpret_cast<const float4*>(fc + j * kNsMax + k);
+            yr[j] = fmaf(-yr[k], u.x, fmaf(yi[k], u.y, yr[j]));
+            yi[j] = fmaf(-yr[k], u.y, fmaf(-yi[k], u.x, yi[j]));
+            if (k + 1 < j) {
+              yr[j] = fmaf(-yr[k + 1], u.z, fmaf(yi[k + 1], u.w, yr[j]));
+              yi[j] = fmaf(-yr[k + 1], u.w, fmaf(-yi[k + 1], u.z, yi[j]));
+            }
           }
         }
 #pragma unroll
       for (int j = NSM - 1; j >= 0; --j)
         if (j < ns) {
           float tr = yr[j], ti = yi[j];
+          float2 p = make_float2(0.f, 0.f);
 #pragma unroll
-          for (int k = j + 1; k < NSM; ++k)
+          for (int k = j & ~1; k < NSM; k += 2)
             if (k < ns) {
-              const float lr = Lr[k * kNsMax + j], li = Li[k * kNsMax + j];
-              tr = fmaf(-yr[k], lr, fmaf(yi[k], li, tr));
-              ti = fmaf(-yr[k], li, fmaf(-yi[k], lr, ti));
+              const float4 l = *reinterpret_cast<const float4*>(fc + j * kNsMax + k);
+              if (k == j) p = make_float2(l.x, l.y);
+              if (k + 1 == j) p = make_float2(l.z, l.w);
+              if (k > j) {
+                tr = fmaf(-yr[k], l.x, fmaf(yi[k], l.y, tr));
+                ti = fmaf(-yr[k], l.y, fmaf(-yi[k], l.x, ti));
+              }
+              if (k + 1 > j && k + 1 < ns) {
+                tr = fmaf(-yr[k + 1], l.z, fmaf(yi[k + 1], l.w, tr));
+                ti = fmaf(-yr[k + 1], l.w, fmaf(-yi[k + 1], l.z, ti));
+              }
             }
-          const float pr_ = Lr[j * kNsMax + j], pi_ = Li[j * kNsMax + j];
-          yr[j] = fmaf(tr, pr_, -ti * pi_);
-          yi[j] = fmaf(tr, pi_, ti * pr_);
+          yr[j] = fmaf(tr, p.x, -ti * p.y);
+          yi[j] = fmaf(tr, p.y, ti * p.x);
         }
       const unsigned long long pw = s_perm[sp];
 #pragma unroll
@@ -946,7 +1001,7 @@ size_t smem_fast_overlap(const Ctx& c, bool fp64_copy = true, bool given = false
   const size_t aug = small ? 2 * 2 * 8 * 8 : 2 * 2 * kNsMax * kLd;
   // the FP32 update factorises in the FP32 factor arrays: no FP64 copy of Phi, no FP64 factors
   return sizeof(double) * (fp64_copy ? 2 * nmp + aug : given ? aug : 0) +
-         sizeof(float) * (2 * nmp + 2 * 2 * kNsMax * kNsMax);
+         sizeof(float) * (2 * nmp + 4 + 4 * 2 * kNsMax * kNsMax);
 }
 size_t smem_mgs_warp(const Ctx& c) { return sizeof(double) * 4 * (size_t)c.N * c.M; }   // two walkers
 
