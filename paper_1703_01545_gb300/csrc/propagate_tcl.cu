@@ -15,8 +15,8 @@
 // written in that form by the V_HS contraction) stream through a TMA ring for every round, 32 KB (a hi
 // tile and its lo tile) a stage.  A hi tile is consumed by two MMAs per 16-wide K step (hi * T_hi,
 // hi * T_lo), a lo tile by one (lo * T_hi): the three split products, accumulated in FP32 in tensor
-// memory.  The running sum S of the series lives in tensor memory beside the accumulator, so the
-// epilogue threads hold no more than 16 columns at a time.
+// memory.  The series runs by Horner's rule, so a round reads T_0 (S, in tensor memory beside the
+// accumulator) and writes nothing back to it; the epilogue threads hold no more than 16 columns at a time.
 //
 // The streamed form at M = 200, N = 18 fills 512 KB of stages a Taylor round (26 bytes a cycle per SM at
 // the measured time, near what L2 delivers to all SMs at once) for 156 MMAs of some 45 cycles.  Scalar
@@ -707,7 +707,7 @@ __global__ void __launch_bounds__(64 + 32 * EPI * G, EPI == 4 ? 2 : 1)
         if (pre && q == 0) okw = okw && !*abort_flag && mbar_wait(xreadg, kw & 1, err, wait_ns);
         if (!__all_sync(0xffffffffu, okw)) { fail(); ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const float inv = (q >= 1 && q <= sh.order) ? 1.f / (float)q : 1.f;
+        const float inv = q >= 1 && q <= sh.order ? 1.f / (float)(sh.order + 1 - q) : 1.f;
         for (int t = 0; t < sh.MT && ok; ++t) {
           if (t && sh.bbuf) {
             okw = !*abort_flag && mbar_wait(dfull1, rq & 1, err, wait_ns);
@@ -734,16 +734,15 @@ __global__ void __launch_bounds__(64 + 32 * EPI * G, EPI == 4 ? 2 : 1)
                 tmem_st_frag(tl + sreg + (uint32_t)(t * dcol + c0), sv);
                 if (in_b) put_block(x, i0b, c0, true, rq + 1);
               } else if (!last) {
-                // T_q = A T_{q-1} / q; S += T_q; operand = T_q, or S after the last term
-                float y[8];
+                // Horner's rule: operand = T_0 + (A operand) / m, m = order + 1 - q; the last one, the sum of
+                // the series, becomes S
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                  x[j] = __uint_as_float(dv[j]) * inv;
-                  y[j] = __uint_as_float(sv[j]) + x[j];
-                  sv[j] = __float_as_uint(y[j]);
+                  x[j] = fmaf(__uint_as_float(dv[j]), inv, __uint_as_float(sv[j]));
+                  sv[j] = __float_as_uint(x[j]);
                 }
-                tmem_st_frag(tl + sreg + (uint32_t)(t * dcol + c0), sv);
-                if (in_b) put_block(q < sh.order ? x : y, i0b, c0, q < sh.order, rq + 1);
+                if (q == sh.order) tmem_st_frag(tl + sreg + (uint32_t)(t * dcol + c0), sv);
+                if (in_b) put_block(x, i0b, c0, q < sh.order, rq + 1);
               } else {
                 // Phi' = S + (E - I) S
 #pragma unroll
