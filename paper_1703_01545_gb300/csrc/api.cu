@@ -189,7 +189,7 @@ afqmc_status setup_mixed(Ctx* h, cudaStream_t s) {
   cudaError_t e = afq::launch_transpose(h->L, tmp, X, (int)MM, s);
   if (e == cudaSuccess) e = afq::split_bf16(tmp, X, (int)MM, X, h->tc_L->Kp, h->tc_L->hi, h->tc_L->lo, s);
   if (e == cudaSuccess && afq::propagate_tcl_ok(*h) &&
-      afq::vhs_tri_ok(M, 2 * Nw, h->tc_U->rows)) {
+      afq::vhs_tri_ok(M, 2 * Nw)) {
     // the lower-triangle blocks of the V_HS rows, for the split output the large-M
     // tensor-core propagator reads (V_HS is symmetric: the kernel writes the mirror half)
     if ((st = make_operand(h, &h->tc_Ltri, afq::vhs_tri_rows(M), X, s)) != AFQMC_OK) {

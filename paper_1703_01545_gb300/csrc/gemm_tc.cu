@@ -259,7 +259,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                  : "memory");
 }
 
-// Persistent variant for large outputs (the V_HS contraction): 128 x 256 tiles, grid = one CTA
+// Persistent variant for one row tile and many columns (where a pair would leave a CTA without rows):
+// 128 x 256 tiles, grid = one CTA
 // per SM looping over tiles, 10 warps.
 //   warp 8 / lane 0  TMA producer over all of the CTA's tiles (2-stage ring of 96 KB stages)
 //   warp 9 / lane 0  MMA issuer: tile i accumulates into TMEM buffer i & 1 (2 x 256 columns),
@@ -798,17 +799,27 @@ cudaError_t split_bf16_tri(const double* in, int64_t ld_in, int M, int K, int Kp
   return cudaGetLastError();
 }
 
-// The persistent kernels take a product of at least two 128 x 256 tiles per SM whose B rows are whole
-// 256-row tiles.
-bool tc_persistent_ok(int Md, int Nd, int b_rows) {
+static bool tc_persistent_ok(int Md, int Nd, int b_rows) {
   const int64_t tiles = (int64_t)((Md + BM - 1) / BM) * ((Nd + PBN - 1) / PBN);
   return tiles >= 2 * 152 && b_rows % PBN == 0;
 }
 
-// The lower-triangle output is the pair kernel's.
-bool vhs_tri_ok(int M, int Nd, int b_rows) {
-  return tc_persistent_ok(vhs_tri_rows(M), Nd, b_rows) && find_pair_clusters() > 0;
+// Whether 256 x 256 tiles by pairs of SMs beat 128 x 128 tiles by single ones (of Md1 rows: all M^2 for a
+// lower triangle), in whole waves: a 64-wide k slice takes a pair's tile about 1.6 k cycles (its MMAs) and a
+// single's 1.3 k (its 64 KB from L2).  Steps with the old line (two 128 x 256 tiles an SM, whole 256-column
+// tiles) and this one: M = 200, 300 walkers 484 -> 370 us, M = 150, 800 walkers 691 -> 605, M = 128, 300
+// walkers 231 -> 204, 100 walkers 168 -> 149, M = 101, 777 walkers 315 -> 291; the force bias at M = 128 and
+// 4096 walkers (6 x 64 single tiles, three waves; 96 pairs, two) 133 -> 124 us.  M = 90, 200 walkers and
+// M = 64, 2048 walkers' force bias (three row tiles, one wave either way) stay with single tiles.
+static bool pair_pays(int64_t Md, int64_t Nd, int64_t Md1) {
+  const int np = find_pair_clusters();
+  const int64_t pt = (Md + 2 * BM - 1) / (2 * BM) * ((Nd + PBN - 1) / PBN);
+  const int64_t t1 = (Md1 + BM - 1) / BM * ((Nd + 127) / 128);
+  return np > 0 && (pt + np - 1) / np * 6 < (t1 + 151) / 152 * 5;
 }
+
+// The lower-triangle output is the pair kernel's.
+bool vhs_tri_ok(int M, int Nd) { return pair_pays(vhs_tri_rows(M), Nd, (int64_t)M * M); }
 
 // A operand boxes are BM = 128 rows; B operand boxes are tc_bn() rows.  Operand buffers
 // hold pad_rows(rows) rows (zero-filled beyond `rows`).
@@ -820,21 +831,19 @@ cudaError_t gemm_f32_or_split(const TcOperand& A, const TcOperand& B, int Md, in
                               float* C, int64_t ldc, const SplitOut& so, int* err, cudaStream_t s) {
   if (A.Kp != B.Kp || Md > A.rows || Nd > B.rows) return cudaErrorInvalidValue;
   if (Md <= 0 || Nd <= 0) return cudaSuccess;
-  // at least two 128 x 256 tiles per SM: the persistent kernel, whose epilogue overlaps the
-  // next tile's MMAs; B tiles of 256 rows stay inside the operand's padded rows (a multiple of
-  // 256 here), or read the TMA fill value beyond them
-  const int64_t tiles = (int64_t)((Md + BM - 1) / BM) * ((Nd + PBN - 1) / PBN);
-  if (so.tri && !vhs_tri_ok(so.M, Nd, B.rows)) return cudaErrorInvalidValue;
-  // by pairs of SMs unless an odd last row tile would leave a CTA idle for more than a tenth of the work
-  const int mt = (Md + BM - 1) / BM, np = find_pair_clusters();
-  if (tc_persistent_ok(Md, Nd, B.rows) && (mt % 2 == 0 || mt > 9) && np > 0) {
-    const int64_t pt = (int64_t)((mt + 1) / 2) * ((Nd + PBN - 1) / PBN);
-    k_gemm_bf16x3_tc_pair<<<2 * (int)std::min<int64_t>(pt, np), QTHREADS, QLayout::SMEM_BYTES, s>>>(
+  if (so.tri && !vhs_tri_ok(so.M, Nd)) return cudaErrorInvalidValue;
+  if (so.tri || pair_pays(Md, Nd, Md)) {
+    const int64_t pt = (int64_t)((Md + 2 * BM - 1) / (2 * BM)) * ((Nd + PBN - 1) / PBN);
+    k_gemm_bf16x3_tc_pair<<<2 * (int)std::min<int64_t>(pt, find_pair_clusters()), QTHREADS, QLayout::SMEM_BYTES, s>>>(
         A.map_hi, A.map_lo, B.map_hi, B.map_lo, Md, Nd, A.Kp / BK, alpha, C, ldc, so, err,
         kWaitLimitNs);
     return cudaGetLastError();
   }
+  // at least two 128 x 256 tiles per SM (here: a single row tile): the persistent kernel, whose epilogue
+  // overlaps the next tile's MMAs; B tiles of 256 rows stay inside the operand's padded rows (a multiple of
+  // 256 here)
   if (tc_persistent_ok(Md, Nd, B.rows)) {
+    const int64_t tiles = (int64_t)((Md + BM - 1) / BM) * ((Nd + PBN - 1) / PBN);
     const int grid = (int)std::min<int64_t>(tiles, 152);
     k_gemm_bf16x3_tc_persist<<<grid, PTHREADS, PLayoutG::SMEM_BYTES, s>>>(
         A.map_hi, A.map_lo, B.map_hi, B.map_lo, Md, Nd, A.Kp / BK, alpha, C, ldc, so, err,

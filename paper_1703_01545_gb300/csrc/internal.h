@@ -257,8 +257,7 @@ struct SplitOut {
 // (i in 16 a + 8 h + [0, 8), j in 16 b + [0, 16), h = 0, 1); V_HS[j][i] = V_HS[i][j] gives
 // the rest.
 int vhs_tri_rows(int M);
-bool tc_persistent_ok(int Md, int Nd, int b_rows);
-bool vhs_tri_ok(int M, int Nd, int b_rows);
+bool vhs_tri_ok(int M, int Nd);
 cudaError_t split_bf16_tri(const double* in, int64_t ld_in, int M, int K, int Kp, __nv_bfloat16* hi,
                            __nv_bfloat16* lo, cudaStream_t s);
 cudaError_t gemm_bf16x3_split_out(const TcOperand& A, const TcOperand& B, int Md, int Nd,

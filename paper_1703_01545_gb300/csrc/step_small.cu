@@ -429,6 +429,9 @@ SmemLimits g_small_limits;
 }  // namespace
 
 // M <= 16 and blocks of at most 8, with the constants and kSteps snapshots within 96 KB (two CTAs per SM).
+// us per step, separate kernels -> this one, 40 steps a call: M = 8, X = 24, 2/2: 66 -> 16 (128 walkers),
+// 235 -> 169 (4096), 1825 -> 1579 (40000); M = 12, X = 40, 3/3, 256 walkers: 87 -> 41; one step a call: 74 ->
+// 41, 245 -> 242, 1838 -> 2076 (the constants are staged for one step only), 96 -> 64.
 bool step_small_ok(const Ctx& c) {
   return c.opt.precision == AFQMC_FP64 && c.n_det == 0 && c.M <= 16 && c.n_up <= kNs && c.N - c.n_up <= kNs &&
          c.X >= 1 && c.X <= 4096 && sizeof(double) * (size_t)layout(c.M, c.N, c.X, (int)c.P, kSteps).total <= 96 * 1024;

@@ -1,6 +1,6 @@
 """Split-BF16 contraction by pairs of SMs (256 x 256 tiles over two CTAs) at the edges of its rule, against
-numpy float64: an even and an odd number of 128-row tiles (the last pair's second CTA empty), the smallest
-odd number it takes and the largest it leaves to one CTA per tile, rows and columns that end inside a
+numpy float64: an even and an odd number of 128-row tiles (the last pair's second CTA empty), two waves of
+pairs where single tiles take three, a single row tile (one CTA per tile), rows and columns that end inside a
 tile, one k slice, fewer slices than the ring, K that is no multiple of 64.
 
 Bound as for the other split-BF16 contractions: operands to 2^-17, lo * lo dropped (2^-18), FP32 sums:
@@ -15,7 +15,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("Md,Nd,K", [
     (2560, 4096, 64), (2500, 4352, 130), (1408, 7168, 200), (1301, 7100, 1), (1152, 8704, 100),
-    (256, 39000, 72), (130, 38912, 300)])
+    (256, 39000, 72), (130, 38912, 300),
+    (768, 8192, 330), (1000, 4096, 200), (100, 78000, 64)])
 def test_pair_contraction(Md, Nd, K):
     need_gpu()
     from paper_1703_01545_gb300 import _lib
