@@ -16,7 +16,8 @@
 struct afqmc_ctx : afq::Ctx {};
 
 namespace afq {
-afqmc_status run_step(Ctx* h, const double* fields_t, cudaStream_t s);
+afqmc_status run_step(Ctx* h, const double* fields_t, cudaStream_t s);     // leaves rhobar, U, A, aux, Phi2
+afqmc_status plain_step(Ctx* h, const double* fields_t, cudaStream_t s);   // the step afqmc_propagate takes
 afqmc_status pair_ortho(Ctx* h, cudaStream_t s);
 }  // namespace afq
 
@@ -209,7 +210,7 @@ afqmc_status adjoint_body(Ctx* h, Arena& ar, int n_steps, const double* fields, 
   // ---- forward pass, checkpoint every K steps ----
   for (int t = 0; t < n_steps; ++t) {
     if (t % K == 0) ADJ_CK(copy_state(c, ck[t / K], cur, s));
-    ADJ_ST(afq::run_step(h, field_t(t), s));
+    ADJ_ST(afq::plain_step(h, field_t(t), s));
     if (mgs_at(t)) ADJ_ST(afq::pair_ortho(h, s));
   }
   ADJ_CK(copy_state(c, fin, cur, s));
@@ -223,7 +224,7 @@ afqmc_status adjoint_body(Ctx* h, Arena& ar, int n_steps, const double* fields, 
     ADJ_CK(afq::launch_overlap(c, nullptr, afq::OV_REFRESH, s));
     for (int t = s0; t < s1; ++t) {
       ADJ_CK(copy_state(c, tape[t - s0], cur, s));
-      ADJ_ST(afq::run_step(h, field_t(t), s));
+      ADJ_ST(afq::plain_step(h, field_t(t), s));
       if (mgs_at(t)) ADJ_ST(afq::pair_ortho(h, s));
     }
     for (int t = s1 - 1; t >= s0; --t) {

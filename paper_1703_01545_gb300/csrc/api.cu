@@ -453,6 +453,7 @@ afqmc_status check_opts(const afqmc_options* o, std::string& why) {
 namespace afq {
 afqmc_status pair_steps(Ctx* h, int n, cudaStream_t s) { return steps_launch(h, n, nullptr, s); }
 afqmc_status run_step(Ctx* h, const double* fields_t, cudaStream_t s) { return step_launch(h, fields_t, s); }
+afqmc_status plain_step(Ctx* h, const double* fields_t, cudaStream_t s) { return steps_launch(h, 1, fields_t, s); }
 afqmc_status pair_ortho(Ctx* h, cudaStream_t s) { return ortho_launch(h, s); }
 afqmc_status pair_energy(Ctx* h, cudaStream_t s) { return energy_launch(h, s); }
 afqmc_status pair_check(Ctx* h) { return check_tc(h); }

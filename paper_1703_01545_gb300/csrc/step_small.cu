@@ -15,7 +15,7 @@
 // Constants (packed Cholesky tensor, half-rotated tensor, e^{-dt K/2}, trial) are staged once per launch.
 // Still bound by the chains of dependent FP64 instructions (a term of the series about 2 us with two CTAs on
 // an SM, the LU of a 2 x 2 block 5 us).  M = 8, X = 24, 2/2, 128 walkers: 16 us a step (51 us of eight
-// kernels); the pair with 2/1, 40 steps and 8 measurements: 2.83 -> 2.04 ms.
+// kernels); the pair with 2/1, 40 steps and 8 measurements: 2.83 -> 1.51 ms.
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
@@ -142,9 +142,10 @@ __global__ void __launch_bounds__(kT) k_steps_small(const SmallArgs g) {
   }
   __syncthreads();
 
-  // out(o, sum_k term(o, k)) for o < count: S lanes per output, whole warps without outputs skipped
-  auto outputs = [&](int count, int K, auto term, auto out) {
-    const int S = lanes_for(count);
+  // out(o, sum_k term(o, k)) for o < count: S lanes per output (0: as many as there are), whole warps
+  // without outputs skipped
+  auto outputs = [&](int count, int K, int S, auto term, auto out) {
+    if (S == 0) S = lanes_for(count);
     for (int b = 0; b < count * S; b += kT) {
       if (b + (tid & ~31) >= count * S) break;
       const int o = (b + tid) / S, part = (b + tid) & (S - 1);
@@ -163,7 +164,7 @@ __global__ void __launch_bounds__(kT) k_steps_small(const SmallArgs g) {
     double* thn = phn + l.nm2;
     // rhobar_g (Eq. 9)
     if (!g.free_proj) {
-      outputs(2 * X, NM,
+      outputs(2 * X, NM, 0,
               [&](int o, int k, double v) { return fma(sm[l.ltil + (o >> 1) * l.ldn + k], th[(o & 1) * NM + k], v); },
               [&](int o, double v) { sm[l.rb + (o & 1) * X + (o >> 1)] = v; });
       __syncthreads();
@@ -200,7 +201,7 @@ __global__ void __launch_bounds__(kT) k_steps_small(const SmallArgs g) {
       if (lane == 0) sm[l.aux + 4 * t + warp] = v;
     }
     // A = sum_g U_g L_g (Eq. 11), both halves of the symmetric matrix
-    outputs(2 * P, X,
+    outputs(2 * P, X, 0,
             [&](int o, int k, double v) { return fma(sm[l.lt + (o >> 1) * l.ldx + k], sm[l.u + (o & 1) * X + k], v); },
             [&](int o, double v) {
               double* a = sm + l.a + (o & 1) * M * l.ldm;
@@ -210,7 +211,7 @@ __global__ void __launch_bounds__(kT) k_steps_small(const SmallArgs g) {
             });
     // e^{-dt K/2} Phi
     auto onebody = [&](const double* src, double* dst, double* dst2) {
-      outputs(2 * NM, M,
+      outputs(2 * NM, M, 0,
               [&](int o, int k, double v) {
                 const int r = o % NM, i = r % M;
                 return fma(sm[l.ek + i * l.ldm + k], src[o - i + k], v);
@@ -260,9 +261,10 @@ __global__ void __launch_bounds__(kT) k_steps_small(const SmallArgs g) {
     }
     onebody(sm + l.acc, phn, nullptr);
     __syncthreads();
-    // O_s = Psi_s^T Phi_s
+    // O_s = Psi_s^T Phi_s, by 4 lanes an entry, as k_overlap64: O, its factors and Theta then have the bits
+    // that a refresh of the same walker gives
     const int nn = nu * nu + nd * nd;
-    outputs(2 * nn, M,
+    outputs(2 * nn, M, 4,
             [&](int o, int k, double v) {
               const int p = o & 1, e = o >> 1, sp = e >= nu * nu, ns = sp ? nd : nu, e2 = sp ? e - nu * nu : e;
               const int n0 = sp ? nu : 0;
