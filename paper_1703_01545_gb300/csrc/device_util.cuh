@@ -5,6 +5,13 @@
 
 namespace afq {
 
+// First statement of a kernel launched by launch_after: waits for the kernel before it in the stream (a
+// no-op after an ordinary launch), then lets the next one be scheduled.  Nothing before it touches memory.
+__device__ __forceinline__ void after_previous() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 struct cplx { double re, im; };
 __device__ __forceinline__ cplx cmul(cplx a, cplx b) {
   return {fma(a.re, b.re, -a.im * b.im), fma(a.re, b.im, a.im * b.re)};

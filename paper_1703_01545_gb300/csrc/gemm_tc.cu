@@ -25,6 +25,7 @@
 #include <cstdint>
 #include <mutex>
 
+#include "device_util.cuh"
 #include "internal.h"
 #include "tc_device.cuh"
 
@@ -157,6 +158,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                      const __grid_constant__ CUtensorMap tmBh, const __grid_constant__ CUtensorMap tmBl,
                      int Md, int Nd, int nkb, float alpha, TC* __restrict__ C, int64_t ldc,
                      SplitOut so, int* err, uint64_t wait_ns, int skip_producer) {
+  after_previous();
   using Lay = TcLayout<BN, STAGES>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -304,6 +306,7 @@ __global__ void __launch_bounds__(PTHREADS, 1)
                              const __grid_constant__ CUtensorMap tmBh, const __grid_constant__ CUtensorMap tmBl,
                              int Md, int Nd, int nkb, float alpha, float* __restrict__ C, int64_t ldc,
                              SplitOut so, int* err, uint64_t wait_ns) {
+  after_previous();
   using Lay = PLayoutG;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -510,6 +513,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(QTHREADS, 1)
                           const __grid_constant__ CUtensorMap tmBh, const __grid_constant__ CUtensorMap tmBl,
                           int Md, int Nd, int nkb, float alpha, float* __restrict__ C, int64_t ldc,
                           SplitOut so, int* err, uint64_t wait_ns) {
+  after_previous();
   using Lay = QLayout;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -743,10 +747,8 @@ cudaError_t launch_tc(const TcOperand& A, const TcOperand& B, int Md, int Nd, fl
   using Lay = TcLayout<BN, STAGES>;
   dim3 grid((Md + BM - 1) / BM, (Nd + BN - 1) / BN);
   if (grid.y > 65535u) return cudaErrorInvalidConfiguration;
-  k_gemm_bf16x3_tc<BN, STAGES, TC><<<grid, NTHREADS, Lay::SMEM_BYTES, s>>>(
-      A.map_hi, A.map_lo, B.map_hi, B.map_lo, Md, Nd, A.Kp / BK, alpha, C, ldc, so, err, wait_ns,
-      skip_producer);
-  return cudaGetLastError();
+  return launch_after(k_gemm_bf16x3_tc<BN, STAGES, TC>, grid, NTHREADS, Lay::SMEM_BYTES, s, A.map_hi, A.map_lo,
+                      B.map_hi, B.map_lo, Md, Nd, A.Kp / BK, alpha, C, ldc, so, err, wait_ns, skip_producer);
 }
 
 }  // namespace
@@ -834,10 +836,9 @@ cudaError_t gemm_f32_or_split(const TcOperand& A, const TcOperand& B, int Md, in
   if (so.tri && !vhs_tri_ok(so.M, Nd)) return cudaErrorInvalidValue;
   if (so.tri || pair_pays(Md, Nd, Md)) {
     const int64_t pt = (int64_t)((Md + 2 * BM - 1) / (2 * BM)) * ((Nd + PBN - 1) / PBN);
-    k_gemm_bf16x3_tc_pair<<<2 * (int)std::min<int64_t>(pt, find_pair_clusters()), QTHREADS, QLayout::SMEM_BYTES, s>>>(
-        A.map_hi, A.map_lo, B.map_hi, B.map_lo, Md, Nd, A.Kp / BK, alpha, C, ldc, so, err,
-        kWaitLimitNs);
-    return cudaGetLastError();
+    return launch_after(k_gemm_bf16x3_tc_pair, 2 * (int)std::min<int64_t>(pt, find_pair_clusters()), QTHREADS,
+                        QLayout::SMEM_BYTES, s, A.map_hi, A.map_lo, B.map_hi, B.map_lo, Md, Nd, A.Kp / BK, alpha, C,
+                        ldc, so, err, kWaitLimitNs);
   }
   // at least two 128 x 256 tiles per SM (here: a single row tile): the persistent kernel, whose epilogue
   // overlaps the next tile's MMAs; B tiles of 256 rows stay inside the operand's padded rows (a multiple of
@@ -845,10 +846,8 @@ cudaError_t gemm_f32_or_split(const TcOperand& A, const TcOperand& B, int Md, in
   if (tc_persistent_ok(Md, Nd, B.rows)) {
     const int64_t tiles = (int64_t)((Md + BM - 1) / BM) * ((Nd + PBN - 1) / PBN);
     const int grid = (int)std::min<int64_t>(tiles, 152);
-    k_gemm_bf16x3_tc_persist<<<grid, PTHREADS, PLayoutG::SMEM_BYTES, s>>>(
-        A.map_hi, A.map_lo, B.map_hi, B.map_lo, Md, Nd, A.Kp / BK, alpha, C, ldc, so, err,
-        kWaitLimitNs);
-    return cudaGetLastError();
+    return launch_after(k_gemm_bf16x3_tc_persist, grid, PTHREADS, PLayoutG::SMEM_BYTES, s, A.map_hi, A.map_lo,
+                        B.map_hi, B.map_lo, Md, Nd, A.Kp / BK, alpha, C, ldc, so, err, kWaitLimitNs);
   }
   return launch_tc<128, 3, float>(A, B, Md, Nd, alpha, C, ldc, err, s, kWaitLimitNs, 0, so);
 }

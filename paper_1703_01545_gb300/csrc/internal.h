@@ -10,6 +10,31 @@
 
 namespace afq {
 
+// Launches a kernel of the split-precision step so that its start overlaps the end of the kernel before it
+// in the stream: it may be scheduled once every CTA of that one has passed its own after_previous()
+// (device_util.cuh), and waits there for its memory.  Every kernel launched so begins with
+// after_previous().  A step of a small system is seven kernels of 5 to 90 us with 3 to 4 us between two of
+// them: M = 64, 2048 walkers, ten steps 2.29 -> 2.17 ms; M = 101, 777 walkers, five steps 1.600 -> 1.593 ms.
+// Under capture the launch is an ordinary one (a graph's nodes already run back to back).
+template <class... P, class... A>
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamIsCapturing(s, &cap);
+  if (e != cudaSuccess) return e;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = cap == cudaStreamCaptureStatusNone ? 1 : 0;
+  e = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+  return e == cudaSuccess ? cudaGetLastError() : e;
+}
+
 // Packed upper triangle (i <= j) of a symmetric M x M matrix, row-major:
 // idx(i, j) = i*M - i*(i-1)/2 + (j - i).
 inline int64_t packed_size(int M) { return (int64_t)M * (M + 1) / 2; }

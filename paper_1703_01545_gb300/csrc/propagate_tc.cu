@@ -25,6 +25,7 @@
 #include <algorithm>
 #include <cstdint>
 
+#include "device_util.cuh"
 #include "internal.h"
 #include "tc_device.cuh"
 
@@ -58,6 +59,7 @@ __global__ void __launch_bounds__(128, 3)
                    const uint32_t* __restrict__ emI_pk, double* phi_out,
                    float* __restrict__ phi_out32, const int* __restrict__ alive, int M, int N,
                    int Nw, int order, int* err, uint64_t wait_ns) {
+  after_previous();
   using Lay = PLayout;
   extern __shared__ uint8_t psm_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(psm_raw) + 1023) &
@@ -305,10 +307,9 @@ cudaError_t launch_propagate_tc(const Ctx& c, double* out, float* out32, cudaStr
   if (!propagate_tc_ok(c)) return cudaErrorInvalidValue;
   const int grid = std::min(c.Nw, 152 * 3);
   if (!c.emI_pk) return cudaErrorInvalidValue;
-  k_propagate_tc<<<grid, 128, PLayout::SMEM_BYTES, s>>>(c.phi, c.Avhs32, c.emI_pk, out, out32,
+  return launch_after(k_propagate_tc, grid, 128, PLayout::SMEM_BYTES, s, c.phi, c.Avhs32, c.emI_pk, out, out32,
                                                         out == c.phi ? c.alive : nullptr, c.M, c.N,
                                                         c.Nw, c.opt.taylor_order, c.d_tc_err, kPWaitNs);
-  return cudaGetLastError();
 }
 
 }  // namespace afq

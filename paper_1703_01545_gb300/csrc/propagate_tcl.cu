@@ -254,6 +254,7 @@ __global__ void __launch_bounds__(64 + 32 * EPI * G, EPI == 4 ? 2 : 1)
                     const TclShape sh, const double* phi_in, double* phi_out,
                     float* __restrict__ phi_out32, const int* __restrict__ alive, int* err,
                     uint64_t wait_ns) {
+  after_previous();
   extern __shared__ uint8_t tsm_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(tsm_raw) + 1023) &
                                              ~uintptr_t(1023));
@@ -957,20 +958,13 @@ cudaError_t launch_propagate_tcl(const Ctx& c, double* out, float* out32, cudaSt
   if (!propagate_tcl_ok(c) || !c.tcl_maps) return cudaErrorInvalidValue;
   const TclShape sh = plan(c);
   const int* al = out == c.phi ? c.alive : nullptr;
-  if (sh.G == 2) {
-    groups_kernel((c.M + 15) / 16, sh.Np)<<<std::min(c.Nw, 152), 64 + 32 * 16, sh.smem_bytes, s>>>(
-        c.tcl_maps[0], c.tcl_maps[1], c.tcl_maps[2], c.tcl_maps[3], sh, c.phi, out, out32, al,
-        c.d_tc_err, kWaitNs);
-  } else if (two_per_sm(sh)) {
-    k_propagate_tcl<4, 1, 0, 0><<<std::min(c.Nw, 2 * 152), 64 + 32 * 4, sh.smem_bytes, s>>>(
-        c.tcl_maps[0], c.tcl_maps[1], c.tcl_maps[2], c.tcl_maps[3], sh, c.phi, out, out32, al,
-        c.d_tc_err, kWaitNs);
-  } else {
-    k_propagate_tcl<8, 1, 0, 0><<<std::min(c.Nw, 152), 64 + 32 * 8, sh.smem_bytes, s>>>(
-        c.tcl_maps[0], c.tcl_maps[1], c.tcl_maps[2], c.tcl_maps[3], sh, c.phi, out, out32, al,
-        c.d_tc_err, kWaitNs);
-  }
-  return cudaGetLastError();
+  auto go = [&](GroupsKernel k, int grid, int threads) {
+    return launch_after(k, std::min(c.Nw, grid), threads, (size_t)sh.smem_bytes, s, c.tcl_maps[0], c.tcl_maps[1],
+                        c.tcl_maps[2], c.tcl_maps[3], sh, c.phi, out, out32, al, c.d_tc_err, kWaitNs);
+  };
+  if (sh.G == 2) return go(groups_kernel((c.M + 15) / 16, sh.Np), 152, 64 + 32 * 16);
+  return two_per_sm(sh) ? go(k_propagate_tcl<4, 1, 0, 0>, 2 * 152, 64 + 32 * 4)
+                        : go(k_propagate_tcl<8, 1, 0, 0>, 152, 64 + 32 * 8);
 }
 
 }  // namespace afq

@@ -139,6 +139,7 @@ __device__ __forceinline__ void overlap_sums(const float* __restrict__ psih, con
 // 16 (one warp per block, ROWS = ceil(ns / (32 / ns)) rows per lane, 4 or 8).
 template <int ROWS, int NSM>
 __global__ void __launch_bounds__(256) k_overlap_fast(FastOvArgs a) {
+  after_previous();
   extern __shared__ double smo[];
   const int wk = blockIdx.x, tid = threadIdx.x, M = a.M, N = a.N, NM = N * M;
   // shared copies of Phi keep each column M + 4 apart: the overlap sums read 8 columns per
@@ -595,6 +596,7 @@ __global__ void __launch_bounds__(256) k_overlap64(FastOvArgs a) {
 
 // Per walker, after k_overlap_fast or k_overlap64: log det O, the overlap ratio and the weight update.
 __global__ void __launch_bounds__(32) k_overlap_weights(FastOvArgs a) {
+  after_previous();
   const int wk = blockIdx.x * blockDim.x + threadIdx.x;
   if (wk >= a.Nw) return;
   const bool upd = (a.mode == OV_UPDATE) && a.alive[wk] != 0;
@@ -1115,12 +1117,11 @@ cudaError_t launch_overlap_fast(const Ctx& c, const double* src, int mode, cudaS
   // the FP32 update (FP32-pair sums, smaller shared footprint) runs more CTAs of 128 threads
   // per SM, so more LU warps overlap; the FP64 sums of the other modes use 256
   const int nt = a.fp64_copy ? 256 : 128;
-  if (nmax <= 8) k_overlap_fast<4, 8><<<c.Nw, nt, sm, s>>>(a);
-  else if (need <= 4) k_overlap_fast<4, 16><<<c.Nw, nt, sm, s>>>(a);
-  else k_overlap_fast<8, 16><<<c.Nw, nt, sm, s>>>(a);
+  const cudaError_t e = launch_after(nmax <= 8 ? k_overlap_fast<4, 8> : need <= 4 ? k_overlap_fast<4, 16> : k_overlap_fast<8, 16>,
+                                     c.Nw, nt, sm, s, a);
+  if (e != cudaSuccess) return e;
   // one warp per CTA: the FP64 chain of each warp gets an SM's FP64 pipe to itself
-  if (with_weights) k_overlap_weights<<<(c.Nw + 31) / 32, 32, 0, s>>>(a);
-  return cudaGetLastError();
+  return with_weights ? launch_after(k_overlap_weights, (c.Nw + 31) / 32, 32, 0, s, a) : cudaSuccess;
 }
 
 namespace {
@@ -1228,6 +1229,7 @@ __device__ __forceinline__ void put_split(__nv_bfloat16* hi, __nv_bfloat16* lo, 
 }
 
 __global__ void __launch_bounds__(128) k_fields_mixed(FieldArgsM a) {
+  after_previous();
   __shared__ float2 red[4][4];   // per warp: the 4 sums as FP32 pairs
   const int wk = blockIdx.x, X = a.X;
   const uint32_t t = (uint32_t)(*a.step);
@@ -1322,8 +1324,7 @@ cudaError_t launch_fields_mixed(const Ctx& c, const double* fields, cudaStream_t
   a.k0 = (uint32_t)c.opt.walker_offset;
   a.X = c.X; a.Nw = c.Nw; a.free_proj = c.opt.mode == AFQMC_FREE;
   a.sqrt_dt = (float)c.sqrt_dt; a.fb_cap = (float)c.opt.fb_cap;
-  k_fields_mixed<<<c.Nw, 128, 0, s>>>(a);
-  return cudaGetLastError();
+  return launch_after(k_fields_mixed, c.Nw, 128, 0, s, a);
 }
 
 }  // namespace afq

@@ -658,6 +658,7 @@ __global__ void __launch_bounds__(256) k_mixed_sum(const double* __restrict__ w,
 }
 
 __global__ void k_step_advance(unsigned long long* step, int n, int* meas, int bump_meas) {
+  after_previous();
   if (threadIdx.x == 0 && blockIdx.x == 0) {
     if (step) *step += (unsigned long long)n;
     if (meas && bump_meas) *meas += 1;
@@ -818,8 +819,7 @@ cudaError_t launch_meas_advance(int* meas, cudaStream_t s) {
 }
 
 cudaError_t launch_step_advance(const Ctx& c, cudaStream_t s, int n_steps) {
-  k_step_advance<<<1, 32, 0, s>>>(c.d_step, n_steps, nullptr, 0);
-  return cudaGetLastError();
+  return launch_after(k_step_advance, 1, 32, 0, s, c.d_step, n_steps, nullptr, 0);
 }
 
 }  // namespace afq
