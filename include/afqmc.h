@@ -467,6 +467,18 @@ afqmc_status afqmc_local_energy_static(const double* h1, const double* L, const 
 afqmc_status afqmc_test_gemm(int impl, int Md, int Nd, int K, const double* A, const double* B,
                              double alpha, double* C, cudaStream_t stream);
 
+/*
+ * afqmc_plan_value -- testing and reporting aid (no counterpart in the paper): a size or choice
+ * that the library's rules give for an FP64 system of this shape (taylor_order 6), without a
+ * handle and without device memory.  `arg` is unused unless stated.  -1: unknown `what` or bad shape.
+ */
+enum {
+  AFQMC_PLAN_ENERGY_DIGITS = 0,     /* 1: local energies in digit form                          */
+  AFQMC_PLAN_ENERGY_T = 1,          /* doubles for the half-rotated products of a walker chunk  */
+  AFQMC_PLAN_TANGENT_T = 2          /* of these, how many tangent mode fills                    */
+};
+int64_t afqmc_plan_value(int what, int M, int X, int n_up, int n_dn, int n_walkers, int arg);
+
 /* Flyvbjerg-Petersen reblocking error of the mean of series[n] (host only): the
  * largest block-level estimate among levels with >= 16 blocks. */
 double afqmc_reblock_error(const double* series, int n);

@@ -70,6 +70,7 @@ SIGNATURES = {
                                                  VP]),
     "afqmc_test_gemm": (ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_int, VP,
                                        VP, ctypes.c_double, VP, VP]),
+    "afqmc_plan_value": (ctypes.c_int64, [ctypes.c_int] * 7),
     "afqmc_time_kernel": (ctypes.c_int, [VP, ctypes.c_int, ctypes.c_int,
                                          ctypes.POINTER(ctypes.c_double), VP]),
 }

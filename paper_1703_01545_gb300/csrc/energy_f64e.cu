@@ -347,9 +347,35 @@ size_t energy_f64e_scratch(const Ctx& c) {
   const size_t t = 2 * (size_t)c.X * ns * ns * chunk_walkers(c);
   return sizeof(double) * (t + 4 * (size_t)c.Nw * c.X + 4 * (size_t)kMaxSplit * c.Nw);
 }
-// tangent mode: traces of T and dT of both spins and their exchange sums (T and dT share the T chunk)
+
+// Tangent mode: T and dT share the T chunk of c.e64, half of its walkers each; c.e64_tan holds the traces of
+// both and both spins, then the exchange sums.  A chunk of one walker has no room for its dT (one walker in
+// all, or a T above half of kTBytes), which then follows the sums in c.e64_tan.
+struct TanPlace {
+  int nwc;                    // walkers at a time
+  size_t len, ex, dt;         // doubles of T; offsets in c.e64_tan of the sums, and of dT or the end
+  bool own;                   // dT in c.e64_tan
+};
+static TanPlace tan_place(const Ctx& c) {
+  const int ns = std::max(c.n_up, c.N - c.n_up), chunk = chunk_walkers(c);
+  TanPlace t;
+  t.own = chunk < 2;
+  t.nwc = t.own ? 1 : chunk / 2;
+  t.len = 2 * (size_t)c.X * ns * ns * t.nwc;
+  t.ex = 8 * (size_t)c.Nw * c.X;
+  t.dt = t.ex + 8 * (size_t)kMaxSplit * c.Nw;
+  return t;
+}
 size_t energy_tan_f64e_scratch(const Ctx& c) {
-  return sizeof(double) * (8 * (size_t)c.Nw * c.X + 8 * (size_t)kMaxSplit * c.Nw);
+  const TanPlace t = tan_place(c);
+  return sizeof(double) * (t.dt + (t.own ? t.len : 0));
+}
+// doubles at the head of c.e64 that hold T of a chunk, and that tangent mode fills with T and dT
+int64_t energy_chunk_doubles(const Ctx& c, bool tangent) {
+  const int ns = std::max(c.n_up, c.N - c.n_up);
+  if (!tangent) return 2 * (int64_t)c.X * ns * ns * chunk_walkers(c);
+  const TanPlace t = tan_place(c);
+  return (int64_t)(t.own ? t.len : 2 * t.len);
 }
 size_t energy_f64e_ws(const Ctx& c) {
   const int ns = std::max(c.n_up, c.N - c.n_up);
@@ -402,12 +428,12 @@ cudaError_t chunk_of(const Ctx& c, const F64Ws& ws, const double* theta, const D
 
 // E_L and dE_L of every walker from Theta and dTheta (tangent mode)
 cudaError_t launch_energy_tan_f64e(const Ctx& c, cudaStream_t s) {
-  const int NM = c.N * c.M, nwc = std::max(1, chunk_walkers(c) / 2), nsmax = std::max(c.n_up, c.N - c.n_up);
-  const int nsplit = splits(c, nwc);
+  const TanPlace at = tan_place(c);
+  const int NM = c.N * c.M, nwc = at.nwc, nsplit = splits(c, nwc);
   double* T = c.e64;
-  double* dT = T + 2 * (size_t)c.X * nsmax * nsmax * nwc;
+  double* dT = at.own ? c.e64_tan + at.dt : T + at.len;
   double* tr = c.e64_tan;
-  double* ex = tr + 8 * (size_t)c.Nw * c.X;
+  double* ex = tr + at.ex;
   cudaError_t e = cudaSuccess;
   int sp = 0;
   for (int s0 = 0; s0 < 2 && e == cudaSuccess; ++s0) {

@@ -1,0 +1,24 @@
+"""Sizes and choices of the library's rules that need no device (afqmc_plan_value)."""
+import pytest
+
+ENERGY_DIGITS, ENERGY_T, TANGENT_T = range(3)
+
+
+@pytest.fixture(scope="module")
+def plan():
+    from paper_1703_01545_gb300 import _lib
+    from paper_1703_01545_gb300.build import build
+    build()
+    return lambda what, shape, nw, arg=0: _lib.load().afqmc_plan_value(what, *shape, nw, arg)
+
+
+# one walker's products take 1.1 MB at the first shape, 40 MB and more at the last two
+@pytest.mark.parametrize("shape", [(96, 480, 12, 12), (128, 768, 16, 16), (64, 320, 8, 8), (66, 130, 32, 30),
+                                   (64, 2500, 32, 1), (64, 3000, 32, 32)])
+@pytest.mark.parametrize("nw", [1, 2, 3, 5, 36, 37, 300])
+def test_tangent_products_stay_inside_the_energy_scratch(plan, shape, nw):
+    held, filled = plan(ENERGY_T, shape, nw), plan(TANGENT_T, shape, nw)
+    M, X, nu, nd = shape
+    assert held % (2 * X * max(nu, nd) ** 2) == 0 and 0 < filled <= held
+    if nw <= 2 and shape in ((96, 480, 12, 12), (128, 768, 16, 16)):
+        assert plan(ENERGY_DIGITS, shape, nw) == 1   # a handle this small does take the digit form
