@@ -1315,7 +1315,7 @@ afqmc_status afqmc_test_gemm(int impl, int Md, int Nd, int K, const double* A, c
   return e == cudaSuccess ? AFQMC_OK : AFQMC_ERR_CUDA;
 }
 
-int64_t afqmc_plan_value(int what, int M, int X, int n_up, int n_dn, int n_walkers, int) {
+int64_t afqmc_plan_value(int what, int M, int X, int n_up, int n_dn, int n_walkers, int arg) {
   const int64_t N = (int64_t)n_up + n_dn;
   if (M < 1 || X < 1 || n_up < 0 || n_dn < 0 || N < 1 || n_up > M || n_dn > M || n_up > 32 || n_dn > 32 ||
       N * M > 4096 || n_walkers < 1)
@@ -1329,6 +1329,7 @@ int64_t afqmc_plan_value(int what, int M, int X, int n_up, int n_dn, int n_walke
     case AFQMC_PLAN_ENERGY_DIGITS: return afq::energy_f64e_ok(M, X, n_up, n_dn, n_walkers);
     case AFQMC_PLAN_ENERGY_T: return afq::energy_chunk_doubles(c, false);
     case AFQMC_PLAN_TANGENT_T: return afq::energy_chunk_doubles(c, true);
+    case AFQMC_PLAN_EXCHANGE_SMEM: return afq::exchange_smem(std::max(n_up, n_dn), arg != 0);
   }
   return -1;
 }

@@ -28,6 +28,10 @@ constexpr size_t kStage = 40 * 1024;           // staged T of one step of k_exch
 constexpr int kMaxSplit = 16;                  // ranges of g that share a walker's exchange sum
 constexpr int kEx = 256;
 
+// Row length of gb staged Cholesky vectors: odd, so that the staging writes spread over the banks too (single
+// vectors are staged in their order as they are).
+__host__ __device__ constexpr int staged_row(int gb) { return gb > 1 ? gb + 1 : 1; }
+
 // Exchange sums and traces of one spin for walkers w0 .. w0 + gridDim.x - 1; T[(p, wl, b)][(g, a)]
 // with rows of ldt = X ns.  CTA (wl, q) takes the q-th range of g, gb (a power of two up to 32) of
 // them staged at a time (one coalesced read) as [p][b][a][g]: the lanes of a warp are consecutive g
@@ -42,7 +46,7 @@ __global__ void __launch_bounds__(kEx) k_exchange(const double* __restrict__ T, 
   __shared__ double red[2 * (kEx / 32)];
   const int wl = blockIdx.x, nwc = gridDim.x, q = blockIdx.y, tid = threadIdx.x, w = w0 + wl;
   const int g0 = (int)((int64_t)X * q / gridDim.y), g1 = (int)((int64_t)X * (q + 1) / gridDim.y);
-  const int np = ns * (ns + 1) / 2, gs = gb + 1;   // odd row length: the staging writes spread too
+  const int np = ns * (ns + 1) / 2, gs = staged_row(gb);
   const int pl = ns * ns * gs;                     // imaginary plane
   const int lg = tid & (gb - 1), slot = tid / gb, nslot = kEx / gb;
   // sums over a = b (xr^2 - xi^2, xr xi) and over a < b (T_ab T_ba), doubled where due at the end
@@ -138,7 +142,7 @@ __global__ void __launch_bounds__(kEx) k_exchange_tan(const double* __restrict__
   __shared__ double red[4 * (kEx / 32)];
   const int wl = blockIdx.x, nwc = gridDim.x, q = blockIdx.y, tid = threadIdx.x, w = w0 + wl;
   const int g0 = (int)((int64_t)X * q / gridDim.y), g1 = (int)((int64_t)X * (q + 1) / gridDim.y);
-  const int nsq = ns * ns, gs = gb + 1, pl = nsq * gs;   // planes: T re, T im, dT re, dT im
+  const int nsq = ns * ns, gs = staged_row(gb), pl = nsq * gs;   // planes: T re, T im, dT re, dT im
   const int lg = tid & (gb - 1), slot = tid / gb, nslot = kEx / gb;
   double acc[4] = {0.0, 0.0, 0.0, 0.0};
   for (int gc = g0; gc < g1; gc += gb) {
@@ -406,10 +410,12 @@ cudaError_t products_of(const Ctx& c, const F64Ws& ws, const double* theta, cons
   return digit_gemm(da, db, g, s);
 }
 
-// Cholesky vectors staged at a time by the exchange kernels: a power of two within kStage
+// Cholesky vectors staged at a time by the exchange kernels: a power of two within kStage.  A single one takes
+// 32 KB at most (4 planes, ns = 32), so no launch asks for more than the 48 KB that need no attribute.
+size_t staged_bytes(int ns, int planes, int gb) { return (size_t)planes * ns * ns * staged_row(gb) * sizeof(double); }
 int staged(int ns, int planes) {
   int gb = 32;
-  while (gb > 1 && (size_t)planes * ns * ns * (gb + 1) * sizeof(double) > kStage) gb /= 2;
+  while (gb > 1 && staged_bytes(ns, planes, gb) > kStage) gb /= 2;
   return gb;
 }
 
@@ -419,12 +425,14 @@ cudaError_t chunk_of(const Ctx& c, const F64Ws& ws, const double* theta, const D
   const cudaError_t e = products_of(c, ws, theta, da, cols, n0, ns, w0, nw, T, s);
   if (e != cudaSuccess) return e;
   const int gb = staged(ns, 2);
-  k_exchange<<<dim3(nw, nsplit), kEx, (size_t)2 * ns * ns * (gb + 1) * sizeof(double), s>>>(
+  k_exchange<<<dim3(nw, nsplit), kEx, staged_bytes(ns, 2, gb), s>>>(
       T, c.X * ns, ns, c.X, w0, c.Nw, gb, ex + (size_t)sp * nsplit * 2 * c.Nw, tr + (size_t)sp * 2 * c.Nw * c.X);
   return cudaGetLastError();
 }
 
 }  // namespace
+
+int64_t exchange_smem(int ns, bool tangent) { return (int64_t)staged_bytes(ns, tangent ? 4 : 2, staged(ns, tangent ? 4 : 2)); }
 
 // E_L and dE_L of every walker from Theta and dTheta (tangent mode)
 cudaError_t launch_energy_tan_f64e(const Ctx& c, cudaStream_t s) {
@@ -447,7 +455,7 @@ cudaError_t launch_energy_tan_f64e(const Ctx& c, cudaStream_t s) {
       e = products_of(c, c.ws64, c.theta, da, cols, n0, ns, w0, nw, T, s);
       if (e == cudaSuccess) e = products_of(c, c.ws64, c.dtheta, da, cols, n0, ns, w0, nw, dT, s);
       if (e != cudaSuccess) break;
-      k_exchange_tan<<<dim3(nw, nsplit), kEx, (size_t)4 * ns * ns * (gb + 1) * sizeof(double), s>>>(
+      k_exchange_tan<<<dim3(nw, nsplit), kEx, staged_bytes(ns, 4, gb), s>>>(
           T, dT, c.X * ns, ns, c.X, w0, c.Nw, gb, ex + (size_t)sp * nsplit * 4 * c.Nw,
           tr + (size_t)sp * 4 * c.Nw * c.X);
       e = cudaGetLastError();

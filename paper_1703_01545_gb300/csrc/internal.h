@@ -229,6 +229,7 @@ size_t energy_f64e_scratch(const Ctx& c);
 size_t energy_f64e_ws(const Ctx& c);
 size_t energy_tan_f64e_scratch(const Ctx& c);   // beside c.e64, for tangent mode (c.e64_tan)
 int64_t energy_chunk_doubles(const Ctx& c, bool tangent);   // of c.e64: T of a chunk, what tangent mode fills
+int64_t exchange_smem(int ns, bool tangent);   // shared memory of its exchange kernels for a spin block of ns
 cudaError_t launch_energy_tan_f64e(const Ctx& c, cudaStream_t s);
 cudaError_t launch_energy_f64e(const Ctx& c, cudaStream_t s);
 cudaError_t digit_gemm(const DigitOp& rows, const DigitOp& cols, const DigitGemm& g, cudaStream_t s);

@@ -1,7 +1,7 @@
 """Sizes and choices of the library's rules that need no device (afqmc_plan_value)."""
 import pytest
 
-ENERGY_DIGITS, ENERGY_T, TANGENT_T = range(3)
+ENERGY_DIGITS, ENERGY_T, TANGENT_T, EXCHANGE_SMEM = range(4)
 
 
 @pytest.fixture(scope="module")
@@ -22,3 +22,10 @@ def test_tangent_products_stay_inside_the_energy_scratch(plan, shape, nw):
     assert held % (2 * X * max(nu, nd) ** 2) == 0 and 0 < filled <= held
     if nw <= 2 and shape in ((96, 480, 12, 12), (128, 768, 16, 16)):
         assert plan(ENERGY_DIGITS, shape, nw) == 1   # a handle this small does take the digit form
+
+
+@pytest.mark.parametrize("tangent", [0, 1])
+def test_exchange_sums_fit_the_shared_memory_of_every_launch(plan, tangent):
+    """48 KB need no raised limit, and every spin block up to the largest (32) is dispatched to them."""
+    for ns in range(1, 33):
+        assert 0 < plan(EXCHANGE_SMEM, (64, 130, ns, 0), 40, tangent) <= 48 * 1024
