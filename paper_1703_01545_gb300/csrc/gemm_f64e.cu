@@ -711,16 +711,17 @@ size_t gemm_f64e_bytes(int64_t Md, int64_t Nd, int Kd, size_t col_cap) {
 }
 
 cudaError_t prepare_gemm_f64e() {
-  static cudaError_t st = cudaErrorNotReady;
-  static std::once_flag once;
-  std::call_once(once, []() {
-    const auto at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    st = cudaFuncSetAttribute(k_gemm_f64e<16>, at, ELay<16>::kSmem);
-    if (st == cudaSuccess) st = cudaFuncSetAttribute(k_gemm_f64e<32>, at, ELay<32>::kSmem);
-    if (st == cudaSuccess) st = cudaFuncSetAttribute(k_gemm_f64e<48>, at, ELay<48>::kSmem);
-    if (st == cudaSuccess) st = cudaFuncSetAttribute(k_gemm_f64e<64>, at, ELay<64>::kSmem);
-  });
-  return st;
+  static SmemLimits limits;   // per device: a handle of another device raises its own
+  auto raise = [&](int slot, auto k, int bytes) {
+    return limits.raise(slot, (size_t)bytes, [&] {
+      return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    });
+  };
+  cudaError_t e = raise(0, k_gemm_f64e<16>, ELay<16>::kSmem);
+  if (e == cudaSuccess) e = raise(1, k_gemm_f64e<32>, ELay<32>::kSmem);
+  if (e == cudaSuccess) e = raise(2, k_gemm_f64e<48>, ELay<48>::kSmem);
+  if (e == cudaSuccess) e = raise(3, k_gemm_f64e<64>, ELay<64>::kSmem);
+  return e;
 }
 
 // B goes through the workspace in chunks of rows when its digits do not fit beside A's.

@@ -883,26 +883,21 @@ cudaError_t gemm_bf16x3_wait_selftest(const TcOperand& A, const TcOperand& B, in
   return launch_tc<128, 3, float>(A, B, Md, Nd, 1.0f, C, ldc, err, s, wait_ns, 1);
 }
 
-// Once per process, before any launch or capture: the ring needs ~194 KB of shared memory.
+// Once per device, before any launch or capture: the rings need up to ~217 KB of shared memory.
 cudaError_t prepare_tc_kernels() {
-  static cudaError_t st = cudaErrorNotReady;
-  static std::once_flag once;
-  std::call_once(once, []() {
-    using Lay = TcLayout<128, 3>;
-    st = cudaFuncSetAttribute(k_gemm_bf16x3_tc<128, 3, float>,
-                              cudaFuncAttributeMaxDynamicSharedMemorySize, Lay::SMEM_BYTES);
-    if (st == cudaSuccess)
-      st = cudaFuncSetAttribute(k_gemm_bf16x3_tc<128, 3, double>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, Lay::SMEM_BYTES);
-    if (st == cudaSuccess)
-      st = cudaFuncSetAttribute(k_gemm_bf16x3_tc_persist, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                PLayoutG::SMEM_BYTES);
-    if (st == cudaSuccess)
-      st = cudaFuncSetAttribute(k_gemm_bf16x3_tc_pair, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                QLayout::SMEM_BYTES);
-    find_pair_clusters();   // asked for here, not under a capture
-  });
-  return st;
+  static SmemLimits limits;
+  auto raise = [&](int slot, auto k, int bytes) {
+    return limits.raise(slot, (size_t)bytes, [&] {
+      return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    });
+  };
+  using Lay = TcLayout<128, 3>;
+  cudaError_t e = raise(0, k_gemm_bf16x3_tc<128, 3, float>, Lay::SMEM_BYTES);
+  if (e == cudaSuccess) e = raise(1, k_gemm_bf16x3_tc<128, 3, double>, Lay::SMEM_BYTES);
+  if (e == cudaSuccess) e = raise(2, k_gemm_bf16x3_tc_persist, PLayoutG::SMEM_BYTES);
+  if (e == cudaSuccess) e = raise(3, k_gemm_bf16x3_tc_pair, QLayout::SMEM_BYTES);
+  if (e == cudaSuccess) find_pair_clusters();   // asked for here, after the limit and not under a capture
+  return e;
 }
 
 }  // namespace afq
