@@ -476,7 +476,8 @@ enum {
   AFQMC_PLAN_ENERGY_DIGITS = 0,     /* 1: local energies in digit form                          */
   AFQMC_PLAN_ENERGY_T = 1,          /* doubles for the half-rotated products of a walker chunk  */
   AFQMC_PLAN_TANGENT_T = 2,         /* of these, how many tangent mode fills                    */
-  AFQMC_PLAN_EXCHANGE_SMEM = 3      /* shared memory of the exchange sums (arg 1: tangent mode) */
+  AFQMC_PLAN_EXCHANGE_SMEM = 3,     /* shared memory of the exchange sums (arg 1: tangent mode) */
+  AFQMC_PLAN_STEPS_SMALL = 4        /* 1: arg steps of a call run in the kernel for small systems */
 };
 int64_t afqmc_plan_value(int what, int M, int X, int n_up, int n_dn, int n_walkers, int arg);
 

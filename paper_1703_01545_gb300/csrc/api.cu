@@ -383,7 +383,7 @@ afqmc_status step_launch(Ctx* h, const double* fields_t, cudaStream_t s) {
 
 // n_steps steps; fields [n_steps][Nw][X] or null.
 afqmc_status steps_launch(Ctx* h, int n_steps, const double* fields, cudaStream_t s) {
-  if (!h->tangent_on && afq::step_small_ok(*h)) {
+  if (!h->tangent_on && afq::step_small_pays(*h, n_steps)) {
     AFQ_CK(afq::launch_steps_small(*h, n_steps, fields, s));
     return AFQMC_OK;
   }
@@ -1329,6 +1329,7 @@ int64_t afqmc_plan_value(int what, int M, int X, int n_up, int n_dn, int n_walke
     case AFQMC_PLAN_ENERGY_DIGITS: return afq::energy_f64e_ok(M, X, n_up, n_dn, n_walkers);
     case AFQMC_PLAN_ENERGY_T: return afq::energy_chunk_doubles(c, false);
     case AFQMC_PLAN_TANGENT_T: return afq::energy_chunk_doubles(c, true);
+    case AFQMC_PLAN_STEPS_SMALL: return afq::step_small_pays(c, arg);
     case AFQMC_PLAN_EXCHANGE_SMEM: return afq::exchange_smem(std::max(n_up, n_dn), arg != 0);
   }
   return -1;

@@ -445,7 +445,8 @@ cudaError_t launch_mixed_sum(const Ctx& c, double* out, const int* slot, int slo
                              cudaStream_t s);
 cudaError_t launch_step_advance(const Ctx& c, cudaStream_t s, int n_steps = 1);
 // Whole FP64 steps of small systems in one kernel (step_small.cu)
-bool step_small_ok(const Ctx& c);
+bool step_small_ok(const Ctx& c);              // the shapes it takes
+bool step_small_pays(const Ctx& c, int n);     // and whether a call of n steps does
 cudaError_t prepare_step_small(const Ctx& c);
 cudaError_t launch_steps_small(const Ctx& c, int n_steps, const double* fields, cudaStream_t s);
 

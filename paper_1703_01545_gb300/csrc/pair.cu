@@ -80,12 +80,14 @@ afqmc_status record_block(afqmc_ctx* A, afqmc_ctx* B, Res* r, F last) {
   afqmc_status st = AFQMC_OK;
   cudaError_t ce = cudaEventRecord(r->fork, r->cs);
   if (ce == cudaSuccess) ce = cudaStreamWaitEvent(r->cs2, r->fork, 0);
-  // steps of A and B recorded in turn, or all up to the orthonormalisation where a kernel takes several
-  const int run = afq::step_small_ok(*A) && afq::step_small_ok(*B) ? r->me : 1;
+  // steps of A and B recorded in turn, all up to the orthonormalisation at once where a kernel takes several
+  const bool one_a = afq::step_small_pays(*A, r->me), one_b = afq::step_small_pays(*B, r->me);
   for (int j = 0; j < r->ee && st == AFQMC_OK && ce == cudaSuccess; j += r->me) {   // ee is a multiple of me
-    for (int k = 0; k < r->me && st == AFQMC_OK; k += run) {
-      st = afq::pair_steps(A, run, r->cs);
-      if (st == AFQMC_OK) st = afq::pair_steps(B, run, r->cs2);
+    if (one_a) st = afq::pair_steps(A, r->me, r->cs);
+    if (st == AFQMC_OK && one_b) st = afq::pair_steps(B, r->me, r->cs2);
+    for (int k = 0; k < r->me && st == AFQMC_OK; ++k) {
+      if (!one_a) st = afq::pair_steps(A, 1, r->cs);
+      if (st == AFQMC_OK && !one_b) st = afq::pair_steps(B, 1, r->cs2);
     }
     if (st == AFQMC_OK) st = afq::pair_ortho(A, r->cs);
     if (st == AFQMC_OK) st = afq::pair_ortho(B, r->cs2);

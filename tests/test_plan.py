@@ -1,7 +1,7 @@
 """Sizes and choices of the library's rules that need no device (afqmc_plan_value)."""
 import pytest
 
-ENERGY_DIGITS, ENERGY_T, TANGENT_T, EXCHANGE_SMEM = range(4)
+ENERGY_DIGITS, ENERGY_T, TANGENT_T, EXCHANGE_SMEM, STEPS_SMALL = range(5)
 
 
 @pytest.fixture(scope="module")
@@ -29,3 +29,13 @@ def test_exchange_sums_fit_the_shared_memory_of_every_launch(plan, tangent):
     """48 KB need no raised limit, and every spin block up to the largest (32) is dispatched to them."""
     for ns in range(1, 33):
         assert 0 < plan(EXCHANGE_SMEM, (64, 130, ns, 0), 40, tangent) <= 48 * 1024
+
+
+@pytest.mark.parametrize("shape,nw,steps,small", [
+    ((8, 24, 2, 2), 128, 1, 1), ((8, 24, 2, 2), 128, 40, 1), ((8, 24, 2, 2), 1000, 1, 1),
+    ((8, 24, 2, 2), 8000, 1, 0), ((8, 24, 2, 2), 40000, 1, 0), ((8, 24, 2, 2), 8000, 2, 1),
+    ((8, 24, 2, 2), 40000, 2, 0), ((8, 24, 2, 2), 40000, 5, 1), ((12, 40, 3, 3), 300, 1, 1),
+    ((12, 40, 3, 3), 1000, 1, 0), ((12, 40, 3, 3), 1000, 5, 1), ((12, 40, 3, 3), 4000, 8, 0),
+    ((17, 40, 3, 3), 64, 5, 0)])
+def test_whole_steps_of_small_systems_where_they_were_measured_faster(plan, shape, nw, steps, small):
+    assert plan(STEPS_SMALL, shape, nw, steps) == small
