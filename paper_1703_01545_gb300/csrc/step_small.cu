@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(kT) k_steps_small(const SmallArgs g) {
     const double* q = sm + l.aux + 4 * t;
     bool bad = d[6] != 0.0 || d[7] != 0.0;
     const double pr = fma(d[0], d[2], -d[1] * d[3]), pi = fma(d[0], d[3], d[1] * d[2]);
-    ld_re = 0.5 * log(fma(pr, pr, pi * pi)) + (d[4] + d[5]) * M_LN2;
+    ld_re = fma(d[4] + d[5], M_LN2, 0.5 * log(fma(pr, pr, pi * pi)));
     ld_im = atan2(pi, pr);
     bad = bad || !isfinite(ld_re) || !isfinite(ld_im);
     double pv_re = __shfl_up_sync(0xffffffffu, ld_re, 1), pv_im = __shfl_up_sync(0xffffffffu, ld_im, 1);

@@ -439,16 +439,74 @@ __global__ void __launch_bounds__(256) k_overlap_fast(FastOvArgs a) {
   }
 }
 
+// Of a walker, from the record dt of its determinants (FastOvArgs.det): log det O, the overlap ratio and the
+// weight update.  row: determinant (mode OV_DET).
+__device__ __forceinline__ void overlap_weights(const FastOvArgs& a, int wk, int row, const double* dt) {
+  const bool upd = (a.mode == OV_UPDATE) && a.alive[wk] != 0;
+  if (a.mode == OV_UPDATE && !upd) return;
+  double* logO = a.logO + row * a.det_logO;
+  const bool bad = dt[5] != 0.0;
+  // log det O = log(d_up d_dn) + (e_up + e_dn) ln 2
+  const double d0r = dt[0], d0i = dt[1], d1r = dt[2], d1i = dt[3];
+  const double pr_ = fma(d0r, d1r, -d0i * d1i), pi_ = fma(d0r, d1i, d0i * d1r);
+  const double ld_re = fma(dt[4], M_LN2, 0.5 * log(fma(pr_, pr_, pi_ * pi_)));   // (spelt out: the same bits in every kernel)
+  const double ld_im = atan2(pi_, pr_);
+  if (bad || !isfinite(ld_re) || !isfinite(ld_im)) {
+    if (a.mode == OV_DET) {   // this determinant contributes nothing to the trial
+      logO[wk] = -INFINITY;
+      logO[a.Nw + wk] = 0.0;
+      return;
+    }
+    atomicAdd(a.flags, 1);
+    if (upd || a.mode == OV_REFRESH) {
+      a.w[wk] = 0.0;
+      a.w[a.Nw + wk] = 0.0;
+      a.alive[wk] = 0;
+    }
+    return;
+  }
+  if (!upd) {
+    logO[wk] = ld_re;
+    logO[a.Nw + wk] = ld_im;
+    return;
+  }
+  const double* x = a.aux + 4 * (int64_t)wk;
+  const double lr_re = x[0] + ld_re - a.logO[wk];
+  const double lr_im = x[1] + ld_im - a.logO[a.Nw + wk];
+  const double li_re = lr_re + x[2] + a.log_shift;
+  const double li_im = lr_im + x[3];
+  a.logO[wk] = ld_re;
+  a.logO[a.Nw + wk] = ld_im;
+  if (a.free_proj) {
+    const double mag = exp(li_re);
+    double sn, cs;
+    sincos(li_im, &sn, &cs);
+    const cplx nw = cmul({a.w[wk], a.w[a.Nw + wk]}, {mag * cs, mag * sn});
+    a.w[wk] = nw.re;
+    a.w[a.Nw + wk] = nw.im;
+  } else {
+    const double nw = a.w[wk] * exp(li_re) * fmax(0.0, cos(lr_im));
+    if (nw > 0.0) {
+      a.w[wk] = nw;
+    } else {
+      a.w[wk] = 0.0;
+      a.alive[wk] = 0;
+    }
+    a.w[a.Nw + wk] = 0.0;
+  }
+}
+
 // The FP64 path's overlap, determinant and Theta for spin blocks of at most 16, everything in
 // float64: the sums of O_s = Psi_s^T Phi_s (4 lanes an entry), the warp LU above, and Theta_s =
 // Phi_s O_s^{-1} by triangular solves, one orbital row of a spin per thread (half the operations of
 // forming the inverse and multiplying).  Bound by the FP64 pipe (2 multiply-adds per clock and SM):
 // at M = 64, 8/8 about 52 k of them per walker, 0.18 ms for 2048 walkers; measured 0.23 ms, against
 // 0.52 ms of the block-wide Gauss-Jordan kernel (k_overlap, now for larger blocks only), which waits at
-// its barriers for as long again.  128 walkers at M = 8, 2/2: 22 -> 9.4 us.
+// its barriers for as long again.  150 walkers at M = 16, 2/2, with the weights: 22.5 -> 9.0 us.
 // Modes as k_overlap: OV_UPDATE takes src as the walker if it lives, else recomputes from Phi
 // (Theta's buffer held the propagated walkers); OV_DET: grid row = determinant, no walker changes.
-template <int ROWS, int NSM>
+// WEIGHTS: the walker's log O and weight too, by a thread beside the solves, instead of k_overlap_weights.
+template <int ROWS, int NSM, bool WEIGHTS>
 __global__ void __launch_bounds__(256) k_overlap64(FastOvArgs a) {
   extern __shared__ double smo[];
   const int wk = blockIdx.x, tid = threadIdx.x, M = a.M, N = a.N, NM = N * M;
@@ -537,6 +595,11 @@ __global__ void __launch_bounds__(256) k_overlap64(FastOvArgs a) {
     s_perm[tid] = pw;
   }
   __syncthreads();
+  if (WEIGHTS && tid == (int)blockDim.x - 32) {   // (the last warp has the fewest rows to solve)
+    const double dt[6] = {s_det[0][0], s_det[0][1], s_det[1][0], s_det[1][1], (double)(s_dexp[0] + s_dexp[1]),
+                          bad ? 1.0 : 0.0};
+    overlap_weights(a, wk, blockIdx.y, dt);
+  }
   if (bad) {
     for (int e = tid; e < NM; e += blockDim.x) theta[wbase + e] = theta[plane + wbase + e] = 0.0;
   } else {
@@ -586,7 +649,7 @@ __global__ void __launch_bounds__(256) k_overlap64(FastOvArgs a) {
         }
     }
   }
-  if (tid < 6) {
+  if (!WEIGHTS && tid < 6) {
     double v = bad ? 1.0 : 0.0;
     if (tid < 4) v = s_det[tid >> 1][tid & 1];
     else if (tid == 4) v = (double)(s_dexp[0] + s_dexp[1]);
@@ -594,64 +657,11 @@ __global__ void __launch_bounds__(256) k_overlap64(FastOvArgs a) {
   }
 }
 
-// Per walker, after k_overlap_fast or k_overlap64: log det O, the overlap ratio and the weight update.
+// The same for one walker a thread, after k_overlap_fast or k_overlap64.
 __global__ void __launch_bounds__(32) k_overlap_weights(FastOvArgs a) {
   after_previous();
   const int wk = blockIdx.x * blockDim.x + threadIdx.x;
-  if (wk >= a.Nw) return;
-  const bool upd = (a.mode == OV_UPDATE) && a.alive[wk] != 0;
-  if (a.mode == OV_UPDATE && !upd) return;
-  const double* dt = a.det + blockIdx.y * a.det_det + 8 * (int64_t)wk;
-  double* logO = a.logO + blockIdx.y * a.det_logO;
-  const bool bad = dt[5] != 0.0;
-  // log det O = log(d_up d_dn) + (e_up + e_dn) ln 2
-  const double d0r = dt[0], d0i = dt[1], d1r = dt[2], d1i = dt[3];
-  const double pr_ = fma(d0r, d1r, -d0i * d1i), pi_ = fma(d0r, d1i, d0i * d1r);
-  const double ld_re = 0.5 * log(fma(pr_, pr_, pi_ * pi_)) + dt[4] * M_LN2;
-  const double ld_im = atan2(pi_, pr_);
-  if (bad || !isfinite(ld_re) || !isfinite(ld_im)) {
-    if (a.mode == OV_DET) {   // this determinant contributes nothing to the trial
-      logO[wk] = -INFINITY;
-      logO[a.Nw + wk] = 0.0;
-      return;
-    }
-    atomicAdd(a.flags, 1);
-    if (upd || a.mode == OV_REFRESH) {
-      a.w[wk] = 0.0;
-      a.w[a.Nw + wk] = 0.0;
-      a.alive[wk] = 0;
-    }
-    return;
-  }
-  if (!upd) {
-    logO[wk] = ld_re;
-    logO[a.Nw + wk] = ld_im;
-    return;
-  }
-  const double* x = a.aux + 4 * (int64_t)wk;
-  const double lr_re = x[0] + ld_re - a.logO[wk];
-  const double lr_im = x[1] + ld_im - a.logO[a.Nw + wk];
-  const double li_re = lr_re + x[2] + a.log_shift;
-  const double li_im = lr_im + x[3];
-  a.logO[wk] = ld_re;
-  a.logO[a.Nw + wk] = ld_im;
-  if (a.free_proj) {
-    const double mag = exp(li_re);
-    double sn, cs;
-    sincos(li_im, &sn, &cs);
-    const cplx nw = cmul({a.w[wk], a.w[a.Nw + wk]}, {mag * cs, mag * sn});
-    a.w[wk] = nw.re;
-    a.w[a.Nw + wk] = nw.im;
-  } else {
-    const double nw = a.w[wk] * exp(li_re) * fmax(0.0, cos(lr_im));
-    if (nw > 0.0) {
-      a.w[wk] = nw;
-    } else {
-      a.w[wk] = 0.0;
-      a.alive[wk] = 0;
-    }
-    a.w[a.Nw + wk] = 0.0;
-  }
+  if (wk < a.Nw) overlap_weights(a, wk, blockIdx.y, a.det + blockIdx.y * a.det_det + 8 * (int64_t)wk);
 }
 
 // Modified Gram-Schmidt, one warp per spin block: columns in order, each projection
@@ -1125,6 +1135,14 @@ cudaError_t launch_overlap_fast(const Ctx& c, const double* src, int mode, cudaS
 }
 
 namespace {
+// Whether a walker's CTA takes its weight too.  The chain of some 250 FP64 instructions holds an SM's FP64 pipe
+// as long for one lane as for 32, so a second launch pays from some CTAs an SM on.  A refresh, us in one kernel
+// / in two (k_overlap before them, in brackets), of 150, 600, 1200 and 2400 walkers:
+//   M = 12, one electron  7.1 / 11.0 (7.6)    9.0 / 11.7 (8.1)    14.1 / 13.7 (15.3)  24.3 / 18.4 (24.9)
+//   M = 16, 2/2           9.0 / 13.4 (22.5)   11.5 / 14.1 (24.6)  18.1 / 17.8 (48.3)  32.3 / 26.6 (76.8)
+//   M = 40, 6/5           22.8 / 27.2 (58.0)  41.7 / 43.2 (77.3)  72.7 / 72.2 (159)   141 / 136 (273)
+bool overlap64_fused(int Nw, int n_det) { return (int64_t)Nw * n_det <= 152 * 4; }
+
 size_t smem_overlap64(const Ctx& c) {
   const int nmax = std::max(c.n_up, c.N - c.n_up);
   return sizeof(double) * (2 * (size_t)c.N * (c.M + 1) + 4 * (nmax <= 8 ? 8 * 8 : kNsMax * kLd));
@@ -1143,9 +1161,12 @@ cudaError_t prepare_overlap64(const Ctx& c) {
       return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     });
   };
-  cudaError_t e = raise(0, k_overlap64<4, 8>);
-  if (e == cudaSuccess) e = raise(1, k_overlap64<4, 16>);
-  if (e == cudaSuccess) e = raise(2, k_overlap64<8, 16>);
+  cudaError_t e = raise(0, k_overlap64<4, 8, false>);
+  if (e == cudaSuccess) e = raise(1, k_overlap64<4, 16, false>);
+  if (e == cudaSuccess) e = raise(2, k_overlap64<8, 16, false>);
+  if (e == cudaSuccess) e = raise(3, k_overlap64<4, 8, true>);
+  if (e == cudaSuccess) e = raise(4, k_overlap64<4, 16, true>);
+  if (e == cudaSuccess) e = raise(5, k_overlap64<8, 16, true>);
   return e;
 }
 
@@ -1174,10 +1195,12 @@ cudaError_t launch_overlap64(const Ctx& c, const double* src, int mode, cudaStre
   const int rows = nmax > 0 ? (nmax + (32 / nmax) - 1) / (32 / nmax) : 1;   // LU rows of a lane
   // as many threads as the entries' lanes or the solves' rows can use
   const int nt = std::max(64, std::min(256, std::max(2 * c.M, 4 * nmax * nmax) / 32 * 32));
-  if (nmax <= 8) k_overlap64<4, 8><<<grid, nt, sm, s>>>(a);
-  else if (rows <= 4) k_overlap64<4, 16><<<grid, nt, sm, s>>>(a);
-  else k_overlap64<8, 16><<<grid, nt, sm, s>>>(a);
-  k_overlap_weights<<<dim3((c.Nw + 31) / 32, nd), 32, 0, s>>>(a);
+  const bool fused = overlap64_fused(c.Nw, nd);
+  auto k = nmax <= 8 ? (fused ? k_overlap64<4, 8, true> : k_overlap64<4, 8, false>)
+           : rows <= 4 ? (fused ? k_overlap64<4, 16, true> : k_overlap64<4, 16, false>)
+                       : (fused ? k_overlap64<8, 16, true> : k_overlap64<8, 16, false>);
+  k<<<grid, nt, sm, s>>>(a);
+  if (!fused) k_overlap_weights<<<dim3((c.Nw + 31) / 32, nd), 32, 0, s>>>(a);
   return cudaGetLastError();
 }
 
