@@ -1,4 +1,6 @@
 // Small element-wise kernels used once per afqmc_setup / afqmc_set_walkers.
+#include <algorithm>
+
 #include "device_util.cuh"
 #include "internal.h"
 
@@ -113,23 +115,27 @@ __global__ void k_init_weights(double* w, int* alive, const double* w_in, int Nw
 }
 
 // external [2][Nw][M][N] <-> internal [2][Nw][N][M]
-// [i][n] <-> [n][i] of every walker and plane: a CTA per matrix, through shared memory, so that both
+// [i][n] <-> [n][i] of every walker and plane: a CTA for `mats` matrices, through shared memory, so that both
 // sides are read and written along their rows (N M <= 4096 numbers).  Bound by memory: 537 MB at
 // M = 128, N = 32, 4096 walkers, 123 us when one side went to memory element by element.
+// MANY: small matrices share a CTA, which one of them would leave mostly idle: N M = 12, 2400 walkers, 4.3 us
+// with a CTA each, 1.9 so; N M = 64: 4.5 and 3.5.  From N M = 144 on (5.1, 5.0; N M = 440: 7.9, 10.9) they do not.
+template <bool MANY>
 __global__ void __launch_bounds__(256) k_phi_layout(const double* __restrict__ in, double* __restrict__ out, int M,
-                                                    int N, int to_internal) {
+                                                    int N, int to_internal, int n_mat, int mats) {
   extern __shared__ double sm[];
   const int per = M * N, rin = to_internal ? M : N, cin = to_internal ? N : M;   // in: [rin][cin]
-  const int ld = rin | 1;
-  const int64_t base = (int64_t)blockIdx.x * per;
-  for (int e = threadIdx.x; e < per; e += blockDim.x) {
-    const int r = e / cin, c = e - r * cin;
-    sm[c * ld + r] = in[base + e];
+  const int ld = rin | 1, pl = cin * ld, m0 = blockIdx.x * mats;
+  const int total = MANY ? per * min(mats, n_mat - m0) : per;
+  const int64_t base = (int64_t)m0 * per;
+  for (int e = threadIdx.x; e < total; e += blockDim.x) {
+    const int m = MANY ? e / per : 0, x = e - m * per, r = x / cin, c = x - r * cin;
+    sm[m * pl + c * ld + r] = in[base + e];
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < per; e += blockDim.x) {
-    const int c = e / rin, r = e - c * rin;
-    out[base + e] = sm[c * ld + r];
+  for (int e = threadIdx.x; e < total; e += blockDim.x) {
+    const int m = MANY ? e / per : 0, x = e - m * per, c = x / rin, r = x - c * rin;
+    out[base + e] = sm[m * pl + c * ld + r];
   }
 }
 
@@ -184,8 +190,14 @@ cudaError_t launch_init_weights(double* w, int* alive, const double* w_in, int N
 }
 cudaError_t launch_phi_layout(const double* in, double* out, int Nw, int M, int N, int to_internal,
                               cudaStream_t s) {
-  const int ld = (to_internal ? M : N) | 1, cols = to_internal ? N : M;
-  k_phi_layout<<<2 * Nw, 256, sizeof(double) * (size_t)cols * ld, s>>>(in, out, M, N, to_internal);
+  const int ld = (to_internal ? M : N) | 1, cols = to_internal ? N : M, n_mat = 2 * Nw;
+  // matrices of at most 128 numbers: about 1024 a CTA, while there are CTAs for two an SM
+  const int mats = M * N <= 128 ? std::max(1, std::min(1024 / (M * N), n_mat / (2 * 152))) : 1;
+  const size_t sm = sizeof(double) * (size_t)cols * ld * mats;
+  if (mats > 1)
+    k_phi_layout<true><<<(n_mat + mats - 1) / mats, 256, sm, s>>>(in, out, M, N, to_internal, n_mat, mats);
+  else
+    k_phi_layout<false><<<n_mat, 256, sm, s>>>(in, out, M, N, to_internal, n_mat, 1);
   return cudaGetLastError();
 }
 
