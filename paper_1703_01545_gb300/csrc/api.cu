@@ -305,13 +305,13 @@ afqmc_status energy_launch(Ctx* h, cudaStream_t s) {
   return AFQMC_OK;
 }
 
-// After a synchronisation: report an expired tensor-core wait.
-afqmc_status check_tc(Ctx* h) {
-  if (!h->d_tc_err) return AFQMC_OK;
-  int v = 0;
-  AFQ_CK(cudaMemcpy(&v, h->d_tc_err, sizeof(int), cudaMemcpyDeviceToHost));
-  if (v) return set_err(h, AFQMC_ERR_TIMEOUT, "a tensor-core kernel's bounded wait expired");
-  return AFQMC_OK;
+// The flag of expired waits, read on the stream: ask_tc before the caller's synchronisation, tc_status after.
+cudaError_t ask_tc(const Ctx* h, int* flag, cudaStream_t s) {
+  *flag = 0;
+  return h->d_tc_err ? cudaMemcpyAsync(flag, h->d_tc_err, sizeof(int), cudaMemcpyDeviceToHost, s) : cudaSuccess;
+}
+afqmc_status tc_status(Ctx* h, int flag) {
+  return flag ? set_err(h, AFQMC_ERR_TIMEOUT, "a tensor-core kernel's bounded wait expired") : AFQMC_OK;
 }
 
 afqmc_status step_launch_mixed(Ctx* h, const double* fields_t, cudaStream_t s);
@@ -456,7 +456,8 @@ afqmc_status run_step(Ctx* h, const double* fields_t, cudaStream_t s) { return s
 afqmc_status plain_step(Ctx* h, const double* fields_t, cudaStream_t s) { return steps_launch(h, 1, fields_t, s); }
 afqmc_status pair_ortho(Ctx* h, cudaStream_t s) { return ortho_launch(h, s); }
 afqmc_status pair_energy(Ctx* h, cudaStream_t s) { return energy_launch(h, s); }
-afqmc_status pair_check(Ctx* h) { return check_tc(h); }
+cudaError_t pair_ask_tc(const Ctx* h, int* flag, cudaStream_t s) { return ask_tc(h, flag, s); }
+afqmc_status pair_tc_status(Ctx* h, int flag) { return tc_status(h, flag); }
 }  // namespace afq
 
 extern "C" {
@@ -869,8 +870,10 @@ afqmc_status afqmc_get_state(afqmc_handle h, double* phi, double* logO, double* 
   if (logO) AFQ_CK(cudaMemcpyAsync(logO, h->logO, sizeof(double) * 2 * h->Nw, cudaMemcpyDefault, s));
   if (w) AFQ_CK(cudaMemcpyAsync(w, h->w, sizeof(double) * 2 * h->Nw, cudaMemcpyDefault, s));
   if (alive) AFQ_CK(cudaMemcpyAsync(alive, h->alive, sizeof(int) * h->Nw, cudaMemcpyDefault, s));
+  int expired;
+  AFQ_CK(ask_tc(h, &expired, s));
   AFQ_CK(cudaStreamSynchronize(s));
-  return check_tc(h);
+  return tc_status(h, expired);
 }
 
 afqmc_status afqmc_get_info(afqmc_handle h, afqmc_info* info, cudaStream_t s) {
@@ -884,11 +887,13 @@ afqmc_status afqmc_get_info(afqmc_handle h, afqmc_info* info, cudaStream_t s) {
   info->n_det = h->n_det;
   std::vector<int> al(h->Nw);
   AFQ_CK(cudaMemcpyAsync(al.data(), h->alive, sizeof(int) * h->Nw, cudaMemcpyDeviceToHost, s));
+  int expired;
+  AFQ_CK(ask_tc(h, &expired, s));
   AFQ_CK(cudaStreamSynchronize(s));
   int n = 0;
   for (int a : al) n += a != 0;
   info->n_alive = n;
-  return check_tc(h);
+  return tc_status(h, expired);
 }
 
 afqmc_status afqmc_propagate(afqmc_handle h, int n_steps, const double* fields, cudaStream_t s) {
@@ -933,6 +938,8 @@ afqmc_status afqmc_energy(afqmc_handle h, double* e_local, double* e_mixed, doub
     AFQ_CK(afq::launch_mixed_sum(*h, h->esum, nullptr, 0, s));
     std::vector<double> es(4 * (size_t)h->R);
     AFQ_CK(cudaMemcpyAsync(es.data(), h->esum, sizeof(double) * es.size(), cudaMemcpyDeviceToHost, s));
+    int expired;
+    AFQ_CK(ask_tc(h, &expired, s));
     AFQ_CK(cudaStreamSynchronize(s));
     std::vector<double> em(h->R), ws(h->R);
     for (int r = 0; r < h->R; ++r) {
@@ -944,7 +951,7 @@ afqmc_status afqmc_energy(afqmc_handle h, double* e_local, double* e_mixed, doub
     if (e_mixed) AFQ_CK(cudaMemcpyAsync(e_mixed, em.data(), sizeof(double) * h->R, cudaMemcpyDefault, s));
     if (w_sum) AFQ_CK(cudaMemcpyAsync(w_sum, ws.data(), sizeof(double) * h->R, cudaMemcpyDefault, s));
     AFQ_CK(cudaStreamSynchronize(s));
-    return check_tc(h);
+    return tc_status(h, expired);
   } else if (e_local && !is_device_ptr(e_local)) {
     AFQ_CK(cudaStreamSynchronize(s));
   }
@@ -1183,6 +1190,8 @@ afqmc_status afqmc_energy_tangent(afqmc_handle h, double* de_local, double* e_mi
   AFQ_CK(afq::launch_mixed_sum_tan(*h, h->desum, s));
   std::vector<double> es(4 * (size_t)h->R);
   AFQ_CK(cudaMemcpyAsync(es.data(), h->desum, sizeof(double) * es.size(), cudaMemcpyDeviceToHost, s));
+  int expired;
+  AFQ_CK(ask_tc(h, &expired, s));
   AFQ_CK(cudaStreamSynchronize(s));
   std::vector<double> em(h->R), dm(h->R);
   for (int r = 0; r < h->R; ++r) {
@@ -1192,7 +1201,7 @@ afqmc_status afqmc_energy_tangent(afqmc_handle h, double* de_local, double* e_mi
   }
   if (e_mixed) AFQ_CK(cudaMemcpy(e_mixed, em.data(), sizeof(double) * h->R, cudaMemcpyDefault));
   if (de_mixed) AFQ_CK(cudaMemcpy(de_mixed, dm.data(), sizeof(double) * h->R, cudaMemcpyDefault));
-  return AFQMC_OK;
+  return tc_status(h, expired);
 }
 
 afqmc_status afqmc_get_tangent_state(afqmc_handle h, double* dlogw, cudaStream_t s) {
