@@ -385,13 +385,10 @@ def measure_kernels(afq, A, dA, nw, precision, workload, stream):
                                   "k_gemm_bf16x3_tc / k_gemm_bf16x3_tc_pair (force bias, split-BF16 tcgen05)",
                                   mma=3 * 2.0 * pad(X, 128) * pad(N * M, 64) * 2 * nw,
                                   traffic=tr("gemm_tc.cu", "force_bias_tc"))
-        # with the large-M tensor-core propagator the contraction covers only the
-        # lower-triangle 16 x 16 blocks of index pairs (two 128-row tiles each), when whole waves of
-        # 256 x 256 tiles by pairs of SMs beat those of 128 x 128 tiles over all M^2 rows
-        nb = (M + 15) // 16
-        tri_rows = nb * (nb + 1) // 2 * 256
-        pairs, singles = tri_rows // 256 * -(-2 * nw // 256), -(-M * M // 128) * -(-2 * nw // 128)
-        tri = pv == 4 and -(-pairs // 76) * 6 < -(-singles // 152) * 5
+        # with the large-M tensor-core propagator the contraction may cover only the lower-triangle
+        # 16 x 16 blocks of index pairs: the library's rule for this device
+        tri_rows = afq.afqmc_plan_value(afq.PLAN_VHS_TRI, M, X, nu, nd, nw)
+        tri = pv == 4 and tri_rows > 0
         vhs_rows = tri_rows if tri else pad(M * M, 128)
         out["vhs"] = entry(afq.K_VHS, STEPS_PER_BLOCK, vhs, "tensor", bf16,
                            "k_gemm_bf16x3_tc_pair (V_HS, split-BF16 tcgen05, "

@@ -469,15 +469,17 @@ afqmc_status afqmc_test_gemm(int impl, int Md, int Nd, int K, const double* A, c
 
 /*
  * afqmc_plan_value -- testing and reporting aid (no counterpart in the paper): a size or choice
- * that the library's rules give for an FP64 system of this shape (taylor_order 6), without a
- * handle and without device memory.  `arg` is unused unless stated.  -1: unknown `what` or bad shape.
+ * that the library's rules give for a system of this shape (FP64 unless stated, taylor_order 6),
+ * without a handle and without device memory.  `arg` is unused unless stated.  -1: unknown `what` or bad shape.
  */
 enum {
   AFQMC_PLAN_ENERGY_DIGITS = 0,     /* 1: local energies in digit form                          */
   AFQMC_PLAN_ENERGY_T = 1,          /* doubles for the half-rotated products of a walker chunk  */
   AFQMC_PLAN_TANGENT_T = 2,         /* of these, how many tangent mode fills                    */
   AFQMC_PLAN_EXCHANGE_SMEM = 3,     /* shared memory of the exchange sums (arg 1: tangent mode) */
-  AFQMC_PLAN_STEPS_SMALL = 4        /* 1: arg steps of a call run in the kernel for small systems */
+  AFQMC_PLAN_STEPS_SMALL = 4,       /* 1: arg steps of a call run in the kernel for small systems */
+  AFQMC_PLAN_VHS_TRI = 5            /* split precision, on the current device: rows of the V_HS contraction
+                                       over lower-triangle blocks, 0: it takes all M^2 rows       */
 };
 int64_t afqmc_plan_value(int what, int M, int X, int n_up, int n_dn, int n_walkers, int arg);
 

@@ -188,6 +188,13 @@ def afqmc_time_kernel(h, which, reps, stream=None):
     return ms.value
 
 
+PLAN_ENERGY_DIGITS, PLAN_ENERGY_T, PLAN_TANGENT_T, PLAN_EXCHANGE_SMEM, PLAN_STEPS_SMALL, PLAN_VHS_TRI = range(6)
+
+
+def afqmc_plan_value(what, M, X, n_up, n_dn, n_walkers, arg=0):
+    return _lib.load().afqmc_plan_value(what, M, X, n_up, n_dn, n_walkers, arg)
+
+
 def afqmc_reblock_error(series):
     s = np.ascontiguousarray(series, dtype=np.float64)
     return float(_lib.load().afqmc_reblock_error(_ptr(s), s.size))

@@ -1339,6 +1339,8 @@ int64_t afqmc_plan_value(int what, int M, int X, int n_up, int n_dn, int n_walke
     case AFQMC_PLAN_ENERGY_T: return afq::energy_chunk_doubles(c, false);
     case AFQMC_PLAN_TANGENT_T: return afq::energy_chunk_doubles(c, true);
     case AFQMC_PLAN_STEPS_SMALL: return afq::step_small_pays(c, arg);
+    case AFQMC_PLAN_VHS_TRI:
+      return afq::propagate_tcl_ok(c) && afq::vhs_tri_ok(M, 2 * n_walkers) ? afq::vhs_tri_rows(M) : 0;
     case AFQMC_PLAN_EXCHANGE_SMEM: return afq::exchange_smem(std::max(n_up, n_dn), arg != 0);
   }
   return -1;
