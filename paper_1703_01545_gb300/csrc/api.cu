@@ -90,7 +90,7 @@ void free_ctx(Ctx* h) {
   for (double* b : {h->Bneg, h->dexpK, h->htilP, h->dphi, h->dphi2, h->dtheta, h->drhobar, h->dU,
                     h->dAvhs, h->dlogO, h->dlogw, h->daux, h->deloc, h->desum})
     if (b) cudaFree(b);
-  for (float* b : {h->Avhs32, h->phi32, h->expK32, h->Ltil32, h->theta32, h->LtT, h->psi32h, h->psi32l,
+  for (float* b : {h->Avhs32, h->phi32, h->expK32, h->Ltil32, h->theta32, h->LtT, h->psi32,
                    h->rhobar32, h->rho_mf32})
     if (b) cudaFree(b);
   if (h->d_tc_err) cudaFree(h->d_tc_err);
@@ -158,8 +158,7 @@ afqmc_status setup_mixed(Ctx* h, cudaStream_t s) {
   if ((st = dalloc(h, &h->d_tc_err, 1)) != AFQMC_OK) return st;
   if ((st = dalloc(h, &h->theta32, 2 * (size_t)Nw * NM)) != AFQMC_OK) return st;
   if ((st = dalloc(h, &h->LtT, (size_t)afq::LtT_size(*h))) != AFQMC_OK) return st;
-  if ((st = dalloc(h, &h->psi32h, (size_t)NM)) != AFQMC_OK) return st;
-  if ((st = dalloc(h, &h->psi32l, (size_t)NM)) != AFQMC_OK) return st;
+  if ((st = dalloc(h, &h->psi32, (size_t)NM)) != AFQMC_OK) return st;
   if ((st = dalloc(h, &h->ovdet, 8 * (size_t)Nw)) != AFQMC_OK) return st;
   if ((st = dalloc(h, &h->rhobar32, 2 * (size_t)Nw * X)) != AFQMC_OK) return st;
   if ((st = dalloc(h, &h->rho_mf32, (size_t)X)) != AFQMC_OK) return st;
@@ -205,7 +204,7 @@ afqmc_status setup_mixed(Ctx* h, cudaStream_t s) {
   if (e == cudaSuccess) e = afq::to_float(h->expK, h->expK32, MM, s);
   if (e == cudaSuccess) e = afq::to_float(h->Ltil, h->Ltil32, (int64_t)X * NM, s);
   if (e == cudaSuccess) e = afq::build_LtT(*h, h->LtT, s);
-  if (e == cudaSuccess) e = afq::split_f32(h->psi, h->psi32h, h->psi32l, NM, s);
+  if (e == cudaSuccess) e = afq::to_float(h->psi, h->psi32, NM, s);
   if (e == cudaSuccess) e = afq::to_float(h->rho_mf, h->rho_mf32, X, s);
   if (e == cudaSuccess && afq::propagate_tc_ok(*h)) {
     if (dalloc(h, &h->emI_pk, 64 * 64) != AFQMC_OK) return AFQMC_ERR_NOMEM;

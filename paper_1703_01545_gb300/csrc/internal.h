@@ -126,7 +126,7 @@ struct Ctx {
   float* Ltil32 = nullptr;    // [X][N][M]
   float* theta32 = nullptr;   // [2][Nw][N][M]  Theta in FP32 (split-precision mode)
   float* LtT = nullptr;       // [X][M][NPT]    Psi_s^T L_g transposed, spin-padded (FP32)
-  float *psi32h = nullptr, *psi32l = nullptr;   // [N][M]  psi = psi32h + psi32l (FP32 pair)
+  float* psi32 = nullptr;     // [N][M]  psi in FP32
   double* ovdet = nullptr;    // [Nw][8]  per-walker determinant factors between the overlap kernels
   uint32_t* emI_pk = nullptr; // [64][64] e^{-dt K/2} - I as split-bf16 words (tensor-core propagator)
   // large-M tensor-core propagator (propagate_tcl.cu): V_HS as split bf16 [2][Nw][M][Mp] (written
@@ -303,7 +303,6 @@ cudaError_t launch_taylor_f32(const Ctx& c, float* phi32, const float* A32, cuda
 cudaError_t launch_energy_f32(const Ctx& c, const float* Ltil32, cudaStream_t s, int n_walkers = -1);
 cudaError_t to_float(const double* in, float* out, int64_t n, cudaStream_t s);
 // hi = fl32(in), lo = fl32(in - hi)
-cudaError_t split_f32(const double* in, float* hi, float* lo, int64_t n, cudaStream_t s);
 cudaError_t prepare_mixed_kernels2(const Ctx& c);
 cudaError_t build_LtT(const Ctx& c, float* LtT, cudaStream_t s);
 int64_t LtT_size(const Ctx& c);

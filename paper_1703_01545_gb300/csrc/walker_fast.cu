@@ -1,8 +1,9 @@
-// Latency-oriented FP64 walker kernels for the split-precision step: overlap / LU / weight
-// update and modified Gram-Schmidt with the small dense linear algebra (N_s <= 16) in one
-// warp, synchronised with __syncwarp only.  Overlaps (FP64, or FP32 pairs when Phi is
-// FP32-exact), determinants, ratios, weights and Gram-Schmidt are FP64; Theta = Phi O^{-1}
-// is formed in FP32.  Also the fields kernel of the split-precision step.
+// Latency-oriented walker kernels: overlap / LU / weight update and orthonormalisation with the small dense
+// linear algebra (N_s <= 16) in one warp, synchronised with __syncwarp only.  The split-precision step's
+// update (k_overlap_fast with an FP32 walker) sums, factorises and solves in FP32; its refresh sums and
+// factorises in FP64 and solves in FP32; FP64 handles' form (k_overlap64) is FP64 throughout.  Log
+// determinants, ratios and weights are FP64 in all of them.  Also Gram-Schmidt (FP64), the Cholesky QR (FP32)
+// and the fields kernel of the split-precision step.
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
@@ -32,10 +33,8 @@ __device__ __forceinline__ void cp_async4(uint32_t dst, const void* src) {
 
 struct FastOvArgs {
   const double* src;  // [2][Nw][N][M]  (propagated walkers in update mode)
-  const float* src32; // the same in FP32 (update mode, may be null): no conversions needed,
-                      // and the overlap is summed in double-float FP32 arithmetic
-  const float* psih;  // psi = psih + psil (FP32 pair, [N][M])
-  const float* psil;
+  const float* src32; // the same in FP32 (update mode, may be null): overlap, LU and solves in FP32
+  const float* psih;  // psi in FP32, [N][M]
   double* phi;
   float* theta32;
   __nv_bfloat16* op_hi;
@@ -1104,9 +1103,9 @@ cudaError_t launch_overlap_fast(const Ctx& c, const double* src, int mode, cudaS
                                 const float* src32, bool with_weights) {
   FastOvArgs a{};
   a.src = src;
-  a.src32 = c.psi32h ? src32 : nullptr;
-  a.psih = c.psi32h;
-  a.psil = c.psi32l; a.phi = c.phi; a.theta32 = c.theta32;
+  a.src32 = c.psi32 ? src32 : nullptr;
+  a.psih = c.psi32;
+  a.phi = c.phi; a.theta32 = c.theta32;
   a.op_hi = c.tc_Theta->hi; a.op_lo = c.tc_Theta->lo; a.Kp = c.tc_Theta->Kp;
   a.psi = c.psi; a.logO = c.logO; a.w = c.w; a.alive = c.alive; a.aux = c.aux; a.flags = c.d_flags;
   a.det = c.ovdet;
