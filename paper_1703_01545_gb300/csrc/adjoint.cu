@@ -292,7 +292,7 @@ afqmc_status adjoint_body(Ctx* h, Arena& ar, int n_steps, const double* fields, 
   ADJ_CK(cudaMemcpyAsync(&E, e_acc, sizeof(double), cudaMemcpyDeviceToHost, s));
   if (dE_dh1) ADJ_CK(cudaMemcpyAsync(dE_dh1, h1bar, sizeof(double) * MM, cudaMemcpyDefault, s));
   int expired = 0;
-  if (ws.err) ADJ_CK(cudaMemcpyAsync(&expired, ws.err, sizeof(int), cudaMemcpyDeviceToHost, s));
+  if (ws.err) ADJ_CK(cudaMemcpyAsync(&expired, ws.err, sizeof(int), cudaMemcpyDefault, s));
   ADJ_CK(cudaStreamSynchronize(s));
   if (expired) return fail(h, AFQMC_ERR_TIMEOUT, "a tensor-core kernel's bounded wait expired");
   if (e_mixed) *e_mixed = E;

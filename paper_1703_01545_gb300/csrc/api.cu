@@ -45,6 +45,18 @@ afqmc_status dalloc(Ctx* h, T** p, size_t count) {
   return AFQMC_OK;
 }
 
+// A flag that kernels set and the host reads after a synchronisation: host memory that the device writes, so
+// that a call pays no copy for it.
+int* alloc_flag() {
+  int* p = nullptr;
+  if (cudaHostAlloc(&p, sizeof(int), cudaHostAllocDefault) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  *p = 0;
+  return p;
+}
+
 bool is_device_ptr(const void* p) {
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
@@ -93,7 +105,7 @@ void free_ctx(Ctx* h) {
   for (float* b : {h->Avhs32, h->phi32, h->expK32, h->Ltil32, h->theta32, h->LtT, h->psi32,
                    h->rhobar32, h->rho_mf32})
     if (b) cudaFree(b);
-  if (h->d_tc_err) cudaFree(h->d_tc_err);
+  if (h->tc_err) cudaFreeHost(h->tc_err);
   if (h->ws64.buf) cudaFree(h->ws64.buf);
   if (h->e64) cudaFree(h->e64);
   if (h->ov_O) cudaFree(h->ov_O);
@@ -155,14 +167,13 @@ afqmc_status setup_mixed(Ctx* h, cudaStream_t s) {
   if ((st = dalloc(h, &h->phi32, 2 * (size_t)Nw * NM)) != AFQMC_OK) return st;
   if ((st = dalloc(h, &h->expK32, (size_t)MM)) != AFQMC_OK) return st;
   if ((st = dalloc(h, &h->Ltil32, (size_t)X * NM)) != AFQMC_OK) return st;
-  if ((st = dalloc(h, &h->d_tc_err, 1)) != AFQMC_OK) return st;
+  if (!(h->tc_err = alloc_flag())) return set_err(h, AFQMC_ERR_NOMEM, "cannot allocate page-locked memory");
   if ((st = dalloc(h, &h->theta32, 2 * (size_t)Nw * NM)) != AFQMC_OK) return st;
   if ((st = dalloc(h, &h->LtT, (size_t)afq::LtT_size(*h))) != AFQMC_OK) return st;
   if ((st = dalloc(h, &h->psi32, (size_t)NM)) != AFQMC_OK) return st;
   if ((st = dalloc(h, &h->ovdet, 8 * (size_t)Nw)) != AFQMC_OK) return st;
   if ((st = dalloc(h, &h->rhobar32, 2 * (size_t)Nw * X)) != AFQMC_OK) return st;
   if ((st = dalloc(h, &h->rho_mf32, (size_t)X)) != AFQMC_OK) return st;
-  AFQ_CK(cudaMemsetAsync(h->d_tc_err, 0, sizeof(int), s));
   if (afq::fast_walker_kernels_ok(*h) && afq::refresh_f64e_ok(*h)) {
     // without the memory the refresh sums run in its kernel
     const size_t nu = h->n_up, nd = N - h->n_up, need = afq::refresh_f64e_ws(*h);
@@ -171,7 +182,7 @@ afqmc_status setup_mixed(Ctx* h, cudaStream_t s) {
       h->ws64.buf = nullptr;
     } else {
       h->ws64.bytes = need;
-      h->ws64.err = h->d_tc_err;
+      h->ws64.err = h->tc_err;
       if (cudaMalloc(&h->ov_O, sizeof(double) * 2 * Nw * (nu * nu + nd * nd)) != cudaSuccess) h->ov_O = nullptr;
     }
     cudaGetLastError();
@@ -274,7 +285,7 @@ afqmc_status step_launch_mixed(Ctx* h, const double* fields_t, cudaStream_t s) {
   if (h->opt.mode == AFQMC_PHASELESS) {
     // the Theta operand was written by the last overlap kernel
     AFQ_CK(afq::gemm_bf16x3(*h->tc_Ltil, *h->tc_Theta, X, 2 * Nw, 1.0f, h->rhobar32, X,
-                            h->d_tc_err, s));
+                            h->tc_err, s));
   }
   AFQ_CK(afq::launch_fields_mixed(*h, fields_t, s));
   const int pv = afq::propagation_variant(*h);
@@ -304,13 +315,10 @@ afqmc_status energy_launch(Ctx* h, cudaStream_t s) {
   return AFQMC_OK;
 }
 
-// The flag of expired waits, read on the stream: ask_tc before the caller's synchronisation, tc_status after.
-cudaError_t ask_tc(const Ctx* h, int* flag, cudaStream_t s) {
-  *flag = 0;
-  return h->d_tc_err ? cudaMemcpyAsync(flag, h->d_tc_err, sizeof(int), cudaMemcpyDeviceToHost, s) : cudaSuccess;
-}
-afqmc_status tc_status(Ctx* h, int flag) {
-  return flag ? set_err(h, AFQMC_ERR_TIMEOUT, "a tensor-core kernel's bounded wait expired") : AFQMC_OK;
+// After a synchronisation: report an expired tensor-core wait.
+afqmc_status check_tc(Ctx* h) {
+  if (!h->tc_err || !*static_cast<volatile int*>(h->tc_err)) return AFQMC_OK;
+  return set_err(h, AFQMC_ERR_TIMEOUT, "a tensor-core kernel's bounded wait expired");
 }
 
 afqmc_status step_launch_mixed(Ctx* h, const double* fields_t, cudaStream_t s);
@@ -455,8 +463,7 @@ afqmc_status run_step(Ctx* h, const double* fields_t, cudaStream_t s) { return s
 afqmc_status plain_step(Ctx* h, const double* fields_t, cudaStream_t s) { return steps_launch(h, 1, fields_t, s); }
 afqmc_status pair_ortho(Ctx* h, cudaStream_t s) { return ortho_launch(h, s); }
 afqmc_status pair_energy(Ctx* h, cudaStream_t s) { return energy_launch(h, s); }
-cudaError_t pair_ask_tc(const Ctx* h, int* flag, cudaStream_t s) { return ask_tc(h, flag, s); }
-afqmc_status pair_tc_status(Ctx* h, int flag) { return tc_status(h, flag); }
+afqmc_status pair_check(Ctx* h) { return check_tc(h); }
 }  // namespace afq
 
 extern "C" {
@@ -594,11 +601,7 @@ afqmc_status afqmc_setup(afqmc_handle* out, const double* h1_in, const double* L
     if (tay) need = std::max(need, afq::taylor_f64e_ws(M, N, (int)Nw));
     if (need > 0) {
       AFQ_SCK(afq::prepare_gemm_f64e());
-      int* err = nullptr;
-      if (cudaMalloc(&err, sizeof(int)) == cudaSuccess) {
-        h->d_tc_err = err;
-        h->ws64.err = err;
-        AFQ_SCK(cudaMemsetAsync(err, 0, sizeof(int), s));
+      if ((h->ws64.err = h->tc_err = alloc_flag())) {
         if (cudaMalloc(&h->ws64.buf, need) == cudaSuccess) h->ws64.bytes = need;
         else h->ws64.buf = nullptr;
         h->taylor_dig = tay && h->ws64.buf;
@@ -869,10 +872,8 @@ afqmc_status afqmc_get_state(afqmc_handle h, double* phi, double* logO, double* 
   if (logO) AFQ_CK(cudaMemcpyAsync(logO, h->logO, sizeof(double) * 2 * h->Nw, cudaMemcpyDefault, s));
   if (w) AFQ_CK(cudaMemcpyAsync(w, h->w, sizeof(double) * 2 * h->Nw, cudaMemcpyDefault, s));
   if (alive) AFQ_CK(cudaMemcpyAsync(alive, h->alive, sizeof(int) * h->Nw, cudaMemcpyDefault, s));
-  int expired;
-  AFQ_CK(ask_tc(h, &expired, s));
   AFQ_CK(cudaStreamSynchronize(s));
-  return tc_status(h, expired);
+  return check_tc(h);
 }
 
 afqmc_status afqmc_get_info(afqmc_handle h, afqmc_info* info, cudaStream_t s) {
@@ -886,13 +887,11 @@ afqmc_status afqmc_get_info(afqmc_handle h, afqmc_info* info, cudaStream_t s) {
   info->n_det = h->n_det;
   std::vector<int> al(h->Nw);
   AFQ_CK(cudaMemcpyAsync(al.data(), h->alive, sizeof(int) * h->Nw, cudaMemcpyDeviceToHost, s));
-  int expired;
-  AFQ_CK(ask_tc(h, &expired, s));
   AFQ_CK(cudaStreamSynchronize(s));
   int n = 0;
   for (int a : al) n += a != 0;
   info->n_alive = n;
-  return tc_status(h, expired);
+  return check_tc(h);
 }
 
 afqmc_status afqmc_propagate(afqmc_handle h, int n_steps, const double* fields, cudaStream_t s) {
@@ -937,8 +936,6 @@ afqmc_status afqmc_energy(afqmc_handle h, double* e_local, double* e_mixed, doub
     AFQ_CK(afq::launch_mixed_sum(*h, h->esum, nullptr, 0, s));
     std::vector<double> es(4 * (size_t)h->R);
     AFQ_CK(cudaMemcpyAsync(es.data(), h->esum, sizeof(double) * es.size(), cudaMemcpyDeviceToHost, s));
-    int expired;
-    AFQ_CK(ask_tc(h, &expired, s));
     AFQ_CK(cudaStreamSynchronize(s));
     std::vector<double> em(h->R), ws(h->R);
     for (int r = 0; r < h->R; ++r) {
@@ -950,7 +947,7 @@ afqmc_status afqmc_energy(afqmc_handle h, double* e_local, double* e_mixed, doub
     if (e_mixed) AFQ_CK(cudaMemcpyAsync(e_mixed, em.data(), sizeof(double) * h->R, cudaMemcpyDefault, s));
     if (w_sum) AFQ_CK(cudaMemcpyAsync(w_sum, ws.data(), sizeof(double) * h->R, cudaMemcpyDefault, s));
     AFQ_CK(cudaStreamSynchronize(s));
-    return tc_status(h, expired);
+    return check_tc(h);
   } else if (e_local && !is_device_ptr(e_local)) {
     AFQ_CK(cudaStreamSynchronize(s));
   }
@@ -983,7 +980,7 @@ afqmc_status afqmc_time_kernel(afqmc_handle h, int which, int reps, double* ms, 
         if (h->n_det > 0) return afq::md_force_bias(*h, s);
         if (h->tc_Ltil)
           return afq::gemm_bf16x3(*h->tc_Ltil, *h->tc_Theta, X, 2 * Nw, 1.0f, h->rhobar32, X,
-                                  h->d_tc_err, s);
+                                  h->tc_err, s);
         return afq::gemm_tn_f64(X, 2 * Nw, (int)NM, 1.0, h->Ltil, NM, 0, h->theta, NM, 0, 0.0,
                                 h->rhobar, X, 0, 1, s, afq::GEMM_FORCE_BIAS, &h->ws64);
       case AFQMC_K_OVERLAP_UPDATE:   // Phi <- Phi (unchanged), Theta from the FP32 walkers
@@ -1189,8 +1186,6 @@ afqmc_status afqmc_energy_tangent(afqmc_handle h, double* de_local, double* e_mi
   AFQ_CK(afq::launch_mixed_sum_tan(*h, h->desum, s));
   std::vector<double> es(4 * (size_t)h->R);
   AFQ_CK(cudaMemcpyAsync(es.data(), h->desum, sizeof(double) * es.size(), cudaMemcpyDeviceToHost, s));
-  int expired;
-  AFQ_CK(ask_tc(h, &expired, s));
   AFQ_CK(cudaStreamSynchronize(s));
   std::vector<double> em(h->R), dm(h->R);
   for (int r = 0; r < h->R; ++r) {
@@ -1200,7 +1195,7 @@ afqmc_status afqmc_energy_tangent(afqmc_handle h, double* de_local, double* e_mi
   }
   if (e_mixed) AFQ_CK(cudaMemcpy(e_mixed, em.data(), sizeof(double) * h->R, cudaMemcpyDefault));
   if (de_mixed) AFQ_CK(cudaMemcpy(de_mixed, dm.data(), sizeof(double) * h->R, cudaMemcpyDefault));
-  return tc_status(h, expired);
+  return check_tc(h);
 }
 
 afqmc_status afqmc_get_tangent_state(afqmc_handle h, double* dlogw, cudaStream_t s) {
@@ -1253,8 +1248,9 @@ afqmc_status afqmc_test_gemm(int impl, int Md, int Nd, int K, const double* A, c
   const int Kp = afq::pad64(K);
   auto cleanup = [&]() {
     for (void* p : {(void*)dA, (void*)dB, (void*)dC, (void*)fC, (void*)ah, (void*)al, (void*)bh,
-                    (void*)bl, (void*)err, wbuf})
+                    (void*)bl, wbuf})
       if (p) cudaFree(p);
+    if (err) cudaFreeHost(err);
   };
   afqmc_status st = AFQMC_OK;
   cudaError_t e = cudaSuccess;
@@ -1262,8 +1258,7 @@ afqmc_status afqmc_test_gemm(int impl, int Md, int Nd, int K, const double* A, c
     if ((e = cudaMalloc(&dA, sizeof(double) * Md * (size_t)K)) != cudaSuccess) break;
     if ((e = cudaMalloc(&dB, sizeof(double) * Nd * (size_t)K)) != cudaSuccess) break;
     if ((e = cudaMalloc(&dC, sizeof(double) * Md * (size_t)Nd)) != cudaSuccess) break;
-    if ((e = cudaMalloc(&err, sizeof(int))) != cudaSuccess) break;
-    if ((e = cudaMemsetAsync(err, 0, sizeof(int), s)) != cudaSuccess) break;
+    if (!(err = alloc_flag())) { e = cudaErrorMemoryAllocation; break; }
     if ((e = cudaMemcpyAsync(dA, A, sizeof(double) * Md * (size_t)K, cudaMemcpyDefault, s)) != cudaSuccess) break;
     if ((e = cudaMemcpyAsync(dB, B, sizeof(double) * Nd * (size_t)K, cudaMemcpyDefault, s)) != cudaSuccess) break;
     if (impl == 0) {
@@ -1276,10 +1271,8 @@ afqmc_status afqmc_test_gemm(int impl, int Md, int Nd, int K, const double* A, c
         ws.buf = static_cast<uint8_t*>(wbuf);
       }
       if ((e = afq::gemm_tn_f64(Md, Nd, K, alpha, dA, K, 0, dB, K, 0, 0.0, dC, Md, 0, 1, s, afq::GEMM_GENERIC, &ws)) != cudaSuccess) break;
-      int herr = 0;
-      if ((e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess) break;
       if ((e = cudaStreamSynchronize(s)) != cudaSuccess) break;
-      if (herr) { st = AFQMC_ERR_TIMEOUT; break; }
+      if (*static_cast<volatile int*>(err)) { st = AFQMC_ERR_TIMEOUT; break; }
     } else {
       if ((e = afq::prepare_tc_kernels()) != cudaSuccess) break;
       const int Mp = afq::tc_pad_rows(Md), Np = afq::tc_pad_rows(Nd);
@@ -1307,10 +1300,8 @@ afqmc_status afqmc_test_gemm(int impl, int Md, int Nd, int K, const double* A, c
       }
       std::vector<float> hf((size_t)Md * Nd);
       if ((e = cudaMemcpyAsync(hf.data(), fC, sizeof(float) * hf.size(), cudaMemcpyDeviceToHost, s)) != cudaSuccess) break;
-      int herr = 0;
-      if ((e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess) break;
       if ((e = cudaStreamSynchronize(s)) != cudaSuccess) break;
-      if (herr) { st = AFQMC_ERR_TIMEOUT; break; }
+      if (*static_cast<volatile int*>(err)) { st = AFQMC_ERR_TIMEOUT; break; }
       std::vector<double> hd(hf.begin(), hf.end());
       if ((e = cudaMemcpy(C, hd.data(), sizeof(double) * hd.size(), cudaMemcpyDefault)) != cudaSuccess) break;
       break;

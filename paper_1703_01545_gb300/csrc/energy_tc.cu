@@ -962,12 +962,12 @@ cudaError_t launch_spin(const Ctx& c, const EnergyTc& et, int n_walkers, cudaStr
     const int grid = std::min(2 * CTs * NG, 152);
     k_energy_tc_spin2<16><<<grid, EPTHREADS, ES2Layout<16>::SMEM_BYTES, s>>>(
         et.A->map_hi, et.A->map_lo, et.B->map_hi, et.B->map_lo, RTs, CTs, rg, NG, et.part, et.NwP,
-        c.d_tc_err, kEWaitNs, reinterpret_cast<float2*>(et.trs), c.X, c.Nw);
+        c.tc_err, kEWaitNs, reinterpret_cast<float2*>(et.trs), c.X, c.Nw);
   } else {
     const int grid = std::min(2 * RTs * CTs, 152);
     k_energy_tc<NPS, true><<<grid, EPTHREADS, Lay::SMEM_BYTES, s>>>(
         et.A->map_hi, et.A->map_lo, et.B->map_hi, et.B->map_lo, et.Kp / EBK, RTs, CTs, et.part,
-        et.NwP, c.d_tc_err, kEWaitNs, reinterpret_cast<float2*>(et.trs), c.X, c.Nw);
+        et.NwP, c.tc_err, kEWaitNs, reinterpret_cast<float2*>(et.trs), c.X, c.Nw);
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_energy_tc_reduce<<<(nw + 7) / 8, 256, 0, s>>>(et.part, nparts, et.NwP, c.theta32, et.hh, et.hl, c.eloc,
@@ -994,12 +994,12 @@ cudaError_t launch_np(const Ctx& c, const EnergyTc& et, int n_walkers, cudaStrea
     const int grid = std::min(ct * nparts, 152);
     k_energy_tc_bres<NP><<<grid, EBLayout<NP>::THREADS, EBLayout<NP>::SMEM_BYTES, s>>>(
         et.A->map_hi, et.A->map_lo, et.B->map_hi, et.B->map_lo, et.RT, ct, rg, nparts, et.part, et.NwP,
-        c.d_tc_err, kEWaitNs);
+        c.tc_err, kEWaitNs);
   } else {
     const int grid = std::min(et.RT * ct, 152);
     k_energy_tc<NP, false><<<grid, EPTHREADS, Lay::SMEM_BYTES, s>>>(
         et.A->map_hi, et.A->map_lo, et.B->map_hi, et.B->map_lo, et.Kp / EBK, et.RT, ct, et.part,
-        et.NwP, c.d_tc_err, kEWaitNs, nullptr, c.X, c.Nw);
+        et.NwP, c.tc_err, kEWaitNs, nullptr, c.X, c.Nw);
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_energy_tc_reduce<<<(nw + 7) / 8, 256, 0, s>>>(et.part, nparts, et.NwP, c.theta32, et.hh, et.hl, c.eloc,

@@ -136,7 +136,7 @@ struct Ctx {
   CUtensorMap* tcl_maps = nullptr;
   float* rhobar32 = nullptr;  // [2][Nw][X]  force bias of the split-precision step (FP32 GEMM output)
   float* rho_mf32 = nullptr;  // [X]         <rho_g>_T in FP32
-  int* d_tc_err = nullptr;    // set by a tensor-core kernel whose bounded wait expired
+  int* tc_err = nullptr;      // page-locked host memory, set by a tensor-core kernel whose bounded wait expired
   EnergyTc* etc = nullptr;    // tensor-core local energy (null when the shape is unsupported)
   // autotuned variants (autotune.cpp); -1 = not tuned, use the default
   int tune_energy_wb = -1;    // local energy: 0 tensor cores, else walkers per CTA of the FP32 kernel (2, 4, 8)

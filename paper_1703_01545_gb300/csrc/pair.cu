@@ -18,8 +18,7 @@ namespace afq {
 afqmc_status pair_steps(Ctx* h, int n, cudaStream_t s);
 afqmc_status pair_ortho(Ctx* h, cudaStream_t s);
 afqmc_status pair_energy(Ctx* h, cudaStream_t s);
-cudaError_t pair_ask_tc(const Ctx* h, int* flag, cudaStream_t s);
-afqmc_status pair_tc_status(Ctx* h, int flag);
+afqmc_status pair_check(Ctx* h);
 cudaError_t launch_meas_advance(int* meas, cudaStream_t s);
 }  // namespace afq
 
@@ -269,9 +268,6 @@ extern "C" afqmc_status afqmc_pair_delta_E(afqmc_handle A, afqmc_handle B, int n
     AFQ_PCK(cudaMemcpyAsync(ser.data(), r->series, sizeof(double) * ser.size(), cudaMemcpyDeviceToHost, cs));
   AFQ_PCK(cudaMemcpyAsync(alA.data(), A->alive, sizeof(int) * A->Nw, cudaMemcpyDeviceToHost, cs));
   AFQ_PCK(cudaMemcpyAsync(alB.data(), B->alive, sizeof(int) * B->Nw, cudaMemcpyDeviceToHost, cs));
-  int expired[2];
-  AFQ_PCK(afq::pair_ask_tc(A, &expired[0], cs));
-  AFQ_PCK(afq::pair_ask_tc(B, &expired[1], cs));
   if (n_meas > 0) {
     AFQ_PCK(cudaEventRecord(r->done, cs));
     AFQ_PCK(cudaStreamWaitEvent(s, r->done, 0));   // the caller's stream sees the whole run
@@ -298,8 +294,8 @@ extern "C" afqmc_status afqmc_pair_delta_E(afqmc_handle A, afqmc_handle B, int n
   if (dE_sigma) AFQ_PCK(cudaMemcpy(dE_sigma, &est[1], sizeof(double), cudaMemcpyDefault));
   if (tau_at_min) AFQ_PCK(cudaMemcpy(tau_at_min, &est[2], sizeof(double), cudaMemcpyDefault));
 #undef AFQ_PCK
-  afqmc_status tcs = afq::pair_tc_status(A, expired[0]);
-  if (tcs == AFQMC_OK) tcs = afq::pair_tc_status(B, expired[1]);
+  afqmc_status tcs = afq::pair_check(A);
+  if (tcs == AFQMC_OK) tcs = afq::pair_check(B);
   if (tcs != AFQMC_OK) return tcs;
   int na = 0, nb = 0;
   for (int a : alA) na += a != 0;

@@ -309,7 +309,7 @@ cudaError_t launch_propagate_tc(const Ctx& c, double* out, float* out32, cudaStr
   if (!c.emI_pk) return cudaErrorInvalidValue;
   return launch_after(k_propagate_tc, grid, 128, PLayout::SMEM_BYTES, s, c.phi, c.Avhs32, c.emI_pk, out, out32,
                                                         out == c.phi ? c.alive : nullptr, c.M, c.N,
-                                                        c.Nw, c.opt.taylor_order, c.d_tc_err, kPWaitNs);
+                                                        c.Nw, c.opt.taylor_order, c.tc_err, kPWaitNs);
 }
 
 }  // namespace afq

@@ -960,7 +960,7 @@ cudaError_t launch_propagate_tcl(const Ctx& c, double* out, float* out32, cudaSt
   const int* al = out == c.phi ? c.alive : nullptr;
   auto go = [&](GroupsKernel k, int grid, int threads) {
     return launch_after(k, std::min(c.Nw, grid), threads, (size_t)sh.smem_bytes, s, c.tcl_maps[0], c.tcl_maps[1],
-                        c.tcl_maps[2], c.tcl_maps[3], sh, c.phi, out, out32, al, c.d_tc_err, kWaitNs);
+                        c.tcl_maps[2], c.tcl_maps[3], sh, c.phi, out, out32, al, c.tc_err, kWaitNs);
   };
   if (sh.G == 2) return go(groups_kernel((c.M + 15) / 16, sh.Np), 152, 64 + 32 * 16);
   return two_per_sm(sh) ? go(k_propagate_tcl<4, 1, 0, 0>, 2 * 152, 64 + 32 * 4)
