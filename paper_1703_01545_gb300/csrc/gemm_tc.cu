@@ -165,6 +165,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                                              ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Lay::BAR_OFFSET);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 1);
+  volatile int* s_fail = reinterpret_cast<volatile int*>(tmem_slot + 1);   // a wait for operands expired
   const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + STAGES),
                  done = smem_u32(bars + 2 * STAGES);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -176,6 +177,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       mbar_init(empty0 + 8 * s, 1);
     }
     mbar_init(done, 1);
+    *s_fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -213,7 +215,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     const uint32_t idesc = idesc_bf16<BN>();
     for (int kb = 0; kb < nkb; ++kb) {
       const int s = kb % STAGES, use = kb / STAGES;
-      if (!mbar_wait(full0 + 8 * s, use & 1, err, wait_ns)) break;
+      if (!mbar_wait(full0 + 8 * s, use & 1, err, wait_ns)) {
+        *s_fail = 1;
+        __threadfence_block();
+        break;
+      }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t st = smem_u32(smem + s * Lay::STAGE_BYTES);
       const uint64_t ah = sw128_desc(st), al = sw128_desc(st + Lay::A_BYTES);
@@ -237,7 +243,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   __syncwarp();
   const int m = m0 + warp * 32 + lane;
-  if (__all_sync(0xffffffffu, ok && *(volatile int*)err == 0)) {
+  if (__all_sync(0xffffffffu, ok && *s_fail == 0)) {
     for (int c0 = 0; c0 < BN; c0 += 32) {
       uint32_t v[32];
       tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
