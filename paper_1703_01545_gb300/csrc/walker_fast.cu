@@ -136,8 +136,10 @@ __device__ __forceinline__ void overlap_sums(const float* __restrict__ psih, con
 // read one float at a time.  1024 walkers: 115 -> 88 us; 4096 beside the other system's kernels 373 -> 304 us.
 // NSM: the larger spin block is at most 8 (both blocks factorised by warp 0, 16 lanes each) or
 // 16 (one warp per block, ROWS = ceil(ns / (32 / ns)) rows per lane, 4 or 8).
-template <int ROWS, int NSM>
-__global__ void __launch_bounds__(256) k_overlap_fast(FastOvArgs a) {
+// SUMS: how the FP32 update sums the overlaps, and the registers a thread may take (rules at overlap_form).
+enum OverlapSums { kEntries, kTiles, kTilesWide };
+template <int ROWS, int NSM, int SUMS>
+__global__ void __launch_bounds__(256, SUMS == kTilesWide ? 1 : NSM == 8 ? 5 : 4) k_overlap_fast(FastOvArgs a) {
   after_previous();
   extern __shared__ double smo[];
   const int wk = blockIdx.x, tid = threadIdx.x, M = a.M, N = a.N, NM = N * M;
@@ -229,39 +231,63 @@ __global__ void __launch_bounds__(256) k_overlap_fast(FastOvArgs a) {
       ar[r * LDA + c] = o[(int64_t)wk * ns];
       ar[PLN + r * LDA + c] = o[((int64_t)a.Nw + wk) * ns];
     }
-  if (f32) {
-    // phi is FP32 here (the propagator's FP32 output): FP32 products of psi (rounded to FP32) and phi,
-    // summed in FP32 (~2^-24 relative to sum |terms| per part; the log determinant then carries ~1e-6 of
-    // rounding, far below the step's other FP32 and split-BF16 errors)
+  // FP32 update: phi is FP32 (the propagator's FP32 output), so FP32 products of psi (rounded to FP32) and phi,
+  // summed in FP32 (~2^-24 relative to sum |terms| per part; the log determinant then carries ~1e-6 of
+  // rounding, far below the step's other FP32 and split-BF16 errors)
+  if (SUMS != kEntries && f32) {
     if ((warp >> 1 ? nd : nu) > 0) overlap_sums<NSM / 4>(a.psih, pfr, pfi, invf, M, MP, nu, nd, warp, lane);
   } else
   for (int base = 0; base < (a.O ? 0 : nn * 4); base += blockDim.x) {
     const int q = base + tid, ent = q >> 2, part = q & 3;
     double re = 0.0, im = 0.0;
+    float sr = 0.f, cr = 0.f, si = 0.f, ci = 0.f;   // FP32 pairs
     int sp = 0, r = 0, c = 0;
     if (ent < nn) {
       if (ent < nu * nu) { r = ent / nu; c = ent % nu; }
       else { sp = 1; const int e2 = ent - nu * nu; r = e2 / nd; c = e2 % nd; }
       const int n0 = sp ? nu : 0;
-      const double* ps = a.psi + (int64_t)(n0 + r) * M;
-      const double* fr = pr + (n0 + c) * MP;
-      const double* fi = pi + (n0 + c) * MP;
-      for (int i = part; i < M; i += 4) {
-        const double p = __ldg(ps + i);
-        re = fma(p, fr[i], re);
-        im = fma(p, fi[i], im);
+      if (f32) {
+        const float* hs = a.psih + (int64_t)(n0 + r) * M;
+        const float* xr = pfr + (n0 + c) * MP;
+        const float* xi = pfi + (n0 + c) * MP;
+        for (int i = part; i < M; i += 4) {
+          const float h = __ldg(hs + i);
+          sr = fmaf(h, xr[i], sr);
+          si = fmaf(h, xi[i], si);
+        }
+      } else {
+        const double* ps = a.psi + (int64_t)(n0 + r) * M;
+        const double* fr = pr + (n0 + c) * MP;
+        const double* fi = pi + (n0 + c) * MP;
+        for (int i = part; i < M; i += 4) {
+          const double p = __ldg(ps + i);
+          re = fma(p, fr[i], re);
+          im = fma(p, fi[i], im);
+        }
       }
     }
-    // combine the 4 partial sums of each entry (every lane takes part in the shuffles)
-    re += __shfl_xor_sync(0xffffffffu, re, 1);
-    im += __shfl_xor_sync(0xffffffffu, im, 1);
-    re += __shfl_xor_sync(0xffffffffu, re, 2);
-    im += __shfl_xor_sync(0xffffffffu, im, 2);
-    if (ent < nn && part == 0) {
-      double* ar = aug + sp * SPB;
-      double* ai = ar + PLN;
-      ar[r * LDA + c] = re;
-      ai[r * LDA + c] = im;
+    // combine the 4 partial sums of each entry (every lane takes part in the shuffles); FP32: with error-free
+    // additions, part 0 keeps the real sum and part 1 the imaginary one
+    if (f32) {
+#pragma unroll
+      for (int o = 1; o <= 2; o <<= 1) {
+        const float s2r = __shfl_xor_sync(0xffffffffu, sr, o), c2r = __shfl_xor_sync(0xffffffffu, cr, o);
+        const float s2i = __shfl_xor_sync(0xffffffffu, si, o), c2i = __shfl_xor_sync(0xffffffffu, ci, o);
+        df_add(sr, cr, s2r, c2r);
+        df_add(si, ci, s2i, c2i);
+      }
+      const bool odd = part & 1;
+      if (ent < nn && part < 2)
+        invf[sp * 2 * kNsMax * kNsMax + (odd ? kNsMax * kNsMax : 0) + r * kNsMax + c] = (odd ? si : sr) + (odd ? ci : cr);
+    } else {
+      re += __shfl_xor_sync(0xffffffffu, re, 1);
+      im += __shfl_xor_sync(0xffffffffu, im, 1);
+      re += __shfl_xor_sync(0xffffffffu, re, 2);
+      im += __shfl_xor_sync(0xffffffffu, im, 2);
+      if (ent < nn && part == 0) {
+        aug[sp * SPB + r * LDA + c] = re;
+        aug[sp * SPB + PLN + r * LDA + c] = im;
+      }
     }
   }
   __syncthreads();
@@ -1016,6 +1042,37 @@ size_t smem_fast_overlap(const Ctx& c, bool fp64_copy = true, bool given = false
 }
 size_t smem_mgs_warp(const Ctx& c) { return sizeof(double) * 4 * (size_t)c.N * c.M; }   // two walkers
 
+template <int SUMS>
+auto overlap_kernel(int nmax, int rows) {
+  return nmax <= 8 ? k_overlap_fast<4, 8, SUMS> : rows <= 4 ? k_overlap_fast<4, 16, SUMS> : k_overlap_fast<8, 16, SUMS>;
+}
+
+// Form of the FP32 update: an overlap entry per four lanes (kEntries), or register tiles, which fill their
+// 8 x 8 or 16 x 16 lanes' tiles from about a third of the entries on.  Tiles take 60 or 80 registers a thread:
+// where shared memory leaves room for more CTAs than these would, they are held to 48 or 64 (kTiles), else not
+// (kTilesWide).  us per launch, 2829 walkers, launches one after another (before the tiles: one entry per four
+// lanes, 48 or 64 registers, factors read one float at a time):
+//                  before   kEntries  kTiles  kTilesWide
+//   M = 19,  2/1     12.6     12.2      13.3     15.6
+//   M = 64,  2/2     14.4     14.1      17.2     18.6
+//   M = 32,  4/4     16.4     16.0      17.3     20.6
+//   M = 48,  5/4     22.6     22.0      21.7
+//   M = 48,  6/6     26.7     26.5      24.2     27.3
+//   M = 64,  8/8     37.0     37.9      33.0     36.2
+//   M = 128, 8/8     59.4     66.9      60.1     57.4
+//   M = 64,  10/9    72.6     68.6      70.0     76.1
+//   M = 128, 10/10   118.8    112.3     113.7    119.3
+//   M = 64,  11/9    82.3     81.9      80.5
+//   M = 60,  12/12   151      148       90       96
+//   M = 128, 12/12   147      159       153      141
+//   M = 64,  16/3    102.5    103.5     97.2     109.2
+//   M = 128, 16/16   234      227       186      185
+OverlapSums overlap_form(int nu, int nd, size_t smem) {
+  const bool small = std::max(nu, nd) <= 8;
+  if (nu * nu + nd * nd < (small ? 41 : 202)) return kEntries;
+  return (int)(227 * 1024 / (smem + 1024)) >= (small ? 10 : 7) ? kTiles : kTilesWide;
+}
+
 }  // namespace
 
 bool fast_walker_kernels_ok(const Ctx& c) {
@@ -1027,7 +1084,10 @@ cudaError_t prepare_fast_walker_kernels(const Ctx& c) {
   static SmemLimits lim;
   const size_t so = smem_fast_overlap(c), sm = smem_mgs_warp(c);
   cudaError_t e = lim.raise(0, so, [&] {
-    for (auto* f : {k_overlap_fast<4, 8>, k_overlap_fast<4, 16>, k_overlap_fast<8, 16>}) {
+    for (auto* f : {overlap_kernel<kEntries>(8, 1), overlap_kernel<kEntries>(16, 4), overlap_kernel<kEntries>(16, 8),
+                    overlap_kernel<kTiles>(8, 1), overlap_kernel<kTiles>(16, 4), overlap_kernel<kTiles>(16, 8),
+                    overlap_kernel<kTilesWide>(8, 1), overlap_kernel<kTilesWide>(16, 4),
+                    overlap_kernel<kTilesWide>(16, 8)}) {
       cudaError_t r = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)so);
       if (r != cudaSuccess) return r;
     }
@@ -1126,8 +1186,10 @@ cudaError_t launch_overlap_fast(const Ctx& c, const double* src, int mode, cudaS
   // the FP32 update (FP32-pair sums, smaller shared footprint) runs more CTAs of 128 threads
   // per SM, so more LU warps overlap; the FP64 sums of the other modes use 256
   const int nt = a.fp64_copy ? 256 : 128;
-  const cudaError_t e = launch_after(nmax <= 8 ? k_overlap_fast<4, 8> : need <= 4 ? k_overlap_fast<4, 16> : k_overlap_fast<8, 16>,
-                                     c.Nw, nt, sm, s, a);
+  const OverlapSums form = a.fp64_copy || a.O ? kEntries : overlap_form(c.n_up, c.N - c.n_up, sm);
+  auto k = form == kEntries ? overlap_kernel<kEntries>(nmax, need)
+           : form == kTiles ? overlap_kernel<kTiles>(nmax, need) : overlap_kernel<kTilesWide>(nmax, need);
+  const cudaError_t e = launch_after(k, c.Nw, nt, sm, s, a);
   if (e != cudaSuccess) return e;
   // one warp per CTA: the FP64 chain of each warp gets an SM's FP64 pipe to itself
   return with_weights ? launch_after(k_overlap_weights, (c.Nw + 31) / 32, 32, 0, s, a) : cudaSuccess;
