@@ -861,7 +861,11 @@ __global__ void __launch_bounds__(64) k_mgs_reg(double* __restrict__ phi, const 
 // number costs nothing.  One 128-thread CTA per walker; shared memory holds the walker as rows
 // of float2 (re, im) with a stride of N + 1, the upper triangle of S factorised in place, R as
 // float2 and the reciprocals of its diagonal.
-__global__ void __launch_bounds__(128) k_mgs_chol(double* __restrict__ phi, const int* __restrict__ alive,
+// NSM: largest spin block, 8 or 16.  The substitution keeps a row in registers, and a thread's registers
+// bound the CTAs of an SM where the walkers are small.  us per launch, 2829 walkers, a row of 16 / of NSM:
+// M = 19, one electron 20.5 / 16.4; M = 64, 8/8: 51.2 / 43.0; M = 128, 4/4: 47.1 / 36.9.
+template <int NSM>
+__global__ void __launch_bounds__(128, NSM == 8 ? 10 : 8) k_mgs_chol(double* __restrict__ phi, const int* __restrict__ alive,
                                                   double* __restrict__ logO, int M, int N, int n_up,
                                                   int Nw) {
   extern __shared__ __align__(16) unsigned char smc[];
@@ -997,11 +1001,11 @@ __global__ void __launch_bounds__(128) k_mgs_chol(double* __restrict__ phi, cons
     const bool dn = it >= M;
     const int i = dn ? it - M : it, ns = dn ? nd : nu, o = dn ? nu : 0;
     float2* row = X2 + (size_t)i * RS + o;
-    float2 q[kNsMax];   // the row in registers: the R entries are all that is read per product
+    float2 q[NSM];   // the row in registers: the R entries are all that is read per product
 #pragma unroll
-    for (int j = 0; j < kNsMax; ++j) q[j] = j < ns ? row[j] : make_float2(0.f, 0.f);
+    for (int j = 0; j < NSM; ++j) q[j] = j < ns ? row[j] : make_float2(0.f, 0.f);
 #pragma unroll
-    for (int j = 0; j < kNsMax; ++j)
+    for (int j = 0; j < NSM; ++j)
       if (j < ns) {
         float2 x = q[j];
 #pragma unroll
@@ -1014,7 +1018,7 @@ __global__ void __launch_bounds__(128) k_mgs_chol(double* __restrict__ phi, cons
         q[j] = make_float2(x.x * inv, x.y * inv);
       }
 #pragma unroll
-    for (int j = 0; j < kNsMax; ++j)
+    for (int j = 0; j < NSM; ++j)
       if (j < ns) row[j] = q[j];
   }
   __syncthreads();
@@ -1101,7 +1105,9 @@ cudaError_t prepare_fast_walker_kernels(const Ctx& c) {
   const size_t sc = smem_mgs_chol(c);
   if (sc > 200 * 1024) return cudaSuccess;   // too large: the Gram-Schmidt kernels serve
   return lim.raise(2, sc, [&] {
-    return cudaFuncSetAttribute(k_mgs_chol, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sc);
+    cudaError_t r = cudaFuncSetAttribute(k_mgs_chol<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sc);
+    if (r == cudaSuccess) r = cudaFuncSetAttribute(k_mgs_chol<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sc);
+    return r;
   });
 }
 
@@ -1272,7 +1278,7 @@ bool mgs_chol_ok(const Ctx& c) {
 cudaError_t launch_mgs_warp(const Ctx& c, cudaStream_t s, bool update_logO) {
   double* lo = update_logO ? c.logO : nullptr;
   if (c.tune_mgs == 1 && mgs_chol_ok(c)) {
-    k_mgs_chol<<<c.Nw, 128, smem_mgs_chol(c), s>>>(c.phi, c.alive, lo, c.M, c.N, c.n_up, c.Nw);
+    (std::max(c.n_up, c.N - c.n_up) <= 8 ? k_mgs_chol<8> : k_mgs_chol<16>)<<<c.Nw, 128, smem_mgs_chol(c), s>>>(c.phi, c.alive, lo, c.M, c.N, c.n_up, c.Nw);
     return cudaGetLastError();
   }
   if (c.M <= 64 && c.n_up <= 8 && c.N - c.n_up <= 8)
