@@ -840,15 +840,17 @@ cudaError_t gemm_f32_or_split(const TcOperand& A, const TcOperand& B, int Md, in
   if (A.Kp != B.Kp || Md > A.rows || Nd > B.rows) return cudaErrorInvalidValue;
   if (Md <= 0 || Nd <= 0) return cudaSuccess;
   if (so.tri && !vhs_tri_ok(so.M, Nd)) return cudaErrorInvalidValue;
-  if (so.tri || pair_pays(Md, Nd, Md)) {
+  if (so.tri || (A.pairs && pair_pays(Md, Nd, Md))) {
     const int64_t pt = (int64_t)((Md + 2 * BM - 1) / (2 * BM)) * ((Nd + PBN - 1) / PBN);
     return launch_after(k_gemm_bf16x3_tc_pair, 2 * (int)std::min<int64_t>(pt, find_pair_clusters()), QTHREADS,
                         QLayout::SMEM_BYTES, s, A.map_hi, A.map_lo, B.map_hi, B.map_lo, Md, Nd, A.Kp / BK, alpha, C,
                         ldc, so, err, kWaitLimitNs);
   }
-  // at least two 128 x 256 tiles per SM (here: a single row tile): the persistent kernel, whose epilogue
-  // overlaps the next tile's MMAs; B tiles of 256 rows stay inside the operand's padded rows (a multiple of
-  // 256 here)
+  // at least two 128 x 256 tiles per SM (here: a single row tile, X <= 128 or M <= 11): the persistent kernel,
+  // whose epilogue overlaps the next tile's MMAs; B tiles of 256 rows stay inside the operand's padded rows (a
+  // multiple of 256 here).  Force bias, us: this kernel / pairs of SMs / 128 x 128 tiles: X = 128, K = 192,
+  // 39000 walkers 23.7 / 30.4 / 34.5, 60000 34.8 / 44.4 / 51.9, 77000 37.9 / 50.6 / 63.2; X = 90, K = 128, 50000
+  // walkers 21.0 / 31.9 / 35.5; X = 120, K = 512, 60000 walkers 63.0 / 63.6 / 74.6
   if (tc_persistent_ok(Md, Nd, B.rows)) {
     const int64_t tiles = (int64_t)((Md + BM - 1) / BM) * ((Nd + PBN - 1) / PBN);
     const int grid = (int)std::min<int64_t>(tiles, 152);

@@ -256,6 +256,7 @@ struct TcOperand {
   __nv_bfloat16* hi = nullptr;
   __nv_bfloat16* lo = nullptr;
   int rows = 0, Kp = 0;
+  bool pairs = true;   // of an A operand: its products may go to pairs of SMs where these pay
 };
 cudaError_t tc_make_operand(TcOperand& op, __nv_bfloat16* hi, __nv_bfloat16* lo, int rows, int Kp,
                             int box_rows);
