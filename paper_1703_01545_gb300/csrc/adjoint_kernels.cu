@@ -843,15 +843,17 @@ bool adjoint_fits(const Ctx& c) {
 }
 
 cudaError_t prepare_adjoint_kernels(const Ctx& c) {
-  cudaError_t e;
-  if ((e = cudaFuncSetAttribute(k_inv_overlap, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem_inv_overlap(c))) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(k_taylor_rev, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem_taylor_rev(c))) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(k_overlap_rev, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem_overlap_rev(c))) != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_energy_rev, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)smem_energy_rev(c));
+  static SmemLimits limits;
+  auto raise = [&](int slot, auto k, size_t bytes) {
+    return limits.raise(slot, bytes, [&] {
+      return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    });
+  };
+  cudaError_t e = raise(0, k_inv_overlap, smem_inv_overlap(c));
+  if (e == cudaSuccess) e = raise(1, k_taylor_rev, smem_taylor_rev(c));
+  if (e == cudaSuccess) e = raise(2, k_overlap_rev, smem_overlap_rev(c));
+  if (e == cudaSuccess) e = raise(3, k_energy_rev, smem_energy_rev(c));
+  return e;
 }
 
 cudaError_t adj_inv_overlap(const Ctx& c, const double* phi, double* Y, double* logO, double* theta,

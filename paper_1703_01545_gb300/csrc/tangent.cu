@@ -626,15 +626,17 @@ bool tangent_fits(const Ctx& c) {
 }
 
 cudaError_t prepare_tangent_kernels(const Ctx& c) {
-  cudaError_t e;
-  if ((e = cudaFuncSetAttribute(k_overlap_tan, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem_overlap_tan(c))) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(k_taylor_tan, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem_taylor_tan(c))) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(k_mgs_tan, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem_mgs_tan(c))) != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_energy_tan, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)smem_energy_tan(c));
+  static SmemLimits limits;   // only grow: a later, smaller handle leaves the launches of this one valid
+  auto raise = [&](int slot, auto k, size_t bytes) {
+    return limits.raise(slot, bytes, [&] {
+      return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    });
+  };
+  cudaError_t e = raise(0, k_overlap_tan, smem_overlap_tan(c));
+  if (e == cudaSuccess) e = raise(1, k_taylor_tan, smem_taylor_tan(c));
+  if (e == cudaSuccess) e = raise(2, k_mgs_tan, smem_mgs_tan(c));
+  if (e == cudaSuccess) e = raise(3, k_energy_tan, smem_energy_tan(c));
+  return e;
 }
 
 cudaError_t launch_fields_tan(const Ctx& c, const double* fields, cudaStream_t s) {
