@@ -531,8 +531,10 @@ __device__ __forceinline__ void overlap_weights(const FastOvArgs& a, int wk, int
 // Modes as k_overlap: OV_UPDATE takes src as the walker if it lives, else recomputes from Phi
 // (Theta's buffer held the propagated walkers); OV_DET: grid row = determinant, no walker changes.
 // WEIGHTS: the walker's log O and weight too, by a thread beside the solves, instead of k_overlap_weights.
+// Blocks above 8 would take 102 registers a thread and so two CTAs an SM; held to 80, three fit: M = 143, 10/9,
+// 1046 walkers 580 -> 523 us (k_overlap 565), M = 200, 10/10, 795 -> 714 (769), M = 100, 16/15, 804 -> 680 (1119).
 template <int ROWS, int NSM, bool WEIGHTS>
-__global__ void __launch_bounds__(256) k_overlap64(FastOvArgs a) {
+__global__ void __launch_bounds__(256, NSM == 16 ? 3 : 1) k_overlap64(FastOvArgs a) {
   extern __shared__ double smo[];
   const int wk = blockIdx.x, tid = threadIdx.x, M = a.M, N = a.N, NM = N * M;
   const int MP = M + 1, NMP = N * MP;   // columns M + 1 apart: the solves' and sums' reads spread
