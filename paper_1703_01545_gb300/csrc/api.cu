@@ -33,11 +33,27 @@ afqmc_status cuda_fail(Ctx* h, const char* what, cudaError_t e) {
     if (e_ != cudaSuccess) return cuda_fail(h, #call, e_); \
   } while (0)
 
+// Gives back what a handle under setup can do without (the digit forms' scratch); false if it holds none.
+bool drop_scratch(Ctx* h) {
+  if (h->live || !h->ws64.buf) return false;
+  for (void* p : {(void*)h->ws64.buf, (void*)h->e64, (void*)h->ov_O})
+    if (p) cudaFree(p);
+  h->ws64.buf = nullptr;
+  h->ws64.bytes = 0;
+  h->e64 = h->ov_O = nullptr;
+  h->taylor_dig = 0;
+  return true;
+}
+
 template <class T>
 afqmc_status dalloc(Ctx* h, T** p, size_t count) {
   *p = nullptr;
   if (count == 0) count = 1;
   cudaError_t e = cudaMalloc((void**)p, count * sizeof(T));
+  if (e != cudaSuccess && drop_scratch(h)) {
+    cudaGetLastError();
+    e = cudaMalloc((void**)p, count * sizeof(T));
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     return set_err(h, AFQMC_ERR_NOMEM, std::string("cudaMalloc failed: ") + cudaGetErrorString(e));
@@ -690,6 +706,7 @@ afqmc_status afqmc_setup(afqmc_handle* out, const double* h1_in, const double* L
   }
   cleanup_tmp();
 #undef AFQ_SCK
+  h->live = true;
   *out = h;
   return AFQMC_OK;
 }
@@ -717,6 +734,7 @@ afqmc_status afqmc_setup_multidet(afqmc_handle* out, const double* h1, const dou
   afqmc_handle h = nullptr;
   afqmc_status st = afqmc_setup(&h, h1, L, dets, M, X, n_up, n_dn, opt, s);
   if (st != AFQMC_OK) return st;
+  h->live = false;   // the determinants' memory goes before the scratch of the first one's setup
   const int N = h->N, Nw = h->Nw;
   const int64_t NM = (int64_t)N * M;
   auto fail_with = [&](afqmc_status code) {
@@ -771,6 +789,7 @@ afqmc_status afqmc_setup_multidet(afqmc_handle* out, const double* h1, const dou
     cuda_fail(h, "afqmc_setup_multidet", e);
     return fail_with(AFQMC_ERR_CUDA);
   }
+  h->live = true;
   h->n_det = n_det;
   if ((st = overlap_launch(h, nullptr, afq::OV_REFRESH, s)) != AFQMC_OK) return fail_with(st);
   int flags = 0;

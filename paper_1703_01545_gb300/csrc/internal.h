@@ -147,6 +147,7 @@ struct Ctx {
   double* e64_tan = nullptr;  // traces and exchange sums of the tangent local energy in digit form
   double* e64 = nullptr;      // scratch of the FP64 local energy in digit form
   F64Ws ws64;                 // digits of the FP64 contractions' operands (FP64 handles)
+  bool live = false;          // set up: kernels and captured graphs may hold the pointers above
   // tangent mode (tangent.cu): derivative along h1 -> h1 + lambda P, FP64 path only
   bool tangent_on = false;
   double* Bneg = nullptr;     // [M][M]  -dt K / 2 (kept from setup)
