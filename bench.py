@@ -429,8 +429,7 @@ def measure_kernels(afq, A, dA, nw, precision, workload, stream):
                                           "solves 8 M sum N_s^2")
         if A.info().tuned_orthonormalise == 1:
             out["mgs"] = entry(afq.K_MGS, 1, mgs, "alu", f32,
-                               "k_mgs_chol (Cholesky QR: Gram matrix and Q in FP32, FP64 factor "
-                               "and log det)",
+                               "k_mgs_chol (Cholesky QR: Gram matrix, factor and Q in FP32, FP64 log det)",
                                traffic=tr("walker_fast.cu", "mgs_chol"))
         else:
             out["mgs"] = entry(afq.K_MGS, 1, mgs, "alu", f64,
@@ -450,19 +449,21 @@ def measure_kernels(afq, A, dA, nw, precision, workload, stream):
                               "k_energy_B + k_energy_tc (split-BF16 tcgen05 local energy)",
                               mma=emma, traffic=tr("energy_tc.cu", "energy_tc"))
     else:
-        out["force_bias"] = entry(afq.K_FORCE_BIAS, STEPS_PER_BLOCK, fb, "alu", f64,
-                                  "k_gemm_f64_force_bias (FP64)")
-        out["vhs"] = entry(afq.K_VHS, STEPS_PER_BLOCK, vhs, "alu", f64,
-                           "k_gemm_f64_vhs (V_HS, packed symmetric L, FP64)",
-                           traffic=tr("gemm_f64.cu", "vhs_gemm"))
-        out["propagator"] = entry(afq.K_TAYLOR, STEPS_PER_BLOCK, 8.0 * order * M * M * N * nw, "alu",
-                                  f64, "k_taylor (Taylor exponential, FP64; the one-body half steps "
-                                  "run as separate FP64 GEMMs)", traffic=tr("walker_kernels.cu", "taylor_f64"))
+        # FP64: the large contractions as BF16 digit products, 36 for one (small ones on the FP64 pipe)
+        dig = ("MEASURED_PEAKS.json bf16_tflops / 36 digit products", BF16_PEAK_TFLOPS / 36)
+        out["force_bias"] = entry(afq.K_FORCE_BIAS, STEPS_PER_BLOCK, fb, "tensor", dig,
+                                  "k_digits + k_gemm_f64e (small: k_gemm_f64*)")
+        out["vhs"] = entry(afq.K_VHS, STEPS_PER_BLOCK, vhs, "tensor", dig,
+                           "k_digits + k_gemm_f64e (V_HS, packed symmetric L; small: k_gemm_f64*)")
+        out["propagator"] = entry(afq.K_TAYLOR, STEPS_PER_BLOCK, 8.0 * order * M * M * N * nw, "tensor",
+                                  dig, "k_vhs_digits + k_term + k_gemm_f64e (Taylor exponential; small: "
+                                  "k_taylor*; the one-body half steps run as separate contractions)")
         out["overlap"] = entry(afq.K_OVERLAP, STEPS_PER_BLOCK,
-                               (12.0 * M * N2 + 8.0 * N3) * nw, "alu", f64,
-                               "k_overlap (FP64 overlap, Gauss-Jordan inverse, Theta; refresh form)")
+                               (12.0 * M * N2 + 8.0 / 3.0 * N3) * nw, "alu", f64,
+                               "k_overlap64 (FP64 overlap, LU, Theta; blocks above 16: k_overlap; refresh form)")
         out["mgs"] = entry(afq.K_MGS, 1, mgs, "alu", f64, "k_mgs + overlap refresh (FP64)")
-        out["energy"] = entry(afq.K_EXCHANGE, 1, en, "alu", f64, "k_energy (FP64 local energy)")
+        out["energy"] = entry(afq.K_EXCHANGE, 1, en, "tensor", dig,
+                              "k_digits + k_gemm_f64e + k_exchange (small: k_energy)")
     return out
 
 

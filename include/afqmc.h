@@ -50,7 +50,12 @@ enum { AFQMC_PHASELESS = 0, AFQMC_FREE = 1 };
  *   AFQMC_FP64:   every contraction, the determinants and MGS to float64 accuracy; the large
  *                 contractions as error-free sums of BF16 digit products on the tensor cores
  *                 (operands to 62 bits of their row's largest element, one rounding of the
- *                 result), the rest on the FP64 pipe.
+ *                 result), the rest on the FP64 pipe.  That accuracy is relative to the rows'
+ *                 largest elements (K 2^-57 max |a| max |b| at most for a sum of K products, beside
+ *                 its rounding): elements more than 2^9 below their row's largest keep fewer bits
+ *                 than a float64 of their own, which shows where only such elements meet.  A walker with an
+ *                 infinity in it gets NaN from these contractions' energies, series and
+ *                 derivatives, where float64 sums give infinities or NaN; others are unaffected.
  *   AFQMC_BF16X3: every product over the Cholesky index or the orbital basis runs on the
  *                 tensor cores with split operands x = hi + lo (two bf16), three MMAs per
  *                 product (hi*hi + hi*lo + lo*hi) accumulated in FP32: the force bias
