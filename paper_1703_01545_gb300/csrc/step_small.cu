@@ -439,25 +439,27 @@ bool step_small_ok(const Ctx& c) {
 // Whether a call of n steps takes this kernel, of a handle that can.  A few waves of CTAs are latency, where it
 // beats the separate kernels two to four times.  Beyond, it pays per walker and step (the separate kernels:
 // 65 to 75 us plus 46 ns at M = 8, 100 ns at M = 12), so what it stages and draws per launch (a third of a
-// one-step launch) and how many CTAs an SM holds count.  us per step, separate kernels -> this one:
-//   M = 8, X = 24, 2/2 (7 to 9 CTAs an SM)     n = 1        n = 2         n = 5         n = 8
+// one-step launch) and how many CTAs an SM holds (4 by registers, fewer above 56 KB) count.  us per step, separate kernels -> this one:
+//   M = 8, X = 24, 2/2 (23 to 32 KB a CTA)      n = 1        n = 2         n = 5         n = 8
 //     128 walkers                              74 -> 38     70 -> 27      67 -> 19      67 -> 17
 //     1000                                     105 -> 82    101 -> 64     98 -> 54      98 -> 52
 //     2000                                     148 -> 150   144 -> 121    142 -> 106    141 -> 102
 //     8000                                     437 -> 481   434 -> 400    431 -> 358    430 -> 352
 //     40000                                    1832 -> 2244 1826 -> 1885  1825 -> 1689  1825 -> 1654
-//   M = 12, X = 40, 3/3 (2 to 3 CTAs an SM)
+//   M = 12, X = 40, 3/3 (67 to 85 KB)
 //     300                                      94 -> 63     90 -> 51      88 -> 43      87 -> 42
 //     1000                                     177 -> 203   174 -> 176    172 -> 165    171 -> 162
 //     2000                                     296 -> 330   291 -> 288    289 -> 288    288 -> 282
 //     4000                                     486 -> 586   481 -> 517    479 -> 572    478 -> 561
-// Hence one wave for single steps, seven for two steps or fewer than 6 CTAs an SM, and any number else.
+// The populations at which the two meet grow with the number of CTAs whose memory an SM's would hold, up to
+// some 10 (M = 4, X = 8, 1/1, single steps: 2000 walkers), so they are counted in waves of these: one for single
+// steps, seven for two steps or where fewer than 6 fit, and any number else.
 bool step_small_pays(const Ctx& c, int n) {
   if (!step_small_ok(c)) return false;
   const size_t sm = sizeof(double) * (size_t)layout(c.M, c.N, c.X, (int)c.P, std::min(n, kSteps)).total + 2048;
-  const int res = (int)std::min<size_t>(10, (size_t)228 * 1024 / sm);   // (registers allow 10)
-  const int waves = (c.Nw + 152 * res - 1) / (152 * res);
-  return n <= 1 ? waves <= 1 : (n == 2 || res < 6) ? waves <= 7 : true;
+  const int fit = (int)std::min<size_t>(10, (size_t)228 * 1024 / sm);
+  const int waves = (c.Nw + 152 * fit - 1) / (152 * fit);
+  return n <= 1 ? waves <= 1 : (n == 2 || fit < 6) ? waves <= 7 : true;
 }
 
 cudaError_t prepare_step_small(const Ctx& c) {
