@@ -531,10 +531,11 @@ __device__ __forceinline__ void overlap_weights(const FastOvArgs& a, int wk, int
 // Modes as k_overlap: OV_UPDATE takes src as the walker if it lives, else recomputes from Phi
 // (Theta's buffer held the propagated walkers); OV_DET: grid row = determinant, no walker changes.
 // WEIGHTS: the walker's log O and weight too, by a thread beside the solves, instead of k_overlap_weights.
-// Blocks above 8 would take 102 registers a thread and so two CTAs an SM; held to 80, three fit: M = 143, 10/9,
+// Registers for four CTAs an SM (72 a thread would leave three: M = 64, 8/8, 2048 walkers 232 -> 263 us).  Blocks
+// above 8 would take 102 and so two CTAs; held to 80, three fit: M = 143, 10/9,
 // 1046 walkers 580 -> 523 us (k_overlap 565), M = 200, 10/10, 795 -> 714 (769), M = 100, 16/15, 804 -> 680 (1119).
 template <int ROWS, int NSM, bool WEIGHTS>
-__global__ void __launch_bounds__(256, NSM == 16 ? 3 : 1) k_overlap64(FastOvArgs a) {
+__global__ void __launch_bounds__(256, NSM == 16 ? 3 : 4) k_overlap64(FastOvArgs a) {
   extern __shared__ double smo[];
   const int wk = blockIdx.x, tid = threadIdx.x, M = a.M, N = a.N, NM = N * M;
   const int MP = M + 1, NMP = N * MP;   // columns M + 1 apart: the solves' and sums' reads spread
@@ -1054,25 +1055,26 @@ auto overlap_kernel(int nmax, int rows) {
 }
 
 // Form of the FP32 update: an overlap entry per four lanes (kEntries), or register tiles, which fill their
-// 8 x 8 or 16 x 16 lanes' tiles from about a third of the entries on.  Tiles take 60 or 80 registers a thread:
-// where shared memory leaves room for more CTAs than these would, they are held to 48 or 64 (kTiles), else not
+// 8 x 8 or 16 x 16 lanes' tiles from about a third of the entries on.  Tiles would take 72 or 127 registers a
+// thread: where shared memory leaves room for more CTAs than that, they are held to 48 or 64 (kTiles), else not
 // (kTilesWide).  us per launch, 2829 walkers, launches one after another (before the tiles: one entry per four
 // lanes, 48 or 64 registers, factors read one float at a time):
 //                  before   kEntries  kTiles  kTilesWide
-//   M = 19,  2/1     12.6     12.2      13.3     15.6
-//   M = 64,  2/2     14.4     14.1      17.2     18.6
-//   M = 32,  4/4     16.4     16.0      17.3     20.6
+//   M = 19,  2/1     12.6     12.2      13.3
+//   M = 64,  2/2     14.4     14.1      17.2
+//   M = 32,  4/4     16.4     16.0      17.3
 //   M = 48,  5/4     22.6     22.0      21.7
-//   M = 48,  6/6     26.7     26.5      24.2     27.3
-//   M = 64,  8/8     37.0     37.9      33.0     36.2
-//   M = 128, 8/8     59.4     66.9      60.1     57.4
-//   M = 64,  10/9    72.6     68.6      70.0     76.1
-//   M = 128, 10/10   118.8    112.3     113.7    119.3
+//   M = 48,  6/6     26.7     26.5      24.2
+//   M = 128, 7/7     55.1     62.1      54.7     52.0
+//   M = 64,  8/8     37.0     37.9      33.0
+//   M = 128, 8/8     59.4     66.9      60.1     57.1
+//   M = 64,  10/9    72.6     68.6      70.0
+//   M = 128, 10/10   118.8    112.3     113.7
 //   M = 64,  11/9    82.3     81.9      80.5
-//   M = 60,  12/12   151      148       90       96
-//   M = 128, 12/12   147      159       153      141
-//   M = 64,  16/3    102.5    103.5     97.2     109.2
-//   M = 128, 16/16   234      227       186      185
+//   M = 60,  12/12   151      148       90
+//   M = 128, 12/12   147      159       153      142
+//   M = 64,  16/3    102.5    103.5     97.2
+//   M = 128, 16/16   233      227       186      179
 OverlapSums overlap_form(int nu, int nd, size_t smem) {
   const bool small = std::max(nu, nd) <= 8;
   if (nu * nu + nd * nd < (small ? 41 : 202)) return kEntries;
