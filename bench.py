@@ -286,7 +286,8 @@ def step_hbm_report(precision, workload, propagation_variant, ms_per_block):
         return None
     steps = 2 * STEPS_PER_BLOCK            # propagation steps of both systems in one block
     items = [("walker_fast.cu", "overlap_fast_C2", steps), ("gemm_tc.cu", "vhs_tc_C2", steps),
-             ("energy_tc.cu", "energy_tc_C2", 2), ("walker_fast.cu", "mgs_reg_C2", 2)]
+             ("gemm_tc.cu", "force_bias_tc_C2", steps),
+             ("energy_tc.cu", "energy_tc_C2", 2), ("walker_fast.cu", "mgs_chol_C2", 2)]
     if propagation_variant == 3:
         items.insert(0, ("propagate_tc.cu", "propagate_tc_C2", steps))
     counted, total = {}, 0.0

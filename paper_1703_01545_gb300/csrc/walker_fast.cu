@@ -131,9 +131,9 @@ __device__ __forceinline__ void overlap_sums(const float* __restrict__ psih, con
 // One CTA (128 or 256 threads) per walker.  Shared: phi [2][N][M + kPad] in FP64 (not in the
 // FP32 update), per spin the overlap matrix factorised in place (re and im [NSM][LDA], FP64),
 // FP32 copies of phi and of the factors.
-// The FP32 update is bound by instruction issue and latency (41 % of the issue slots at 4 to 5 CTAs an SM):
+// The FP32 update is bound by instruction issue and latency (41 % of the issue slots at 4 CTAs an SM):
 // at M = 128, 16/16 a walker takes 41 k warp instructions, 56 k with one overlap entry a thread and factors
-// read one float at a time.  1024 walkers: 115 -> 88 us; 4096 beside the other system's kernels 373 -> 304 us.
+// read one float at a time.  1024 walkers: 115 -> 79 us; 4096 (CUDA events, alone): 330 -> 251 us.
 // NSM: the larger spin block is at most 8 (both blocks factorised by warp 0, 16 lanes each) or
 // 16 (one warp per block, ROWS = ceil(ns / (32 / ns)) rows per lane, 4 or 8).
 // SUMS: how the FP32 update sums the overlaps, and the registers a thread may take (rules at overlap_form).
