@@ -189,7 +189,9 @@ afqmc_status afqmc_set_walkers(afqmc_handle h, const double* phi, const double* 
  * afqmc_set_walkers this resumes a run from a checkpoint: the state between steps is
  * (Phi, w, t) for a given seed and walker offset, so a handle restored at a step right after
  * an orthonormalisation continues along the same fields as the run that wrote it.  FP64
- * handles then continue bit for bit, because log O and Theta are recomputed from Phi in both.
+ * handles then continue bit for bit, because log O and Theta are recomputed from Phi in both
+ * (large populations of systems of at most 16 orbitals: in calls of the same numbers of steps,
+ * which choose their kernel).
  * Split-precision handles continue within rounding: they lower log O by log det R at
  * orthonormalisation instead.  Asynchronous on the stream.  Errors: ARG (h NULL), CUDA.
  */
