@@ -177,10 +177,6 @@ afqmc_status setup_mixed(Ctx* h, cudaStream_t s) {
   AFQ_CK(afq::prepare_propagate_tcl());
   if ((st = make_operand(h, &h->tc_L, (int)MM, X, s)) != AFQMC_OK) return st;
   if ((st = make_operand(h, &h->tc_Ltil, X, (int)NM, s)) != AFQMC_OK) return st;
-  // Blocks above 16 run the block-wide overlap kernel, whose CTAs hold the SMs for most of a step: beside the
-  // other system of a pair a cluster waits for two free SMs, and the pair run loses what V_HS gains alone
-  // (M = 75, 20/19, 293 walkers, five steps: 11.90 ms with single tiles, 12.24 by pairs; one system 4.26, 4.26).
-  h->tc_L->pairs = h->tc_Ltil->pairs = afq::fast_walker_kernels_ok(*h);
   if ((st = make_operand(h, &h->tc_U, 2 * Nw, X, s)) != AFQMC_OK) return st;
   if ((st = make_operand(h, &h->tc_Theta, 2 * Nw, (int)NM, s)) != AFQMC_OK) return st;
   if ((st = dalloc(h, &h->Avhs32, 2 * (size_t)Nw * MM)) != AFQMC_OK) return st;
@@ -291,6 +287,11 @@ afqmc_status setup_mixed(Ctx* h, cudaStream_t s) {
   }
   if (e == cudaSuccess && h->opt.autotune)
     e = afq::autotune_mixed(*h, h->opt.autotune_cache, s);
+  // Beside the other system of a pair a cluster waits for two free SMs, which kernels of many small CTAs hardly
+  // leave: the block-wide overlap kernel (blocks above 16) and the FP32 propagation.  Pair runs then lose what the
+  // contractions gain alone (M = 75, 20/19, 293 walkers, five steps: 11.90 ms with single tiles, 12.24 by pairs of
+  // SMs; M = 61, 5/3, FP32 propagation, 2177 walkers: 4.61 and 4.85; one system 4.26 and 4.26 at the first).
+  h->tc_L->pairs = h->tc_Ltil->pairs = afq::fast_walker_kernels_ok(*h) && afq::propagation_variant(*h) >= 3;
   if (own) {
     cudaStreamSynchronize(s);
     cudaFree(tmp);
