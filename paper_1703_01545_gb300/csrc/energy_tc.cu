@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(EPTHREADS, 1)
         tile_of(t, m0, n0, rt_all, ct);
         for (int kb = 0; kb < nkb; ++kb, ++g) {
           const int s = g % ESTAGES, use = g / ESTAGES;
-          if (g >= ESTAGES && !mbar_wait(empty0 + 8 * s, (use - 1) & 1, err, wait_ns)) { ok = false; break; }
+          if (g >= ESTAGES && !mbar_poll(empty0 + 8 * s, (use - 1) & 1, err, wait_ns)) { ok = false; break; }
           const uint32_t st = smem_u32(smem + s * Lay::STAGE_BYTES), fb = full0 + 8 * s;
           const int kx = kb * EBK;
           mbar_expect_tx(fb, Lay::STAGE_BYTES);
@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(EPTHREADS, 1)
       }
       // every issued stage must have landed before the CTA may exit
       for (int q = (g > ESTAGES ? g - ESTAGES : 0); q < g; ++q)
-        mbar_wait(full0 + 8 * (q % ESTAGES), (q / ESTAGES) & 1, err, wait_ns);
+        mbar_poll(full0 + 8 * (q % ESTAGES), (q / ESTAGES) & 1, err, wait_ns);
     }
   } else if (warp == EWARPS + 1) {
     if (lane == 0) {
@@ -235,12 +235,12 @@ __global__ void __launch_bounds__(EPTHREADS, 1)
       bool ok = true;
       for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++i) {
         const int b = i & 1;
-        if (i >= 2 && !mbar_wait(tempty0 + 8 * b, ((i >> 1) - 1) & 1, err, wait_ns)) break;
+        if (i >= 2 && !mbar_poll(tempty0 + 8 * b, ((i >> 1) - 1) & 1, err, wait_ns)) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t d = tmem + (uint32_t)(b * EBN);
         for (int kb = 0; kb < nkb; ++kb, ++g) {
           const int s = g % ESTAGES, use = g / ESTAGES;
-          if (!mbar_wait(full0 + 8 * s, use & 1, err, wait_ns)) { ok = false; break; }
+          if (!mbar_poll(full0 + 8 * s, use & 1, err, wait_ns)) { ok = false; break; }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t st = smem_u32(smem + s * Lay::STAGE_BYTES);
           const uint64_t ah = sw128_desc(st), al = sw128_desc(st + Lay::A_BYTES);
@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(EPTHREADS, 1)
       tile_of(t, m0_, n0_, rt_all, ct_t);
       const int b = i & 1;
       float* rb = red + b * (4 * WPT * 2);
-      const bool ok = mbar_wait(tfull0 + 8 * b, (i >> 1) & 1, err, wait_ns);
+      const bool ok = mbar_poll(tfull0 + 8 * b, (i >> 1) & 1, err, wait_ns);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       if (__all_sync(0xffffffffu, ok)) {
         for (int gg = 0; gg < NGH; ++gg) {
@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(EPTHREADS, 1)
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0) mbar_wait(done, 0, err, wait_ns);   // no MMA may still write TMEM
+  if (threadIdx.x == 0) mbar_poll(done, 0, err, wait_ns);   // no MMA may still write TMEM
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0)

@@ -55,6 +55,26 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* er
   return false;
 }
 
+// The same without the time hint: the thread polls.  For the per-tile local energy (k_energy_tc), whose waits are
+// short and whose epilogue does not contend with the issuing warp: M = 194, 10/9, 932 walkers 1255 -> 1221 us.
+__device__ __forceinline__ bool mbar_poll(uint32_t bar, uint32_t parity, int* err, uint64_t limit_ns) {
+  const uint64_t t0 = global_ns();
+  for (uint32_t it = 0;; ++it) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (ok) return true;
+    if ((it & 255u) == 255u && global_ns() - t0 > limit_ns) break;
+  }
+  atomicOr(err, 1);
+  return false;
+}
+
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
