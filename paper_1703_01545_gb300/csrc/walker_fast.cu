@@ -1207,12 +1207,13 @@ cudaError_t launch_overlap_fast(const Ctx& c, const double* src, int mode, cudaS
 
 namespace {
 // Whether a walker's CTA takes its weight too.  The chain of some 250 FP64 instructions holds an SM's FP64 pipe
-// as long for one lane as for 32, so a second launch pays from some CTAs an SM on.  A refresh, us in one kernel
-// / in two (k_overlap before them, in brackets), of 150, 600, 1200 and 2400 walkers:
-//   M = 12, one electron  7.1 / 11.0 (7.6)    9.0 / 11.7 (8.1)    14.1 / 13.7 (15.3)  24.3 / 18.4 (24.9)
-//   M = 16, 2/2           9.0 / 13.4 (22.5)   11.5 / 14.1 (24.6)  18.1 / 17.8 (48.3)  32.3 / 26.6 (76.8)
-//   M = 40, 6/5           22.8 / 27.2 (58.0)  41.7 / 43.2 (77.3)  72.7 / 72.2 (159)   141 / 136 (273)
-bool overlap64_fused(int Nw, int n_det) { return (int64_t)Nw * n_det <= 152 * 4; }
+// as long for one lane as for 32, so a second launch pays from some seven CTAs an SM on.  A refresh, us in one
+// kernel / in two (k_overlap before them, in brackets), of 700, 900, 1100 and 1400 walkers:
+//   M = 16, one electron  10.1 / 12.1 (9.3)   11.4 / 12.7 (10.1)  14.0 / 13.6 (15.9)  16.7 / 15.0 (18.0)
+//   M = 16, 2/2           12.8 / 15.0 (27.0)  14.7 / 15.8 (29.5)  18.0 / 17.7 (48.0)  21.6 / 20.0 (55.5)
+//   M = 40, 6/5           49.9 / 51.0 (89.4)  58.0 / 59.2 (103)   72.4 / 71.8 (159)   102 / 106 (175)
+//   M = 64, 9/8           167 / 180 (203)     191 / 191 (236)     282 / 266 (339)     354 / 347 (392)
+bool overlap64_fused(int Nw, int n_det) { return (int64_t)Nw * n_det <= 152 * 6; }
 
 size_t smem_overlap64(const Ctx& c) {
   const int nmax = std::max(c.n_up, c.N - c.n_up);

@@ -7,7 +7,7 @@ from gpu_util import need_gpu
 from test_gpu_step_small import system
 
 pytestmark = pytest.mark.gpu
-FEW, MANY = 608, 609   # walkers up to which an SM's four CTAs take the weights too
+FEW, MANY = 912, 913   # six walkers' CTAs an SM: up to there they take the weights too
 
 
 # (M, X, n_up, n_dn): one electron, blocks of 8, 9 to 10 and 16 (the kernel's three forms); M above 16, where a
@@ -36,20 +36,20 @@ def test_one_and_two_kernels_give_the_same_bits(M, X, nu, nd, mode):
 
 
 def test_few_determinants_match_many():
-    """The records of a multi-determinant trial: 76 walkers of 8 determinants, against 77."""
+    """The records of a multi-determinant trial: 114 walkers of 8 determinants, against 115."""
     afq = need_gpu()
     M, X, nu, nd, ndet = 17, 5, 3, 2, 8
-    h1, L, trial, phi, w, rng = system(M, X, nu, nd, 77, 3)
+    h1, L, trial, phi, w, rng = system(M, X, nu, nd, 115, 3)
     q = np.linalg.qr(rng.standard_normal((M, M)))[0]
     dets = np.stack([trial + 0.3 * np.concatenate([q[:, k:k + nu], q[:, k:k + nd]], axis=1) for k in range(ndet)])
     out = []
-    for nw in (76, 77):
+    for nw in (114, 115):
         g = afq.System(h1, L, None, nu, nd, dt=0.05, n_walkers=nw, dets=dets, coeffs=1.0 / np.arange(1, ndet + 1))
         g.set_walkers(phi[:nw], w[:nw])
         g.propagate(1, np.full((1, nw, X), 0.3))
         out.append(g.state())
     for k in ("logO", "w", "alive", "phi"):
-        np.testing.assert_array_equal(out[0][k], out[1][k][:76])
+        np.testing.assert_array_equal(out[0][k], out[1][k][:114])
 
 
 def test_few_walkers_take_a_launch_less():
